@@ -1,308 +1,247 @@
-// Depthwise task (groups == C == K), 3x3 or 5x5 (MobileNetV2 and MnasNet, paper Sec. 4.1): memory-bound, CUDA
-// cores.  bf16 NHWC in and out with padded channels, float32 arithmetic, fused bias + activation (+ residual).
+// Depthwise task (groups == C == K), 3x3 or 5x5, stride 1 or 2 (MobileNetV2 and MnasNet, paper Sec. 4.1), CUDA cores.
+// bf16 NHWC in and out with padded channels, float32 arithmetic, fused bias + activation (+ residual).
 //
-// One CTA computes TH x TW output pixels of one image for one block of 64 channels.  Its input
-// patch ((TH-1)*stride+3) x ((TW-1)*stride+3) pixels x 64 channels comes in with a single tiled
-// TMA load (out-of-bounds pixels and channels read as zero, which is the padding), so every input
-// byte is fetched from L2/HBM once per CTA and the nine taps are served from shared memory.
-// A thread owns 8 channels of one output column and walks down the TH rows; threads of a warp
-// cover the 8 channel groups of 4 neighbouring columns, i.e. four contiguous 128-byte pixels.
-// Several CTAs share an SM, so one CTA's load overlaps the arithmetic of the others.  The wait
-// on the load is bounded like every other device-side wait of the library.
+// A CTA keeps one block of up to 72 channels (its taps stay in registers) and works through tiles of output pixels of
+// that block: CTAs that fit the chip at once share the tiles out (persistent, two patch buffers: the next tile's patch is
+// on its way while one is computed).  A tile's input patch comes in with a single tiled TMA load (out-of-bounds pixels and
+// channels read as zero, which is the padding), so every input byte is fetched from L2/HBM once per tile and all taps are
+// served from shared memory.  A thread owns CH channels of COLS neighbouring output columns and walks down TR output rows.
+// It reads and widens every pixel of its window once: an input row feeds all the output rows it overlaps, so
+// NACC = ceil(R / STRIDE) rows of accumulators are alive, and the row loop is unrolled NACC times so that their rotation
+// costs no moves.  The waits on the loads are bounded like every other device-side wait.
+//
+// What bounds it: the instructions of a row step (about 105 per 8 outputs of a thread: 36 packed FMAs, 16 conversions, the
+// clamp and packing, loads, stores) at three warps per scheduler, before memory does.  C 108, 56x56, batch 64, stride 1,
+// cold: 23.4 us = 3.7 TB/s (a thread per column of 8 channels, one tile per CTA: 30.9 us); 5x5, C 288, 14x14, batch 20:
+// 6.6 us (22.0 us with the taps in shared memory).  Packed FMAs: 23.4 against 26.4 us with scalar ones.  Streaming row
+// chunks through a ring instead of whole patches: 29 us; loads straight from global memory: 35 us.
+
 #include <cstring>
 
 #include "common.cuh"
 #include "plan.h"
+#include "sm100_ptx.cuh"
 
 namespace cprune {
 
 struct DwParams {
-    const bf16x8 *w;   // [3][3][c8]
+    const uint32_t *w;     // bf16 pairs [R][R][c2]
     const float *b;
-    const bf16x8 *res;
-    bf16x8 *y;
-    int P, Q, pad, act, R;
-    int c8;            // c_pad / 8
-    int G;             // channel groups (of 8) per CTA: min(8, c8)
-    int TH, TW, IH, IW;
+    const uint32_t *res;
+    uint32_t *y;
+    int P, Q, pad;
+    int c2;                // c_pad / 2: words per pixel
+    int G;                 // channel groups (of 8) per CTA
+    int strips, segs, TR;  // per CTA: column strips (COLS columns each), row segments (TR output rows each)
+    int IH, IW;            // input patch
     int tiles_h, tiles_w, cblocks;
+    int tiles, ctas;       // tiles per channel block (all images), CTAs that share them
+    int dn, dth, dtw;      // `ctas` as images, tile rows, tile columns: the distance between a CTA's tiles
+    int patch_bytes;       // stride of the two patch buffers
     int *status;
 };
 
-__device__ __forceinline__ uint32_t dw_smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// a0 += x.lo * w.lo, a1 += x.hi * w.hi for two packed bf16 pairs: the mixed-precision fused multiply-add takes bf16
-// factors and a float32 addend.  A product of two bf16 values is exact in float32, so the result is the one
-// fmaf(float(x), float(w), a) gives, without the two conversions per pair.
-__device__ __forceinline__ void fma_bf16x2(float &a0, float &a1, uint32_t x, uint32_t w) {
-    asm("{\n\t"
-        ".reg .b16 xl, xh, wl, wh;\n\t"
-        "mov.b32 {xl, xh}, %2;\n\t"
-        "mov.b32 {wl, wh}, %3;\n\t"
-        "fma.rn.f32.bf16 %0, xl, wl, %0;\n\t"
-        "fma.rn.f32.bf16 %1, xh, wh, %1;\n\t"
-        "}"
-        : "+f"(a0), "+f"(a1)
-        : "r"(x), "r"(w));
+// x * w + a on a pair of float32 values: one instruction issues both fused multiply-adds
+__device__ __forceinline__ unsigned long long fma2(unsigned long long x, unsigned long long w, unsigned long long a) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(x), "l"(w), "l"(a));
+    return d;
 }
-
-template <int STRIDE>
-__global__ void __launch_bounds__(256) depthwise3x3_kernel(const __grid_constant__ CUtensorMap tm_x, const DwParams p) {
-    extern __shared__ __align__(128) uint8_t dw_smem[];
-    __shared__ __align__(8) unsigned long long bar;
-    __shared__ int failed;
-
-    pdl_trigger();
-    pdl_wait();
-    int bid = blockIdx.x;
-    const int cb = bid % p.cblocks; bid /= p.cblocks;
-    const int tw = bid % p.tiles_w; bid /= p.tiles_w;
-    const int th = bid % p.tiles_h;
-    const int n = bid / p.tiles_h;
-    const int p0 = th * p.TH, q0 = tw * p.TW;
-    const int G = p.G;
-
-    const uint32_t bar_a = dw_smem_u32(&bar);
-    if (threadIdx.x == 0) {
-        failed = 0;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_a) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        const uint32_t bytes = (uint32_t)(p.IH * p.IW * G * 16);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_a), "r"(bytes) : "memory");
-        asm volatile(
-            "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-            :
-            : "r"(dw_smem_u32(dw_smem)), "l"(&tm_x), "r"(bar_a), "r"(cb * G * 8), "r"(q0 * STRIDE - p.pad),
-              "r"(p0 * STRIDE - p.pad), "r"(n)
-            : "memory");
-    }
-    __syncthreads();   // the barrier is initialised before anyone polls it
-
-    const int cg = threadIdx.x % G;          // channel group within the CTA's channel block
-    const int qq = threadIdx.x / G;          // output column within the tile
-    const int cgg = cb * G + cg;             // channel group within the tensor
-    const bool active = qq < p.TW && q0 + qq < p.Q && cgg < p.c8;
-
-    // filter taps (bf16 pairs, as packed) and bias of this thread's 8 channels (overlaps the load)
-    bf16x8 wq[9];
-    float bf[8];
-    if (active) {
-#pragma unroll
-        for (int t = 0; t < 9; ++t) wq[t] = ldg8(p.w + (size_t)t * p.c8 + cgg);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) bf[i] = __ldg(p.b + cgg * 8 + i);
-    }
-
-    // bounded wait for the patch
-    {
-        uint32_t ok = 0;
-        long long t0 = clock64();
-        while (true) {
-            asm volatile(
-                "{\n\t.reg .pred q;\n\t"
-                "mbarrier.try_wait.parity.shared::cta.b64 q, [%1], 0;\n\t"
-                "selp.u32 %0, 1, 0, q;\n\t}"
-                : "=r"(ok)
-                : "r"(bar_a)
-                : "memory");
-            if (ok) break;
-            if (clock64() - t0 > (1LL << 31)) {
-                atomicOr(p.status, STATUS_TIMEOUT);
-                failed = 1;
-                break;
-            }
-        }
-    }
-    __syncthreads();
-    if (failed) {
-        for (int i = 0; i < 200; ++i) __nanosleep(1000);   // let a late copy land before the CTA's memory goes away
-        return;
-    }
-    if (!active) return;
-
-    const bf16x8 *patch = reinterpret_cast<const bf16x8 *>(dw_smem) + cg;   // [IH][IW][G groups]
-    const size_t out_row = (size_t)p.Q * p.c8;
-    const size_t o0 = (((size_t)n * p.P + p0) * p.Q + q0 + qq) * p.c8 + cgg;
-
-    auto finish = [&](float *acc, int pp) {
-        const size_t o = o0 + (size_t)pp * out_row;
-        if (p.res) {
-            float rf[8];
-            unpack8(ldg8(p.res + o), rf);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) acc[i] += rf[i];
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i] = apply_act(acc[i], p.act);
-        p.y[o] = pack8(acc);
-    };
-
-    if (STRIDE == 1) {
-        // walk down the input rows; each row feeds the three output rows it overlaps.  An input value is used three
-        // times here, so it is converted to float32 once (measured: faster than the mixed-precision form below, and
-        // than packed float32 pairs with rotating accumulators)
-        const int rows = min(p.TH, p.P - p0);       // output rows of this tile
-        float wf[9][8];
-#pragma unroll
-        for (int t = 0; t < 9; ++t) unpack8(wq[t], wf[t]);
-        float a0[8], a1[8], a2[8];                  // accumulators of output rows h-2, h-1, h
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { a0[i] = bf[i]; a1[i] = bf[i]; a2[i] = bf[i]; }
-        for (int h = 0; h < rows + 2; ++h) {
-            const bf16x8 *row = patch + ((size_t)h * p.IW + qq) * G;
-            float x[3][8];
-#pragma unroll
-            for (int s = 0; s < 3; ++s) unpack8(row[s * G], x[s]);
-#pragma unroll
-            for (int s = 0; s < 3; ++s)
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    a0[i] = fmaf(x[s][i], wf[6 + s][i], a0[i]);   // this row is tap row 2 of output row h-2
-                    a1[i] = fmaf(x[s][i], wf[3 + s][i], a1[i]);   // tap row 1 of output row h-1
-                    a2[i] = fmaf(x[s][i], wf[s][i], a2[i]);       // tap row 0 of output row h
-                }
-            if (h >= 2) finish(a0, h - 2);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) { a0[i] = a1[i]; a1[i] = a2[i]; a2[i] = bf[i]; }
-        }
+__device__ __forceinline__ unsigned long long widen2(uint32_t v) {       // the float32 values of a bf16 pair
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(v << 16), "r"(v & 0xffff0000u));
+    return r;
+}
+__device__ __forceinline__ float2 split2(unsigned long long a) {
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(a));
+    return f;
+}
+template <int NW>
+__device__ __forceinline__ void load_words(const uint32_t *p, uint32_t *v) {
+    if constexpr (NW == 2) {
+        const uint2 t = *reinterpret_cast<const uint2 *>(p);
+        v[0] = t.x; v[1] = t.y;
     } else {
-        // an input value is used once per output row here: the mixed-precision FMA saves its conversion
-        for (int pp = 0; pp < p.TH && p0 + pp < p.P; ++pp) {
-            float acc[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) acc[i] = bf[i];
-#pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                const bf16x8 *row = patch + ((size_t)(pp * STRIDE + r) * p.IW + qq * STRIDE) * G;
-#pragma unroll
-                for (int s = 0; s < 3; ++s) {
-                    const bf16x8 x = row[s * G];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) fma_bf16x2(acc[2 * j], acc[2 * j + 1], x.w[j], wq[r * 3 + s].w[j]);
-                }
-            }
-            finish(acc, pp);
-        }
+        v[0] = *p;
     }
 }
 
-// R x R taps for filters too large to keep in registers (5x5): the same tiling and patch load as above; the CTA's
-// filter taps are converted to float32 in shared memory once, and a thread (8 channels of one output column) walks
-// down the tile's rows, reading every tap of its window from the patch.
-template <int STRIDE, int R>
-__global__ void __launch_bounds__(256) depthwise_rxr_kernel(const __grid_constant__ CUtensorMap tm_x, const DwParams p) {
+template <int R, int STRIDE, int CH, int COLS, int ACT>
+__global__ void __launch_bounds__(256, 2) depthwise_kernel(const __grid_constant__ CUtensorMap tm_x, const DwParams p) {
     extern __shared__ __align__(128) uint8_t dw_smem[];
-    __shared__ __align__(8) unsigned long long bar;
-    __shared__ int failed;
-    __shared__ __align__(16) float wsm[R * R][9][8];      // [tap][channel group of the CTA][channel]
+    __shared__ __align__(8) unsigned long long bars[2];
+    __shared__ int abort_word;
+    constexpr int NACC = (R + STRIDE - 1) / STRIDE;      // output rows one input row can belong to
+    constexpr int NPX = (COLS - 1) * STRIDE + R;         // input pixels per row of a thread's window
+    constexpr int NW = CH / 2;                           // words (channel pairs) per pixel
 
     pdl_trigger();
-    pdl_wait();
-    int bid = blockIdx.x;
-    const int cb = bid % p.cblocks; bid /= p.cblocks;
-    const int tw = bid % p.tiles_w; bid /= p.tiles_w;
-    const int th = bid % p.tiles_h;
-    const int n = bid / p.tiles_h;
-    const int p0 = th * p.TH, q0 = tw * p.TW;
     const int G = p.G;
-
-    const uint32_t bar_a = dw_smem_u32(&bar);
-    if (threadIdx.x == 0) {
-        failed = 0;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_a) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        const uint32_t bytes = (uint32_t)(p.IH * p.IW * G * 16);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_a), "r"(bytes) : "memory");
-        asm volatile(
-            "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-            :
-            : "r"(dw_smem_u32(dw_smem)), "l"(&tm_x), "r"(bar_a), "r"(cb * G * 8), "r"(q0 * STRIDE - p.pad),
-              "r"(p0 * STRIDE - p.pad), "r"(n)
-            : "memory");
-    }
-    // filter taps of the CTA's channel groups (overlaps the load); groups beyond the tensor read as zero
-    for (int e = threadIdx.x; e < R * R * G; e += blockDim.x) {
-        const int t = e / G, g = e - t * G;
-        float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (cb * G + g < p.c8) unpack8(ldg8(p.w + (size_t)t * p.c8 + cb * G + g), f);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) wsm[t][g][i] = f[i];
-    }
-    __syncthreads();   // the barrier is initialised and the taps are in place before anyone goes on
-
-    const int cg = threadIdx.x % G;
-    const int qq = threadIdx.x / G;
-    const int cgg = cb * G + cg;
-    const bool active = qq < p.TW && q0 + qq < p.Q && cgg < p.c8;
-    float bf[8];
-    if (active) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) bf[i] = __ldg(p.b + cgg * 8 + i);
-    }
+    const int first = blockIdx.x / p.cblocks, cb = blockIdx.x - first * p.cblocks;
+    int n, th, tw;
     {
-        uint32_t ok = 0;
-        long long t0 = clock64();
-        while (true) {
-            asm volatile(
-                "{\n\t.reg .pred q;\n\t"
-                "mbarrier.try_wait.parity.shared::cta.b64 q, [%1], 0;\n\t"
-                "selp.u32 %0, 1, 0, q;\n\t}"
-                : "=r"(ok)
-                : "r"(bar_a)
-                : "memory");
-            if (ok) break;
-            if (clock64() - t0 > (1LL << 31)) {
-                atomicOr(p.status, STATUS_TIMEOUT);
-                failed = 1;
-                break;
-            }
-        }
+        const int r = first / p.tiles_w;
+        tw = first - r * p.tiles_w;
+        n = r / p.tiles_h;
+        th = r - n * p.tiles_h;
     }
-    __syncthreads();
-    if (failed) {
-        for (int i = 0; i < 200; ++i) __nanosleep(1000);   // let a late copy land before the CTA's memory goes away
-        return;
+    auto advance = [&](int &n_, int &th_, int &tw_) {
+        tw_ += p.dtw;
+        if (tw_ >= p.tiles_w) { tw_ -= p.tiles_w; ++th_; }
+        th_ += p.dth;
+        if (th_ >= p.tiles_h) { th_ -= p.tiles_h; ++n_; }
+        n_ += p.dn;
+    };
+    int ln = n, lth = th, ltw = tw, ltile = first;       // next tile to load (thread 0)
+    auto load_tile = [&](int buf) {
+        const uint32_t bar = smem_u32(&bars[buf]);
+        mbar_expect_tx(bar, (uint32_t)(p.IH * p.IW * G * 16));
+        tma_load_4d(smem_u32(dw_smem) + (uint32_t)(buf * p.patch_bytes), &tm_x, bar, cb * G * 8,
+                    ltw * p.strips * COLS * STRIDE - p.pad, lth * p.segs * p.TR * STRIDE - p.pad, ln);
+        advance(ln, lth, ltw);
+        ltile += p.ctas;
+    };
+    if (threadIdx.x == 0) {
+        abort_word = 0;
+        mbar_init(smem_u32(&bars[0]), 1);
+        mbar_init(smem_u32(&bars[1]), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        pdl_wait();
+        load_tile(0);
+        if (ltile < p.tiles) load_tile(1);
     }
-    if (!active) return;
+    __syncthreads();   // the barriers are initialised before anyone polls them
 
-    const bf16x8 *patch = reinterpret_cast<const bf16x8 *>(dw_smem) + cg;   // [IH][IW][G groups]
-    const size_t out_row = (size_t)p.Q * p.c8;
-    const size_t o0 = (((size_t)n * p.P + p0) * p.Q + q0 + qq) * p.c8 + cgg;
-    for (int pp = 0; pp < p.TH && p0 + pp < p.P; ++pp) {
-        float acc[8];
+    const int lanes = G * 8 / CH;                        // threads per strip: neighbouring channels
+    const int sc = threadIdx.x / lanes;
+    const int cq = threadIdx.x - sc * lanes;
+    const int seg = sc / p.strips, strip = sc - seg * p.strips;
+    const int word = cb * G * 4 + cq * NW;               // first channel pair of this thread
+    const bool in_tile = seg < p.segs && word < p.c2;
+
+    // taps and bias were written when the task was packed, not by the preceding kernel (overlaps the load)
+    unsigned long long wf[R][R][NW], bf[NW];
+    if (in_tile) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i] = bf[i];
+        for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const bf16x8 *row = patch + ((size_t)(pp * STRIDE + r) * p.IW + qq * STRIDE) * G;
+            for (int s = 0; s < R; ++s) {
+                uint32_t t[NW];
+                load_words<NW>(p.w + (r * R + s) * p.c2 + word, t);
 #pragma unroll
-            for (int s2 = 0; s2 < R; ++s2) {
-                float xf[8];
-                unpack8(row[s2 * G], xf);
-                const float4 w0 = *reinterpret_cast<const float4 *>(&wsm[r * R + s2][cg][0]);
-                const float4 w1 = *reinterpret_cast<const float4 *>(&wsm[r * R + s2][cg][4]);
-                acc[0] = fmaf(xf[0], w0.x, acc[0]); acc[1] = fmaf(xf[1], w0.y, acc[1]);
-                acc[2] = fmaf(xf[2], w0.z, acc[2]); acc[3] = fmaf(xf[3], w0.w, acc[3]);
-                acc[4] = fmaf(xf[4], w1.x, acc[4]); acc[5] = fmaf(xf[5], w1.y, acc[5]);
-                acc[6] = fmaf(xf[6], w1.z, acc[6]); acc[7] = fmaf(xf[7], w1.w, acc[7]);
+                for (int k = 0; k < NW; ++k) wf[r][s][k] = widen2(t[k]);
+            }
+#pragma unroll
+        for (int k = 0; k < NW; ++k) bf[k] = *reinterpret_cast<const unsigned long long *>(p.b + 2 * (word + k));
+    }
+
+    const bool has_res = p.res != nullptr;
+    if (has_res) pdl_wait();                             // the residual is the result of an earlier kernel of the chain
+
+    const __nv_bfloat162 zero2 = __floats2bfloat162_rn(0.f, 0.f), six2 = __floats2bfloat162_rn(6.f, 6.f);
+    const uint32_t pix = (uint32_t)G * 4u;               // words per pixel of the patch
+    const uint32_t row_words = (uint32_t)p.IW * pix;
+    const uint32_t in0 = (uint32_t)(seg * p.TR * STRIDE) * row_words + (uint32_t)(strip * COLS * STRIDE) * pix + cq * NW;
+    const uint32_t out_step = (uint32_t)p.Q * (uint32_t)p.c2;
+    uint32_t buf = 0, phase = 0;
+    for (int tile = first; tile < p.tiles; tile += p.ctas) {
+        const bool ok = mbar_wait(smem_u32(&bars[buf]), phase, &abort_word, p.status);
+        const int ps = (th * p.segs + seg) * p.TR, qs = (tw * p.strips + strip) * COLS;
+        const int rows = min(p.TR, p.P - ps);
+        if (ok && in_tile && rows > 0 && qs < p.Q) {
+            const uint32_t *in = reinterpret_cast<const uint32_t *>(dw_smem + buf * p.patch_bytes) + in0;
+            unsigned long long acc[NACC][COLS][NW];
+#pragma unroll
+            for (int a = 0; a < NACC; ++a)
+#pragma unroll
+                for (int c = 0; c < COLS; ++c)
+#pragma unroll
+                    for (int k = 0; k < NW; ++k) acc[a][c][k] = 0ull;
+            const size_t o0 = (((size_t)n * p.P + ps) * p.Q + qs) * p.c2 + word;
+            uint32_t *dst = p.y + o0;
+            const uint32_t *rsrc = p.res + o0;
+            const int steps = rows + NACC - 1;           // STRIDE input rows each; step t completes output row t - NACC + 1
+            for (int t0 = 0; t0 < steps; t0 += NACC) {
+#pragma unroll
+                for (int u = 0; u < NACC; ++u) {
+                    const int t = t0 + u;
+                    if (t >= steps) break;
+#pragma unroll
+                    for (int j = 0; j < STRIDE; ++j) {
+                        if (j > 0 && t * STRIDE + j >= (rows - 1) * STRIDE + R) break;      // below the last row the segment needs
+#pragma unroll
+                        for (int k = 0; k < NPX; ++k) {
+                            uint32_t raw[NW];
+                            unsigned long long xv[NW];
+                            load_words<NW>(in + k * pix, raw);
+#pragma unroll
+                            for (int q = 0; q < NW; ++q) xv[q] = widen2(raw[q]);
+#pragma unroll
+                            for (int a = 0; a < NACC; ++a) {
+                                const int r = a * STRIDE + j;    // this input row is tap row r of output row t - a
+                                if (r < R) {
+#pragma unroll
+                                    for (int c = 0; c < COLS; ++c) {
+                                        const int s = k - c * STRIDE;
+                                        if (s >= 0 && s < R) {
+#pragma unroll
+                                            for (int q = 0; q < NW; ++q) {
+                                                unsigned long long &d = acc[(u - a + NACC) % NACC][c][q];
+                                                d = fma2(xv[q], wf[r][s][q], (r == 0 && s == 0) ? bf[q] : d);    // an output row starts from the bias
+                                            }
+                                        }
+                                    }
+                                }
+                            }
+                        }
+                        in += row_words;
+                        if (j == 0 && t >= NACC - 1) {
+                            // output row t - NACC + 1 is complete (R is odd: its last tap row is the first row of a step)
+                            unsigned long long (&fin)[COLS][NW] = acc[(u + 1) % NACC];
+#pragma unroll
+                            for (int c = 0; c < COLS; ++c) {
+                                if (c == 0 || qs + c < p.Q) {
+                                    uint32_t o[NW];
+#pragma unroll
+                                    for (int q = 0; q < NW; ++q) {
+                                        float2 f = split2(fin[c][q]);
+                                        if (has_res) {
+                                            const uint32_t rv = rsrc[(uint32_t)c * p.c2 + q];
+                                            f.x += __uint_as_float(rv << 16);
+                                            f.y += __uint_as_float(rv & 0xffff0000u);
+                                        }
+                                        // 0 and 6 are bf16 values, so the clamp commutes with the rounding
+                                        __nv_bfloat162 v = __floats2bfloat162_rn(f.x, f.y);
+                                        if (ACT != CPRUNE_ACT_NONE) v = __hmax2(v, zero2);
+                                        if (ACT == CPRUNE_ACT_RELU6) v = __hmin2(v, six2);
+                                        o[q] = *reinterpret_cast<const uint32_t *>(&v);
+                                    }
+                                    uint32_t *d = dst + (uint32_t)c * p.c2;
+                                    if constexpr (NW == 2) *reinterpret_cast<uint2 *>(d) = make_uint2(o[0], o[1]);
+                                    else *d = o[0];
+                                }
+                            }
+                            dst += out_step;
+                            rsrc += out_step;
+                        }
+                    }
+                }
             }
         }
-        const size_t o = o0 + (size_t)pp * out_row;
-        if (p.res) {
-            float rf[8];
-            unpack8(ldg8(p.res + o), rf);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) acc[i] += rf[i];
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i] = apply_act(acc[i], p.act);
-        p.y[o] = pack8(acc);
+        advance(n, th, tw);
+        if (__syncthreads_or(ok ? 0 : 1)) break;         // the buffer has been read by everyone (or somebody gave up)
+        if (threadIdx.x == 0 && ltile < p.tiles) load_tile(buf);
+        buf ^= 1u;
+        if (buf == 0) phase ^= 1u;
+    }
+    if (*(volatile int *)&abort_word) {
+        for (int i = 0; i < 200; ++i) __nanosleep(1000);   // let a late copy land before the CTA's memory goes away
     }
 }
 
-// Tile of output pixels per CTA and channel groups per CTA.
-// Channel groups (of 8 channels) per CTA: between 4 and 9, whichever wastes the fewest lanes in
-// the last channel block (c_pad/8 = 18 -> 9, 14 -> 7, 4 -> 4); larger wins ties.
+// Channel groups (of 8 channels) per CTA: between 4 and 9, whichever wastes the fewest lanes in the last channel block
+// (c_pad/8 = 18 -> 9, 14 -> 7, 4 -> 4); larger wins ties.
 int depthwise_groups(int c8) {
     if (c8 <= 9) return c8;
     int best = 8;
@@ -314,34 +253,115 @@ int depthwise_groups(int c8) {
     return best;
 }
 
-// Tile of output pixels per CTA and channel groups per CTA.
-static void dw_tile(const cprune_plan_info &i, int *TH, int *TW, int *G) {
+constexpr int DW_MAX_PATCH = 64 * 1024;
+
+// Channels and columns per thread.  3x3: the nine taps of four channels fit the registers beside the accumulators (two or
+// eight channels, one or four columns measured 3 to 40 % slower); 5x5: those of two channels.
+static void dw_config(int R, int *ch, int *cols) { *ch = R == 3 ? 4 : 2; *cols = 2; }
+
+// Chooses the tile (column strips x row segments x rows per segment) and the number of CTAs.  The model prices an SM's share
+// of the tiles: the row steps of its warps (dearer when few warps share the SM or few CTAs cover each other's loads) and the
+// patch bytes, plus a start-up per resident warp.  Its constants were fitted to a sweep of 55 to 420 tilings of 35 layers
+// (batch 1 to 64) on B200; the tiling it picks is within 3 % of the best of the sweep on average, 8 % at worst.
+cprune_status plan_depthwise(cprune_plan *plan) {
+    const cprune_plan_info &i = plan->info;
+    DwTiling &d = plan->dw;
+    int ch, cols;
+    dw_config(i.R, &ch, &cols);
+    const bool s1 = i.stride == 1;
+    const double step_cycles = s1 ? 0.37 * i.R * i.R + 34.3 : 0.5 * i.R * i.R + 41.7;
+    const double step_extra = s1 ? 1.0 : 0.54, warps_needed = s1 ? 12.0 : 15.7, load_rate = s1 ? 50.0 : 100.0;
+    const double warp_start = s1 ? 268.0 : 130.0, average_share = s1 ? 0.217 : 0.31, cover = s1 ? 0.055 : 0.09;
     const int c8 = i.c_pad / 8;
-    *G = depthwise_groups(c8);
-    int tw = 112 / *G;                      // about 112 threads per CTA: small patches, several CTAs per SM
-    if (i.stride == 2 && tw > 28) tw = 28;  // keeps the input patch small
-    *TW = i.Q < tw ? i.Q : tw;
-    int th = i.stride == 1 ? 14 : (*TW <= 14 ? 7 : 4);
-    if (i.R > 3 && i.stride == 2 && *TW > 14) *TW = 14;      // larger filters: keep the input patch within shared memory
-    *TH = i.P < th ? i.P : th;
+    d.G = depthwise_groups(c8);
+    d.cblocks = (c8 + d.G - 1) / d.G;
+    const int lanes = d.G * 8 / ch;
+    const int nacc = (i.R + i.stride - 1) / i.stride;
+    const int all_strips = (i.Q + cols - 1) / cols;
+    double best = 1e30;
+    for (int ns = 1; ns <= all_strips && ns * lanes <= 256; ++ns) {
+        const int tiles_w = (all_strips + ns - 1) / ns;
+        if (ns > 1 && tiles_w == (all_strips + ns - 2) / (ns - 1)) continue;      // narrower tiles, as many of them
+        const int IW = (ns * cols - 1) * i.stride + i.R;
+        if (IW > 256) break;
+        for (int tr = 1; tr <= i.P && tr <= 28; ++tr) {
+            for (int ng = 1; ng * ns * lanes <= 256; ++ng) {
+                if (ng > 1 && (ng - 1) * tr >= i.P) break;
+                const int IH = (ng * tr - 1) * i.stride + i.R;
+                const int patch = round_up(IH * IW * d.G * 16, 128);
+                if (IH > 256 || patch > DW_MAX_PATCH) break;
+                const int tiles_h = (i.P + ng * tr - 1) / (ng * tr);
+                const long long tiles = (long long)i.N * tiles_w * tiles_h;
+                const int warps = (ng * ns * lanes + 31) / 32;
+                int resident = 220 * 1024 / (2 * patch + 1024);
+                if (resident > 18 / warps) resident = 18 / warps;                // by registers
+                if (resident < 1) continue;
+                long long ctas = 148LL * resident / d.cblocks;
+                if (ctas < 1) ctas = 1;
+                if (ctas > tiles) ctas = tiles;
+                const double on_sm = (double)ceil_div(ctas * d.cblocks, 148), active = on_sm * warps;
+                const double share = (double)ceil_div(tiles, ctas) * on_sm * (1.0 - average_share) + (double)tiles * d.cblocks / 148.0 * average_share;
+                const double hide = (active < warps_needed ? warps_needed / active : 1.0) * (1.0 + cover / on_sm);
+                const double work = share * warps * (tr + nacc - 1 + step_extra) * step_cycles * (s1 ? 1.0 : 0.85) * hide;
+                const double load = share * patch / load_rate;
+                const double t = (work > load ? work + 0.3 * load : load + 0.3 * work) + active * warp_start;
+                if (t < best) {
+                    best = t;
+                    d.strips = ns; d.segs = ng; d.TR = tr; d.IH = IH; d.IW = IW; d.tiles_w = tiles_w; d.tiles_h = tiles_h;
+                    d.tiles = tiles; d.ctas = (int)ctas; d.patch_bytes = patch;
+                }
+            }
+        }
+    }
+    return best < 1e30 ? CPRUNE_OK : CPRUNE_ERR_UNSUPPORTED;
+}
+
+template <int R, int STRIDE, int CH, int COLS, int ACT>
+static cprune_status launch_dw_act(const CUtensorMap &tm, const DwParams &p, unsigned blocks, cudaStream_t st) {
+    const int threads = (p.strips * p.segs * (p.G * 8 / CH) + 31) / 32 * 32;
+    const size_t smem = (size_t)p.patch_bytes * (p.tiles > p.ctas ? 2 : 1);
+    static std::mutex attr_mu;
+    static bool attr_set[64] = {false};    // the shared-memory limit of a kernel is a per-device attribute
+    {
+        int dev = 0;
+        CPRUNE_CUDA_CHECK(cudaGetDevice(&dev));
+        if (dev < 0 || dev >= 64) return CPRUNE_ERR_UNSUPPORTED;
+        std::lock_guard<std::mutex> lock(attr_mu);
+        if (!attr_set[dev]) {
+            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(depthwise_kernel<R, STRIDE, CH, COLS, ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * DW_MAX_PATCH));
+            attr_set[dev] = true;
+        }
+    }
+    CPRUNE_CUDA_CHECK(launch_chained(depthwise_kernel<R, STRIDE, CH, COLS, ACT>, dim3(blocks), dim3(threads), smem, st, tm, p));
+    CPRUNE_LAUNCH_CHECK("depthwise kernel");
+    return CPRUNE_OK;
+}
+
+template <int R, int STRIDE, int CH, int COLS>
+static cprune_status launch_dw(int act, const CUtensorMap &tm, const DwParams &p, unsigned blocks, cudaStream_t st) {
+    if (act == CPRUNE_ACT_NONE) return launch_dw_act<R, STRIDE, CH, COLS, CPRUNE_ACT_NONE>(tm, p, blocks, st);
+    if (act == CPRUNE_ACT_RELU) return launch_dw_act<R, STRIDE, CH, COLS, CPRUNE_ACT_RELU>(tm, p, blocks, st);
+    return launch_dw_act<R, STRIDE, CH, COLS, CPRUNE_ACT_RELU6>(tm, p, blocks, st);
 }
 
 cprune_status launch_depthwise(cprune_plan *plan, const void *x, const void *w, const float *b, const void *res,
                                void *y, cudaStream_t st) {
     const cprune_plan_info &i = plan->info;
+    const DwTiling &d = plan->dw;
     DwParams p;
-    p.w = (const bf16x8 *)w;
+    p.w = (const uint32_t *)w;
     p.b = b;
-    p.res = (const bf16x8 *)res;
-    p.y = (bf16x8 *)y;
-    p.P = i.P; p.Q = i.Q; p.pad = i.pad; p.act = plan->opts.activation; p.R = i.R;
-    p.c8 = i.c_pad / 8;
-    dw_tile(i, &p.TH, &p.TW, &p.G);
-    p.IH = (p.TH - 1) * i.stride + i.R;
-    p.IW = (p.TW - 1) * i.stride + i.S;
-    p.tiles_h = (i.P + p.TH - 1) / p.TH;
-    p.tiles_w = (i.Q + p.TW - 1) / p.TW;
-    p.cblocks = (p.c8 + p.G - 1) / p.G;
+    p.res = (const uint32_t *)res;
+    p.y = (uint32_t *)y;
+    p.P = i.P; p.Q = i.Q; p.pad = i.pad;
+    const int act = plan->opts.activation;
+    p.c2 = i.c_pad / 2;
+    p.G = d.G; p.strips = d.strips; p.segs = d.segs; p.TR = d.TR; p.IH = d.IH; p.IW = d.IW;
+    p.tiles_h = d.tiles_h; p.tiles_w = d.tiles_w; p.cblocks = d.cblocks;
+    p.tiles = (int)d.tiles; p.ctas = d.ctas; p.patch_bytes = d.patch_bytes;
+    p.dn = d.ctas / (d.tiles_h * d.tiles_w);
+    p.dth = (d.ctas - p.dn * d.tiles_h * d.tiles_w) / d.tiles_w;
+    p.dtw = d.ctas - (p.dn * d.tiles_h + p.dth) * d.tiles_w;
     p.status = device_status_word();
     if (!p.status) return cuda_fail(cudaGetLastError(), "status word");
     CUtensorMap tm;
@@ -359,37 +379,10 @@ cprune_status launch_depthwise(cprune_plan *plan, const void *x, const void *w, 
         }
         std::memcpy(&tm, &plan->tm_a, sizeof(CUtensorMap));
     }
-    const long long blocks = (long long)i.N * p.tiles_h * p.tiles_w * p.cblocks;
-    if (blocks == 0) return CPRUNE_OK;
-    if (blocks > 0x7fffffffLL || p.IW > 256 || p.IH > 256) return CPRUNE_ERR_UNSUPPORTED;
-    const int smem = p.IH * p.IW * p.G * 16;
-    static std::mutex attr_mu;
-    static int attr_set[64] = {0};     // the shared-memory limit of a kernel is a per-device attribute
-    {
-        int dev = 0;
-        CPRUNE_CUDA_CHECK(cudaGetDevice(&dev));
-        if (dev < 0 || dev >= 64) return CPRUNE_ERR_UNSUPPORTED;
-        std::lock_guard<std::mutex> lock(attr_mu);
-        if (!attr_set[dev]) {
-            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(depthwise3x3_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
-            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(depthwise3x3_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
-            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(depthwise_rxr_kernel<1, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
-            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(depthwise_rxr_kernel<2, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
-            attr_set[dev] = 1;
-        }
-    }
-    if (smem > 100 * 1024) return CPRUNE_ERR_UNSUPPORTED;
-    const int threads = ((p.TW * p.G + 31) / 32) * 32;
-    if (i.R == 5) {
-        if (i.stride == 1) CPRUNE_CUDA_CHECK(launch_chained(depthwise_rxr_kernel<1, 5>, dim3((unsigned)blocks), dim3(threads), (size_t)smem, st, tm, p));
-        else CPRUNE_CUDA_CHECK(launch_chained(depthwise_rxr_kernel<2, 5>, dim3((unsigned)blocks), dim3(threads), (size_t)smem, st, tm, p));
-    } else if (i.stride == 1) {
-        CPRUNE_CUDA_CHECK(launch_chained(depthwise3x3_kernel<1>, dim3((unsigned)blocks), dim3(threads), (size_t)smem, st, tm, p));
-    } else {
-        CPRUNE_CUDA_CHECK(launch_chained(depthwise3x3_kernel<2>, dim3((unsigned)blocks), dim3(threads), (size_t)smem, st, tm, p));
-    }
-    CPRUNE_LAUNCH_CHECK("depthwise kernel");
-    return CPRUNE_OK;
+    if (d.tiles > 0x3fffffffLL) return CPRUNE_ERR_UNSUPPORTED;
+    const long long blocks = (long long)d.ctas * d.cblocks;
+    if (i.R == 3) return i.stride == 1 ? launch_dw<3, 1, 4, 2>(act, tm, p, (unsigned)blocks, st) : launch_dw<3, 2, 4, 2>(act, tm, p, (unsigned)blocks, st);
+    return i.stride == 1 ? launch_dw<5, 1, 2, 2>(act, tm, p, (unsigned)blocks, st) : launch_dw<5, 2, 2, 2>(act, tm, p, (unsigned)blocks, st);
 }
 
 }  // namespace cprune

@@ -53,10 +53,10 @@ static cprune_status build_plan(const PlanKey &key, cprune_plan **out) {
     if (depthwise) {
         if (family != CPRUNE_KERNEL_AUTO && family != CPRUNE_KERNEL_DEPTHWISE) st = CPRUNE_ERR_UNSUPPORTED;
         family = CPRUNE_KERNEL_DEPTHWISE;
-        // output pixels per CTA (rows x columns) are chosen at launch, see depthwise.cu
         i.tile_m = i.stride == 1 ? 14 : 4;
         i.tile_n = 14;
         i.tile_k = 8;
+        if (st == CPRUNE_OK) st = plan_depthwise(pl);
     } else {
         if (family == CPRUNE_KERNEL_DEPTHWISE) st = CPRUNE_ERR_UNSUPPORTED;
         // 3-channel stems run on the tensor cores too when their filters fit the 128-row side

@@ -20,6 +20,17 @@ struct PatchTiling {
     int dense_pitch;                        // dense staging: bytes between neighbouring pixels in the staging buffer
 };
 
+// Tiling of the depthwise kernel (depthwise.cu)
+struct DwTiling {
+    int G, cblocks;              // channel groups (of 8) per CTA, CTAs along the channels
+    int strips, segs, TR;        // tile: column strips x row segments of TR output rows
+    int IH, IW;                  // input patch
+    int tiles_h, tiles_w;
+    long long tiles;             // tiles of one channel block, all images
+    int ctas;                    // CTAs that share them
+    int patch_bytes;
+};
+
 struct cprune_plan {
     cprune_plan_info info;
     cprune_task_opts opts;
@@ -50,6 +61,7 @@ struct cprune_plan {
     int narrow = 0;                 // patch kernel on a regrouped 16-channel input (stems with few channels)
     size_t pre_bytes = 0;           // regrouped input in the workspace
     PatchTiling pt = {};
+    DwTiling dw = {};
     double est_us = 0.0;            // the planner's cost-model estimate of the task's time
 };
 
@@ -58,11 +70,12 @@ namespace cprune {
 // CUDA-core direct convolution, any dense shape (fallback family and small-C stems)
 cprune_status launch_conv_direct(const cprune_plan *plan, const void *x, const void *w, const float *b,
                                  const void *res, void *y, cudaStream_t st);
-// depthwise 3x3
+// depthwise 3x3 and 5x5
 cprune_status launch_depthwise(cprune_plan *plan, const void *x, const void *w, const float *b,
                                const void *res, void *y, cudaStream_t st);
 // channel groups (of 8 channels) one depthwise CTA handles, for c8 groups in the tensor
 int depthwise_groups(int c8);
+cprune_status plan_depthwise(cprune_plan *plan);    // fills plan->dw
 // tcgen05 implicit GEMM
 cprune_status plan_conv_tensor(cprune_plan *plan);  // fills tile fields of plan->info; UNSUPPORTED if not eligible
 cprune_status launch_conv_tensor(cprune_plan *plan, const void *x, const void *w, const float *b, const void *res,

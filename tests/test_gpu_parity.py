@@ -442,6 +442,14 @@ def test_depthwise_5x5_task_parity(cp, C, H, W, stride):
     check_task(cp, 1, C, H, W, C, 5, stride, 2, groups=C, act="none", with_res=(stride == 1))
 
 
+@pytest.mark.parametrize("N,C,H,W,R,stride,res", [(40, 20, 57, 55, 3, 1, False), (40, 200, 29, 31, 3, 2, False), (26, 72, 33, 61, 5, 1, True),
+                                                  (30, 136, 23, 40, 5, 2, False), (1, 8, 1, 1, 3, 1, False), (1, 72, 40, 2, 5, 1, False)])
+def test_depthwise_tiles_of_a_persistent_block(cp, N, C, H, W, R, stride, res):
+    # several tiles per thread block (both patch buffers refilled), odd extents against the two-column strips and the row
+    # segments, a last channel block that is not full, and images smaller than a strip or a segment
+    check_task(cp, N, C, H, W, C, R, stride, R // 2, groups=C, act="relu6", with_res=res)
+
+
 def test_task_runs_are_deterministic(cp):
     x, w, b, _ = wl.conv_task_tensors(5, 2, 89, 14, 14, 128, 3, 3)
     plan = cp.cprune_task_plan(2, 89, 14, 14, 128, 3, 3, 1, 1)
