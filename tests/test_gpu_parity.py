@@ -609,6 +609,20 @@ def test_mnasnet_parity(cp):
     model_parity(cp, "mnasnet1_0", 16, hw=96, oracle_images=4)
 
 
+@pytest.mark.parametrize("N,inn,out,act", [(1, 3, 1, "none"), (16, 40, 10, "relu"), (17, 243, 130, "none"), (33, 1300, 24, "relu6"), (70, 2600, 9, "none")])
+def test_fully_connected_tiles(cp, N, inn, out, act):
+    # edges of the 16- and 32-image tiles, of the eight-feature blocks and of the input pieces dealt to eight warps (fewer than
+    # one piece each, several rounds); float32 sums of exact bf16 products against float64: error far below 1e-5 of the scale
+    x, w, b = wl.normal_f32(91, 0, (N, inn)), wl.normal_f32(91, 1, (out, inn), 0.1), wl.normal_f32(91, 2, (out,), 0.05)
+    xb = cp.cprune_cast_input(_dev(x.reshape(N, 1, 1, inn))).reshape(N, -1)
+    y = cp.cprune_fc(xb, inn, *cp.cprune_fc_pack(_dev(w), _dev(b)), out, act, out_f32=True).cpu().numpy()
+    xr, wr = oracle.round_bf16(x).astype(np.float64), oracle.round_bf16(w).astype(np.float64)
+    ref, scale = xr @ wr.T + b, np.abs(xr) @ np.abs(wr).T + np.abs(b)
+    if act != "none":
+        ref = np.clip(ref, 0, 6 if act == "relu6" else None)
+    assert np.max(np.abs(y - ref) / scale) <= 1e-5
+
+
 def block_tensors(seed, N, C_in, H, W, hidden, C_out):
     x = wl.normal_f32(seed, 0, (N, H, W, C_in))
     we = wl.normal_f32(seed, 1, (hidden, C_in, 1, 1), np.sqrt(2.0 / C_in))
