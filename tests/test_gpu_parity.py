@@ -115,6 +115,23 @@ def test_select_filters_bit_exact(cp, K, C, R, keep):
     assert g.cpu().numpy().tobytes() == rb.tobytes()
 
 
+@pytest.mark.parametrize("K,C,R,keep,nxt", [(1, 1, 1, 1, (3, 1)), (257, 3, 3, 255, (2, 3)), (1280, 30, 1, 700, (900, 1)), (8192, 2, 1, 4000, (1, 5)),
+                                            (8200, 1, 1, 7000, (2, 1)), (300, 64, 3, 150, None)])
+def test_select_and_slice_edges(cp, K, C, R, keep, nxt):
+    # radix selection with exact ties and equal norms everywhere, rows copied as vectors and as single elements, several blocks
+    # per consumer row, a depthwise consumer (None), and more filters than the one-kernel path holds (8200)
+    w = wl.normal_f32(93, 1, (K, C, R, R), 0.05)
+    w[: K // 2] = w[K // 3]                                     # half of the filters tie exactly
+    b = wl.normal_f32(93, 2, (K,), 0.01)
+    wn = wl.normal_f32(93, 3, (K, 1, 3, 3) if nxt is None else (nxt[0], K, nxt[1], nxt[1]), 0.05)
+    kept, wo, bo, wno = cp.cprune_select_filters(_dev(w), keep, _dev(b), _dev(wn), nxt is None)
+    cp.cprune_poll_device_status()
+    idx = oracle.select_indices(w, keep)
+    assert np.array_equal(kept.cpu().numpy(), idx)
+    assert np.array_equal(wo.cpu().numpy(), w[idx]) and np.array_equal(bo.cpu().numpy(), b[idx])
+    assert np.array_equal(wno.cpu().numpy(), wn[idx] if nxt is None else wn[:, idx])
+
+
 def test_select_every_keep_count_nests(cp):
     w = wl.normal_f32(22, 1, (64, 64, 3, 3), 0.06)
     dw = _dev(w)
