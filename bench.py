@@ -278,18 +278,18 @@ def main():
     if rank == 0 and not args.no_task_times:
         peaks = measured_peaks()
         per_task = net_task_times(cp, net, table)
-        # the tensor family has two kernels; the roofline object describes the one that takes more of the step
+        # the tensor family has three kernels; the roofline object describes the one that takes more of the step
         tens_all = [t for t in per_task if t["kernel"] == "tensor"]
-        by_variant = {v: [t for t in tens_all if min(t["variant"], 1) == v] for v in (0, 1)}   # variants 1 and 2: the patch kernel
-        top = max((0, 1), key=lambda v: sum(t["ms"] for t in by_variant[v]))
+        by_variant = {v: [t for t in tens_all if {2: 1}.get(t["variant"], t["variant"]) == v] for v in (0, 1, 3)}   # 1, 2: the patch kernel
+        top = max((0, 1, 3), key=lambda v: sum(t["ms"] for t in by_variant[v]))
         tens = by_variant[top]
-        tens_name = "conv_patch_kernel" if top == 1 else "conv_tc_kernel"
+        tens_name = {0: "conv_tc_kernel", 1: "conv_patch_kernel", 3: "conv_small_kernel"}[top]
         dw = [t for t in per_task if t["kernel"] == "depthwise"]
         t_tens, t_dw = sum(t["ms"] for t in tens), sum(t["ms"] for t in dw)
         if t_dw > t_tens and dw:
             gb = sum(t["bytes"] for t in dw) / 1e9
             ach = gb / (t_dw * 1e-3)
-            roof = {"kernel": "depthwise3x3_kernel", "bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"],
+            roof = {"kernel": "depthwise_kernel", "bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"],
                     "unit": "GB/s", "frac": ach / peaks["hbm_gbs"], "traffic": None, "peak_source": peaks["source"],
                     "launches_per_step": len(dw), "ms_per_step": t_dw}
         elif tens:

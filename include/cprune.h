@@ -163,7 +163,9 @@ typedef struct {
     int variant;              /* tensor family: 0 = operands gathered per filter tap (im2col loads), 1 = the input patch
                                  of a tile stays in shared memory and every tap reads it (stride-1 tasks, stems),
                                  2 = as 1, for 1x1 tasks whose output tile is one contiguous range of y: staged as it
-                                 lies in memory and stored by a single bulk copy */
+                                 lies in memory and stored by a single bulk copy,
+                                 3 = few pixels (small batches): small tiles over the whole contraction, operands straight
+                                 from global memory */
     int splits;               /* slices of the reduction that go to different CTAs (1: no split); > 1 adds a second launch */
     /* How the program splits the two iterators that run over the filters (paper Sec. 3.5): the compute iterator
      * (filter tiles x instruction-sized groups per tile) and the store iterator (filter tiles x pieces of the memory

@@ -68,6 +68,8 @@ static cprune_status build_plan(const PlanKey &key, cprune_plan **out) {
                 family = CPRUNE_KERNEL_DIRECT;
             }
         }
+        if (st == CPRUNE_OK && pl->opts.kernel == CPRUNE_KERNEL_AUTO && plan_conv_small(pl, family == CPRUNE_KERNEL_DIRECT))
+            family = CPRUNE_KERNEL_TENSOR;
         if (family == CPRUNE_KERNEL_DIRECT) {
             i.tile_m = 1; i.tile_n = 8; i.tile_k = 8; i.stages = 0;
             i.tiles_m = i.N * i.P * i.Q; i.tiles_n = i.k_pad / 8;
@@ -81,7 +83,12 @@ static cprune_status build_plan(const PlanKey &key, cprune_plan **out) {
                                  (double)i.K * (i.C / i.groups) * rs) + 4.0 * i.K;
     // how the program splits the filter axis (see cprune_prune_step)
     i.splits = family == CPRUNE_KERNEL_TENSOR ? pl->splits : 1;
-    if (family == CPRUNE_KERNEL_TENSOR && (pl->patch || pl->orient == 0)) {
+    if (family == CPRUNE_KERNEL_TENSOR && pl->small) {
+        // filter tiles x 8-filter instruction groups per tile, stored in the same pieces
+        i.unit_compute = i.unit_store = 8;
+        i.split_compute[0] = i.split_store[0] = i.tiles_n;
+        i.split_compute[1] = i.split_store[1] = i.tile_n / 8;
+    } else if (family == CPRUNE_KERNEL_TENSOR && (pl->patch || pl->orient == 0)) {
         // filters on the MMA's column side: tiles_n tiles of tile_n filters, built from 16-filter instruction groups
         // (64-filter groups when there are several tiles: tiles end on store-box boundaries), stored in pieces of the
         // memory layout's granule (8 filters = 16 bytes up to 128 filters, 16 filters above)
@@ -105,7 +112,7 @@ static cprune_status build_plan(const PlanKey &key, cprune_plan **out) {
         i.split_compute[1] = i.split_store[1] = i.k_pad / i.unit_store;
         if (family == CPRUNE_KERNEL_DIRECT) pl->est_us = i.flops / 15.0e6 + 4.0;
     }
-    i.variant = (family == CPRUNE_KERNEL_TENSOR && pl->patch) ? (pl->pt.dense ? 2 : 1) : 0;
+    i.variant = pl->small ? 3 : (family == CPRUNE_KERNEL_TENSOR && pl->patch) ? (pl->pt.dense ? 2 : 1) : 0;
     const int s_packed = (family == CPRUNE_KERNEL_TENSOR && pl->s_packed > 0) ? pl->s_packed : i.S;
     i.packed_weight_bytes = depthwise ? (size_t)(rs * i.c_pad * 2) : (size_t)i.k_alloc * i.R * s_packed * i.c_pad * 2;
     if (family == CPRUNE_KERNEL_TENSOR && pl->patch && pl->narrow) i.packed_weight_bytes = packed_weight_bytes_patch(pl);
@@ -134,7 +141,7 @@ cprune_status task_run_internal(cprune_plan *plan, const void *x, const void *w_
     void *partial = (plan->partial_bytes || plan->pre_bytes) ? (void *)((char *)workspace + plan->pool_bytes) : nullptr;
     cprune_status s;
     switch (i.kernel) {
-        case CPRUNE_KERNEL_TENSOR: s = launch_conv_tensor(plan, x, w_packed, b_packed, residual, conv_out, partial, st, input_regrouped); break;
+        case CPRUNE_KERNEL_TENSOR: s = plan->small ? launch_conv_small(plan, x, w_packed, b_packed, residual, conv_out, st) : launch_conv_tensor(plan, x, w_packed, b_packed, residual, conv_out, partial, st, input_regrouped); break;
         case CPRUNE_KERNEL_DIRECT: s = launch_conv_direct(plan, x, w_packed, b_packed, residual, conv_out, st); break;
         case CPRUNE_KERNEL_DEPTHWISE: s = launch_depthwise(plan, x, w_packed, b_packed, residual, conv_out, st); break;
         default: return CPRUNE_ERR_INTERNAL;

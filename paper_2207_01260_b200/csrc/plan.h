@@ -62,6 +62,8 @@ struct cprune_plan {
     size_t pre_bytes = 0;           // regrouped input in the workspace
     PatchTiling pt = {};
     DwTiling dw = {};
+    int small = 0;                  // 1: task of few pixels on conv_small.cu: 8 / small_kw groups of 16 * small_mt pixels x 8 * small_nt
+    int small_mt = 0, small_nt = 0, small_kw = 0;   // filters per block, small_kw warps to a group
     double est_us = 0.0;            // the planner's cost-model estimate of the task's time
 };
 
@@ -80,6 +82,10 @@ cprune_status plan_depthwise(cprune_plan *plan);    // fills plan->dw
 cprune_status plan_conv_tensor(cprune_plan *plan);  // fills tile fields of plan->info; UNSUPPORTED if not eligible
 cprune_status launch_conv_tensor(cprune_plan *plan, const void *x, const void *w, const float *b, const void *res,
                                  void *y, void *partial, cudaStream_t st, bool input_regrouped = false);
+// tasks of few pixels (part of the tensor family; warp-level MMAs)
+bool plan_conv_small(cprune_plan *plan, bool other_is_direct);     // takes the planned task over where it is faster
+cprune_status launch_conv_small(const cprune_plan *plan, const void *x, const void *w, const float *b, const void *res, void *y,
+                                cudaStream_t st);
 // stride-1 R x S > 1 tasks with the input patch resident in shared memory (part of the tensor family)
 cprune_status plan_conv_patch(cprune_plan *plan);   // UNSUPPORTED if the task is not eligible or would waste the tile
 cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w, const float *b, const void *res,

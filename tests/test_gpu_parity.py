@@ -241,6 +241,20 @@ def test_pointwise_tasks_as_flat_matrix_products(cp):
         assert plan.variant == variant, case
 
 
+@pytest.mark.parametrize("case", [
+    # N, C, H, W, K, R, stride, pad, act, residual, pool: one and several warps to a contraction, contractions shorter than a
+    # warp's first loads and longer than several refills, ragged last pixel and filter tiles, windows that leave the image on
+    # every side, pools over whole and partial tiles, a 3-channel layer, a contraction of 1134 pieces and one beyond the table of 1700
+    (1, 3, 32, 32, 45, 3, 1, 1, "relu", False, None), (1, 8, 5, 5, 9, 1, 1, 0, "none", False, None), (1, 64, 1, 1, 300, 1, 1, 0, "relu6", True, None),
+    (2, 207, 2, 2, 243, 3, 1, 1, "relu", False, "max2x2"), (1, 45, 30, 26, 58, 3, 1, 1, "relu6", False, "max2x2"), (3, 44, 17, 13, 64, 3, 1, 1, "relu", True, None),
+    (1, 75, 15, 16, 130, 5, 2, 2, "relu", False, None), (2, 256, 14, 14, 358, 3, 2, 1, "relu", False, None), (1, 1000, 7, 7, 24, 3, 1, 1, "none", True, None),
+    (1, 1536, 3, 3, 16, 3, 1, 1, "relu", False, None), (4, 432, 14, 14, 96, 1, 1, 0, "none", True, None), (1, 16, 9, 40, 20, 7, 1, 3, "relu", False, None)])
+def test_few_pixel_tasks(cp, case):
+    N, C, H, W, K, R, stride, pad, act, res, pool = case
+    plan = check_task(cp, N, C, H, W, K, R, stride, pad, act=act, with_res=res, pool=pool)
+    assert (plan.variant == 3) == (C < 1536) and (plan.variant != 3 or plan.workspace_bytes == 0)
+
+
 def test_stems_on_the_patch_kernel(cp):
     # enough tiles for the patch kernel: the input is regrouped into 16-channel pixels (stride 1 and 2)
     plan = check_task(cp, 16, 3, 64, 64, 64, 7, 2, 3, kernel="tensor")
