@@ -59,21 +59,32 @@ static cprune_status enqueue(cprune_model *m, const float *x, float *logits, cud
     return s;
 }
 
-// True when the model's input is read by its first task only and that task is a stem that works on a regrouped
-// input: the float32 image is then cast and regrouped in one pass and the bf16 NHWC copy is never written.
-static bool stem_reads_image_directly(const cprune_model *m) {
-    if (m->tasks.empty()) return false;
+// How the model's first task gets at the float32 image when it is the only reader of the input: straight (the stem kernel
+// casts on the way in), through the regrouped copy of the patch kernel (cast and regrouping in one pass), or, otherwise,
+// from the bf16 NHWC copy that every model can make.
+enum { INPUT_CAST = 0, INPUT_REGROUP = 1, INPUT_DIRECT = 2 };
+static int input_path(const cprune_model *m) {
+    if (m->tasks.empty()) return INPUT_CAST;
     const cprune_task_desc &d0 = m->tasks[0];
-    if (d0.op != CPRUNE_OP_CONV || d0.in != 0 || !d0.plan || !d0.plan->patch || !d0.plan->narrow) return false;
+    if (d0.op != CPRUNE_OP_CONV || d0.in != 0 || !d0.plan) return INPUT_CAST;
     for (size_t t = 1; t < m->tasks.size(); ++t)
-        if (m->tasks[t].in == 0 || m->tasks[t].res == 0) return false;
-    return true;
+        if (m->tasks[t].in == 0 || m->tasks[t].res == 0) return INPUT_CAST;
+    if (d0.plan->stem.ok) return INPUT_DIRECT;
+    return d0.plan->patch && d0.plan->narrow ? INPUT_REGROUP : INPUT_CAST;
+}
+
+// Kernels that one run of a conv task enqueues.
+static int conv_launches(const cprune_plan *plan) {
+    const bool tensor = plan->info.kernel == CPRUNE_KERNEL_TENSOR;
+    return 1 + (plan->opts.pool && !(tensor && plan->fused_pool) ? 1 : 0) + (plan->splits > 1 ? 1 : 0) + (plan->patch && plan->narrow ? 1 : 0);
 }
 
 static cprune_status enqueue_chain(cprune_model *m, const float *x, float *logits, cudaStream_t st) {
-    const bool direct = stem_reads_image_directly(m);
-    cprune_status s = direct ? regroup_stem_input(m->tasks[0].plan, x, 1, stem_scratch(m->tasks[0].plan, m->workspace), st)
-                             : cprune_cast_input(x, (size_t)m->N * m->H * m->W, m->C, tensor_ptr(m, 0), st);
+    int path = input_path(m);
+    if (path == INPUT_DIRECT && ((uintptr_t)x & 15)) path = INPUT_CAST;      // bulk copies need 16-byte alignment
+    cprune_status s = CPRUNE_OK;
+    if (path == INPUT_REGROUP) s = regroup_stem_input(m->tasks[0].plan, x, 1, stem_scratch(m->tasks[0].plan, m->workspace), st);
+    else if (path == INPUT_CAST) s = cprune_cast_input(x, (size_t)m->N * m->H * m->W, m->C, tensor_ptr(m, 0), st);
     if (s != CPRUNE_OK) return s;
     for (size_t t = 0; t < m->tasks.size(); ++t) {
         const cprune_task_desc &d = m->tasks[t];
@@ -83,8 +94,9 @@ static cprune_status enqueue_chain(cprune_model *m, const float *x, float *logit
         void *pout = last ? (void *)logits : tensor_ptr(m, d.out);
         switch (d.op) {
             case CPRUNE_OP_CONV:
-                s = task_run_internal(d.plan, pin, d.w, d.b, d.res >= 0 ? tensor_ptr(m, d.res) : nullptr, pout, m->workspace, st,
-                                      t == 0 && direct);
+                if (t == 0 && path == INPUT_DIRECT) s = launch_conv_stem(d.plan, x, d.w, d.b, pout, st);
+                else s = task_run_internal(d.plan, pin, d.w, d.b, d.res >= 0 ? tensor_ptr(m, d.res) : nullptr, pout, m->workspace, st,
+                                           t == 0 && path == INPUT_REGROUP);
                 break;
             case CPRUNE_OP_BLOCK:
                 s = cprune_block_run(d.block, pin, d.w, d.b, pout, m->workspace, st);
@@ -148,8 +160,7 @@ cprune_status cprune_model_create(int N, int H, int W, int C, const cprune_task_
                 }
                 o.h = i.out_h; o.w = i.out_w; o.c = i.K;
                 if (i.workspace_bytes > m->workspace_bytes) m->workspace_bytes = i.workspace_bytes;
-                m->launches += ((d.plan->opts.pool && !(i.kernel == CPRUNE_KERNEL_TENSOR && d.plan->fused_pool)) ? 2 : 1) + (d.plan->splits > 1 ? 1 : 0) +
-                               ((d.plan->patch && d.plan->narrow) ? 1 : 0);
+                m->launches += conv_launches(d.plan);
                 break;
             }
             case CPRUNE_OP_BLOCK: {
@@ -191,7 +202,9 @@ cprune_status cprune_model_create(int N, int H, int W, int C, const cprune_task_
         m->tensors[d.out] = o;
     }
     if (st != CPRUNE_OK) { delete m; return st; }
-    if (stem_reads_image_directly(m)) m->launches -= 1;     // one pass casts and regroups the image
+    const int path = input_path(m);
+    if (path != INPUT_CAST) m->launches -= 1;               // no separate cast of the image
+    if (path == INPUT_DIRECT) m->launches += 1 - conv_launches(m->tasks[0].plan);
     size_t off = 0;
     for (auto &kv : m->tensors) {
         kv.second.bytes = (size_t)kv.second.n * kv.second.h * kv.second.w * kv.second.c_pad * 2;

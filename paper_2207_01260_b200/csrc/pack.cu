@@ -100,6 +100,10 @@ cprune_status cprune_pack_weights(const cprune_plan *plan, const float *w, const
         CPRUNE_LAUNCH_CHECK("pad_bias_kernel");
         return CPRUNE_OK;
     }
+    if (plan->stem.ok) {
+        const cprune_status s = pack_conv_stem(plan, w, (char *)w_packed + plan->stem.weight_offset, st);
+        if (s != CPRUNE_OK) return s;
+    }
     if (i.kernel == CPRUNE_KERNEL_TENSOR && plan->patch && plan->narrow) {
         pad_bias_kernel<<<(i.k_alloc + 255) / 256, 256, 0, st>>>(b, i.K, i.k_alloc, b_packed);
         CPRUNE_LAUNCH_CHECK("pad_bias_kernel");

@@ -116,6 +116,13 @@ static cprune_status build_plan(const PlanKey &key, cprune_plan **out) {
     const int s_packed = (family == CPRUNE_KERNEL_TENSOR && pl->s_packed > 0) ? pl->s_packed : i.S;
     i.packed_weight_bytes = depthwise ? (size_t)(rs * i.c_pad * 2) : (size_t)i.k_alloc * i.R * s_packed * i.c_pad * 2;
     if (family == CPRUNE_KERNEL_TENSOR && pl->patch && pl->narrow) i.packed_weight_bytes = packed_weight_bytes_patch(pl);
+    if (!depthwise) {
+        plan_conv_stem(pl);
+        if (pl->stem.ok) {
+            pl->stem.weight_offset = (i.packed_weight_bytes + 255) / 256 * 256;
+            i.packed_weight_bytes = pl->stem.weight_offset + pl->stem.weight_bytes;
+        }
+    }
     i.packed_bias_bytes = (size_t)i.k_alloc * sizeof(float);
     // workspace: [unpooled conv output if a pool follows][split-K partial sums]
     const bool separate_pool = pl->opts.pool != CPRUNE_POOL_NONE && !(family == CPRUNE_KERNEL_TENSOR && pl->fused_pool);

@@ -31,6 +31,15 @@ struct DwTiling {
     int patch_bytes;
 };
 
+// Tiling of the stem kernel that reads a model's float32 image (conv_stem.cu): a step is D conv rows of KF filters each
+struct StemTiling {
+    int ok;
+    int D, KF, RH, N, ktot;                  // input rows per step, MMA columns, packed row length
+    int per, slot, tiles, adv;               // input rows per operand tile, bytes of a window, tiles a step reads, tiles from step to step
+    int row_bytes, tile_bytes, raw_bytes, ring, stage_bytes, xch_words, smem_bytes, steps_per_img;
+    size_t weight_offset, weight_bytes;      // its filters behind the task's own in the packed weights
+};
+
 struct cprune_plan {
     cprune_plan_info info;
     cprune_task_opts opts;
@@ -62,6 +71,7 @@ struct cprune_plan {
     size_t pre_bytes = 0;           // regrouped input in the workspace
     PatchTiling pt = {};
     DwTiling dw = {};
+    StemTiling stem = {};
     int small = 0;                  // 1: task of few pixels on conv_small.cu: 8 / small_kw groups of 16 * small_mt pixels x 8 * small_nt
     int small_mt = 0, small_nt = 0, small_kw = 0;   // filters per block, small_kw warps to a group
     double est_us = 0.0;            // the planner's cost-model estimate of the task's time
@@ -98,6 +108,10 @@ cprune_status task_run_internal(cprune_plan *plan, const void *x, const void *w_
                                 void *y, void *workspace, cudaStream_t st, bool input_regrouped);
 // where in a task's workspace the regrouped stem input lives
 inline void *stem_scratch(const cprune_plan *plan, void *workspace) { return (char *)workspace + plan->pool_bytes; }
+// a model's first task straight from the float32 image (fills plan->stem; stem.ok == 0 where it is not supported)
+void plan_conv_stem(cprune_plan *plan);
+cprune_status pack_conv_stem(const cprune_plan *plan, const float *w, void *w_stem, cudaStream_t st);
+cprune_status launch_conv_stem(const cprune_plan *plan, const float *x, const void *w_packed, const float *b, void *y, cudaStream_t st);
 // filters of a regrouped stem (plan->narrow) and their size
 cprune_status pack_conv_patch(const cprune_plan *plan, const float *w, void *w_packed, cudaStream_t st);
 size_t packed_weight_bytes_patch(const cprune_plan *plan);

@@ -265,6 +265,39 @@ def test_stems_on_the_patch_kernel(cp):
 
 
 @pytest.mark.parametrize("case", [
+    # N, H, W, K, R, stride, pad, act, pool: 1, 2 and 4 conv rows per step, images whose steps are dealt unevenly to the blocks
+    # (with the pool: one conv row above recomputed), ragged last step, rows and columns outside the image on every side,
+    # windows of 32, 64 and 128 bytes, filters that fill 32, 64 and 128 rows
+    (9, 64, 64, 45, 3, 1, 1, "relu", None), (5, 224, 224, 32, 3, 2, 1, "relu6", None), (4, 64, 136, 64, 7, 2, 3, "relu", "max3x3s2"),
+    (20, 32, 132, 48, 7, 2, 3, "relu6", "max3x3s2"), (9, 68, 76, 24, 5, 1, 2, "none", None), (17, 70, 132, 100, 5, 2, 2, "relu", None),
+    (40, 63, 132, 8, 3, 2, 0, "none", None), (20, 36, 132, 40, 4, 2, 1, "none", "max3x3s2"), (9, 64, 68, 120, 3, 1, 1, "relu", None)])
+def test_stems_straight_from_the_image(cp, case):
+    N, H, W, K, R, stride, pad, act, pool = case
+    x, w, b, _ = wl.conv_task_tensors(95, N, 3, H, W, K, R, R)
+    plan = cp.cprune_task_plan(N, 3, H, W, K, R, R, stride, pad, 1, act, False, pool)
+    packed, fc = cp.cprune_pack_weights(plan, _dev(w), _dev(b)), cp.cprune_fc_pack(torch.ones((8, K), device="cuda"))
+    tasks = [cp.TaskDesc(op=cp.OP_CONV, in_=0, out=1, res=-1, plan=plan.handle, w=packed[0].data_ptr(), b=packed[1].data_ptr()),
+             cp.TaskDesc(op=cp.OP_GAP, in_=1, out=2, res=-1),
+             cp.TaskDesc(op=cp.OP_FC, in_=2, out=3, res=-1, w=fc[0].data_ptr(), b=fc[1].data_ptr(), p0=K, p1=8)]
+    model = cp.cprune_model_create(N, H, W, 3, tasks, keep_alive=(plan, packed, fc))
+    assert model.launches == 3
+    cp.cprune_model_run(model, _dev(x))
+    y = model.copy_tensor(1).float().cpu().numpy()
+    cp.cprune_poll_device_status()
+    ref, bound = _pooled(*oracle.conv2d(x, w, b, stride, pad, 1, act, None, with_bound=True), pool)
+    rb = oracle.round_bf16
+    ref_m, bound_m = _pooled(*oracle.conv2d(rb(x), rb(w), b, stride, pad, 1, act, None, with_bound=True), pool)
+    assert y.shape[:3] == ref.shape[:3] and np.all(y[..., K:] == 0)
+    check_values("stem %s" % (case,), y[..., :K], ref, bound, ref_m, bound_m)
+    # an image that is not 16-byte aligned takes the bf16 copy; the same values up to the order of the sums
+    odd = torch.empty(x.size + 1, device="cuda")[1:].view(x.shape)
+    odd.copy_(_dev(x))
+    cp.cprune_model_run(model, odd)
+    y2 = model.copy_tensor(1).float().cpu().numpy()
+    check_values("stem, unaligned image %s" % (case,), y2[..., :K], ref, bound, ref_m, bound_m)
+
+
+@pytest.mark.parametrize("case", [
     # N, C, H, W, K, R, stride, pad: fused in the patch kernel (tiles around whole 3x3 windows, even and odd extents),
     # and as a separate pass (few tiles; a task with wrap-around slots)
     (16, 3, 64, 64, 64, 7, 2, 3), (12, 3, 60, 52, 40, 7, 2, 3), (40, 3, 30, 30, 24, 3, 1, 1),
