@@ -21,11 +21,11 @@
 //                64 filters brings the residual tile in through the same ring;
 //   warps 1, 2   filter loads, one per (channel block, tap), taken in turn; small filter sets
 //                stay resident in shared memory for the whole kernel;
-//   warps 3, 12  tcgen05.mma issue, one warp per accumulator block; the residual tile is added by
+//   warps 3, 12  tcgen05.mma issue (3 and 20 with sixteen epilogue warps), one warp per accumulator block; the residual tile is added by
 //                one more MMA against a 64 x 64 identity held in shared memory (bf16 x 1.0 into an
 //                fp32 accumulator is exact), so the epilogue never touches global memory for it
 //                (the 1x1 instantiation, whose tile is flat, still adds it in the epilogue);
-//   warps 4..11  epilogue: tcgen05.ld, bias, activation, bf16 into a swizzled staging
+//   warps 4..11  epilogue (4..19 for flat 1x1 tasks): tcgen05.ld, bias, activation, bf16 into a swizzled staging
 //                buffer, then ONE TMA store per group of 64 filters whose box is the tile's rows x
 //                Wp pixels (wrap-around columns, rows below the image and filters beyond k_pad lie
 //                outside the tensor map and are not written).  With a fused max-pool the staged
@@ -43,14 +43,15 @@
 
 namespace cprune {
 
-constexpr int PK_THREADS = 13 * 32;       // general kernel: 5 role warps + 8 epilogue warps
-constexpr int PK_THREADS_DENSE = 21 * 32; // dense-staging kernel: 16 epilogue warps (its epilogue bounds the tile; it needs few registers)
 constexpr int PK_POOL_WARPS = 8;          // 3x3-pool kernel: these warps pool the staged tile while the epilogue warps stage the next one
-constexpr int PK_THREADS_POOL3 = (13 + PK_POOL_WARPS) * 32;
 // kernel instantiations
-constexpr int PK_GENERAL = 0, PK_DENSE = 1, PK_POOL3 = 2;
-__host__ __device__ constexpr int pk_threads(int mode) { return mode == PK_DENSE ? PK_THREADS_DENSE : (mode == PK_POOL3 ? PK_THREADS_POOL3 : PK_THREADS); }
-__host__ __device__ constexpr int pk_epi_warps(bool dense) { return dense ? 16 : 8; }
+constexpr int PK_GENERAL = 0, PK_DENSE = 1, PK_POOL3 = 2, PK_FLAT = 3;
+// Epilogue warps.  A flat tile has little for the MMAs to do, so its epilogue bounds it: a warp spends about 300 cycles on 16
+// filters of 128 pixels, mostly the latencies of a chain of 50 instructions, and sixteen warps hide twice as many of them as
+// eight (64 images, 1x1 24 -> 108 of 56x56: 23.1 -> 19.9 us; 32 -> 16 of 112x112: 26.3 -> 19.1 us).  The other tasks are bound by
+// their MMAs and lose with sixteen (3x3 131 -> 203 of 28x28: 37.8 -> 39.6 us); beside the pooling warps there is room for eight.
+__host__ __device__ constexpr int pk_epi_warps(int mode) { return mode == PK_DENSE || mode == PK_FLAT ? 16 : 8; }
+__host__ __device__ constexpr int pk_threads(int mode) { return (5 + pk_epi_warps(mode) + (mode == PK_POOL3 ? PK_POOL_WARPS : 0)) * 32; }
 constexpr int PK_MMA_WARP = 3;
 constexpr int PK_FIRST_EPI = 4;
 // (the warp after the epilogue warps issues for the second accumulator block when MT = 2)
@@ -74,6 +75,8 @@ struct PatchParams {
     int dense;             // the staged tile is [slot][k_pad] as in memory and leaves by one bulk copy (flat tasks, one filter tile)
     int dense_pitch;       // ... bytes per slot in the staging buffer: k_pad * 2, or 16 more (then the tile leaves by a tiled copy)
     int stage_bytes;       // shared memory of one staging buffer
+    int flat;              // 1x1 tasks: one image of one row
+    uint32_t img_mul, row_mul;   // ceil(2^32 / tiles_per_img), ceil(2^32 / tiles_w), or 0
     int res_blocks;        // residual added on the tensor core: 64-filter blocks of the residual tile per item (0: none)
     const float *bias;
     const __nv_bfloat16 *res;
@@ -93,6 +96,36 @@ __device__ __forceinline__ uint4 bf16x8_max(uint4 a, uint4 b) {
     __nv_bfloat162 *pr = reinterpret_cast<__nv_bfloat162 *>(&r);
 #pragma unroll
     for (int i = 0; i < 4; ++i) pr[i] = __hmax2(pa[i], pb[i]);
+    return r;
+}
+
+// Eight accumulator values of one pixel + bias -> activated bf16.  Two sums per instruction; 0 and 6 are bf16 values, so that
+// the clamps commute with the rounding (ReLU is part of the conversion).
+__device__ __forceinline__ unsigned long long pair64(uint32_t lo, uint32_t hi) {
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
+    return d;
+}
+__device__ __forceinline__ bf16x8 bias_act8(const uint32_t *v, const unsigned long long *bias, int act) {
+    bf16x8 r;
+    float lo[4], hi[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        unsigned long long t;
+        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(pair64(v[2 * j], v[2 * j + 1])), "l"(bias[j]));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(lo[j]), "=f"(hi[j]) : "l"(t));
+    }
+    if (act == CPRUNE_ACT_NONE) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r.w[j]) : "f"(hi[j]), "f"(lo[j]));
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(r.w[j]) : "f"(hi[j]), "f"(lo[j]));
+        if (act == CPRUNE_ACT_RELU6) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) asm("min.bf16x2 %0, %0, %1;" : "+r"(r.w[j]) : "r"(0x40C040C0u));
+        }
+    }
     return r;
 }
 
@@ -145,12 +178,18 @@ __device__ __forceinline__ void issue_row(uint32_t d_tmem, uint32_t a_lo, uint32
 }
 
 // First output pixel (may be -1 with the 3x3 pool, whose windows reach one pixel outside the tile's own pooled
-// pixels) and image of tile tm.
+// pixels) and image of tile tm.  The divisions are multiplications with reciprocals that the host has checked for every
+// tile number (mul == 0: by division); flat tasks (one image, one row of tiles) need none.
+__device__ __forceinline__ int quotient(int v, int d, uint32_t mul) { return mul ? (int)__umulhi((uint32_t)v, mul) : v / d; }
 __device__ __forceinline__ void tile_origin(const PatchParams &p, int tm, int &n, int &p0, int &q0) {
-    n = tm / p.tiles_per_img;
+    if (p.flat) {
+        n = 0; p0 = 0; q0 = tm * p.step_w;
+        return;
+    }
+    n = quotient(tm, p.tiles_per_img, p.img_mul);
     const int r = tm - n * p.tiles_per_img;
     int ty = r, tx = 0;
-    if (p.tiles_w > 1) { ty = r / p.tiles_w; tx = r - ty * p.tiles_w; }
+    if (p.tiles_w > 1) { ty = quotient(r, p.tiles_w, p.row_mul); tx = r - ty * p.tiles_w; }
     p0 = ty * p.step_h + p.org;
     q0 = tx * p.step_w + p.org;
 }
@@ -162,7 +201,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     extern __shared__ uint8_t smem_raw[];
     constexpr bool DENSE = MODE == PK_DENSE;
     constexpr bool SPLIT = MODE == PK_POOL3;      // staging by the epilogue warps, pooling by PK_POOL_WARPS further warps
-    constexpr int EPI_WARPS = pk_epi_warps(DENSE);
+    constexpr int EPI_WARPS = pk_epi_warps(MODE);
     constexpr int MMA_WARP2 = PK_FIRST_EPI + EPI_WARPS;
     pdl_trigger();
     if (threadIdx.x == 0) {
@@ -476,8 +515,12 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         }
     } else {
         // ------------------------------------------------------------------ epilogue
+        constexpr int EPI_THREADS = EPI_WARPS * 32;
+        constexpr int SUBS = EPI_WARPS / 4;            // warps that share a quarter of the accumulator lanes
+        constexpr int WCOLS = 64 / SUBS;               // ... each takes this many filters of a 64-filter group
+        constexpr int UNITS = WCOLS / 16;              // 16-filter units of a warp per accumulator block
         const int quarter = warp & 3;
-        const int half = (warp - PK_FIRST_EPI) >> 2;
+        const int sub = (warp - PK_FIRST_EPI) >> 2;
         const int trow = quarter * 32 + lane;          // accumulator lane = slot within its 128-slot block
         const int etid = threadIdx.x - PK_FIRST_EPI * 32;
         int acc = 0;
@@ -492,45 +535,29 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         };
         // the task's bias into shared memory, while the first tile is being computed
         if (bias_staged) {
-            for (int e = etid; e < k_all; e += EPI_WARPS * 32) bias_s[e] = __ldg(p.bias + e);
+            for (int e = etid; e < k_all; e += EPI_THREADS) bias_s[e] = __ldg(p.bias + e);
             ok = epi_sync();
         }
-        // activation as a clamp: no branches in the per-element code
-        const float act_lo = p.act == CPRUNE_ACT_NONE ? -INFINITY : 0.f, act_hi = p.act == CPRUNE_ACT_RELU6 ? 6.f : INFINITY;
         const bool clamp_lo = p.act != CPRUNE_ACT_NONE;      // results are >= 0
         const bool store_thread = warp == PK_FIRST_EPI && lane == 0;
         const int groups = (p.FT + 63) / 64;
-        // one group and one filter tile: a thread stages the same 32 filters in every tile and keeps their bias in registers
-        const bool bias_const = !DENSE && groups == 1 && p.tiles_n == 1;
-        float bias_r[32];
-        if (bias_const) {
+        // one group and one filter tile: a thread stages the same filters in every tile and keeps their bias in registers
+        const bool bias_const = groups == 1 && p.tiles_n == 1;
+        unsigned long long bias_r[WCOLS / 2];
+        auto load_bias = [&](int c) {                  // filters c .. c + WCOLS - 1
 #pragma unroll
-            for (int j = 0; j < 32; ++j) bias_r[j] = (half * 32 + j < p.FT) ? __ldg(p.bias + half * 32 + j) : 0.f;
-        }
+            for (int j = 0; j < WCOLS / 2; ++j)
+                bias_r[j] = c + j * 2 < k_all ? *reinterpret_cast<const unsigned long long *>(bias_src + c + j * 2) : 0ull;
+        };
+        if (bias_const) load_bias(sub * WCOLS);
         const int n_entries = p.pool == 1 ? (p.TH >> 1) * (p.Q >> 1) : ((p.TH - 1) >> 1) * ((p.TW - 1) >> 1);
-        // 3x3 pool: a thread copies out at most two (pooled pixel, 8 filters) items per tile, the same ones in every tile;
-        // the shared-memory offsets of their nine window slots are worked out once
-        uint32_t win_off[2][9];
-        int win_pi[2] = {0, 0}, win_pj[2] = {0, 0};
-        if (MODE == PK_GENERAL && p.pool == 2) {
-            const int tpc = (p.TW - 1) >> 1;
-#pragma unroll
-            for (int it = 0; it < 2; ++it) {
-                const int e = etid + it * 256;
-                const int ent = e >> 3, chunk = e & 7;
-                win_pi[it] = ent / tpc; win_pj[it] = ent - win_pi[it] * tpc;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    const int sl = (2 * win_pi[it] + k / 3) * p.Wp + 2 * win_pj[it] + k % 3;
-                    win_off[it][k] = (uint32_t)((sl >> 7) * PK_BLOCK_BYTES) + sub_off(sl & 127, chunk);
-                }
-            }
-        }
         // Residuals.  Everywhere but with dense staging the MMA warps add the residual on the tensor core (see there) and
         // the epilogue has nothing to do with it.  Dense staging: the residual of tile item_ (tiles_n == 1, one row of
         // tiles) is one contiguous range of memory, arrives in the staging buffer the tile will use and is added in place.
         const bool with_res = DENSE && p.res != nullptr;
         const bool dense_tiled = DENSE && p.dense_pitch != p.k_pad * 2;
+        const int dense_n16 = (p.k_pad + 15) >> 4, dense_units = dense_n16 * p.MT;
+        const uint32_t dense_block = 128u * (uint32_t)p.dense_pitch;
         auto load_residual_dense = [&](int item_, uint32_t counter) {
             const int q0_ = item_ * p.step_w;
             const uint32_t bytes = (uint32_t)min(p.TW, p.Q - q0_) * (uint32_t)p.k_pad * 2u;
@@ -574,42 +601,34 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                     ok = __all_sync(0xffffffffu, mbar_wait(res_full(b), (group_counter >> 1) & 1u, abort_flag, p.status, false));
                     if (!ok) break;
                 }
-                for (int g = 0; g < groups; ++g) {
-                    const int ch = g * 64 + half * 16;           // this warp's 16 filters of the group (16 epilogue warps)
-                    if (ch >= p.k_pad) continue;
-                    for (int mb = 0; mb < p.MT; ++mb) {
-                        uint8_t *row = buf + (uint32_t)(mb * 128 + trow) * pitch;
-                        uint32_t v[16];
-                        tmem_ld16(t_row + (uint32_t)(mb * p.FT + ch), v);
-                        bf16x8 rv[2];
-                        if (with_res) {
+                // 16-filter units of both accumulator blocks, dealt to the warps of a quarter in turn
+                uint8_t *row = buf + (uint32_t)trow * pitch;
+                auto stage_half = [&](uint8_t *dst, uint32_t *v, int c) {
+                    unsigned long long bb[4];
+                    const ulonglong2 b0 = *reinterpret_cast<const ulonglong2 *>(bias_src + c), b1 = *reinterpret_cast<const ulonglong2 *>(bias_src + c + 4);
+                    bb[0] = b0.x; bb[1] = b0.y; bb[2] = b1.x; bb[3] = b1.y;
+                    if (with_res) {
+                        // (acc + bias) + residual, as everywhere
+                        const bf16x8 rv = *(const bf16x8 *)dst;
 #pragma unroll
-                            for (int j = 0; j < 2; ++j)
-                                if (ch + j * 8 < p.k_pad) rv[j] = *(const bf16x8 *)(row + (ch + j * 8) * 2);
-                        }
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            const int c = ch + q * 8;
-                            if (c < p.k_pad) {
-                                float f[8];
-                                const float4 b0 = *(const float4 *)(bias_src + c);
-                                const float4 b1 = *(const float4 *)(bias_src + c + 4);
-                                const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-                                for (int j = 0; j < 8; ++j) f[j] = __uint_as_float(v[q * 8 + j]) + bb[j];
-                                if (with_res) {
-                                    float rf[8];
-                                    unpack8(rv[q], rf);
-#pragma unroll
-                                    for (int j = 0; j < 8; ++j) f[j] += rf[j];
-                                }
-#pragma unroll
-                                for (int j = 0; j < 8; ++j) f[j] = fminf(fmaxf(f[j], act_lo), act_hi);
-                                *(bf16x8 *)(row + c * 2) = pack8(f);
-                            }
+                        for (int j = 0; j < 4; ++j) {
+                            unsigned long long t;
+                            asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(pair64(v[2 * j], v[2 * j + 1])), "l"(bb[j]));
+                            asm("mov.b64 {%0, %1}, %2;" : "=r"(v[2 * j]), "=r"(v[2 * j + 1]) : "l"(t));
+                            bb[j] = pair64(rv.w[j] << 16, rv.w[j] & 0xffff0000u);
                         }
                     }
+                    *(bf16x8 *)dst = bias_act8(v, bb, p.act);
+                };
+                for (int u = sub; u < dense_units; u += SUBS) {
+                    const bool second = u >= dense_n16;
+                    const int ch = (second ? u - dense_n16 : u) * 16;
+                    uint8_t *dst = row + (second ? dense_block : 0u) + ch * 2;
+                    uint32_t v[16];
+                    tmem_ld16(t_row + (uint32_t)((second ? p.FT : 0) + ch), v);
+                    tmem_ld_wait();
+                    stage_half(dst, v, ch);
+                    if (ch + 8 < p.k_pad) stage_half(dst + 16, v + 8, ch + 8);
                 }
                 // every warp has read what it needs of the accumulator (a warp without filters in the last group too)
                 tc_fence_before();
@@ -632,63 +651,38 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             for (int g = 0; g < groups && ok; ++g) {
                 const uint32_t boff = (p.staging_bufs == 2 ? (group_counter & 1u) : 0u) * stage_buf_bytes;
                 uint8_t *buf = smem + (staging0 - base) + boff;
-                const int ch = g * 64 + half * 32;           // this warp's 32 filters of the group
+                const int ch = g * 64 + sub * WCOLS;         // this warp's filters of the group
                 if constexpr (SPLIT) {
                     // the buffer's previous contents (two groups ago) must have been pooled
                     ok = __all_sync(0xffffffffu, mbar_wait(sempty(group_counter & 1u), ((group_counter >> 1) & 1u) ^ 1u, abort_flag, p.status, false));
                     if (!ok) break;
                 }
-                // Units of 16 filters of one accumulator block: (block 0, first 16), (block 0, second 16), (block 1, ...).
-                // The tensor-memory load of unit u + 1 is in flight while unit u is turned into bf16 and staged, so that
-                // only the first load's latency is exposed; two register buffers alternate.
-                const bool u_ok[4] = {ch < p.FT, ch + 16 < p.FT, p.MT == 2 && ch < p.FT, p.MT == 2 && ch + 16 < p.FT};
-                auto unit_addr = [&](int u) { return t_row + (uint32_t)((u >> 1) * p.FT + ch + (u & 1) * 16); };
-                auto stage_unit = [&](int u, const uint32_t *v) {
-                    const int c0 = ch + (u & 1) * 16;
-                    float f[16];
-                    if (bias_const) {
+                // Units of 16 filters of one accumulator block; the tensor-memory loads of a pair of them are in flight together:
+                // those of the two blocks, or (two units per warp) both of block 0, then both of block 1.
+                if (!bias_const && ch < p.FT) load_bias(k0 + ch);
+                uint32_t va[16], vb[16];
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[j]) + bias_r[(u & 1) * 16 + j];
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const float4 b4 = *(const float4 *)(bias_src + k0 + c0 + q * 4);
-                            f[q * 4 + 0] = __uint_as_float(v[q * 4 + 0]) + b4.x;
-                            f[q * 4 + 1] = __uint_as_float(v[q * 4 + 1]) + b4.y;
-                            f[q * 4 + 2] = __uint_as_float(v[q * 4 + 2]) + b4.z;
-                            f[q * 4 + 3] = __uint_as_float(v[q * 4 + 3]) + b4.w;
-                        }
-                    }
-                    if (p.act == CPRUNE_ACT_RELU) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) f[j] = fmaxf(f[j], 0.f);
-                    } else if (p.act == CPRUNE_ACT_RELU6) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) f[j] = fminf(fmaxf(f[j], 0.f), 6.f);
-                    }
-                    uint8_t *blk = buf + (u >> 1) * PK_BLOCK_BYTES;
-                    *(bf16x8 *)(blk + sub_off(trow, half * 4 + (u & 1) * 2)) = pack8(f);
-                    *(bf16x8 *)(blk + sub_off(trow, half * 4 + (u & 1) * 2 + 1)) = pack8(f + 8);
-                };
-                {
-                    uint32_t va[16], vb[16];
-                    if (u_ok[0]) tmem_ld16(unit_addr(0), va);
+                for (int q = 0; q < UNITS; ++q) {
+                    const int mb_a = UNITS == 1 ? 0 : q, mb_b = UNITS == 1 ? 1 : q, cu_b = UNITS == 1 ? 0 : 1;
+                    const bool do_a = mb_a < p.MT && ch < p.FT, do_b = mb_b < p.MT && ch + cu_b * 16 < p.FT;
+                    if (do_a) tmem_ld16(t_row + (uint32_t)(mb_a * p.FT + ch), va);
+                    if (do_b) tmem_ld16(t_row + (uint32_t)(mb_b * p.FT + ch + cu_b * 16), vb);
                     tmem_ld_wait();
-                    if (u_ok[1]) tmem_ld16(unit_addr(1), vb);
-                    if (u_ok[0]) stage_unit(0, va);
-                    tmem_ld_wait();
-                    if (u_ok[2]) tmem_ld16(unit_addr(2), va);
-                    if (u_ok[1]) stage_unit(1, vb);
-                    tmem_ld_wait();
-                    if (u_ok[3]) tmem_ld16(unit_addr(3), vb);
-                    if (u_ok[2]) stage_unit(2, va);
-                    tmem_ld_wait();
-                    if (g == groups - 1) {     // accumulator fully read: hand it back
+                    if (q == UNITS - 1 && g == groups - 1) {     // accumulator fully read: hand it back
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(tempty(acc));
                     }
-                    if (u_ok[3]) stage_unit(3, vb);
+                    if (do_a) {
+                        uint8_t *blk = buf + mb_a * PK_BLOCK_BYTES;
+                        *(bf16x8 *)(blk + sub_off(trow, sub * (WCOLS / 8))) = bias_act8(va, bias_r, p.act);
+                        *(bf16x8 *)(blk + sub_off(trow, sub * (WCOLS / 8) + 1)) = bias_act8(va + 8, bias_r + 4, p.act);
+                    }
+                    if (do_b) {
+                        uint8_t *blk = buf + mb_b * PK_BLOCK_BYTES;
+                        *(bf16x8 *)(blk + sub_off(trow, sub * (WCOLS / 8) + cu_b * 2)) = bias_act8(vb, bias_r + cu_b * 8, p.act);
+                        *(bf16x8 *)(blk + sub_off(trow, sub * (WCOLS / 8) + cu_b * 2 + 1)) = bias_act8(vb + 8, bias_r + cu_b * 8 + 4, p.act);
+                    }
                 }
                 if constexpr (SPLIT) {
                     // hand the staged group to the pooling warps and go on with the next one
@@ -724,7 +718,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 const int kg = k0 + g * 64;
                 auto staged = [&](int sl, int chunk) { return *(const uint4 *)(buf + (sl >> 7) * PK_BLOCK_BYTES + sub_off(sl & 127, chunk)); };
                 if (p.pool == 1) {
-                    for (int e = etid; e < n_entries * 8; e += 256) {
+                    for (int e = etid; e < n_entries * 8; e += EPI_THREADS) {
                         const int2 l = lut[e >> 3];
                         const int chunk = e & 7;
                         if (l.x >= 0 && (l.x >> 16) < rows_valid && g * 64 + chunk * 8 < p.FT && kg + chunk * 8 < p.k_pad) {
@@ -744,20 +738,19 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                     // after ReLU / ReLU6 all values are >= 0: pixels outside the image can be replaced by 0 (every
                     // window holds a real pixel) and the maximum taken on the bit patterns
                     const uint4 fill = clamp_lo ? make_uint4(0u, 0u, 0u, 0u) : ninf;
-#pragma unroll
-                    for (int it = 0; it < 2; ++it) {
-                        const int e = etid + it * 256;
-                        const int chunk = e & 7;
-                        const int pr = pr0 + win_pi[it], pc = pc0 + win_pj[it];
-                        if (e < n_entries * 8 && pr < p.out_h && pc < p.out_w && g * 64 + chunk * 8 < p.FT && kg + chunk * 8 < p.k_pad) {
-                            const int r0 = p0 + 2 * win_pi[it], c0 = q0 + 2 * win_pj[it];
+                    const int tpc = (p.TW - 1) >> 1;
+                    for (int e = etid; e < n_entries * 8; e += EPI_THREADS) {
+                        const int chunk = e & 7, win_pi = (e >> 3) / tpc, win_pj = (e >> 3) - win_pi * tpc;
+                        const int pr = pr0 + win_pi, pc = pc0 + win_pj;
+                        if (pr < p.out_h && pc < p.out_w && g * 64 + chunk * 8 < p.FT && kg + chunk * 8 < p.k_pad) {
+                            const int r0 = p0 + 2 * win_pi, c0 = q0 + 2 * win_pj;
                             // bit d of a mask: window row / column d lies inside the image
                             const uint32_t rmask = (r0 >= 0 ? 1u : 0u) | 2u | (r0 + 2 < p.P ? 4u : 0u);
                             const uint32_t cmask = (c0 >= 0 ? 1u : 0u) | 2u | (c0 + 2 < p.Q ? 4u : 0u);
                             uint4 w[9];
 #pragma unroll
                             for (int k = 0; k < 9; ++k) {
-                                const uint4 t = *(const uint4 *)(buf + win_off[it][k]);
+                                const uint4 t = staged((2 * win_pi + k / 3) * p.Wp + 2 * win_pj + k % 3, chunk);
                                 w[k] = ((rmask >> (k / 3)) & (cmask >> (k % 3)) & 1u) ? t : fill;
                             }
                             uint4 m;
@@ -1244,6 +1237,7 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
         std::lock_guard<std::mutex> lock(attr_mu);
         if (!attr_set[dev]) {
             CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(conv_patch_kernel<PK_GENERAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(conv_patch_kernel<PK_FLAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
             CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(conv_patch_kernel<PK_DENSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
             CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(conv_patch_kernel<PK_POOL3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
             attr_set[dev] = true;
@@ -1253,6 +1247,13 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
     p.P = g.vP; p.Q = g.vQ; p.Wp = Wp; p.TH = t.TH; p.tiles_per_img = t.tiles_per_img;
     p.TW = t.TW; p.tiles_w = t.tiles_w; p.step_h = t.step_h; p.step_w = t.step_w; p.org = t.org;
     p.out_h = g.vOH; p.out_w = g.vOW;
+    p.flat = g.flat;
+    // v * ceil(2^32 / d) / 2^32 has the integer part v / d as long as v * d < 2^32 (the error of the reciprocal is below 1 / 2^32)
+    const auto reciprocal = [](long long d, long long most) {
+        return d > 1 && d * most < (1ll << 32) ? (uint32_t)(((1ull << 32) + d - 1) / d) : 0u;
+    };
+    p.img_mul = reciprocal(t.tiles_per_img, i.tiles_m);
+    p.row_mul = reciprocal(t.tiles_w, t.tiles_per_img);
     p.tiles_m = i.tiles_m; p.tiles_n = i.tiles_n; p.FT = t.FT; p.MT = t.MT; p.R = g.kR; p.S = g.kS; p.pad = g.pad_lo; p.pad_w = g.pad_w;
     p.cblks = g.cblks;
     p.ksteps_last = g.ksteps_last;
@@ -1282,6 +1283,8 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
     const bool split_pool = p.pool == CPRUNE_POOL_MAX3X3S2 && t.staging_bufs == 2 && !res && !(plan->opts.flags & CPRUNE_FLAG_POOL_ON_EPILOGUE_WARPS);
     if (t.dense)
         CPRUNE_CUDA_CHECK(launch_chained(conv_patch_kernel<PK_DENSE>, dim3(grid), dim3(pk_threads(PK_DENSE)), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, p));
+    else if (g.flat)
+        CPRUNE_CUDA_CHECK(launch_chained(conv_patch_kernel<PK_FLAT>, dim3(grid), dim3(pk_threads(PK_FLAT)), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, p));
     else if (split_pool)
         CPRUNE_CUDA_CHECK(launch_chained(conv_patch_kernel<PK_POOL3>, dim3(grid), dim3(pk_threads(PK_POOL3)), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, p));
     else
