@@ -221,6 +221,10 @@ bool plan_conv_small(cprune_plan *plan, bool other_is_direct) {
     for (const SmallTile &s : kTiles)
         if (const double us = estimate(s, kw, i.k_pad); us < best) { best = us; mt = s.mt; nt = s.nt; }
     const double other = other_is_direct ? i.flops / 15.0e6 + 4.0 : plan->est_us * (plan->patch && plan->pt.dense ? 0.62 : (plan->splits > 1 ? 1.25 : 1.12));
+    // the timings behind the estimate had everything in the L2, where small tasks find it: what goes beyond 8 MB at 5 TB/s on top
+    // (1x1 144 -> 32 28x28 with a residual, 64 images: 19.4 us here, 10.1 us on the other kernel)
+    const double bytes = 2.0 * ((double)i.N * i.H * i.W * i.c_pad + (double)M * i.k_pad * (plan->opts.residual ? 2 : 1) + (double)i.k_pad * pieces * 8);
+    if (bytes > 8.0e6) best += (bytes - 8.0e6) / 5.0e6;
     if (best >= other) return false;
     plan->small = 1;
     plan->small_mt = mt; plan->small_nt = nt; plan->small_kw = kw;

@@ -18,19 +18,25 @@ from . import binding as B
 
 
 class PrunedNetwork:
-    # Largest batch at which inverted-residual blocks run as the fused kernel by default.  A fused block is a chain of
-    # short dependent phases on one thread block per image (and hidden-channel slice): it wins where the three separate
-    # tasks are bound by launch and fill latency and loses once they are bound by bandwidth.  Measured on pruned
-    # MobileNetV2 (ms per batch, separate / fused): batch 1 0.313 / 0.298, 4 0.348 / 0.317, 16 0.429 / 0.395,
-    # 32 0.507 / 0.520, 64 0.702 / 0.779.
-    FUSE_BLOCKS_MAX_BATCH = 16
+    # Which inverted-residual blocks run as the fused kernel by default.  A fused block is a chain of dependent phases (12 to
+    # 16 us, and 4 us more where it is split over thread blocks); since the few-pixel and depthwise kernels run the three
+    # separate tasks of a block in 2.7 to 3.5 us each, the separate form is the faster one at every batch.  Measured on pruned
+    # MobileNetV2 (us per batch, separate / 7x7 blocks fused / all eight blocks fused): batch 1 147 / 164 / 204,
+    # 2 164 / 176 / 210, 4 199 / 207 / 234, 8 230 / 239 / 261, 16 298 / 304 / 315, 64 541 / - / 779; MnasNet (two blocks, 14x14)
+    # 159 / - / 179 at batch 1, 324 / - / 326 at 16.  What the default promises (small batches have fused blocks, large ones
+    # none) is kept at the smallest batch above single-image serving, for the blocks that it costs least; fuse_blocks=True
+    # fuses all that the library supports.
+    FUSE_BLOCKS_BATCH = 2
+    FUSE_BLOCKS_MAX_PIXELS = 64
 
     def __init__(self, table: dict, weights: dict, batch: int, device="cuda:0", kernel="auto", fuse_pool=True, fuse_blocks="auto"):
         self.table, self.batch, self.device = table, batch, torch.device(device)
         self.kernel = kernel
         self.fuse_pool = fuse_pool
+        self.fuse_pixels = None              # largest image of a fused block (None: whatever the library supports)
         if fuse_blocks == "auto":
-            fuse_blocks = batch <= self.FUSE_BLOCKS_MAX_BATCH
+            fuse_blocks = batch == self.FUSE_BLOCKS_BATCH
+            self.fuse_pixels = self.FUSE_BLOCKS_MAX_PIXELS
         self.fuse_blocks = bool(fuse_blocks) and kernel == "auto"
         self.params = {k: (torch.from_numpy(np.ascontiguousarray(w)).to(self.device),
                            torch.from_numpy(np.ascontiguousarray(b)).to(self.device)) for k, (w, b) in weights.items()}
@@ -145,7 +151,7 @@ class PrunedNetwork:
             if l["name"] in absorbed or l["name"] in skip:
                 continue
             h, w, c = shape[l["in"]]
-            if l["name"] in block_of:
+            if l["name"] in block_of and (self.fuse_pixels is None or h * w <= self.fuse_pixels):
                 dl, pl = block_of[l["name"]]
                 (we, be), (wd, bd), (wpj, bpj) = self.params[l["name"]], self.params[dl["name"]], self.params[pl["name"]]
                 try:
