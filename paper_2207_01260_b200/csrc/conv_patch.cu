@@ -15,13 +15,22 @@
 //
 // The accumulator row of a pixel is its "slot" i * Wp + j (i row in the tile, j column); slots with
 // j >= Q are the S - 1 wrap-around columns: they are computed and thrown away.  A tile has MT
-// blocks of 128 slots (MT = 1 or 2, one accumulator each, both fed by the same filter stage).
+// blocks of 128 slots (MT = 1 or 2, one accumulator each, both fed by the same filter stage).  Of images that fit several times
+// (4x4, 7x7, 8x8) a tile takes whole ones, with the zero borders shared between rows and between images (us, 7x7 at 64 images
+// 512 -> 358 filters 23.9 as im2col, 20.0 here; 4x4 at 128 images 163 -> 301 15.1 and 9.3; 8x8 187 -> 171 13.6 and 12.4, there
+// against one image per tile).
+//
+// What bounds it: the shared-memory port, which per tap of 64 channels carries 4 x (128 + filters) x 32 bytes of MMA operands per
+// block and the filters' own arrival, and the issuing warps.  An MMA warp fetches its instructions alone, two MMAs are pending at
+// most, and every wait, commit and counter between taps is exposed (60 to 220 cycles a tap).  Hence one wait per filter row where
+// two rows of filters fit, and one instantiation per kind of ring and epilogue, which keeps the code between the loops short.
 //
 //   warp 0       patch loads (one per channel block); with a residual, one more load per group of
 //                64 filters brings the residual tile in through the same ring;
 //   warps 1, 2   filter loads, one per (channel block, tap), taken in turn; small filter sets
 //                stay resident in shared memory for the whole kernel;
-//   warps 3, 12  tcgen05.mma issue (3 and 20 with sixteen epilogue warps), one warp per accumulator block; the residual tile is added by
+//   warps 3, 12  tcgen05.mma issue (3 and 20 with sixteen epilogue warps), one warp per accumulator
+//                block; the residual tile is added by
 //                one more MMA against a 64 x 64 identity held in shared memory (bf16 x 1.0 into an
 //                fp32 accumulator is exact), so the epilogue never touches global memory for it
 //                (the 1x1 instantiation, whose tile is flat, still adds it in the epilogue);
@@ -45,7 +54,7 @@ namespace cprune {
 
 constexpr int PK_POOL_WARPS = 8;          // 3x3-pool kernel: these warps pool the staged tile while the epilogue warps stage the next one
 // kernel instantiations
-constexpr int PK_GENERAL = 0, PK_DENSE = 1, PK_POOL3 = 2, PK_FLAT = 3;
+constexpr int PK_GENERAL = 0, PK_DENSE = 1, PK_POOL3 = 2, PK_FLAT = 3, PK_TAPS = 4;
 // Epilogue warps.  A flat tile has little for the MMAs to do, so its epilogue bounds it: a warp spends about 300 cycles on 16
 // filters of 128 pixels, mostly the latencies of a chain of 50 instructions, and sixteen warps hide twice as many of them as
 // eight (64 images, 1x1 24 -> 108 of 56x56: 23.1 -> 19.9 us; 32 -> 16 of 112x112: 26.3 -> 19.1 us).  The other tasks are bound by
@@ -67,6 +76,7 @@ struct PatchParams {
     int TW, tiles_w, step_h, step_w, org;   // tile (ty, tx) starts at output (ty * step_h + org, tx * step_w + org) and spans TH x TW
     int out_h, out_w;                       // stored extent (after a fused pool)
     int FT, MT, R, S, pad, pad_w, cblks, ksteps_last, k_pad;   // pad: rows above the image in a patch; pad_w: columns left of it
+    int wgroup;            // taps that share a filter barrier: a filter row, or one
     int act, wstages, pstages, resident, acc_bufs, staging_bufs, pool;
     int patch_bytes;       // shared memory of one patch stage
     int patch_box_bytes;   // bytes one patch load delivers
@@ -76,6 +86,7 @@ struct PatchParams {
     int dense_pitch;       // ... bytes per slot in the staging buffer: k_pad * 2, or 16 more (then the tile leaves by a tiled copy)
     int stage_bytes;       // shared memory of one staging buffer
     int flat;              // 1x1 tasks: one image of one row
+    int ipt, imgs;         // whole images per tile (0: tiles of one image), images of the task
     uint32_t img_mul, row_mul;   // ceil(2^32 / tiles_per_img), ceil(2^32 / tiles_w), or 0
     int res_blocks;        // residual added on the tensor core: 64-filter blocks of the residual tile per item (0: none)
     const float *bias;
@@ -153,9 +164,9 @@ __device__ __forceinline__ void issue_tap(uint32_t d_tmem, uint32_t a_lo, uint32
     __syncwarp();
 }
 
-// A whole filter row (S taps) from one elected block: used when nothing has to be waited for between taps.
+// A whole filter row (S taps) from one elected block: nothing has to be waited for between its taps.
 __device__ __forceinline__ void issue_row(uint32_t d_tmem, uint32_t a_lo, uint32_t w_lo, uint32_t desc_hi, uint32_t idesc,
-                                          uint32_t accumulate, int nk, int S, uint32_t slot_step, uint32_t w_step, uint32_t commit_p) {
+                                          uint32_t accumulate, int nk, int S, uint32_t slot_step, uint32_t w_step, uint32_t commit_w, uint32_t commit_p) {
     if (elect_one()) {
         for (int s = 0; s < S; ++s) {
             if (nk == 4) {
@@ -171,6 +182,7 @@ __device__ __forceinline__ void issue_row(uint32_t d_tmem, uint32_t a_lo, uint32
             accumulate = 1;
             a_lo += slot_step;
             w_lo += w_step;
+            if (commit_w) { umma_commit(commit_w); commit_w += 8u; }     // every tap frees its own stage
         }
         if (commit_p) umma_commit(commit_p);
     }
@@ -186,6 +198,10 @@ __device__ __forceinline__ void tile_origin(const PatchParams &p, int tm, int &n
         n = 0; p0 = 0; q0 = tm * p.step_w;
         return;
     }
+    if (p.ipt) {
+        n = tm * p.ipt; p0 = 0; q0 = 0;
+        return;
+    }
     n = quotient(tm, p.tiles_per_img, p.img_mul);
     const int r = tm - n * p.tiles_per_img;
     int ty = r, tx = 0;
@@ -194,7 +210,7 @@ __device__ __forceinline__ void tile_origin(const PatchParams &p, int tm, int &n
     q0 = tx * p.step_w + p.org;
 }
 
-template <int MODE>
+template <int MODE, bool POOLED = false>
 __global__ void __launch_bounds__(pk_threads(MODE), 1)
 conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                   const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_res, const PatchParams p) {
@@ -250,7 +266,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         if (l < 2) { mbar_init(tfull(l), p.MT); mbar_init(tempty(l), EPI_WARPS); mbar_init(res_full(l), 1); }
         if (l == 2) { mbar_init(epi_bar, EPI_WARPS); *abort_flag = 0; }
         if (SPLIT && l >= 4 && l < 6) { mbar_init(sfull(l - 4), EPI_WARPS); mbar_init(sempty(l - 4), PK_POOL_WARPS); }
-        if (l < p.wstages) { mbar_init(wfull(l), 1); mbar_init(wempty(l), p.MT); }
+        if (l < p.wstages) { mbar_init(wfull(l), p.wgroup); mbar_init(wempty(l), p.MT); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // the bias (written when the task was packed, not by the preceding kernel) in shared memory: a read costs the
@@ -275,13 +291,26 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         }
         fence_async_smem();
     }
+    // Stacked images: each one's bottom and right border is the top border of the next and the left border of the next row.
+    // What the last one lacks follows its patch in the stage and is cleared once (no load writes there).
+    if (p.ipt) {
+        const uint32_t tail = (uint32_t)(p.pad * p.Wp + p.pad) * 8u;      // 16-byte pieces
+        for (uint32_t e = threadIdx.x; e < (uint32_t)p.pstages * tail; e += blockDim.x) {
+            const uint32_t st = e / tail, q = e - st * tail;
+            *(uint4 *)(smem + (patch0 - base) + st * (uint32_t)p.patch_bytes + (uint32_t)p.patch_box_bytes + q * 16u) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        fence_async_smem();
+    }
     // slot table: which accumulator rows hold real output pixels and where they go
-    for (int e = threadIdx.x; e < 256 && p.pool == 1; e += blockDim.x) {
+    for (int e = threadIdx.x; POOLED && e < 256 && p.pool == 1; e += blockDim.x) {
         int2 v = make_int2(-1, 0);
         {
             const int hq = p.Q >> 1;
             const int i2 = e / hq, j2 = e - i2 * hq;
-            if (i2 < (p.TH >> 1)) v = make_int2((2 * i2 * p.Wp + 2 * j2) | ((2 * i2) << 16), (i2 * hq + j2) * p.k_pad);
+            if (p.ipt) {           // the "row" that decides whether the pixel is stored is the image
+                const int hp = p.P >> 1, im = i2 / hp, ii = i2 - im * hp;
+                if (im < p.ipt) v = make_int2(((im * (p.P + p.pad) + 2 * ii) * p.Wp + 2 * j2) | (im << 16), e * p.k_pad);
+            } else if (i2 < (p.TH >> 1)) v = make_int2((2 * i2 * p.Wp + 2 * j2) | ((2 * i2) << 16), (i2 * hq + j2) * p.k_pad);
         }
         lut[e] = v;
     }
@@ -335,7 +364,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         }
     } else if (warp < PK_MMA_WARP) {
         // ------------------------------------------------------------------ filter loads
-        int ws = 0, turn = 0;
+        int ws = 0, wsub = 0, turn = 0;
         uint32_t wphase = 0;
         bool ok = true;
         const int me = warp - 1;
@@ -352,11 +381,13 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                         if (!p.resident) ok = __all_sync(0xffffffffu, mbar_wait(wempty(ws), wphase ^ 1u, abort_flag, p.status));
                         if (!ok) break;
                         if (elect_one()) {
-                            mbar_expect_tx(wfull(ws), w_tx_bytes);
-                            tma_load_3d(w0 + (uint32_t)ws * w_bytes, &tm_w, wfull(ws), cb * 64, tap, k0);
+                            const uint32_t wb = wfull(MODE == PK_GENERAL ? ws - wsub : ws);   // the taps of a row complete one barrier
+                            mbar_expect_tx(wb, w_tx_bytes);
+                            tma_load_3d(w0 + (uint32_t)ws * w_bytes, &tm_w, wb, cb * 64, tap, k0);
                         }
                         __syncwarp();
                     }
+                    if (MODE == PK_GENERAL && ++wsub == p.wgroup) wsub = 0;
                     if (++ws == p.wstages) { ws = 0; wphase ^= 1u; }
                 }
             }
@@ -391,15 +422,28 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 if (!ok) break;
                 const int nk = cb == p.cblks - 1 ? p.ksteps_last : 4;
                 uint32_t tap_lo = patch_lo + (uint32_t)(mb * 128) * slot_step;      // the second block's slots follow the first's
-                if (p.resident && item != (int)blockIdx.x) {
+                if (MODE != PK_TAPS && p.resident && item != (int)blockIdx.x) {
                     // resident filters, loaded during the first tile: nothing to wait for, a filter row per elected block
                     for (int r = 0; r < p.R; ++r) {
-                        issue_row(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, p.S, slot_step, w_step, r == p.R - 1 ? pempty(ps) : 0u);
+                        issue_row(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, p.S, slot_step, w_step, 0u, r == p.R - 1 ? pempty(ps) : 0u);
                         accumulate = 1;
                         tap_lo += (uint32_t)p.Wp * slot_step;
                         w_lo += (uint32_t)p.S * w_step;
                         ws += p.S;
                         if (ws == p.wstages) { ws = 0; w_lo = w_lo0; }
+                    }
+                } else if constexpr (MODE == PK_GENERAL) {
+                    // one wait per filter row, then the row's MMAs from one elected block; every tap frees its own stage
+                    for (int r = 0; r < p.R; ++r) {
+                        ok = __all_sync(0xffffffffu, mbar_wait(wfull(ws), p.resident ? 0u : wphase, abort_flag, p.status));
+                        if (!ok) break;
+                        issue_row(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, p.S, slot_step, w_step, p.resident ? 0u : wempty(ws),
+                                  r == p.R - 1 ? pempty(ps) : 0u);
+                        accumulate = 1;
+                        tap_lo += (uint32_t)p.Wp * slot_step;
+                        w_lo += (uint32_t)p.S * w_step;
+                        ws += p.S;
+                        if (ws == p.wstages) { ws = 0; wphase ^= 1u; w_lo = w_lo0; }
                     }
                 } else {
                     int s = 0;
@@ -550,7 +594,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 bias_r[j] = c + j * 2 < k_all ? *reinterpret_cast<const unsigned long long *>(bias_src + c + j * 2) : 0ull;
         };
         if (bias_const) load_bias(sub * WCOLS);
-        const int n_entries = p.pool == 1 ? (p.TH >> 1) * (p.Q >> 1) : ((p.TH - 1) >> 1) * ((p.TW - 1) >> 1);
+        const int n_entries = p.ipt ? p.ipt * (p.P >> 1) * (p.Q >> 1) : p.pool == 1 ? (p.TH >> 1) * (p.Q >> 1) : ((p.TH - 1) >> 1) * ((p.TW - 1) >> 1);
         // Residuals.  Everywhere but with dense staging the MMA warps add the residual on the tensor core (see there) and
         // the epilogue has nothing to do with it.  Dense staging: the residual of tile item_ (tiles_n == 1, one row of
         // tiles) is one contiguous range of memory, arrives in the staging buffer the tile will use and is added in place.
@@ -581,7 +625,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             int n, p0, q0;
             tile_origin(p, tm, n, p0, q0);
             const int k0 = nt * p.FT;
-            const int rows_valid = p.P - p0;                 // tile rows below this are real image rows
+            const int rows_valid = p.ipt ? p.imgs - n : p.P - p0;    // tile rows (or images) below this are real ones
             // first pooled pixel of the tile (2x2 pool: full-width tiles from an even row)
             __nv_bfloat16 *ytile = p.pool == 1 ? p.y + ((size_t)n * (p.P >> 1) + (p0 >> 1)) * (p.Q >> 1) * p.k_pad : nullptr;
             ok = __all_sync(0xffffffffu, mbar_wait(tfull(acc), acc_phase, abort_flag, p.status, false));
@@ -691,7 +735,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                     ++group_counter;
                     continue;
                 }
-                if (!p.pool) {
+                if constexpr (!POOLED) {
                     // one TMA store per group: the staged slots are TH rows of Wp pixels; the tensor map's box has
                     // that shape, and the wrap-around columns (j >= Q), rows below the image and filters beyond
                     // k_pad fall outside the tensor, where a store writes nothing
@@ -710,8 +754,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                         if (!ok) break;
                     }
                     ++group_counter;
-                    continue;
-                }
+                } else {
                 ok = epi_sync();
                 if (!ok) break;
                 // copy-out: eight threads per output pixel, 16 bytes each
@@ -772,6 +815,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                     if (!ok) break;
                 }
                 ++group_counter;
+                }
             }
             }
             if (p.acc_bufs == 2) { if (++acc == 2) { acc = 0; acc_phase ^= 1u; } }
@@ -890,10 +934,22 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
     PatchTiling bt = {};
     for (int MT = 1; MT <= 2; ++MT) {
       // candidate tile shapes: whole-width rows; for the 3x3 pool (2 tpr + 1) x (2 tpc + 1) conv pixels around tpr x tpc pooled ones
-      const int n_shapes = pool3 ? 32 * 32 : 1;
+      // and whole images next to each other where several fit
+      const int n_shapes = pool3 ? 32 * 32 : 2;
       for (int shape = 0; shape < n_shapes; ++shape) {
+        int ipt = 0;
         int TH, TW = g.vQ, tiles_w = 1, step_h, step_w = g.vQ, org = 0, tiles_per_img, Wp = g.Wp;
-        if (g.flat) {
+        if (!pool3 && shape == 1) {
+            // small images (7x7: four to 256 slots): a pixel row is W + pad slots, an image (H + pad) rows, and each border is
+            // shared by the two rows or images that it lies between
+            if (g.flat || g.stem || i.R != i.S || (i.R & 1) == 0 || i.pad != i.R / 2) continue;
+            Wp = g.vQ + i.pad;
+            ipt = 128 * MT / ((g.vP + i.pad) * Wp);
+            if (ipt < 2) continue;
+            TH = (g.vP + i.pad) * ipt;
+            step_h = TH;
+            tiles_per_img = 1;
+        } else if (g.flat) {
             TH = 1; TW = 128 * MT; Wp = TW; step_h = 1; step_w = TW;
             tiles_w = (g.vQ + TW - 1) / TW;
             tiles_per_img = tiles_w;
@@ -922,7 +978,7 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
             if ((k16 + FT - 1) / FT != tiles_n) continue;
             const int acc_bufs = 2 * MT * FT <= 512 ? 2 : 1;
             const int patch_bytes = round_up((128 * MT + (g.kR - 1) * Wp + g.kS - 1) * RB, 1024);
-            if (patch_bytes < Wp * (TH + g.kR - 1) * RB) continue;
+            if (!ipt && patch_bytes < Wp * (TH + g.kR - 1) * RB) continue;
             // patch ring depth: two stages; up to four when the task has that many channel blocks and the patches are
             // small (1x1 tasks), because each load's latency is otherwise exposed
             // (flat tasks: a tile is little work, and a patch load's latency under a stream of output writes is several
@@ -951,47 +1007,56 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
             // with the pixel pitch made an odd number of 16-byte pieces (no bank conflicts between neighbouring pixels;
             // 32-byte pixels conflict two-way and still gain, measured)
             const int stage_bytes = dense ? dense_bytes : MT * PK_BLOCK_BYTES;
-            int staging_bufs = sb_max, wstages = 0, resident = 0;
+            int staging_bufs = sb_max, wstages = 0, resident = 0, wgroup = g.kS;
             // resident filters when the whole set of this filter tile fits
-            const int sb_res_min = sb_min;
             if (tiles_n == 1 && RS * cblks <= PK_MAX_WSTAGES) {
-                for (int sb = sb_max; sb >= sb_res_min && !resident; --sb)
+                for (int sb = sb_max; sb >= sb_min && !resident; --sb)
                     if (RS * cblks * w_stage + sb * stage_bytes <= budget) { resident = 1; staging_bufs = sb; wstages = RS * cblks; }
             }
             if (!resident) {
-                staging_bufs = sb_max;
-                wstages = (budget - staging_bufs * stage_bytes) / w_stage;
-                if (wstages < 3 && sb_min < sb_max) {
-                    staging_bufs = sb_min;
-                    wstages = (budget - staging_bufs * stage_bytes) / w_stage;
+                // Streamed filters: a ring of filter rows, at least two, with one barrier each (3x3 301 -> 250 4x4 at 128 images
+                // 12.2 us, tap by tap 14.8; 128 -> 89 28x28 at 64 images 17.8 and 19.4).  Taps one by one only where two rows do
+                // not fit (256 filters, for instance), or where the patch ring had to become shallower for it at no gain.
+                for (staging_bufs = sb_max; staging_bufs > sb_min && (budget - staging_bufs * stage_bytes) / w_stage < 2 * wgroup;) --staging_bufs;
+                if ((budget - staging_bufs * stage_bytes) / w_stage < 2 * wgroup) {
+                    wgroup = 1;
+                    for (staging_bufs = sb_max; staging_bufs > sb_min && (budget - staging_bufs * stage_bytes) / w_stage < 3;) --staging_bufs;
                 }
+                wstages = (budget - staging_bufs * stage_bytes) / w_stage;
                 if (wstages < 3) continue;
-                if (wstages > 8) wstages = 8;
+                if (wstages > 12) wstages = 12;
+                wstages -= wstages % wgroup;
             }
             if (dense && staging_bufs != 2) continue;
             // the fused 3x3 pool runs on its own warps only beside two staging buffers, which is worth more than a deeper ring
             if (pool3 && staging_bufs != 2 && pstages > 2) continue;
-            const long long tiles = (long long)g.vN * tiles_per_img * tiles_n;
+            const long long tiles = (ipt ? ceil_div(g.vN, ipt) : (long long)g.vN * tiles_per_img) * tiles_n;
             const double waves = (double)((tiles + 147) / 148);
             double tile = tile_cycles(MT, FT, RS, cblks, ksteps_last, RB, Wp, TH, g.kR, resident != 0, acc_bufs);
+            // between two filter barriers the tensor pipe idles for as long as its queue of two MMAs is shorter than a wait
+            // (measured: 221 cycles with 64 filters, 117 with 128, 65 with 192; the second issuing warp hides most of it)
+            if (!resident && !g.flat) tile += cblks * (RS / wgroup) * (MT == 2 ? 60.0 : FT < 200 ? 280.0 - 1.2 * FT : 40.0);
+            if (ipt) tile -= cblks * Wp * (g.kR - 1) * RB / 128.0;     // (no border rows beside the TH counted)
             if (res_blocks_plan && !dense) tile += res_blocks_plan * (MT * 4 * 48.0 + TH * Wp);   // residual MMAs and their loads
             double t = waves * tile;
             if (resident) t += RS * cblks * FT;    // one-time filter load
+            if (staging_bufs == 1 && !g.flat) t += ((FT + 63) / 64) * 900.0;     // the last tile's stores, one after the other
             if (t < best) {
                 best = t;
-                bt = {MT, TH, FT, tiles_n, tiles_per_img, wstages, resident, acc_bufs, staging_bufs, patch_bytes, TW, tiles_w, step_h, step_w, org, pstages, dense, stage_bytes, dense_pitch};
+                bt = {MT, TH, FT, tiles_n, tiles_per_img, wstages, resident, acc_bufs, staging_bufs, patch_bytes, TW, tiles_w, step_h, step_w, org, pstages, dense, stage_bytes, dense_pitch, ipt, wgroup};
             }
-            break;      // the deepest ring that fits
+            if (resident || wgroup == g.kS) break;      // the deepest patch ring beside which the filters fit
           }
         }
       }
     }
     if (best >= 1e30) return CPRUNE_ERR_UNSUPPORTED;
     // share of accumulator rows that hold real pixels; below one half the im2col kernel is the better choice
-    const double fill = (double)g.vP * g.vQ / ((double)bt.tiles_per_img * 128 * bt.MT);
+    const long long tiles_m = bt.ipt ? ceil_div(g.vN, bt.ipt) : (long long)g.vN * bt.tiles_per_img;
+    const double fill = (double)g.vP * g.vQ * g.vN / ((double)tiles_m * 128 * bt.MT);
     if (fill < 0.5) return CPRUNE_ERR_UNSUPPORTED;
     // too few tiles for the SMs: the im2col kernel can split the reduction over more CTAs
-    if ((long long)g.vN * bt.tiles_per_img * bt.tiles_n < 64) return CPRUNE_ERR_UNSUPPORTED;
+    if (tiles_m * bt.tiles_n < 64) return CPRUNE_ERR_UNSUPPORTED;
     plan->patch = 1;
     plan->pt = bt;
     plan->narrow = g.stem;
@@ -1007,7 +1072,7 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
     i.tile_n = bt.FT;
     i.tile_k = 64;
     i.stages = bt.wstages;
-    i.tiles_m = g.vN * bt.tiles_per_img;
+    i.tiles_m = (int)tiles_m;
     i.tiles_n = bt.tiles_n;
     i.k_alloc = bt.tiles_n * bt.FT;
     const int ksteps = (cblks - 1) * 4 + ksteps_last;
@@ -1153,7 +1218,10 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
     const PatchTiling &t = plan->pt;
     PatchGeometry g;
     if (!patch_geometry(i, &g)) return CPRUNE_ERR_INTERNAL;
-    const int Wp = t.TW + g.kS - 1;    // patch row pitch: the tile's width plus the filter's
+    // patch row pitch: the tile's width plus the filter's; with stacked images a border column is shared by two rows
+    const int Wp = t.ipt ? t.TW + i.pad : t.TW + g.kS - 1;
+    const unsigned box_rows = t.ipt ? (unsigned)(i.P + i.pad) : (unsigned)(t.TH + g.kR - 1), box_out = t.ipt ? box_rows : (unsigned)t.TH;
+    const unsigned box_imgs = t.ipt ? (unsigned)t.ipt : 1u;
     const void *xe = x;        // the tensor the patch loads read
     if (g.stem) {
         if (!scratch) return CPRUNE_ERR_INVALID_ARG;
@@ -1179,7 +1247,7 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
                                                     (unsigned long long)g.vN};
                 const unsigned long long strides[3] = {(unsigned long long)i.c_pad * 2, (unsigned long long)g.vW * i.c_pad * 2,
                                                        (unsigned long long)g.vH * g.vW * i.c_pad * 2};
-                const unsigned box[4] = {64, (unsigned)Wp, (unsigned)(t.TH + g.kR - 1), 1};
+                const unsigned box[4] = {64, (unsigned)Wp, box_rows, box_imgs};
                 cprune_status s = encode_tiled_bf16_swz(&plan->tm_a, xe, 4, dims, strides, box, 128, true);
                 if (s != CPRUNE_OK) return s;
             }
@@ -1205,7 +1273,7 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
                                                    (unsigned long long)g.vOH * g.vOW * i.k_pad * 2};
             const bool dense_tiled = t.dense && t.dense_pitch != i.k_pad * 2;      // the whole staged tile, unswizzled
             const unsigned box[4] = {dense_tiled ? (unsigned)(t.dense_pitch / 2) : 64u, dense_tiled ? (unsigned)t.TW : (unsigned)Wp,
-                                     dense_tiled ? 1u : (unsigned)t.TH, 1};
+                                     dense_tiled ? 1u : box_out, box_imgs};
             cprune_status s = encode_tiled_bf16_swz(&plan->tm_y, y, 4, dims, strides, box, dense_tiled ? 0 : 128, false);
             if (s != CPRUNE_OK) return s;
             plan->map_y = y;
@@ -1217,7 +1285,7 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
                                                    (unsigned long long)g.vP * g.vQ * i.k_pad * 2};
             const bool dense_tiled = t.dense && t.dense_pitch != i.k_pad * 2;
             const unsigned box[4] = {dense_tiled ? (unsigned)(t.dense_pitch / 2) : 64u, dense_tiled ? (unsigned)t.TW : (unsigned)Wp,
-                                     dense_tiled ? 1u : (unsigned)t.TH, 1};
+                                     dense_tiled ? 1u : box_out, box_imgs};
             cprune_status s = encode_tiled_bf16_swz(&plan->tm_res, res, 4, dims, strides, box, dense_tiled ? 0 : 128, true);
             if (s != CPRUNE_OK) return s;
             plan->map_res = res;
@@ -1236,10 +1304,11 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
         if (dev < 0 || dev >= 64) return CPRUNE_ERR_UNSUPPORTED;
         std::lock_guard<std::mutex> lock(attr_mu);
         if (!attr_set[dev]) {
-            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(conv_patch_kernel<PK_GENERAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(conv_patch_kernel<PK_FLAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(conv_patch_kernel<PK_DENSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(conv_patch_kernel<PK_POOL3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+            const void *kernels[] = {(const void *)conv_patch_kernel<PK_GENERAL, false>, (const void *)conv_patch_kernel<PK_GENERAL, true>,
+                                     (const void *)conv_patch_kernel<PK_TAPS, false>,    (const void *)conv_patch_kernel<PK_TAPS, true>,
+                                     (const void *)conv_patch_kernel<PK_FLAT>,           (const void *)conv_patch_kernel<PK_DENSE>,
+                                     (const void *)conv_patch_kernel<PK_POOL3>};
+            for (const void *k : kernels) CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
             attr_set[dev] = true;
         }
     }
@@ -1248,6 +1317,7 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
     p.TW = t.TW; p.tiles_w = t.tiles_w; p.step_h = t.step_h; p.step_w = t.step_w; p.org = t.org;
     p.out_h = g.vOH; p.out_w = g.vOW;
     p.flat = g.flat;
+    p.ipt = t.ipt; p.imgs = g.vN;
     // v * ceil(2^32 / d) / 2^32 has the integer part v / d as long as v * d < 2^32 (the error of the reciprocal is below 1 / 2^32)
     const auto reciprocal = [](long long d, long long most) {
         return d > 1 && d * most < (1ll << 32) ? (uint32_t)(((1ull << 32) + d - 1) / d) : 0u;
@@ -1259,10 +1329,10 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
     p.ksteps_last = g.ksteps_last;
     p.k_pad = i.k_pad;
     p.act = plan->opts.activation;
-    p.wstages = t.wstages; p.pstages = t.pstages; p.resident = t.resident; p.acc_bufs = t.acc_bufs; p.staging_bufs = t.staging_bufs;
+    p.wgroup = t.wgroup; p.wstages = t.wstages; p.pstages = t.pstages; p.resident = t.resident; p.acc_bufs = t.acc_bufs; p.staging_bufs = t.staging_bufs;
     p.pool = plan->fused_pool ? plan->opts.pool : 0;
     p.patch_bytes = t.patch_bytes;
-    p.patch_box_bytes = Wp * (t.TH + g.kR - 1) * 128;
+    p.patch_box_bytes = Wp * (int)(box_rows * box_imgs) * 128;
     p.rb16 = 8;
     p.dense = t.dense; p.stage_bytes = t.stage_bytes; p.dense_pitch = t.dense_pitch;
     p.w_stage_bytes = t.FT * 128;
@@ -1281,14 +1351,20 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
     const int grid = total < sms ? total : sms;
     // a fused 3x3 pool with two staging buffers: the instantiation with separate pooling warps
     const bool split_pool = p.pool == CPRUNE_POOL_MAX3X3S2 && t.staging_bufs == 2 && !res && !(plan->opts.flags & CPRUNE_FLAG_POOL_ON_EPILOGUE_WARPS);
-    if (t.dense)
-        CPRUNE_CUDA_CHECK(launch_chained(conv_patch_kernel<PK_DENSE>, dim3(grid), dim3(pk_threads(PK_DENSE)), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, p));
-    else if (g.flat)
-        CPRUNE_CUDA_CHECK(launch_chained(conv_patch_kernel<PK_FLAT>, dim3(grid), dim3(pk_threads(PK_FLAT)), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, p));
-    else if (split_pool)
-        CPRUNE_CUDA_CHECK(launch_chained(conv_patch_kernel<PK_POOL3>, dim3(grid), dim3(pk_threads(PK_POOL3)), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, p));
-    else
-        CPRUNE_CUDA_CHECK(launch_chained(conv_patch_kernel<PK_GENERAL>, dim3(grid), dim3(pk_threads(PK_GENERAL)), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, p));
+    // One instantiation per kind of epilogue and of filter ring: a role is one warp that fetches its instructions alone, and each
+    // of them is faster the less code lies between its loops (64 images: 1x1 24 -> 108 56x56 20.2 -> 17.8 us, 96 -> 432 14x14 10.7 ->
+    // 10.0 us, 3x3 131 -> 203 28x28 37.0 -> 36.3 us).
+    const auto launch = [&](auto kernel, int mode) {
+        return launch_chained(kernel, dim3(grid), dim3(pk_threads(mode)), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, p);
+    };
+    const bool taps = t.wgroup == 1 && !t.resident;
+    if (t.dense) CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_DENSE>, PK_DENSE));
+    else if (g.flat) CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_FLAT>, PK_FLAT));
+    else if (split_pool) CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_POOL3>, PK_POOL3));
+    else if (taps && p.pool) CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_TAPS, true>, PK_TAPS));
+    else if (taps) CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_TAPS, false>, PK_TAPS));
+    else if (p.pool) CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_GENERAL, true>, PK_GENERAL));
+    else CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_GENERAL, false>, PK_GENERAL));
     return CPRUNE_OK;
 }
 

@@ -18,6 +18,8 @@ struct PatchTiling {
     int dense;                              // flat tasks: a tile's output is staged as it lies in memory and stored by one bulk copy
     int stage_bytes;                        // shared memory of one staging buffer
     int dense_pitch;                        // dense staging: bytes between neighbouring pixels in the staging buffer
+    int ipt;                                // whole images per tile where several fit (0: tiles are rows of one image)
+    int wgroup;                             // filter taps under one barrier of the filter ring
 };
 
 // Tiling of the depthwise kernel (depthwise.cu)

@@ -255,6 +255,19 @@ def test_few_pixel_tasks(cp, case):
     assert (plan.variant == 3) == (C < 1536) and (plan.variant != 3 or plan.workspace_bytes == 0)
 
 
+@pytest.mark.parametrize("case", [
+    # N, C, H, W, K, R, act, residual, pool, M tiles: whole images side by side (last tile ragged, images not square, filters of
+    # one and two border pixels, two channel blocks, residual of two 64-filter groups, pooled), then tiles of image rows with
+    # streamed filters, a filter row and a tap at a time, the last channel block of one MMA step
+    (321, 24, 4, 4, 40, 3, "relu", False, None, 65), (129, 72, 7, 7, 72, 3, "none", True, None, 65), (193, 16, 7, 7, 24, 5, "relu6", False, None, 65),
+    (331, 40, 3, 5, 16, 3, "relu", False, None, 67), (193, 20, 8, 8, 24, 3, "none", False, "max2x2", 65), (385, 136, 4, 4, 130, 3, "relu", True, None, 39),
+    (10, 136, 28, 28, 120, 3, "relu", True, None, 70), (10, 40, 28, 28, 208, 5, "none", False, None, 70)])
+def test_patch_tiles_of_whole_images_and_streamed_filter_rows(cp, case):
+    N, C, H, W, K, R, act, res, pool, tiles = case
+    plan = check_task(cp, N, C, H, W, K, R, 1, R // 2, act=act, with_res=res, pool=pool, kernel="tensor")
+    assert plan.variant == 1 and plan.tiles_m == tiles
+
+
 def test_stems_on_the_patch_kernel(cp):
     # enough tiles for the patch kernel: the input is regrouped into 16-channel pixels (stride 1 and 2)
     plan = check_task(cp, 16, 3, 64, 64, 64, 7, 2, 3, kernel="tensor")
