@@ -17,7 +17,7 @@
 // j >= Q are the S - 1 wrap-around columns: they are computed and thrown away.  A tile has MT
 // blocks of 128 slots (MT = 1 or 2, one accumulator each, both fed by the same filter stage).  Of images that fit several times
 // (4x4, 7x7, 8x8) a tile takes whole ones, with the zero borders shared between rows and between images (us, 7x7 at 64 images
-// 512 -> 358 filters 23.9 as im2col, 20.0 here; 4x4 at 128 images 163 -> 301 15.1 and 9.3; 8x8 187 -> 171 13.6 and 12.4, there
+// 512 -> 358 filters 23.9 as im2col, 18.2 here; 4x4 at 128 images 301 -> 250 14.7 and 11.0; 8x8 187 -> 171 13.6 and 11.9, there
 // against one image per tile).
 //
 // What bounds it: the shared-memory port, which per tap of 64 channels carries 4 x (128 + filters) x 32 bytes of MMA operands per
@@ -53,7 +53,8 @@
 namespace cprune {
 
 constexpr int PK_POOL_WARPS = 8;          // 3x3-pool kernel: these warps pool the staged tile while the epilogue warps stage the next one
-// kernel instantiations
+// kernel instantiations: 3x3 and other R x S > 1 with resident filters or a ring of filter rows, 1x1 staged as in memory, fused
+// 3x3 pool on its own warps, other 1x1, and R x S > 1 with a ring of taps
 constexpr int PK_GENERAL = 0, PK_DENSE = 1, PK_POOL3 = 2, PK_FLAT = 3, PK_TAPS = 4;
 // Epilogue warps.  A flat tile has little for the MMAs to do, so its epilogue bounds it: a warp spends about 300 cycles on 16
 // filters of 128 pixels, mostly the latencies of a chain of 50 instructions, and sixteen warps hide twice as many of them as
@@ -85,7 +86,6 @@ struct PatchParams {
     int dense;             // the staged tile is [slot][k_pad] as in memory and leaves by one bulk copy (flat tasks, one filter tile)
     int dense_pitch;       // ... bytes per slot in the staging buffer: k_pad * 2, or 16 more (then the tile leaves by a tiled copy)
     int stage_bytes;       // shared memory of one staging buffer
-    int flat;              // 1x1 tasks: one image of one row
     int ipt, imgs;         // whole images per tile (0: tiles of one image), images of the task
     uint32_t img_mul, row_mul;   // ceil(2^32 / tiles_per_img), ceil(2^32 / tiles_w), or 0
     int res_blocks;        // residual added on the tensor core: 64-filter blocks of the residual tile per item (0: none)
@@ -193,8 +193,9 @@ __device__ __forceinline__ void issue_row(uint32_t d_tmem, uint32_t a_lo, uint32
 // pixels) and image of tile tm.  The divisions are multiplications with reciprocals that the host has checked for every
 // tile number (mul == 0: by division); flat tasks (one image, one row of tiles) need none.
 __device__ __forceinline__ int quotient(int v, int d, uint32_t mul) { return mul ? (int)__umulhi((uint32_t)v, mul) : v / d; }
+template <bool FLAT>
 __device__ __forceinline__ void tile_origin(const PatchParams &p, int tm, int &n, int &p0, int &q0) {
-    if (p.flat) {
+    if (FLAT) {
         n = 0; p0 = 0; q0 = tm * p.step_w;
         return;
     }
@@ -210,7 +211,7 @@ __device__ __forceinline__ void tile_origin(const PatchParams &p, int tm, int &n
     q0 = tx * p.step_w + p.org;
 }
 
-template <int MODE, bool POOLED = false>
+template <int MODE, bool RESIDENT, bool POOLED = false, int WIDTH = 0>
 __global__ void __launch_bounds__(pk_threads(MODE), 1)
 conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                   const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_res, const PatchParams p) {
@@ -256,7 +257,9 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     // the shuffle tells the compiler that the warp number is the same in all lanes, so that the role code below
     // (loop counters, descriptors, TMA coordinates) can live in uniform registers
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const int RS = p.R * p.S;
+    constexpr bool FLAT = MODE == PK_DENSE || MODE == PK_FLAT;      // 1x1 tasks: one image of one row
+    const int FR = FLAT ? 1 : WIDTH ? WIDTH : p.R, FS = FLAT || SPLIT ? 1 : WIDTH ? WIDTH : p.S, RS = FR * FS;
+    const int ipt = FLAT || SPLIT ? 0 : p.ipt;
 
     // barrier set-up, spread over the lanes of warp 0 (one thread doing up to 70 initialisations costs microseconds).
     // Every accumulator block has its own issuing warp: stages are free, and a tile is complete, once all have committed.
@@ -293,7 +296,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     }
     // Stacked images: each one's bottom and right border is the top border of the next and the left border of the next row.
     // What the last one lacks follows its patch in the stage and is cleared once (no load writes there).
-    if (p.ipt) {
+    if (ipt) {
         const uint32_t tail = (uint32_t)(p.pad * p.Wp + p.pad) * 8u;      // 16-byte pieces
         for (uint32_t e = threadIdx.x; e < (uint32_t)p.pstages * tail; e += blockDim.x) {
             const uint32_t st = e / tail, q = e - st * tail;
@@ -307,9 +310,9 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         {
             const int hq = p.Q >> 1;
             const int i2 = e / hq, j2 = e - i2 * hq;
-            if (p.ipt) {           // the "row" that decides whether the pixel is stored is the image
+            if (ipt) {           // the "row" that decides whether the pixel is stored is the image
                 const int hp = p.P >> 1, im = i2 / hp, ii = i2 - im * hp;
-                if (im < p.ipt) v = make_int2(((im * (p.P + p.pad) + 2 * ii) * p.Wp + 2 * j2) | (im << 16), e * p.k_pad);
+                if (im < ipt) v = make_int2(((im * (p.P + p.pad) + 2 * ii) * p.Wp + 2 * j2) | (im << 16), e * p.k_pad);
             } else if (i2 < (p.TH >> 1)) v = make_int2((2 * i2 * p.Wp + 2 * j2) | ((2 * i2) << 16), (i2 * hq + j2) * p.k_pad);
         }
         lut[e] = v;
@@ -337,7 +340,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             int tm = item, nt = 0;
             if (p.tiles_n > 1) { tm = item / p.tiles_n; nt = item - tm * p.tiles_n; }
             int n, p0, q0;
-            tile_origin(p, tm, n, p0, q0);
+            tile_origin<FLAT>(p, tm, n, p0, q0);
             for (int cb = 0; cb < p.cblks; ++cb) {
                 ok = __all_sync(0xffffffffu, mbar_wait(pempty(ps), pphase ^ 1u, abort_flag, p.status));
                 if (!ok) break;
@@ -369,7 +372,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         bool ok = true;
         const int me = warp - 1;
         for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
-            if (p.resident && item != (int)blockIdx.x) break;     // the filters of the first tile stay
+            if (RESIDENT && item != (int)blockIdx.x) break;     // the filters of the first tile stay
             int nt = 0;
             if (p.tiles_n > 1) nt = item % p.tiles_n;
             const int k0 = nt * p.FT;
@@ -378,7 +381,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                     const bool mine = turn == me;
                     turn ^= 1;
                     if (mine) {
-                        if (!p.resident) ok = __all_sync(0xffffffffu, mbar_wait(wempty(ws), wphase ^ 1u, abort_flag, p.status));
+                        if (!RESIDENT) ok = __all_sync(0xffffffffu, mbar_wait(wempty(ws), wphase ^ 1u, abort_flag, p.status));
                         if (!ok) break;
                         if (elect_one()) {
                             const uint32_t wb = wfull(MODE == PK_GENERAL ? ws - wsub : ws);   // the taps of a row complete one barrier
@@ -409,7 +412,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         const uint32_t desc_hi = p.rb16 == 8 ? DESC_HI_SW128 : DESC_HI_SW32;
         const uint32_t slot_step = (uint32_t)p.rb16;                    // descriptor units (16 bytes) per pixel row
         const uint32_t patch_step = (uint32_t)p.patch_bytes >> 4, w_step = w_bytes >> 4;
-        const uint32_t row_step = (uint32_t)(p.Wp - p.S + 1) * slot_step;   // from tap (r, S-1) to (r+1, 0)
+        const uint32_t row_step = (uint32_t)(p.Wp - FS + 1) * slot_step;   // from tap (r, S-1) to (r+1, 0)
         uint32_t patch_lo = patch_lo0, w_lo = w_lo0;
         for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
             ok = __all_sync(0xffffffffu, mbar_wait(tempty(acc), acc_phase ^ 1u, abort_flag, p.status));
@@ -422,43 +425,43 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 if (!ok) break;
                 const int nk = cb == p.cblks - 1 ? p.ksteps_last : 4;
                 uint32_t tap_lo = patch_lo + (uint32_t)(mb * 128) * slot_step;      // the second block's slots follow the first's
-                if (MODE != PK_TAPS && p.resident && item != (int)blockIdx.x) {
+                if (RESIDENT && item != (int)blockIdx.x) {
                     // resident filters, loaded during the first tile: nothing to wait for, a filter row per elected block
-                    for (int r = 0; r < p.R; ++r) {
-                        issue_row(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, p.S, slot_step, w_step, 0u, r == p.R - 1 ? pempty(ps) : 0u);
+                    for (int r = 0; r < FR; ++r) {
+                        issue_row(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, FS, slot_step, w_step, 0u, r == FR - 1 ? pempty(ps) : 0u);
                         accumulate = 1;
                         tap_lo += (uint32_t)p.Wp * slot_step;
-                        w_lo += (uint32_t)p.S * w_step;
-                        ws += p.S;
+                        w_lo += (uint32_t)FS * w_step;
+                        ws += FS;
                         if (ws == p.wstages) { ws = 0; w_lo = w_lo0; }
                     }
                 } else if constexpr (MODE == PK_GENERAL) {
                     // one wait per filter row, then the row's MMAs from one elected block; every tap frees its own stage
-                    for (int r = 0; r < p.R; ++r) {
-                        ok = __all_sync(0xffffffffu, mbar_wait(wfull(ws), p.resident ? 0u : wphase, abort_flag, p.status));
+                    for (int r = 0; r < FR; ++r) {
+                        ok = __all_sync(0xffffffffu, mbar_wait(wfull(ws), RESIDENT ? 0u : wphase, abort_flag, p.status));
                         if (!ok) break;
-                        issue_row(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, p.S, slot_step, w_step, p.resident ? 0u : wempty(ws),
-                                  r == p.R - 1 ? pempty(ps) : 0u);
+                        issue_row(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, FS, slot_step, w_step, RESIDENT ? 0u : wempty(ws),
+                                  r == FR - 1 ? pempty(ps) : 0u);
                         accumulate = 1;
                         tap_lo += (uint32_t)p.Wp * slot_step;
-                        w_lo += (uint32_t)p.S * w_step;
-                        ws += p.S;
+                        w_lo += (uint32_t)FS * w_step;
+                        ws += FS;
                         if (ws == p.wstages) { ws = 0; wphase ^= 1u; w_lo = w_lo0; }
                     }
                 } else {
                     int s = 0;
                     for (int tap = 0; tap < RS; ++tap) {
-                        ok = __all_sync(0xffffffffu, mbar_wait(wfull(ws), p.resident ? 0u : wphase, abort_flag, p.status));
+                        ok = __all_sync(0xffffffffu, mbar_wait(wfull(ws), RESIDENT ? 0u : wphase, abort_flag, p.status));
                         if (!ok) break;
                         {
-                            const uint32_t cw = p.resident ? 0u : wempty(ws), cp = tap == RS - 1 ? pempty(ps) : 0u;
+                            const uint32_t cw = RESIDENT ? 0u : wempty(ws), cp = tap == RS - 1 ? pempty(ps) : 0u;
                             issue_tap(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, cw, cp);
                         }
                         accumulate = 1;
                         w_lo += w_step;
                         if (++ws == p.wstages) { ws = 0; wphase ^= 1u; w_lo = w_lo0; }
                         tap_lo += slot_step;
-                        if (++s == p.S) { s = 0; tap_lo += row_step - slot_step; }
+                        if (++s == FS) { s = 0; tap_lo += row_step - slot_step; }
                     }
                 }
                 patch_lo += patch_step;
@@ -515,7 +518,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             int tm = item, nt = 0;
             if (p.tiles_n > 1) { tm = item / p.tiles_n; nt = item - tm * p.tiles_n; }
             int n, p0, q0;
-            tile_origin(p, tm, n, p0, q0);
+            tile_origin<FLAT>(p, tm, n, p0, q0);
             const int pr0 = (p0 + 1) >> 1, pc0 = (q0 + 1) >> 1;
             for (int g = 0; g < groups && ok; ++g) {
                 const uint32_t b = counter & 1u;
@@ -594,7 +597,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 bias_r[j] = c + j * 2 < k_all ? *reinterpret_cast<const unsigned long long *>(bias_src + c + j * 2) : 0ull;
         };
         if (bias_const) load_bias(sub * WCOLS);
-        const int n_entries = p.ipt ? p.ipt * (p.P >> 1) * (p.Q >> 1) : p.pool == 1 ? (p.TH >> 1) * (p.Q >> 1) : ((p.TH - 1) >> 1) * ((p.TW - 1) >> 1);
+        const int n_entries = ipt ? ipt * (p.P >> 1) * (p.Q >> 1) : p.pool == 1 ? (p.TH >> 1) * (p.Q >> 1) : ((p.TH - 1) >> 1) * ((p.TW - 1) >> 1);
         // Residuals.  Everywhere but with dense staging the MMA warps add the residual on the tensor core (see there) and
         // the epilogue has nothing to do with it.  Dense staging: the residual of tile item_ (tiles_n == 1, one row of
         // tiles) is one contiguous range of memory, arrives in the staging buffer the tile will use and is added in place.
@@ -623,9 +626,9 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             int tm = item, nt = 0;
             if (p.tiles_n > 1) { tm = item / p.tiles_n; nt = item - tm * p.tiles_n; }
             int n, p0, q0;
-            tile_origin(p, tm, n, p0, q0);
+            tile_origin<FLAT>(p, tm, n, p0, q0);
             const int k0 = nt * p.FT;
-            const int rows_valid = p.ipt ? p.imgs - n : p.P - p0;    // tile rows (or images) below this are real ones
+            const int rows_valid = ipt ? p.imgs - n : p.P - p0;    // tile rows (or images) below this are real ones
             // first pooled pixel of the tile (2x2 pool: full-width tiles from an even row)
             __nv_bfloat16 *ytile = p.pool == 1 ? p.y + ((size_t)n * (p.P >> 1) + (p0 >> 1)) * (p.Q >> 1) * p.k_pad : nullptr;
             ok = __all_sync(0xffffffffu, mbar_wait(tfull(acc), acc_phase, abort_flag, p.status, false));
@@ -1015,7 +1018,7 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
             }
             if (!resident) {
                 // Streamed filters: a ring of filter rows, at least two, with one barrier each (3x3 301 -> 250 4x4 at 128 images
-                // 12.2 us, tap by tap 14.8; 128 -> 89 28x28 at 64 images 17.8 and 19.4).  Taps one by one only where two rows do
+                // 12.2 us, tap by tap 14.8; 128 -> 89 28x28 at 64 images 17.9 and 19.4).  Taps one by one only where two rows do
                 // not fit (256 filters, for instance), or where the patch ring had to become shallower for it at no gain.
                 for (staging_bufs = sb_max; staging_bufs > sb_min && (budget - staging_bufs * stage_bytes) / w_stage < 2 * wgroup;) --staging_bufs;
                 if ((budget - staging_bufs * stage_bytes) / w_stage < 2 * wgroup) {
@@ -1304,10 +1307,12 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
         if (dev < 0 || dev >= 64) return CPRUNE_ERR_UNSUPPORTED;
         std::lock_guard<std::mutex> lock(attr_mu);
         if (!attr_set[dev]) {
-            const void *kernels[] = {(const void *)conv_patch_kernel<PK_GENERAL, false>, (const void *)conv_patch_kernel<PK_GENERAL, true>,
-                                     (const void *)conv_patch_kernel<PK_TAPS, false>,    (const void *)conv_patch_kernel<PK_TAPS, true>,
-                                     (const void *)conv_patch_kernel<PK_FLAT>,           (const void *)conv_patch_kernel<PK_DENSE>,
-                                     (const void *)conv_patch_kernel<PK_POOL3>};
+            const void *kernels[] = {(const void *)conv_patch_kernel<PK_GENERAL, false>, (const void *)conv_patch_kernel<PK_GENERAL, false, false, 3>, (const void *)conv_patch_kernel<PK_GENERAL, false, true, 3>, (const void *)conv_patch_kernel<PK_GENERAL, false, true>,
+                                     (const void *)conv_patch_kernel<PK_GENERAL, true>, (const void *)conv_patch_kernel<PK_GENERAL, true, false, 3>, (const void *)conv_patch_kernel<PK_GENERAL, true, true, 3>,  (const void *)conv_patch_kernel<PK_GENERAL, true, true>,
+                                     (const void *)conv_patch_kernel<PK_TAPS, false>,    (const void *)conv_patch_kernel<PK_TAPS, false, true>,
+                                     (const void *)conv_patch_kernel<PK_FLAT, false>,    (const void *)conv_patch_kernel<PK_FLAT, true>,
+                                     (const void *)conv_patch_kernel<PK_DENSE, false>,   (const void *)conv_patch_kernel<PK_DENSE, true>,
+                                     (const void *)conv_patch_kernel<PK_POOL3, false>,   (const void *)conv_patch_kernel<PK_POOL3, true>};
             for (const void *k : kernels) CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
             attr_set[dev] = true;
         }
@@ -1316,7 +1321,6 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
     p.P = g.vP; p.Q = g.vQ; p.Wp = Wp; p.TH = t.TH; p.tiles_per_img = t.tiles_per_img;
     p.TW = t.TW; p.tiles_w = t.tiles_w; p.step_h = t.step_h; p.step_w = t.step_w; p.org = t.org;
     p.out_h = g.vOH; p.out_w = g.vOW;
-    p.flat = g.flat;
     p.ipt = t.ipt; p.imgs = g.vN;
     // v * ceil(2^32 / d) / 2^32 has the integer part v / d as long as v * d < 2^32 (the error of the reciprocal is below 1 / 2^32)
     const auto reciprocal = [](long long d, long long most) {
@@ -1351,20 +1355,24 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
     const int grid = total < sms ? total : sms;
     // a fused 3x3 pool with two staging buffers: the instantiation with separate pooling warps
     const bool split_pool = p.pool == CPRUNE_POOL_MAX3X3S2 && t.staging_bufs == 2 && !res && !(plan->opts.flags & CPRUNE_FLAG_POOL_ON_EPILOGUE_WARPS);
-    // One instantiation per kind of epilogue and of filter ring: a role is one warp that fetches its instructions alone, and each
-    // of them is faster the less code lies between its loops (64 images: 1x1 24 -> 108 56x56 20.2 -> 17.8 us, 96 -> 432 14x14 10.7 ->
-    // 10.0 us, 3x3 131 -> 203 28x28 37.0 -> 36.3 us).
+    // One instantiation per kind of epilogue and of filter set, and for 3x3 filters: a role is one warp that fetches its
+    // instructions alone, and each is faster the less code lies between its loops.  One kernel for all / now (us, 64 images):
+    // 1x1 24 -> 108 56x56 20.2 / 17.6, 96 -> 432 14x14 10.7 / 9.6, 32 -> 16 112x112 19.7 / 18.8, 3x3 512 -> 358 7x7 20.5 / 18.2,
+    // 64 -> 44 56x56 20.8 / 19.9, 131 -> 203 28x28 37.0 / 36.2.
     const auto launch = [&](auto kernel, int mode) {
         return launch_chained(kernel, dim3(grid), dim3(pk_threads(mode)), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, p);
     };
-    const bool taps = t.wgroup == 1 && !t.resident;
-    if (t.dense) CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_DENSE>, PK_DENSE));
-    else if (g.flat) CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_FLAT>, PK_FLAT));
-    else if (split_pool) CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_POOL3>, PK_POOL3));
-    else if (taps && p.pool) CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_TAPS, true>, PK_TAPS));
-    else if (taps) CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_TAPS, false>, PK_TAPS));
-    else if (p.pool) CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_GENERAL, true>, PK_GENERAL));
-    else CPRUNE_CUDA_CHECK(launch(conv_patch_kernel<PK_GENERAL, false>, PK_GENERAL));
+    const bool r = t.resident != 0, pooled = p.pool != 0;
+    cudaError_t e;
+    if (t.dense) e = r ? launch(conv_patch_kernel<PK_DENSE, true>, PK_DENSE) : launch(conv_patch_kernel<PK_DENSE, false>, PK_DENSE);
+    else if (g.flat) e = r ? launch(conv_patch_kernel<PK_FLAT, true>, PK_FLAT) : launch(conv_patch_kernel<PK_FLAT, false>, PK_FLAT);
+    else if (split_pool) e = r ? launch(conv_patch_kernel<PK_POOL3, true>, PK_POOL3) : launch(conv_patch_kernel<PK_POOL3, false>, PK_POOL3);
+    else if (g.kR == 3 && g.kS == 3 && r) e = pooled ? launch(conv_patch_kernel<PK_GENERAL, true, true, 3>, PK_GENERAL) : launch(conv_patch_kernel<PK_GENERAL, true, false, 3>, PK_GENERAL);
+    else if (g.kR == 3 && g.kS == 3 && t.wgroup == 3) e = pooled ? launch(conv_patch_kernel<PK_GENERAL, false, true, 3>, PK_GENERAL) : launch(conv_patch_kernel<PK_GENERAL, false, false, 3>, PK_GENERAL);
+    else if (r) e = pooled ? launch(conv_patch_kernel<PK_GENERAL, true, true>, PK_GENERAL) : launch(conv_patch_kernel<PK_GENERAL, true>, PK_GENERAL);
+    else if (t.wgroup == 1) e = pooled ? launch(conv_patch_kernel<PK_TAPS, false, true>, PK_TAPS) : launch(conv_patch_kernel<PK_TAPS, false>, PK_TAPS);
+    else e = pooled ? launch(conv_patch_kernel<PK_GENERAL, false, true>, PK_GENERAL) : launch(conv_patch_kernel<PK_GENERAL, false>, PK_GENERAL);
+    CPRUNE_CUDA_CHECK(e);
     return CPRUNE_OK;
 }
 
