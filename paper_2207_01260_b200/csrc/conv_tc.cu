@@ -90,7 +90,11 @@ __device__ __forceinline__ void store_pooled(const float *f, uint8_t *dst, int c
 
 // ---------------------------------------------------------------------------------------- kernel
 
-template <int ORIENT, int POOL>
+// One instantiation per orientation, fused pool, kind of input (PLAIN: whole 64-channel blocks; else 3-channel stems) and
+// split of the reduction: the producer and the issuing warp run alone, and faster the less code lies between their loops (us, 64
+// images, one kernel for all / now: 3x3 stride 2 256 -> 358 14x14 15.5 / 13.6, 128 -> 179 28x28 15.3 / 13.9, 1x1 stride 2
+// 256 -> 512 14x14 7.4 / 6.8).
+template <int ORIENT, int POOL, bool PLAIN, bool SPLIT>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 conv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_res,
@@ -147,8 +151,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__
     const uint32_t tmem_base = *tmem_slot;
 
     const int k_alloc = p.tiles_n * p.FT;     // row length of the float32 partial sums (split-K)
-    const int total_tiles = p.tiles_m * p.tiles_n * p.splits;   // work items: (tile, K slice), slice fastest
+    const int total_tiles = p.tiles_m * p.tiles_n * (SPLIT ? p.splits : 1);   // work items: (tile, K slice), slice fastest
     const int PQ = p.P * p.Q;
+    const int res_iters = ORIENT == ORIENT_FILT ? p.res_iters : 0;
 
     if (warp < N_PRODUCERS) {
         // ------------------------------------------------------------------ producers
@@ -162,7 +167,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__
             // the divisions below are skipped in the common cases (no split-K, one filter tile) and done in
             // 32 bits when the pixel count allows: each costs this lone warp a few hundred cycles
             int tile = item, split = 0, it_begin = 0, it_end = p.iters;
-            if (p.splits > 1) {
+            if constexpr (SPLIT) {
                 tile = item / p.splits; split = item - tile * p.splits;
                 it_begin = split * p.ipp; it_end = min(p.iters, it_begin + p.ipp);
             }
@@ -179,12 +184,12 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__
             }
             const int p0 = (int)((uint32_t)rem / (uint32_t)p.Q), q0 = rem - p0 * p.Q;
             const int wc = q0 * p.stride - p.pad, hc = p0 * p.stride - p.pad;
-            if (p.small_c == 2) {
+            if (!PLAIN && p.small_c == 2) {
                 // stride-2 stem read as pixel pairs: the tensor map sees [N][H][W/2][16]; a pair-tap is one im2col
                 // load of PT pixels x 32 bytes = one K step; 4 pair-taps per stage
                 const int taps = p.R * p.pair_taps;
                 const int wcp = q0 - ((p.pad + 1) >> 1);
-                for (int it = 0; it < p.iters - p.res_iters; ++it) {
+                for (int it = 0; it < p.iters - res_iters; ++it) {
                     const bool mine = turn == warp;
                     if (++turn == N_PRODUCERS) turn = 0;
                     if (mine) ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status));
@@ -205,10 +210,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__
                     __syncwarp();
                     if (++stage == p.stages) { stage = 0; phase ^= 1u; }
                 }
-            } else if (p.small_c) {
+            } else if (!PLAIN) {
                 // 8 taps x 8 channels per stage; every tap is its own im2col load of PT pixels x 16 bytes
                 const int taps = p.R * p.S;
-                for (int it = 0; it < p.iters - p.res_iters; ++it) {
+                for (int it = 0; it < p.iters - res_iters; ++it) {
                     const bool mine = turn == warp;
                     if (++turn == N_PRODUCERS) turn = 0;
                     if (mine) ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status));
@@ -239,7 +244,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__
                 tap = it_begin / p.cblks; cb = it_begin - tap * p.cblks;
                 r = tap / p.S; s = tap - r * p.S;
             }
-            const int it_last = it_end - (p.splits == 1 ? p.res_iters : 0);
+            const int it_last = it_end - (SPLIT ? 0 : res_iters);
             const int k0 = nt_f * p.FT;
             for (int it = it_begin; it < it_last; ++it) {
                 const bool mine = turn == warp;
@@ -264,7 +269,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__
             // residual blocks (ORIENT_FILT): the residual tile [PT pixels][64 filters] is the pixel-side
             // operand and a 64-column slice of the identity matrix the filter-side operand, so that the
             // MMA adds residual[pixel][k] to accumulator row k
-            for (int j = 0; j < p.res_iters && ok; ++j) {
+            for (int j = 0; j < res_iters && ok; ++j) {
                 const bool mine = turn == warp;
                 if (++turn == N_PRODUCERS) turn = 0;
                 if (mine) ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status));
@@ -292,12 +297,11 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__
         const uint64_t dx0 = smem_desc_sw128(base), dw0 = smem_desc_sw128(base + (uint32_t)x_bytes);
         const uint64_t stage_step = (uint64_t)(stage_bytes >> 4);     // descriptor start addresses count 16-byte units
         uint64_t dx = dx0, dw = dw0;
-        const int main_iters = p.iters - p.res_iters;
-        const bool plain = p.small_c == 0;
+        const int main_iters = p.iters - res_iters;
         for (int item = blockIdx.x; item < total_tiles && ok; item += gridDim.x) {
             int it_begin = 0, it_end = p.iters;
             int cb = 0;
-            if (p.splits > 1) {
+            if constexpr (SPLIT) {
                 const int split = item % p.splits;
                 it_begin = split * p.ipp;
                 it_end = min(p.iters, it_begin + p.ipp);
@@ -311,8 +315,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__
             for (int it = it_begin; it < it_end; ++it) {
                 ok = __all_sync(0xffffffffu, mbar_wait(full_bar(stage), phase, abort_flag, p.status));
                 if (!ok) break;
-                const bool res_it = it >= main_iters;
-                if (plain || res_it) {
+                const bool res_it = ORIENT == ORIENT_FILT && it >= main_iters;
+                if (PLAIN || res_it) {
                     int nk = BK / 16;
                     if (res_it) {
                         int left = p.k_pad - (it - main_iters) * BK;
@@ -409,7 +413,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__
         };
         for (int item = blockIdx.x; item < total_tiles && ok; item += gridDim.x) {
             int tile = item, split = 0;
-            if (p.splits > 1) { tile = item / p.splits; split = item - tile * p.splits; }
+            if constexpr (SPLIT) { tile = item / p.splits; split = item - tile * p.splits; }
             int mt = tile, nt = 0;
             if (p.tiles_n > 1) { mt = tile / p.tiles_n; nt = tile - mt * p.tiles_n; }
             const long long m0 = (long long)mt * p.PT;
@@ -421,7 +425,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__
             tc_fence_after();
             const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * ACC_STRIDE);
 
-            if (p.splits > 1) {
+            if constexpr (SPLIT) {
                 // split-K: this CTA holds a partial sum; store it as float32, the finalize kernel adds
                 // the slices in a fixed order and applies bias, residual and activation
                 float *part = p.partial + (size_t)split * (size_t)p.M * k_alloc;
@@ -1031,10 +1035,13 @@ cprune_status launch_conv_tensor(cprune_plan *plan, const void *x, const void *w
         if (dev < 0 || dev >= 64) return CPRUNE_ERR_UNSUPPORTED;
         std::lock_guard<std::mutex> lock(attr_mu);
         if (!attr_set[dev]) {
-            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(conv_tc_kernel<ORIENT_PIX, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(conv_tc_kernel<ORIENT_PIX, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(conv_tc_kernel<ORIENT_FILT, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-            CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(conv_tc_kernel<ORIENT_FILT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+            const void *kernels[] = {
+                (const void *)conv_tc_kernel<ORIENT_PIX, 0, true, false>,  (const void *)conv_tc_kernel<ORIENT_PIX, 0, true, true>,
+                (const void *)conv_tc_kernel<ORIENT_PIX, 0, false, false>, (const void *)conv_tc_kernel<ORIENT_PIX, 1, true, false>,
+                (const void *)conv_tc_kernel<ORIENT_PIX, 1, false, false>, (const void *)conv_tc_kernel<ORIENT_FILT, 0, true, false>,
+                (const void *)conv_tc_kernel<ORIENT_FILT, 0, true, true>,  (const void *)conv_tc_kernel<ORIENT_FILT, 0, false, false>,
+                (const void *)conv_tc_kernel<ORIENT_FILT, 1, true, false>, (const void *)conv_tc_kernel<ORIENT_FILT, 1, false, false>};
+            for (const void *k : kernels) CPRUNE_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
             attr_set[dev] = 1;
         }
     }
@@ -1064,13 +1071,17 @@ cprune_status launch_conv_tensor(cprune_plan *plan, const void *x, const void *w
     if (total == 0) return CPRUNE_OK;
     const int grid = total < sm_count() ? total : sm_count();
     const bool pool_in_kernel = plan->fused_pool && !split;
-    if (plan->orient == ORIENT_PIX) {
-        if (pool_in_kernel) CPRUNE_CUDA_CHECK(launch_chained(conv_tc_kernel<ORIENT_PIX, 1>, dim3(grid), dim3(TC_THREADS), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, tm_id, p));
-        else CPRUNE_CUDA_CHECK(launch_chained(conv_tc_kernel<ORIENT_PIX, 0>, dim3(grid), dim3(TC_THREADS), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, tm_id, p));
-    } else {
-        if (pool_in_kernel) CPRUNE_CUDA_CHECK(launch_chained(conv_tc_kernel<ORIENT_FILT, 1>, dim3(grid), dim3(TC_THREADS), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, tm_id, p));
-        else CPRUNE_CUDA_CHECK(launch_chained(conv_tc_kernel<ORIENT_FILT, 0>, dim3(grid), dim3(TC_THREADS), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, tm_id, p));
-    }
+    const auto launch = [&](auto kernel) {
+        return launch_chained(kernel, dim3(grid), dim3(TC_THREADS), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, tm_id, p);
+    };
+    const bool pix = plan->orient == ORIENT_PIX, plain = !plan->small_c;
+    cudaError_t e;
+    if (split) e = pix ? launch(conv_tc_kernel<ORIENT_PIX, 0, true, true>) : launch(conv_tc_kernel<ORIENT_FILT, 0, true, true>);
+    else if (plain && pool_in_kernel) e = pix ? launch(conv_tc_kernel<ORIENT_PIX, 1, true, false>) : launch(conv_tc_kernel<ORIENT_FILT, 1, true, false>);
+    else if (plain) e = pix ? launch(conv_tc_kernel<ORIENT_PIX, 0, true, false>) : launch(conv_tc_kernel<ORIENT_FILT, 0, true, false>);
+    else if (pool_in_kernel) e = pix ? launch(conv_tc_kernel<ORIENT_PIX, 1, false, false>) : launch(conv_tc_kernel<ORIENT_FILT, 1, false, false>);
+    else e = pix ? launch(conv_tc_kernel<ORIENT_PIX, 0, false, false>) : launch(conv_tc_kernel<ORIENT_FILT, 0, false, false>);
+    CPRUNE_CUDA_CHECK(e);
     CPRUNE_LAUNCH_CHECK("conv_tc_kernel");
     if (split) {
         const long long elems = (plan->fused_pool ? p.M / 4 : p.M) * (i.k_pad / 8) * (plan->fused_pool ? 16 : 4);   // threads
