@@ -1027,7 +1027,7 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
                 }
                 wstages = (budget - staging_bufs * stage_bytes) / w_stage;
                 if (wstages < 3) continue;
-                if (wstages > 12) wstages = 12;
+                if (wstages > 8) wstages = wgroup > 4 ? 2 * wgroup : 8;
                 wstages -= wstages % wgroup;
             }
             if (dense && staging_bufs != 2) continue;
