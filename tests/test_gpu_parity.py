@@ -310,6 +310,40 @@ def test_stems_straight_from_the_image(cp, case):
     check_values("stem, unaligned image %s" % (case,), y2[..., :K], ref, bound, ref_m, bound_m)
 
 
+def stem_model(cp, plan, w, b):
+    """A model of one conv task that reads its float32 image, a pool and a small FC layer."""
+    K = plan.K
+    packed, fc = cp.cprune_pack_weights(plan, _dev(w), _dev(b)), cp.cprune_fc_pack(torch.ones((8, K), device="cuda"))
+    tasks = [cp.TaskDesc(op=cp.OP_CONV, in_=0, out=1, res=-1, plan=plan.handle, w=packed[0].data_ptr(), b=packed[1].data_ptr()),
+             cp.TaskDesc(op=cp.OP_GAP, in_=1, out=2, res=-1),
+             cp.TaskDesc(op=cp.OP_FC, in_=2, out=3, res=-1, w=fc[0].data_ptr(), b=fc[1].data_ptr(), p0=K, p1=8)]
+    model = cp.cprune_model_create(plan.N, plan.H, plan.W, 3, tasks, keep_alive=(plan, packed, fc))
+    assert model.launches == 3          # the conv task reads the image itself
+    return model
+
+
+@pytest.mark.parametrize("case", [
+    # N, H, W, K, R, stride, pad, act: images too large for a step of 128 filter rows, so that a step has one or two conv rows of 32
+    # or 64 filters and the other rows of the MMA go nowhere; two or three steps per block (both staging buffers), every step's bias
+    # other than zero
+    (4, 224, 224, 64, 7, 2, 3, "relu"), (3, 224, 224, 48, 7, 2, 3, "none"), (4, 160, 160, 24, 3, 1, 1, "relu6"),
+    (2, 320, 320, 32, 3, 2, 1, "relu")])
+def test_stems_of_large_images_with_fewer_conv_rows_per_step(cp, case):
+    N, H, W, K, R, stride, pad, act = case
+    x, w, b, _ = wl.conv_task_tensors(96, N, 3, H, W, K, R, R)
+    plan = cp.cprune_task_plan(N, 3, H, W, K, R, R, stride, pad, 1, act)
+    model = stem_model(cp, plan, w, b)
+    for _ in range(2):
+        cp.cprune_model_run(model, _dev(x))
+    y = model.copy_tensor(1).float().cpu().numpy()
+    cp.cprune_poll_device_status()
+    ref, bound = oracle.conv2d(x, w, b, stride, pad, 1, act, None, with_bound=True)
+    rb = oracle.round_bf16
+    ref_m, bound_m = oracle.conv2d(rb(x), rb(w), b, stride, pad, 1, act, None, with_bound=True)
+    assert np.all(y[..., K:] == 0)
+    check_values("stem of a large image %s" % (case,), y[..., :K], ref, bound, ref_m, bound_m)
+
+
 @pytest.mark.parametrize("case", [
     # N, C, H, W, K, R, stride, pad: fused in the patch kernel (tiles around whole 3x3 windows, even and odd extents),
     # and as a separate pass (few tiles; a task with wrap-around slots)
