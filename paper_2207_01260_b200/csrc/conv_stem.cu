@@ -306,8 +306,8 @@ __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const __grid_c
         const int quarter = warp & 3, half = warp >> 2;
         const int m = quarter * 32 + lane;
         const int dy = m / p.KF, k = m - dy * p.KF;
-        // rows of filters that a halved D leaves over (D * KF < 128) have no place in the staging buffer
-        const bool k_ok = k < p.k_pad && dy < p.D;
+        // rows of filters that a halved D leaves over (D * KF < 128) have no place in the staging buffer; the pool's D is always 2
+        const bool k_ok = k < p.k_pad && (POOL || dy < p.D);
         const float bias = k_ok ? __ldg(p.bias + k) : 0.f;
         const int units = p.N >> 4;
         const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16);
