@@ -865,6 +865,34 @@ def test_intermediate_activations_match(cp):
         assert rel <= 1e-2, (name, rel)
 
 
+@pytest.mark.parametrize("act", ["none", "relu", "relu6"])
+@pytest.mark.parametrize("case", [
+    # N, C, H, K, R, stride, groups, variant: the patch kernel with resident filters, with a ring of filter rows and of taps, on whole
+    # images, on flat tasks staged by 64 filters and as they lie in memory; im2col in both orientations; depthwise
+    (64, 64, 28, 48, 3, 1, 1, 1), (64, 256, 14, 89, 3, 1, 1, 1), (64, 256, 14, 256, 3, 1, 1, 1), (128, 96, 8, 80, 3, 1, 1, 1),
+    (64, 32, 28, 200, 1, 1, 1, 1), (64, 48, 56, 72, 1, 1, 1, 2), (64, 64, 28, 96, 3, 2, 1, 0), (64, 64, 28, 200, 3, 2, 1, 0),
+    (4, 40, 14, 40, 3, 1, 40, 0)])
+def test_a_nan_pixel_reaches_only_the_outputs_whose_window_holds_it(cp, case, act):
+    # every kernel answers alike: NaN without an activation, 0 under the clamps (the clamp returns the operand that is a number)
+    N, C, H, K, R, stride, groups, variant = case
+    plan = cp.cprune_task_plan(N, C, H, H, K, R, R, stride, R // 2, groups, act)
+    assert plan.variant == variant
+    x, w, b, _ = wl.conv_task_tensors(97, N, C, H, H, K, R, R, groups)
+    wp, bp = cp.cprune_pack_weights(plan, _dev(w), _dev(b))
+    clean = cp.cprune_cast_input(_dev(x))
+    bad, h, v, c = clean.clone(), 4, 5, 3
+    bad[1, h, v, c] = float("nan")
+    a, y = (cp.cprune_task_run(plan, t, wp, bp).clone()[..., :K].float() for t in (clean, bad))
+    cp.cprune_poll_device_status()
+    touched = torch.zeros_like(a, dtype=torch.bool)
+    p = torch.arange(plan.P, device="cuda") * stride - R // 2
+    rows, cols = (p <= h) & (h < p + R), (p <= v) & (v < p + R)
+    touched[1] = (rows[:, None] & cols[None, :])[..., None] & (torch.ones(K, dtype=torch.bool, device="cuda") if groups == 1 else torch.arange(K, device="cuda") == c)
+    assert torch.equal(y[~touched], a[~touched])
+    got = y[touched]
+    assert torch.isnan(got).all() if act == "none" else (got == 0).all()
+
+
 def test_plan_cache_shares_repeated_shapes(cp):
     from paper_2207_01260_b200.pipeline import PrunedNetwork
     table = wl.resnet18()
