@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(CS_WARPS * 32, 2) conv_small_kernel(const Smal
         const int r = e / (COLS / 2), c = (e - r * (COLS / 2)) * 2, k = o0 + c;
         const int m = (POOL ? b0 / 4 : b0) + r;
         if (k >= p.k_pad || m >= (POOL ? p.M / 4 : p.M)) continue;
-        float2 best = make_float2(-INFINITY, -INFINITY);
+        float2 best = make_float2(0.f, 0.f);
 #pragma unroll
         for (int u = 0; u < (POOL ? 4 : 1); ++u) {
             const int row = POOL ? r * 4 + u : r, grp = row / ROWS, lr = row - grp * ROWS;
@@ -172,7 +172,8 @@ __global__ void __launch_bounds__(CS_WARPS * 32, 2) conv_small_kernel(const Smal
                 v.y += __uint_as_float(rv & 0xffff0000u);
             }
             v.x = apply_act(v.x, p.act); v.y = apply_act(v.y, p.act);
-            best.x = fmaxf(best.x, v.x); best.y = fmaxf(best.y, v.y);
+            // (the maximum starts from the window's first value: one with minus infinity would turn a NaN into it)
+            best = u == 0 ? v : make_float2(fmaxf(best.x, v.x), fmaxf(best.y, v.y));
         }
         *reinterpret_cast<__nv_bfloat162 *>(p.y + (size_t)m * p.k_pad + k) = __floats2bfloat162_rn(best.x, best.y);
     }

@@ -871,7 +871,9 @@ def test_intermediate_activations_match(cp):
     # images, on flat tasks staged by 64 filters and as they lie in memory; im2col in both orientations; depthwise
     (64, 64, 28, 48, 3, 1, 1, 1), (64, 256, 14, 89, 3, 1, 1, 1), (64, 256, 14, 256, 3, 1, 1, 1), (128, 96, 8, 80, 3, 1, 1, 1),
     (64, 32, 28, 200, 1, 1, 1, 1), (64, 48, 56, 72, 1, 1, 1, 2), (64, 64, 28, 96, 3, 2, 1, 0), (64, 64, 28, 200, 3, 2, 1, 0),
-    (4, 40, 14, 40, 3, 1, 40, 0)])
+    (4, 40, 14, 40, 3, 1, 40, 0),
+    # few pixels
+    (2, 64, 16, 48, 3, 1, 1, 3), (2, 64, 16, 48, 1, 1, 1, 3), (2, 64, 16, 200, 3, 2, 1, 3)])
 def test_a_nan_pixel_reaches_only_the_outputs_whose_window_holds_it(cp, case, act):
     # every kernel answers alike: NaN without an activation, 0 under the clamps (the clamp returns the operand that is a number)
     N, C, H, K, R, stride, groups, variant = case
@@ -891,6 +893,19 @@ def test_a_nan_pixel_reaches_only_the_outputs_whose_window_holds_it(cp, case, ac
     assert torch.equal(y[~touched], a[~touched])
     got = y[touched]
     assert torch.isnan(got).all() if act == "none" else (got == 0).all()
+
+
+def test_a_nan_in_a_pooled_window_of_few_pixels(cp):
+    # a maximum skips a NaN beside numbers and is a NaN when the whole window is (as the separate pooling pass has it)
+    N, C, H, K = 2, 64, 8, 48
+    x, w, b, _ = wl.conv_task_tensors(98, N, C, H, H, K, 1, 1)
+    x[0, 2, 2, 0] = np.nan                        # one pixel of the pooled pixel (1, 1)
+    x[1, 4:6, 6:8, 5] = np.nan                    # all four of (2, 3)
+    plan = cp.cprune_task_plan(N, C, H, H, K, 1, 1, 1, 0, 1, "none", False, "max2x2")
+    assert plan.variant == 3
+    y = cp.cprune_task_run(plan, cp.cprune_cast_input(_dev(x)), *cp.cprune_pack_weights(plan, _dev(w), _dev(b))).float()[..., :K]
+    assert torch.isnan(y).nonzero()[:, :3].unique(dim=0).tolist() == [[1, 2, 3]] and torch.isnan(y[1, 2, 3]).all()
+    assert torch.isfinite(y[0]).all()
 
 
 def test_plan_cache_shares_repeated_shapes(cp):
