@@ -3,7 +3,8 @@
 // the fused subgraph).
 //
 // The pixels are on the column side of the MMA and the filters on its 128 rows: D = 128 / KF conv rows of KF (32, 64 or 128)
-// filters each, so that the rows are full for the 16 to 64 filters of a pruned stem.  Those D conv rows read the same
+// filters each, so that the rows are full for the 16 to 64 filters of a pruned stem (fewer where the tiles of a large image would not
+// fit; the rows left over go nowhere).  Those D conv rows read the same
 // RH = stride * (D - 1) + R input rows; a filter of conv row dy is packed with zero taps where its window does not reach.
 //   K order     per input row, the S pixels of a window in 4 channel lanes each: 32 bytes (S <= 4) or 64.  A 128-byte operand
 //               row holds the windows of one output column in `per` (1, 2 or 4) neighbouring input rows.
@@ -11,8 +12,11 @@
 //               buffer, and copy every output column's window from there into a swizzled operand tile.  (Overlapping windows
 //               are stored once per column because the MMA fetches one row of its operand's swizzle width per cycle: with
 //               the rows read in place through an unswizzled descriptor the 7x7 stem of 64 images took 55 us.)  Tiles form a
-//               ring; rows outside the image are zeros, as are the columns left and right of it.
-//   MMA         (1 warp) one step = D conv rows: N = Q columns, K = RH windows; filters stay in shared memory.
+//               ring; rows outside the image are zeros, as are the columns left and right of it.  They also say of every tile
+//               whether it holds a pixel that is no number (infinite or NaN as a bf16 value).
+//   MMA         (1 warp) one step = D conv rows: N = Q columns, K = RH windows; filters stay in shared memory.  Conv rows meet the
+//               input rows outside their window with zero taps, which is nothing unless a pixel is no number: the rows of such a
+//               tile go to the accumulator lanes that want them alone (always doing so cost the pooled stem 7 us of 46).
 //   epilogue    (8 warps) a thread owns one filter of one conv row and walks along the pixels, so the pool's horizontal
 //               maximum stays in registers; odd conv rows hand theirs to the even ones through shared memory.  Results are
 //               transposed through shared memory (2-byte stores, neighbouring lanes = neighbouring filters) and leave as one
@@ -50,7 +54,8 @@ struct StemParams {
     int per, tiles, adv;                  // input rows per operand tile, tiles a step reads, tiles from step to step
     int row_bytes, tile_bytes, raw_bytes, ring, stage_bytes, xch_words;
     int steps_per_img, total_steps;
-    int k_pad;
+    int k_pad, S;
+    unsigned long long lanes_on, lanes_new;   // 4 bits per input row of a step: accumulator lanes (32 each) whose window holds it, and begins with it
     int *status;
 };
 
@@ -86,6 +91,12 @@ __device__ __forceinline__ uint32_t max2(uint32_t a, uint32_t b) {
     return *reinterpret_cast<const uint32_t *>(&v);
 }
 
+// a + 0 * v for bf16 pairs: a zero stays a zero unless v is infinite or NaN
+__device__ __forceinline__ uint32_t times_zero2(uint32_t v, uint32_t a) {
+    asm("fma.rn.bf16x2 %0, %1, %2, %0;" : "+r"(a) : "r"(v), "r"(0u));
+    return a;
+}
+
 // CPS: 16-byte pieces of a window
 template <int ACT, bool POOL, int CPS>
 __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const __grid_constant__ CUtensorMap tm_w, const StemParams p) {
@@ -111,6 +122,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const __grid_c
     auto rfull = [&](int s) { return ctrl0 + 256u + 8u * s; };
     uint32_t *tmem_slot = (uint32_t *)(ctrl + 248);
     volatile int *abort_flag = (volatile int *)(ctrl + 252);
+    uint8_t *flags = ctrl + 288;           // 16 tiles (more than the ring and the tiles being converted) x converter warps
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
@@ -190,7 +202,8 @@ __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const __grid_c
             copy_q[u] = q;
             copy_src[u] = cr * p.row_bytes + q * p.stride * 8;
         }
-        int t = t0, slot = 0, rslot = 0, buf = 0;
+        const uint32_t keep = p.S & 1 ? 0u : 0xffffffffu;      // the second pixel of a window's last piece
+        int t = t0, slot = 0, rslot = 0, buf = 0, seq = 0;
         uint32_t phase = 0, rphase = 0, conv_phase = 0;
         bool ok = true;
         StemSegment sg;
@@ -203,6 +216,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const __grid_c
                 uint8_t *rb = rows + buf * row_buf;
                 const uint8_t *src = raw + rslot * p.raw_bytes;
                 const int row0 = b * p.per - p.pad;
+                uint32_t odd[2] = {0u, 0u};                // zeros, or NaN where a pixel is no number
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     if (conv_r[u] < 0) break;
@@ -212,12 +226,21 @@ __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const __grid_c
                         const float4 *s4 = (const float4 *)(src + conv_src[u] + (row0 - r0) * p.W * 12);
                         f0 = s4[0]; f1 = s4[1]; f2 = s4[2];
                     }
+                    const uint2 px[4] = {make_uint2(act_pack2<CPRUNE_ACT_NONE>(f0.x, f0.y), act_pack2<CPRUNE_ACT_NONE>(f0.z, 0.f)),
+                                         make_uint2(act_pack2<CPRUNE_ACT_NONE>(f0.w, f1.x), act_pack2<CPRUNE_ACT_NONE>(f1.y, 0.f)),
+                                         make_uint2(act_pack2<CPRUNE_ACT_NONE>(f1.z, f1.w), act_pack2<CPRUNE_ACT_NONE>(f2.x, 0.f)),
+                                         make_uint2(act_pack2<CPRUNE_ACT_NONE>(f2.y, f2.z), act_pack2<CPRUNE_ACT_NONE>(f2.w, 0.f))};
                     uint2 *dst = (uint2 *)(rb + conv_dst[u]);
-                    dst[0] = make_uint2(act_pack2<CPRUNE_ACT_NONE>(f0.x, f0.y), act_pack2<CPRUNE_ACT_NONE>(f0.z, 0.f));
-                    dst[1] = make_uint2(act_pack2<CPRUNE_ACT_NONE>(f0.w, f1.x), act_pack2<CPRUNE_ACT_NONE>(f1.y, 0.f));
-                    dst[2] = make_uint2(act_pack2<CPRUNE_ACT_NONE>(f1.z, f1.w), act_pack2<CPRUNE_ACT_NONE>(f2.x, 0.f));
-                    dst[3] = make_uint2(act_pack2<CPRUNE_ACT_NONE>(f2.y, f2.z), act_pack2<CPRUNE_ACT_NONE>(f2.w, 0.f));
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        dst[q] = px[q];
+                        odd[0] = times_zero2(px[q].x, odd[0]);
+                        odd[1] = times_zero2(px[q].y, odd[1]);
+                    }
                 }
+                const bool any_odd = __any_sync(0xffffffffu, ((odd[0] | odd[1]) & 0x7fff7fffu) != 0u);
+                if (lane == 0) flags[(seq & 15) * ST_CONV_WARPS + (warp - ST_EPI_WARPS)] = any_odd;
+                ++seq;
                 // everyone has read the float32 rows and written its pixels; the row buffer is written again two tiles on,
                 // behind the next meeting
                 __syncwarp();
@@ -243,6 +266,15 @@ __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const __grid_c
                             v[c] = make_uint4(lo.x, lo.y, hi.x, hi.y);
                         }
                     }
+                    // pixels behind the window's last meet zero taps and have to be numbers: zeros
+                    v[CPS - 1].z &= keep; v[CPS - 1].w &= keep;
+                    if (p.S <= 2 * CPS - 2) {
+#pragma unroll
+                        for (int c = 0; c < CPS; ++c) {
+                            if (2 * c >= p.S) v[c].x = v[c].y = 0u;
+                            if (2 * c + 1 >= p.S) v[c].z = v[c].w = 0u;
+                        }
+                    }
 #pragma unroll
                     for (int c = 0; c < CPS; ++c) *(uint4 *)(dst0 + sub_off(copy_q[u], copy_r[u] * CPS + c)) = v[c];
                 }
@@ -263,8 +295,8 @@ __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const __grid_c
         int t = t0, acc = 0;
         uint32_t acc_phase = 0;
         int head = 0;                                      // ring slot of the oldest tile in use
-        int wslot = 0;                                     // next tile to wait for
-        uint32_t wphase = 0;
+        int wslot = 0, seq = 0;                            // next tile to wait for
+        uint32_t wphase = 0, odd = 0;                      // odd: ring slots whose tile holds a pixel that is no number
         StemSegment sg;
         bool ok = __all_sync(0xffffffffu, mbar_wait(wbar, 0u, abort_flag, p.status));
         while (ok && next_segment<POOL>(p, t, t1, sg)) {
@@ -276,20 +308,38 @@ __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const __grid_c
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * ST_ACC_STRIDE);
                 const bool last = s + 1 == sg.to;
                 int slot = head;
+                bool odd_first = false;                    // the step's first tile is such a one
                 for (int j = 0; j < p.tiles && ok; ++j) {
                     if (have <= (s - sg.first) * p.adv + j) {
                         ok = __all_sync(0xffffffffu, mbar_wait(full(wslot), wphase, abort_flag, p.status));
                         if (!ok) break;
                         tc_fence_after();
+                        const uint32_t bit = 1u << wslot;
+                        odd = *(const volatile unsigned long long *)(flags + (seq++ & 15) * ST_CONV_WARPS) ? odd | bit : odd & ~bit;
                         if (++wslot == p.ring) { wslot = 0; wphase ^= 1u; }
                         ++have;
                     }
                     const int nk = min(p.per, p.RH - j * p.per) * ROW_STEPS;
                     const uint32_t a_lo = a_lo0 + (uint32_t)j * 1024u, b_lo = ring_lo + (uint32_t)slot * tile_step;
+                    const bool odd_tile = (odd >> slot) & 1u;
+                    if (j == 0) odd_first = odd_tile;
                     if (elect_one()) {
+                        if (__builtin_expect(odd_tile || odd_first, 0)) {
+                            // zero times a pixel that is no number is NaN: only the accumulator lanes whose window holds the row.
+                            // A conv row's sums begin with the first tile, which clears all lanes, or with its own first row.
+                            const uint32_t on16 = (uint32_t)(p.lanes_on >> (j * p.per * 4)), new16 = odd_first ? (uint32_t)(p.lanes_new >> (j * p.per * 4)) : 0u;
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            if (k < nk) umma_bf16_words(d_tmem, a_lo + (uint32_t)(2 * k), b_lo + (uint32_t)(2 * k), DESC_HI_SW128, idesc, (j | k) ? 1u : 0u);
+                            for (int k = 0; k < 4; ++k) {
+                                const uint32_t on = (on16 >> (k / ROW_STEPS * 4)) & 15u, fresh = k % ROW_STEPS ? 0u : (new16 >> (k / ROW_STEPS * 4)) & 15u;
+                                const uint32_t a = a_lo + (uint32_t)(2 * k), b = b_lo + (uint32_t)(2 * k);
+                                if (on != fresh) umma_bf16_words_lanes(d_tmem, a, b, DESC_HI_SW128, idesc, 1u, on ^ fresh);
+                                if (fresh) umma_bf16_words_lanes(d_tmem, a, b, DESC_HI_SW128, idesc, 0u, fresh);
+                            }
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                if (k < nk) umma_bf16_words(d_tmem, a_lo + (uint32_t)(2 * k), b_lo + (uint32_t)(2 * k), DESC_HI_SW128, idesc, (j | k) ? 1u : 0u);
+                        }
                         if (j < p.adv || last) umma_commit(empty(slot));      // not needed by the next step
                         if (j + 1 == p.tiles) umma_commit(tfull(acc));
                     }
@@ -557,7 +607,14 @@ cprune_status launch_conv_stem(const cprune_plan *plan, const float *x, const vo
     p.row_bytes = s.row_bytes; p.tile_bytes = s.tile_bytes; p.raw_bytes = s.raw_bytes; p.ring = s.ring; p.stage_bytes = s.stage_bytes;
     p.xch_words = s.xch_words;
     p.steps_per_img = s.steps_per_img; p.total_steps = i.N * s.steps_per_img;
-    p.k_pad = i.k_pad;
+    p.k_pad = i.k_pad; p.S = i.S;
+    p.lanes_on = p.lanes_new = 0;
+    for (int dy = 0; dy < s.D; ++dy)
+        for (int r = 0; r < i.R; ++r) {
+            const unsigned long long lanes = (unsigned long long)((1 << s.KF / 32) - 1) << (dy * s.KF / 32 + 4 * (i.stride * dy + r));
+            p.lanes_on |= lanes;
+            if (r == 0) p.lanes_new |= lanes;
+        }
     p.status = device_status_word();
     if (!p.status) return cuda_fail(cudaGetLastError(), "status word");
     int sms = 148, dev = 0;

@@ -193,6 +193,21 @@ __device__ __forceinline__ void umma_bf16_words(uint32_t d_tmem, uint32_t a_lo, 
         : "memory");
 }
 
+// The same for some of the accumulator's lanes: bit i of `on` enables lanes 32 i to 32 i + 31, the others keep their contents.
+__device__ __forceinline__ void umma_bf16_words_lanes(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
+                                                      uint32_t accumulate, uint32_t on) {
+    const uint32_t m0 = (on & 1u) - 1u, m1 = ((on >> 1) & 1u) - 1u, m2 = ((on >> 2) & 1u) - 1u, m3 = ((on >> 3) & 1u) - 1u;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %4};\n\t"
+        "mov.b64 db, {%2, %4};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, {%6, %7, %8, %9}, p;\n\t}"
+        :
+        : "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(desc_hi), "r"(accumulate), "r"(m0), "r"(m1), "r"(m2), "r"(m3)
+        : "memory");
+}
+
 // Descriptor of a K-major bf16 operand stored without swizzle as 8-row x 16-byte core matrices:
 // rows 16 bytes apart, 8-row groups 128 bytes apart, the next 8 channels `k_stride` bytes away
 // (the layout of one im2col TMA load of 8 channels per pixel; successive taps follow each other).

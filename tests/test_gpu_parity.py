@@ -345,6 +345,40 @@ def test_stems_of_large_images_with_fewer_conv_rows_per_step(cp, case):
 
 
 @pytest.mark.parametrize("case", [
+    # N, H, W, K, R, stride, pad, act, pool: 1, 2 and 4 conv rows per step (two of them with rows of the MMA left over), windows of 32,
+    # 64 and 128 bytes with one to thirteen pixels behind the filter's last
+    (9, 64, 64, 45, 3, 1, 1, "none", None), (5, 224, 224, 32, 3, 2, 1, "none", None), (4, 160, 160, 24, 3, 1, 1, "relu6", None),
+    (3, 224, 224, 48, 7, 2, 3, "none", None), (9, 68, 76, 24, 5, 1, 2, "relu", None), (9, 64, 68, 120, 3, 1, 1, "none", None),
+    (20, 36, 132, 40, 4, 2, 1, "none", "max3x3s2"), (4, 64, 136, 64, 7, 2, 3, "relu", "max3x3s2")])
+def test_a_pixel_that_is_no_number_reaches_only_the_conv_rows_whose_window_holds_it(cp, case):
+    # conv rows of one step share their input rows and windows are stored wider than the filter: neither may be multiplied with zeros
+    N, H, W, K, R, stride, pad, act, pool = case
+    plan = cp.cprune_task_plan(N, 3, H, W, K, R, R, stride, pad, 1, act, False, pool)
+    x, w, b, _ = wl.conv_task_tensors(99, N, 3, H, W, K, R, R)
+    model = stem_model(cp, plan, w, b)
+    bad, pixels = x.copy(), ((1, 21, 30, np.nan), (2, 38 % (H - 2), 61, np.inf))
+    for n, h, v, value in pixels:
+        bad[n, h, v, 1] = value
+    out = []
+    for t in (x, bad):
+        cp.cprune_model_run(model, _dev(t))
+        out.append(model.copy_tensor(1).float().cpu().numpy()[..., :K])
+    cp.cprune_poll_device_status()
+    touched = np.zeros((N, plan.P, plan.Q, 1))
+    for n, h, v, _ in pixels:
+        p, q = np.arange(plan.P) * stride - pad, np.arange(plan.Q) * stride - pad
+        touched[n, ..., 0] = ((p <= h) & (h < p + R))[:, None] & ((q <= v) & (v < q + R))[None, :]
+    if pool:
+        touched = oracle.maxpool(touched, 3, 2, 1)
+    touched = np.broadcast_to(touched > 0, out[0].shape)
+    assert np.array_equal(out[0][~touched], out[1][~touched])
+    if act != "none":
+        assert np.all(np.isfinite(out[1][1])) and (pool or np.all(out[1][1][touched[1]] == 0))
+    elif not pool:
+        assert np.all(np.isnan(out[1][1][touched[1]])) and not np.any(np.isfinite(out[1][2][touched[2]]))
+
+
+@pytest.mark.parametrize("case", [
     # N, C, H, W, K, R, stride, pad: fused in the patch kernel (tiles around whole 3x3 windows, even and odd extents),
     # and as a separate pass (few tiles; a task with wrap-around slots)
     (16, 3, 64, 64, 64, 7, 2, 3), (12, 3, 60, 52, 40, 7, 2, 3), (40, 3, 30, 30, 24, 3, 1, 1),
