@@ -84,8 +84,12 @@ __global__ void __launch_bounds__(256) gap_kernel(const bf16x8 *__restrict__ x, 
 // registers (a thread's 16-byte piece of 8 neighbouring features serves two MMA steps: the order of the contraction index is
 // free as long as both operands use the same), and the first pieces of the weights, which no kernel of the chain writes, are
 // requested before the preceding kernel has finished.
-// Back to back, cold weights: 1280 -> 1000 at 64 images 14.3 us with one warp per 4 features x 8 images on the FMA pipe, 5.0 us
-// with this one; 512 -> 1000 7.0 and 3.7 us; one image 5.2 and 2.9 us.
+// The tensor core truncates where it adds to an accumulator, so that a chain of MMAs loses more than float32 additions do.  Two
+// MMAs (32 features) start from zero and are added to the running sum with a rounded addition; the eight warps' sums meet in
+// float64.  Relative error (2-norm, against 64 bits): 512 features 5.4e-8, 1280 6.5e-8, 4096 9.0e-8, 25088 1.9e-7; as one chain per
+// warp 8.7e-8, 1.5e-7, 4.7e-7, 3.3e-6; float32 fused multiply-adds 6.7e-8, 7.7e-8, 9.8e-8, 2.2e-7.
+// Back to back, cold weights: 1280 -> 1000 at 64 images 14.3 us with one warp per 4 features x 8 images on the FMA pipe, 5.3 us
+// with this one (5.0 as one chain); 512 -> 1000 7.0 and 3.8 us; one image 5.0 and 3.0, 3.2 and 2.5 us.
 constexpr int FC_WARPS = 8, FC_AHEAD = 5;
 
 template <int MT>
@@ -127,8 +131,11 @@ __global__ void __launch_bounds__(FC_WARPS * 32) fc_kernel(const bf16x8 *__restr
         for (int i = 0; i < FC_AHEAD; ++i) {
 #pragma unroll
             for (int m = 0; m < MT; ++m) {
-                mma_16816(acc[m], xq[i][m][0].w[0], xq[i][m][1].w[0], xq[i][m][0].w[1], xq[i][m][1].w[1], wq[i].w[0], wq[i].w[1]);
-                mma_16816(acc[m], xq[i][m][0].w[2], xq[i][m][1].w[2], xq[i][m][0].w[3], xq[i][m][1].w[3], wq[i].w[2], wq[i].w[3]);
+                float s[4] = {0.f, 0.f, 0.f, 0.f};
+                mma_16816(s, xq[i][m][0].w[0], xq[i][m][1].w[0], xq[i][m][0].w[1], xq[i][m][1].w[1], wq[i].w[0], wq[i].w[1]);
+                mma_16816(s, xq[i][m][0].w[2], xq[i][m][1].w[2], xq[i][m][0].w[3], xq[i][m][1].w[3], wq[i].w[2], wq[i].w[3]);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[m][j] += s[j];
             }
             wq[i] = load_w(c0 + (FC_AHEAD + i) * FC_WARPS);
         }
@@ -141,10 +148,14 @@ __global__ void __launch_bounds__(FC_WARPS * 32) fc_kernel(const bf16x8 *__restr
     for (int e = threadIdx.x; e < MT * 16 * 8; e += FC_WARPS * 32) {
         const int r = e >> 3, c = e & 7, n = n0 + r, o = o0 + c;
         if (n >= N) continue;
-        float v = b[o];
+        double s[FC_WARPS];
 #pragma unroll
-        for (int q = 0; q < FC_WARPS; ++q) v += part[q][r][c];
-        v = apply_act(v, act);
+        for (int q = 0; q < FC_WARPS; ++q) s[q] = part[q][r][c];
+#pragma unroll
+        for (int h = FC_WARPS / 2; h > 0; h /= 2)
+#pragma unroll
+            for (int q = 0; q < h; ++q) s[q] += s[q + h];
+        const float v = apply_act((float)(s[0] + b[o]), act);
         if (out_is_f32) {
             if (o < out) ((float *)y)[(size_t)n * out + o] = v;
         } else {

@@ -768,6 +768,22 @@ def test_fully_connected_tiles(cp, N, inn, out, act):
     assert np.max(np.abs(y - ref) / scale) <= 1e-5
 
 
+@pytest.mark.parametrize("N,inn,out", [(1, 512, 1000), (64, 358, 1000), (64, 512, 1000), (16, 1280, 1000), (64, 4096, 200), (8, 25088, 200)])
+def test_fully_connected_sums_are_as_exact_as_float32_additions(cp, N, inn, out):
+    # Relative error of the float32 results, 2-norm: the last rounding (at most 2^-24 of each value) and the running sums of a
+    # warp, n = inn / 256 rounded additions.  Addition k of n rounds a partial sum of sqrt(k / n) of an eighth of the variance
+    # by 0.43 * 2^-24 (rms), which makes (0.43 * 2^-24)^2 * n / 2 for the eight warps together: below (2^-24)^2 * n / 8.
+    bound = 2.0 ** -24 * np.sqrt(1 + inn / 256 / 8)
+    for positive in (True, False):
+        x, w, b = wl.normal_f32(94, 0, (N, inn)), wl.normal_f32(94, 1, (out, inn), 1 / np.sqrt(inn)), wl.normal_f32(94, 2, (out,), 0.01)
+        x = np.abs(x) if positive else x
+        xb = cp.cprune_cast_input(_dev(x.reshape(N, 1, 1, inn))).reshape(N, -1)
+        y = cp.cprune_fc(xb, inn, *cp.cprune_fc_pack(_dev(w), _dev(b)), out, "none", out_f32=True).cpu().numpy().astype(np.float64)
+        ref = oracle.round_bf16(x).astype(np.float64) @ oracle.round_bf16(w).astype(np.float64).T + b
+        rel = np.linalg.norm(y - ref) / np.linalg.norm(ref)
+        assert rel <= bound, (rel, bound)
+
+
 def block_tensors(seed, N, C_in, H, W, hidden, C_out):
     x = wl.normal_f32(seed, 0, (N, H, W, C_in))
     we = wl.normal_f32(seed, 1, (hidden, C_in, 1, 1), np.sqrt(2.0 / C_in))
