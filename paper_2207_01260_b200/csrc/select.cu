@@ -189,6 +189,8 @@ __device__ __forceinline__ void select_list(const long long *key, int K, int kee
         if (lane == 0) atomicOr(&top, ((unsigned long long)hi << 32) | lo);
     }
     __syncthreads();
+    // norms are never negative, unless weights that break the precondition (infinite, NaN) made them so: these rank last
+    const unsigned long long flip = top & (1ull << 63);
     unsigned long long prefix = 0;
     int need = keep_k;                     // how many of the norms that share the prefix are kept
     int shift = top ? (63 - __clzll((long long)top)) / 8 * 8 : 0;
@@ -196,7 +198,7 @@ __device__ __forceinline__ void select_list(const long long *key, int K, int kee
         hist[tid] = 0;
         __syncthreads();
         for (int k = tid; k < K; k += SLICE_THREADS) {
-            const unsigned long long v = (unsigned long long)key[k];
+            const unsigned long long v = (unsigned long long)key[k] ^ flip;
             if (((v ^ prefix) >> shift) < 256) atomicAdd(&hist[(int)((v >> shift) & 255)], 1);
         }
         __syncthreads();
@@ -228,7 +230,7 @@ __device__ __forceinline__ void select_list(const long long *key, int K, int kee
     const int k0 = min(tid * per, K), k1 = min(k0 + per, K);
     int mine = 0;                          // larger norms (upper half) and equal norms (lower half) among this thread's filters
     for (int k = k0; k < k1; ++k) {
-        const unsigned long long v = (unsigned long long)key[k];
+        const unsigned long long v = (unsigned long long)key[k] ^ flip;
         mine += (v > prefix ? 1 << 16 : 0) + (v == prefix ? 1 : 0);
     }
     int incl = mine;
@@ -243,7 +245,7 @@ __device__ __forceinline__ void select_list(const long long *key, int K, int kee
     for (int q = 0; q < warp; ++q) at += warp_sum[q];
     int larger = at >> 16, equal = at & 0xffff;
     for (int k = k0; k < k1; ++k) {
-        const unsigned long long v = (unsigned long long)key[k];
+        const unsigned long long v = (unsigned long long)key[k] ^ flip;
         if (v > prefix) {
             list[larger + min(equal, need)] = k;
             ++larger;

@@ -158,6 +158,26 @@ def test_select_flags_bad_weights_and_bad_arguments(cp):
     assert e.value.status == 3
 
 
+@pytest.mark.parametrize("K", [64, 300, 8200])
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+def test_filters_that_hold_no_numbers_rank_last(cp, K, value):
+    # the data breaks the precondition (and the status word says so), but the order is that of signed norms on both paths: the
+    # integer sums of these filters are negative
+    w = wl.normal_f32(26, 1, (K, 4, 3, 3), 0.05)
+    bad = [7, K // 2, K - 1]
+    for k in bad:
+        w[k, 1, 1, 1] = value
+    zeroed = w.copy()
+    zeroed[bad] = 0
+    for keep in (1, K // 3, K - len(bad)):
+        kept = cp.cprune_select_filters(_dev(w), keep)[0].cpu().numpy()
+        shared = cp.cprune_select_shared([_dev(w)], keep).cpu().numpy()
+        with pytest.raises(cp.CpruneError) as e:
+            cp.cprune_poll_device_status()
+        assert e.value.status == 7
+        assert np.array_equal(kept, oracle.select_indices(zeroed, keep)) and np.array_equal(shared, kept)
+
+
 # ------------------------------------------------------------------ single tasks
 
 def test_config1_single_pruned_task(cp):
