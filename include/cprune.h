@@ -224,7 +224,8 @@ cprune_status cprune_pack_weights(const cprune_plan *plan, const float *w, const
  * The workspace holds what the plan needs besides x and y: float32 partial sums of a split reduction,
  * the unpooled result when the pool runs as a separate pass, the regrouped input of a stem.
  * Enqueue only (at most three launches), no allocation, no synchronisation.  Pointers must be 16-byte
- * aligned.  Errors: INVALID_ARG (null pointer, missing workspace, residual mismatch with the plan), CUDA. */
+ * aligned; a packed bias off the alignment that its kernel reads is refused.  Errors: INVALID_ARG (null or misaligned pointer,
+ * missing workspace, residual mismatch with the plan), CUDA. */
 cprune_status cprune_task_run(cprune_plan *plan, const void *x, const void *w_packed, const float *b_packed,
                               const void *residual, void *y, void *workspace, void *stream);
 

@@ -1074,6 +1074,7 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
     plan->partial_bytes = 0;
     plan->pre_bytes = g.stem ? ((size_t)i.N * g.He * g.WP * 32 + 255) / 256 * 256 : 0;
     plan->fused_pool = (pool || pool3) ? 1 : 0;
+    plan->bias_align = bt.tiles_n * bt.FT <= PK_BIAS_FLOATS ? 4 : 8;      // (more filters: read in pairs from global memory)
     i.tile_m = 128 * bt.MT;
     i.tile_n = bt.FT;
     i.tile_k = 64;

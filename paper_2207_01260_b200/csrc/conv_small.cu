@@ -239,6 +239,7 @@ bool plan_conv_small(cprune_plan *plan, bool other_is_direct) {
     plan->partial_bytes = 0;
     plan->pre_bytes = 0;
     plan->fused_pool = pool ? 1 : 0;
+    plan->bias_align = 4;
     i.tile_m = CS_WARPS / kw * 16 * mt;
     i.tile_n = 8 * nt;
     i.tile_k = 32;

@@ -885,6 +885,7 @@ cprune_status plan_conv_tensor(cprune_plan *plan) {
         if (plan->splits > 1) plan->fused_pool = 1;
         else if (pow2 && i.Q <= (plan->orient == ORIENT_PIX ? 16 : 32)) plan->fused_pool = 1;
     }
+    plan->bias_align = plan->orient == ORIENT_PIX && plan->splits == 1 ? 16 : 4;
     plan->ipp = (iters + plan->splits - 1) / plan->splits;
     plan->partial_bytes = plan->splits > 1 ? (size_t)plan->splits * (size_t)M * i.k_alloc * 4 : 0;
     {

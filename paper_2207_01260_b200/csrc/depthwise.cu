@@ -133,7 +133,10 @@ __global__ void __launch_bounds__(256, 2) depthwise_kernel(const __grid_constant
                 for (int k = 0; k < NW; ++k) wf[r][s][k] = widen2(t[k]);
             }
 #pragma unroll
-        for (int k = 0; k < NW; ++k) bf[k] = *reinterpret_cast<const unsigned long long *>(p.b + 2 * (word + k));
+        for (int k = 0; k < NW; ++k) {
+            const float lo = __ldg(p.b + 2 * (word + k)), hi = __ldg(p.b + 2 * (word + k) + 1);      // (any float32 address)
+            asm("mov.b64 %0, {%1, %2};" : "=l"(bf[k]) : "f"(lo), "f"(hi));
+        }
     }
 
     const bool has_res = p.res != nullptr;

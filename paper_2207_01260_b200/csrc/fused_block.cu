@@ -519,7 +519,7 @@ cprune_status cprune_block_pack(const cprune_block *block, const float *w_expand
 cprune_status cprune_block_run(cprune_block *block, const void *x, const void *w_packed, const float *b_packed, void *y, void *workspace,
                                void *stream) {
     if (!block || !x || !w_packed || !b_packed || !y) return CPRUNE_ERR_INVALID_ARG;
-    if (((uintptr_t)x | (uintptr_t)w_packed | (uintptr_t)y | (uintptr_t)workspace) & 15) return CPRUNE_ERR_INVALID_ARG;
+    if (((uintptr_t)x | (uintptr_t)w_packed | (uintptr_t)b_packed | (uintptr_t)y | (uintptr_t)workspace) & 15) return CPRUNE_ERR_INVALID_ARG;
     if (block->info.workspace_bytes && !workspace) return CPRUNE_ERR_INVALID_ARG;
     const cprune_block_info &i = block->info;
     const int HW = i.H * i.W;

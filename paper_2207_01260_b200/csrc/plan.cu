@@ -141,6 +141,7 @@ cprune_status task_run_internal(cprune_plan *plan, const void *x, const void *w_
     if ((plan->opts.residual != 0) != (residual != nullptr)) return CPRUNE_ERR_INVALID_ARG;
     if (((uintptr_t)x | (uintptr_t)w_packed | (uintptr_t)y | (uintptr_t)residual | (uintptr_t)workspace) & 15)
         return CPRUNE_ERR_INVALID_ARG;
+    if ((uintptr_t)b_packed & (unsigned)(plan->bias_align - 1)) return CPRUNE_ERR_INVALID_ARG;      // (a read of its kernel would fault)
     const cprune_plan_info &i = plan->info;
     const bool pool = plan->opts.pool != CPRUNE_POOL_NONE && !(i.kernel == CPRUNE_KERNEL_TENSOR && plan->fused_pool);
     if (i.workspace_bytes && !workspace) return CPRUNE_ERR_INVALID_ARG;

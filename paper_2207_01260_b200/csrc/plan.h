@@ -76,6 +76,7 @@ struct cprune_plan {
     StemTiling stem = {};
     int small = 0;                  // 1: task of few pixels on conv_small.cu: 8 / small_kw groups of 16 * small_mt pixels x 8 * small_nt
     int small_mt = 0, small_nt = 0, small_kw = 0;   // filters per block, small_kw warps to a group
+    int bias_align = 4;             // alignment of the packed bias that the kernel's widest read of it needs
     double est_us = 0.0;            // the planner's cost-model estimate of the task's time
 };
 

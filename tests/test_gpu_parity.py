@@ -978,6 +978,24 @@ def test_a_nan_in_a_pooled_window_of_few_pixels(cp):
     assert torch.isfinite(y[0]).all()
 
 
+@pytest.mark.parametrize("case", [
+    # N, C, H, K, R, stride, groups: depthwise 3x3 and 5x5, the patch kernel (bias in shared memory; staged as in memory), filters
+    # on the row side of the im2col kernel, few pixels
+    (4, 40, 14, 40, 3, 1, 40), (4, 40, 14, 40, 5, 2, 40), (64, 64, 28, 48, 3, 1, 1), (64, 48, 56, 72, 1, 1, 1), (64, 64, 28, 96, 3, 2, 1),
+    (2, 64, 16, 48, 3, 1, 1)])
+def test_a_packed_bias_at_any_float_address(cp, case):
+    N, C, H, K, R, stride, groups = case
+    plan = cp.cprune_task_plan(N, C, H, H, K, R, R, stride, R // 2, groups)
+    x, w, b, _ = wl.conv_task_tensors(100, N, C, H, H, K, R, R, groups)
+    xb, (wp, bp) = cp.cprune_cast_input(_dev(x)), cp.cprune_pack_weights(plan, _dev(w), _dev(b))
+    y = cp.cprune_task_run(plan, xb, wp, bp)
+    for off in (1, 2, 3):
+        moved = torch.empty(bp.numel() + off, device="cuda")[off:]
+        moved.copy_(bp)
+        assert torch.equal(cp.cprune_task_run(plan, xb, wp, moved), y)
+    cp.cprune_poll_device_status()
+
+
 def test_plan_cache_shares_repeated_shapes(cp):
     from paper_2207_01260_b200.pipeline import PrunedNetwork
     table = wl.resnet18()

@@ -122,6 +122,18 @@ def test_plan_argument_errors(cp):
     assert e.value.status == 1
 
 
+def test_a_bias_off_the_alignment_that_its_kernel_reads_is_refused(cp):
+    # more than 512 filters on the patch kernel are read in pairs, the pixel-major im2col kernel reads four at a time: refused before
+    # anything is launched (the addresses are never touched)
+    for args, variant, align in (((64, 96, 14, 14, 600, 1, 1, 1, 0), 1, 8), ((64, 64, 28, 28, 200, 3, 3, 2, 1), 0, 16)):
+        plan = cp.cprune_task_plan(*args)
+        assert plan.variant == variant and plan.workspace_bytes == 0
+        for off in range(4, align, 4):
+            assert cp.lib().cprune_task_run(plan.handle, 1 << 20, 2 << 20, (3 << 20) + off, None, 4 << 20, None, None) == 1, (args, off)
+    blk = cp.cprune_block_plan(2, 64, 14, 14, 288, 64, residual=True)
+    assert cp.lib().cprune_block_run(blk.handle, 1 << 20, 2 << 20, (3 << 20) + 8, 4 << 20, 5 << 20, None) == 1
+
+
 def test_missing_library_fails_loudly(cp, monkeypatch):
     from paper_2207_01260_b200 import binding
     monkeypatch.setattr(binding, "_lib", None)
