@@ -61,15 +61,15 @@ static cprune_status enqueue(cprune_model *m, const float *x, float *logits, cud
 
 // How the model's first task gets at the float32 image when it is the only reader of the input: straight (the stem kernel
 // casts on the way in), through the regrouped copy of the patch kernel (cast and regrouping in one pass), or, otherwise,
-// from the bf16 NHWC copy that every model can make.
+// from the bf16 NHWC copy that every model can make.  The stem kernel's bulk copies need an image on a 16-byte boundary.
 enum { INPUT_CAST = 0, INPUT_REGROUP = 1, INPUT_DIRECT = 2 };
-static int input_path(const cprune_model *m) {
+static int input_path(const cprune_model *m, bool aligned = true) {
     if (m->tasks.empty()) return INPUT_CAST;
     const cprune_task_desc &d0 = m->tasks[0];
     if (d0.op != CPRUNE_OP_CONV || d0.in != 0 || !d0.plan) return INPUT_CAST;
     for (size_t t = 1; t < m->tasks.size(); ++t)
         if (m->tasks[t].in == 0 || m->tasks[t].res == 0) return INPUT_CAST;
-    if (d0.plan->stem.ok) return INPUT_DIRECT;
+    if (d0.plan->stem.ok && aligned) return INPUT_DIRECT;
     return d0.plan->patch && d0.plan->narrow ? INPUT_REGROUP : INPUT_CAST;
 }
 
@@ -80,8 +80,7 @@ static int conv_launches(const cprune_plan *plan) {
 }
 
 static cprune_status enqueue_chain(cprune_model *m, const float *x, float *logits, cudaStream_t st) {
-    int path = input_path(m);
-    if (path == INPUT_DIRECT && ((uintptr_t)x & 15)) path = INPUT_CAST;      // bulk copies need 16-byte alignment
+    const int path = input_path(m, ((uintptr_t)x & 15) == 0);
     cprune_status s = CPRUNE_OK;
     if (path == INPUT_REGROUP) s = regroup_stem_input(m->tasks[0].plan, x, 1, stem_scratch(m->tasks[0].plan, m->workspace), st);
     else if (path == INPUT_CAST) s = cprune_cast_input(x, (size_t)m->N * m->H * m->W, m->C, tensor_ptr(m, 0), st);

@@ -398,6 +398,25 @@ def test_a_pixel_that_is_no_number_reaches_only_the_conv_rows_whose_window_holds
         assert np.all(np.isnan(out[1][1][touched[1]])) and not np.any(np.isfinite(out[1][2][touched[2]]))
 
 
+def test_an_image_off_a_16_byte_boundary_is_cast_and_regrouped_in_one_pass(cp):
+    N, H, K = 16, 128, 64
+    plan = cp.cprune_task_plan(N, 3, H, H, K, 7, 7, 2, 3, 1)
+    assert plan.variant == 1 and plan.workspace_bytes > 0           # by itself the task runs on a regrouped input
+    x, w, b, _ = wl.conv_task_tensors(101, N, 3, H, H, K, 7, 7)
+    model = stem_model(cp, plan, w, b)
+    mark = _dev(np.full((N, H, H, 3), 7.0, dtype=np.float32))
+    ptr, _ = model.tensor(0)                                        # the bf16 copy of the image, which nobody needs
+    assert cp.lib().cprune_cast_input(mark.data_ptr(), N * H * H, 3, ptr, torch.cuda.current_stream().cuda_stream) == 0
+    odd = torch.empty(x.size + 1, device="cuda")[1:].view(x.shape)
+    odd.copy_(_dev(x))
+    cp.cprune_model_run(model, odd)
+    a = model.copy_tensor(1)
+    assert torch.all(model.copy_tensor(0)[..., :3] == 7.0)
+    y = cp.cprune_task_run(plan, cp.cprune_cast_input(_dev(x)), *cp.cprune_pack_weights(plan, _dev(w), _dev(b)))
+    cp.cprune_poll_device_status()
+    assert torch.equal(a, y)                                        # the task's own kernel on the same values
+
+
 @pytest.mark.parametrize("case", [
     # N, C, H, W, K, R, stride, pad: fused in the patch kernel (tiles around whole 3x3 windows, even and odd extents),
     # and as a separate pass (few tiles; a task with wrap-around slots)
