@@ -278,12 +278,12 @@ def main():
     if rank == 0 and not args.no_task_times:
         peaks = measured_peaks()
         per_task = net_task_times(cp, net, table)
-        # the tensor family has three kernels; the roofline object describes the one that takes more of the step
+        # the tensor family has four kernels; the roofline object describes the one that takes more of the step
+        tens_names = {0: "conv_tc_kernel", 1: "conv_patch_kernel", 3: "conv_small_kernel", STEM_VARIANT: "conv_stem_kernel"}
         tens_all = [t for t in per_task if t["kernel"] == "tensor"]
-        by_variant = {v: [t for t in tens_all if {2: 1}.get(t["variant"], t["variant"]) == v] for v in (0, 1, 3)}   # 1, 2: the patch kernel
-        top = max((0, 1, 3), key=lambda v: sum(t["ms"] for t in by_variant[v]))
-        tens = by_variant[top]
-        tens_name = {0: "conv_tc_kernel", 1: "conv_patch_kernel", 3: "conv_small_kernel"}[top]
+        by_variant = {v: [t for t in tens_all if {2: 1}.get(t["variant"], t["variant"]) == v] for v in tens_names}   # 1, 2: the patch kernel
+        top = max(tens_names, key=lambda v: sum(t["ms"] for t in by_variant[v]))
+        tens, tens_name = by_variant[top], tens_names[top]
         dw = [t for t in per_task if t["kernel"] == "depthwise"]
         t_tens, t_dw = sum(t["ms"] for t in tens), sum(t["ms"] for t in dw)
         if t_dw > t_tens and dw:
@@ -573,24 +573,30 @@ def time_task_cold(cp, plan, wp, bp, with_res, launches=8, reps=3, warmup=2):
     return best, nsets
 
 
+STEM_VARIANT = 4       # here, beside the library's variants: a first task that reads the network's float32 image itself
+
+
 def net_task_times(cp, net, table):
-    """Times every distinct conv task of the network alone, cold (see time_task_cold), with its own packed weights."""
+    """Times every distinct conv task of the network alone, cold (see time_task_cold), with its own packed weights.  A first task
+    that reads the image runs on another kernel in the network than by itself: the model times that one (on one set of buffers)."""
     out, seen = [], {}
     for l in table["layers"]:
         if l["kind"] != "conv" or l["name"] not in net.plans:
             continue
         plan = net.plans[l["name"]]
         key = plan.handle.value
+        image = net.model.reads_image and not out
         if key not in seen:
             wp, bp = net.packed[l["name"]]
-            seen[key] = time_task_cold(cp, plan, wp, bp, l.get("res") is not None)
+            seen[key] = (net.model.time_tasks(8)[0], 1) if image else time_task_cold(cp, plan, wp, bp, l.get("res") is not None)
         ms, nsets = seen[key]
         i = plan.info
+        nbytes = i["algorithmic_bytes"] + (2.0 * i["N"] * i["H"] * i["W"] * i["C"] if image else 0.0)      # four bytes per input value, not two
         out.append({"name": l["name"], "kernel": cp.KERNEL_NAMES[i["kernel"]], "C": i["C"], "K": i["K"],
                     "HW": [i["H"], i["W"]], "R": i["R"], "stride": i["stride"], "ms": ms, "flops": i["flops"],
-                    "variant": i["variant"], "bytes": i["algorithmic_bytes"], "tflops": i["flops"] / ms / 1e9,
-                    "gbs": i["algorithmic_bytes"] / ms / 1e6, "tile_n": i["tile_n"], "tiles": i["tiles_m"] * i["tiles_n"],
-                    "buffer_sets": nsets, "timing": "8 launches per event pair, rotating buffers (cold)"})
+                    "variant": STEM_VARIANT if image else i["variant"], "bytes": nbytes, "tflops": i["flops"] / ms / 1e9,
+                    "gbs": nbytes / ms / 1e6, "tile_n": i["tile_n"], "tiles": i["tiles_m"] * i["tiles_n"],
+                    "buffer_sets": nsets, "timing": "8 launches per event pair, " + ("one buffer set, from the float32 image" if image else "rotating buffers (cold)")})
     return out
 
 

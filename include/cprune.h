@@ -319,6 +319,10 @@ cprune_status cprune_model_tensor(const cprune_model *model, int id, const void 
 cprune_status cprune_model_copy_tensor(const cprune_model *model, int id, void *dst, void *stream);
 /* Kernel launches one cprune_model_run enqueues. */
 int cprune_model_launches(const cprune_model *model);
+/* 1 if the model's first task, a conv task with three input channels, runs straight from the float32 image (cast, convolution and
+ * pool in one kernel), 0 otherwise.  The model then launches another kernel for it than cprune_task_run does with the same plan:
+ * variant, the splits, est_us and cprune_prune_step describe the program of cprune_task_run, cprune_model_time_tasks the model's. */
+int cprune_model_reads_image(const cprune_model *model);
 
 /* The model's task table (paper Sec. 3.4: which subgraphs share which task): one entry per distinct plan among
  * the model's conv tasks, in order of first appearance.  entries (host) receives at most max_entries entries;
@@ -330,7 +334,8 @@ typedef struct {
 } cprune_task_entry;
 cprune_status cprune_model_task_table(const cprune_model *model, cprune_task_entry *entries, int max_entries, int *n_entries);
 /* Times every entry of the task table on the device: the entry's first subgraph is run `reps` times back to back
- * on the model's own buffers between two CUDA events (after one untimed run); ms (host, one value per table entry)
+ * on the model's own buffers between two CUDA events (after one untimed run), the model's first task as the model runs it, from
+ * a float32 image of zeros that takes the place of tensor 0; ms (host, one value per table entry)
  * receives the mean milliseconds per run.  Blocks until the measurements are done.  Feed ms and the counts to
  * cprune_task_order to get the paper's pruning priority. */
 cprune_status cprune_model_time_tasks(cprune_model *model, int reps, double *ms, void *stream);

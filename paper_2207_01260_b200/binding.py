@@ -31,7 +31,7 @@ EXPORTS = [
     "cprune_model_destroy", "cprune_poll_device_status", "cprune_select_shared", "cprune_prune_step",
     "cprune_task_estimate", "cprune_task_order", "cprune_model_task_table", "cprune_model_time_tasks",
     "cprune_selftest_wait_timeout", "cprune_block_plan", "cprune_block_query", "cprune_block_release", "cprune_block_pack",
-    "cprune_block_run",
+    "cprune_block_run", "cprune_model_reads_image",
 ]
 
 
@@ -118,6 +118,7 @@ def lib():
                                           POINTER(c_int), POINTER(c_int)]
         L.cprune_model_copy_tensor.argtypes = [c_void_p, c_int, c_void_p, c_void_p]
         L.cprune_model_launches.argtypes = [c_void_p]
+        L.cprune_model_reads_image.argtypes = [c_void_p]
         L.cprune_model_destroy.argtypes = [c_void_p]
         L.cprune_poll_device_status.argtypes = [c_void_p]
         L.cprune_select_shared.argtypes = [POINTER(c_void_p), POINTER(c_size_t), c_int, c_int, c_int, c_void_p, c_void_p,
@@ -455,6 +456,11 @@ class Model:
     @property
     def launches(self):
         return lib().cprune_model_launches(self.handle)
+
+    @property
+    def reads_image(self):
+        """Whether the first task runs straight from the float32 image."""
+        return bool(lib().cprune_model_reads_image(self.handle))
 
     def tensor(self, tid):
         """bf16 view [n, h, w, c_pad] of an activation buffer (for tests)."""

@@ -398,6 +398,23 @@ def test_a_pixel_that_is_no_number_reaches_only_the_conv_rows_whose_window_holds
         assert np.all(np.isnan(out[1][1][touched[1]])) and not np.any(np.isfinite(out[1][2][touched[2]]))
 
 
+def test_the_task_times_of_a_model_are_those_of_the_kernels_it_launches(cp):
+    # the entry of a first task that reads the image is timed on that kernel, with an image of zeros in the place of the unused bf16 copy
+    N, H, K = 16, 128, 48
+    plan = cp.cprune_task_plan(N, 3, H, H, K, 7, 7, 2, 3, 1)
+    _, w, b, _ = wl.conv_task_tensors(102, 1, 3, 8, 8, K, 7, 7)
+    model = stem_model(cp, plan, w, b)
+    assert model.reads_image
+    cp.cprune_model_run(model, torch.zeros((N, H, H, 3), device="cuda"))
+    a = model.copy_tensor(1)
+    mark = _dev(np.full((N, H, H, 3), 7.0, dtype=np.float32))
+    ptr, _ = model.tensor(0)
+    assert cp.lib().cprune_cast_input(mark.data_ptr(), N * H * H, 3, ptr, torch.cuda.current_stream().cuda_stream) == 0
+    (ms,) = model.time_tasks(2)
+    cp.cprune_poll_device_status()
+    assert torch.equal(model.copy_tensor(1), a) and 0 < ms < 5
+
+
 def test_an_image_off_a_16_byte_boundary_is_cast_and_regrouped_in_one_pass(cp):
     N, H, K = 16, 128, 64
     plan = cp.cprune_task_plan(N, 3, H, H, K, 7, 7, 2, 3, 1)
