@@ -66,7 +66,7 @@ enum { INPUT_CAST = 0, INPUT_REGROUP = 1, INPUT_DIRECT = 2 };
 static int input_path(const cprune_model *m, bool aligned = true) {
     if (m->tasks.empty()) return INPUT_CAST;
     const cprune_task_desc &d0 = m->tasks[0];
-    if (d0.op != CPRUNE_OP_CONV || d0.in != 0 || !d0.plan) return INPUT_CAST;
+    if (d0.op != CPRUNE_OP_CONV || d0.in != 0 || d0.res == 0 || !d0.plan) return INPUT_CAST;
     for (size_t t = 1; t < m->tasks.size(); ++t)
         if (m->tasks[t].in == 0 || m->tasks[t].res == 0) return INPUT_CAST;
     if (d0.plan->stem.ok && aligned) return INPUT_DIRECT;

@@ -415,6 +415,21 @@ def test_the_task_times_of_a_model_are_those_of_the_kernels_it_launches(cp):
     assert torch.equal(model.copy_tensor(1), a) and 0 < ms < 5
 
 
+def test_a_first_task_that_adds_the_image_to_its_result(cp):
+    # the residual is the bf16 copy of the image: it has to be made even where the convolution itself runs on a regrouped input
+    N, H = 64, 128
+    plan = cp.cprune_task_plan(N, 3, H, H, 3, 3, 3, 1, 1, 1, "none", True)
+    x, w, b, _ = wl.conv_task_tensors(103, N, 3, H, H, 3, 3, 3)
+    packed, fc = cp.cprune_pack_weights(plan, _dev(w), _dev(b)), cp.cprune_fc_pack(torch.ones((8, 3), device="cuda"))
+    tasks = [cp.TaskDesc(op=cp.OP_CONV, in_=0, out=1, res=0, plan=plan.handle, w=packed[0].data_ptr(), b=packed[1].data_ptr()),
+             cp.TaskDesc(op=cp.OP_GAP, in_=1, out=2, res=-1),
+             cp.TaskDesc(op=cp.OP_FC, in_=2, out=3, res=-1, w=fc[0].data_ptr(), b=fc[1].data_ptr(), p0=3, p1=8)]
+    model = cp.cprune_model_create(N, H, H, 3, tasks, keep_alive=(plan, packed, fc))
+    cp.cprune_model_run(model, _dev(x))
+    xb = cp.cprune_cast_input(_dev(x))
+    assert plan.variant == 1 and torch.equal(model.copy_tensor(1), cp.cprune_task_run(plan, xb, *packed, xb))
+
+
 def test_an_image_off_a_16_byte_boundary_is_cast_and_regrouped_in_one_pass(cp):
     N, H, K = 16, 128, 64
     plan = cp.cprune_task_plan(N, 3, H, H, K, 7, 7, 2, 3, 1)
