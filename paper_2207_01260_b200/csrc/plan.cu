@@ -84,10 +84,13 @@ static cprune_status build_plan(const PlanKey &key, cprune_plan **out) {
     // how the program splits the filter axis (see cprune_prune_step)
     i.splits = family == CPRUNE_KERNEL_TENSOR ? pl->splits : 1;
     if (family == CPRUNE_KERNEL_TENSOR && pl->small) {
-        // filter tiles x 8-filter instruction groups per tile, stored in the same pieces
-        i.unit_compute = i.unit_store = 8;
-        i.split_compute[0] = i.split_store[0] = i.tiles_n;
-        i.split_compute[1] = i.split_store[1] = i.tile_n / 8;
+        // filter tiles x 8-filter instruction groups per tile; stored in pieces of the memory layout's granule (two tiles of
+        // eight filters share one of sixteen)
+        i.unit_compute = 8;
+        i.split_compute[0] = i.tiles_n; i.split_compute[1] = i.tile_n / 8;
+        i.unit_store = i.K > 128 ? 16 : 8;
+        i.split_store[0] = i.tile_n >= i.unit_store ? i.tiles_n : i.k_pad / i.unit_store;
+        i.split_store[1] = i.tile_n >= i.unit_store ? i.tile_n / i.unit_store : 1;
     } else if (family == CPRUNE_KERNEL_TENSOR && (pl->patch || pl->orient == 0)) {
         // filters on the MMA's column side: tiles_n tiles of tile_n filters, built from 16-filter instruction groups
         // (64-filter groups when there are several tiles: tiles end on store-box boundaries), stored in pieces of the

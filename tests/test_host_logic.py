@@ -164,6 +164,20 @@ def test_prune_step_follows_the_lcm_rule_on_the_plans_own_splits(cp):
     assert cp.cprune_prune_step(p) == 16
 
 
+def test_the_store_unit_of_every_program_is_the_granule_of_the_memory_layout(cp):
+    # 8 filters up to 128, 16 above: fewer filters than that do not shrink the tensor, whatever kernel writes it
+    variants = set()
+    for N in (1, 4, 64):
+        for C, H, R, stride in ((64, 56, 3, 1), (128, 28, 3, 2), (512, 7, 3, 1), (720, 7, 1, 1), (96, 14, 1, 1)):
+            for K in (24, 40, 128, 130, 160, 358, 600):
+                p = cp.cprune_task_plan(N, C, H, H, K, R, R, stride, R // 2)
+                variants.add(p.variant)
+                assert p.unit_store == (16 if K > 128 else 8), (N, C, H, K, p.variant)
+                assert p.split_store[0] * p.split_store[1] * p.unit_store >= p.k_pad
+                assert cp.cprune_prune_step(p) % p.unit_store == 0
+    assert {0, 1, 3} <= variants
+
+
 def test_task_estimate_is_a_staircase_in_the_filter_count(cp):
     p = cp.cprune_task_plan(64, 128, 28, 28, 128, 3, 3, 1, 1)
     est = [cp.cprune_task_estimate(p, k) for k in range(128, 31, -1)]
