@@ -1047,6 +1047,18 @@ def test_a_packed_bias_at_any_float_address(cp, case):
     cp.cprune_poll_device_status()
 
 
+@pytest.mark.parametrize("raw", [True, False])
+def test_calls_go_to_the_current_stream(cp, raw, monkeypatch):
+    # with torch's call for the raw handle, which it does not promise, and without
+    from paper_2207_01260_b200 import binding
+    if not raw:
+        monkeypatch.setattr(binding, "_raw_stream", None)
+    s = torch.cuda.Stream()
+    assert binding._stream() == torch.cuda.current_stream().cuda_stream and binding._stream(s) == s.cuda_stream
+    with torch.cuda.stream(s):
+        assert binding._stream() == s.cuda_stream
+
+
 def test_plan_cache_shares_repeated_shapes(cp):
     from paper_2207_01260_b200.pipeline import PrunedNetwork
     table = wl.resnet18()
