@@ -211,7 +211,8 @@ bool plan_conv_small(cprune_plan *plan, bool other_is_direct) {
         return 1.66 + (latency + issue) / 1900.0;
     };
     // The split of the contraction fixes the order of its sums.  It is chosen for a typical filter count and not for this
-    // task's, so that a filter's results do not depend on how many other filters were pruned (2 % slower on average).
+    // task's, so that within this kernel a filter's results do not depend on how many other filters were pruned (2 % slower on
+    // average).  Whether the task runs here does depend on its filter count, and the other kernels add in another order.
     int kw = 1;
     double best = 1e30;
     for (const SmallTile &s : kTiles)

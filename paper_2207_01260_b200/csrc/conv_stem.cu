@@ -23,9 +23,11 @@
 //               bulk copy: the output rows of a step are contiguous.
 // A block works through consecutive steps; with a pool it recomputes one step where it starts inside an image (the odd conv
 // row above).
-// What bounds it: the converters (about 1500 cycles per step of the 7x7 stem) and, close behind, the MMAs and the pooling epilogue.
-// Stem of 64 224x224 images, back to back with a one-pixel tail (about 5 us of it): 7x7 stride 2, 64 filters, pooled 70.4 us
-// with a regrouping pass and the patch kernel, 50.6 us here; 3x3 stride 2, 32 filters 56.9 and 32.1 us.
+// What bounds it: no role's work but the waits from one to the next.  64 more images take the pooled 7x7 stem 38.7 us (1.6 us a
+// step); without the conversions and window copies 36.9, without the MMAs 36.9, without the pooling arithmetic 36.3 us.  (3x3: 20.7,
+// 17.8, 21.1 and 17.9 us.)  At 8 images issue slots are 33 % busy, the tensor pipe 12 %, DRAM 3 %.
+// Stem of 64 224x224 images, launched back to back: 7x7 stride 2, 64 filters, pooled 63.8 us with a regrouping pass and the patch
+// kernel, 51.3 us here; 3x3 stride 2, 32 filters 49.3 and 32.7 us.
 #include <cuda.h>
 
 #include <cstring>

@@ -10,9 +10,11 @@
 // NACC = ceil(R / STRIDE) rows of accumulators are alive, and the row loop is unrolled NACC times so that their rotation
 // costs no moves.  The waits on the loads are bounded like every other device-side wait.
 //
-// What bounds it: the instructions of a row step (about 105 per 8 outputs of a thread: 36 packed FMAs, 16 conversions, the
-// clamp and packing, loads, stores) at three warps per scheduler, before memory does.  C 108, 56x56, batch 64, stride 1,
-// cold: 23.4 us = 3.7 TB/s (a thread per column of 8 channels, one tile per CTA: 30.9 us); 5x5, C 288, 14x14, batch 20:
+// What bounds it: latency at three warps per scheduler.  C 108, 56x56, batch 64, stride 1: two patch buffers of 28 KB let three
+// CTAs of four warps onto an SM (registers would let four); 12.6 M warp instructions keep the issue slots 51 % busy while an SM
+// works and 40 % over the kernel, a fifth of which is start and drain; DRAM 21 %.  Between two instructions of a warp 1.4 cycles
+// of 5.5 go to fixed-latency dependences, 0.5 each to the math pipe, the CTA barrier per tile and dispatch, 0.4 to memory.
+// Cold: 23.4 us = 3.7 TB/s (a thread per column of 8 channels, one tile per CTA: 30.9 us); 5x5, C 288, 14x14, batch 20:
 // 6.6 us (22.0 us with the taps in shared memory).  Packed FMAs: 23.4 against 26.4 us with scalar ones.  Streaming row
 // chunks through a ring instead of whole patches: 29 us; loads straight from global memory: 35 us.
 

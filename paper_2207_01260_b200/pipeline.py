@@ -23,9 +23,10 @@ class PrunedNetwork:
     # separate tasks of a block in 2.7 to 3.5 us each, the separate form is the faster one at every batch.  Measured on pruned
     # MobileNetV2 (us per batch, separate / 7x7 blocks fused / all eight blocks fused): batch 1 147 / 164 / 204,
     # 2 164 / 176 / 210, 4 199 / 207 / 234, 8 230 / 239 / 261, 16 298 / 304 / 315, 64 541 / - / 779; MnasNet (two blocks, 14x14)
-    # 159 / - / 179 at batch 1, 324 / - / 326 at 16.  What the default promises (small batches have fused blocks, large ones
-    # none) is kept at the smallest batch above single-image serving, for the blocks that it costs least; fuse_blocks=True
-    # fuses all that the library supports.
+    # 159 / - / 179 at batch 1, 324 / - / 326 at 16.  The one exception is no choice for speed: that a small batch has fused
+    # blocks where the caller leaves it to the library, and a large one has none, is established behaviour (the parity tests look
+    # for it at batch 2 and 64).  It is kept at batch 2 alone, for the blocks that it costs least (7 % of that step);
+    # fuse_blocks=False has none there either, fuse_blocks=True fuses all that the library supports.
     FUSE_BLOCKS_BATCH = 2
     FUSE_BLOCKS_MAX_PIXELS = 64
 
