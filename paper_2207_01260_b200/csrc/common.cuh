@@ -33,6 +33,10 @@ cprune_status cuda_fail(cudaError_t e, const char *what);
 // Programmatic dependent launch.  A kernel of a model's launch chain lets its successor start as early as possible
 // (pdl_trigger) and waits for its predecessor's results (pdl_wait) only after its own set-up, so that launch
 // latency and set-up overlap the predecessor's tail.  Both are no-ops in a kernel launched the ordinary way.
+// A chain begins with a kernel that waits BEFORE it lets its successor start (cast, regrouping, stem): everything that was enqueued
+// before the chain is then complete when the second kernel starts.  Kernels may therefore read packed parameters ahead of their wait,
+// even those that a kernel just before the chain packed, and no kernel of a pass starts while the pass before it still reads the
+// same activations (whose lines could stay in an L1).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -40,7 +44,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 bool chain_launch_enabled();
 void set_chain_launch(bool on);
 
-// Launches a kernel that calls pdl_wait() before it touches global memory; inside a chain the launch carries the
+// Launches a kernel that calls pdl_wait() before it touches what its predecessors write; inside a chain the launch carries the
 // programmatic-serialization attribute.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args) {

@@ -1100,8 +1100,8 @@ constexpr int RG_ROWS = 4;     // regrouped rows per block
 template <typename T>
 __global__ void __launch_bounds__(256) regroup_kernel(const T *__restrict__ x, int H, int W, int C, int c_mem, int sf, int pad_lo, int WP,
                                                       uint4 *__restrict__ out) {
+    pdl_wait();        // first kernel of a chain: before its successor may start
     pdl_trigger();
-    pdl_wait();
     // one block per RG_ROWS regrouped rows of one image: their sf * RG_ROWS input rows are contiguous in memory and are
     // brought into shared memory with 16-byte loads first
     extern __shared__ __align__(16) unsigned char rg_smem[];

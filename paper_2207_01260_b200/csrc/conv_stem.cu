@@ -103,7 +103,6 @@ __device__ __forceinline__ uint32_t times_zero2(uint32_t v, uint32_t a) {
 template <int ACT, bool POOL, int CPS>
 __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const __grid_constant__ CUtensorMap tm_w, const StemParams p) {
     extern __shared__ uint8_t smem_raw[];
-    pdl_trigger();
     const uint32_t raw_base = smem_u32(smem_raw);
     const uint32_t base = (raw_base + 1023u) & ~1023u;
     uint8_t *smem = smem_raw + (base - raw_base);
@@ -137,7 +136,9 @@ __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const __grid_c
         mbar_init(conv_bar, ST_CONV_WARPS);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        // the filters were written when the task was packed, not by the preceding kernel
+        // first kernel of a chain: before its successor may start, and before the parameters are read
+        pdl_wait();
+        pdl_trigger();
         mbar_expect_tx(wbar, w_bytes);
         for (int b = 0; b < p.tiles; ++b) tma_load_2d(base + (uint32_t)b * 16384u, &tm_w, wbar, b * 64, 0);
     }
@@ -360,6 +361,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const __grid_c
         const int dy = m / p.KF, k = m - dy * p.KF;
         // rows of filters that a halved D leaves over (D * KF < 128) have no place in the staging buffer; the pool's D is always 2
         const bool k_ok = k < p.k_pad && (POOL || dy < p.D);
+        pdl_wait();
         const float bias = k_ok ? __ldg(p.bias + k) : 0.f;
         const int units = p.N >> 4;
         const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16);

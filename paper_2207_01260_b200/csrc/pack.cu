@@ -41,8 +41,8 @@ __global__ void pad_bias_kernel(const float *__restrict__ b, int K, int k_alloc,
 
 // one thread per (pixel, group of 8 output lanes)
 __global__ void cast_input_kernel(const float *__restrict__ x, size_t pixels, int C, int c_pad, bf16x8 *__restrict__ y) {
+    pdl_wait();        // first kernel of a chain: before its successor may start
     pdl_trigger();
-    pdl_wait();
     int groups = c_pad / 8;
     size_t total = pixels * groups;
     for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {

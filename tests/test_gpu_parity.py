@@ -415,6 +415,42 @@ def test_the_task_times_of_a_model_are_those_of_the_kernels_it_launches(cp):
     assert torch.equal(model.copy_tensor(1), a) and 0 < ms < 5
 
 
+def test_passes_with_new_images_and_newly_packed_filters_follow_each_other_unwaited(cp):
+    # a chain of three short kernels: a pass must see the parameters that the kernel just before it packed, and nothing of the
+    # images of the passes before it
+    N, H, K = 9, 64, 45
+    plan = cp.cprune_task_plan(N, 3, H, H, K, 3, 3, 1, 1, 1)
+    xs = [_dev(wl.conv_task_tensors(104 + j, N, 3, H, H, K, 3, 3)[0]) for j in range(3)]
+    ws = [[_dev(t) for t in wl.conv_task_tensors(107 + j, N, 3, 8, 8, K, 3, 3)[1:3]] for j in range(2)]
+    fc = cp.cprune_fc_pack(_dev(wl.normal_f32(109, 0, (8, K))))
+    packed = cp.cprune_pack_weights(plan, *ws[0])
+    tasks = [cp.TaskDesc(op=cp.OP_CONV, in_=0, out=1, res=-1, plan=plan.handle, w=packed[0].data_ptr(), b=packed[1].data_ptr()),
+             cp.TaskDesc(op=cp.OP_GAP, in_=1, out=2, res=-1),
+             cp.TaskDesc(op=cp.OP_FC, in_=2, out=3, res=-1, w=fc[0].data_ptr(), b=fc[1].data_ptr(), p0=K, p1=8)]
+    model = cp.cprune_model_create(N, H, H, 3, tasks, keep_alive=(plan, packed, fc))
+    assert model.reads_image
+    st = torch.cuda.current_stream().cuda_stream
+
+    def passes(wait):
+        out = []
+        for i in range(24):
+            if i % 4 == 0:
+                w, b = ws[i // 4 % 2]
+                assert cp.lib().cprune_pack_weights(plan.handle, w.data_ptr(), b.data_ptr(), packed[0].data_ptr(), packed[1].data_ptr(), st) == 0
+            if wait:
+                torch.cuda.synchronize()
+            out.append(cp.cprune_model_run(model, xs[i % 3]))
+        torch.cuda.synchronize()
+        return out
+
+    want = passes(True)
+    assert not torch.equal(want[0], want[1]) and not torch.equal(want[0], want[12])
+    for _ in range(20):
+        for a, b in zip(passes(False), want):
+            assert torch.equal(a, b)
+    cp.cprune_poll_device_status()
+
+
 def test_a_first_task_that_adds_the_image_to_its_result(cp):
     # the residual is the bf16 copy of the image: it has to be made even where the convolution itself runs on a regrouped input
     N, H = 64, 128
