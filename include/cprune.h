@@ -212,7 +212,8 @@ cprune_status cprune_task_order(const double *times, const int *counts, int n, i
 /* One-time layout change of a (pruned) layer's parameters for its plan:
  * w float32 [K][C/groups][R][S] -> bfloat16 (round to nearest even) [k_alloc][R][S][c_pad] with zero
  * padding (depthwise: [R][S][c_pad]; stems that the plan runs on a regrouped input: the plan's own
- * order of taps and channels); b float32 [K] (NULL = zeros) -> float32 [k_alloc] zero padded.
+ * order of taps and channels; plans that a model can run straight from its float32 image: those of that
+ * kernel behind them); b float32 [K] (NULL = zeros) -> float32 [k_alloc] zero padded.
  * The packed layout belongs to the plan: pack with the plan the task will run with.
  * All pointers device; w_packed needs packed_weight_bytes, b_packed packed_bias_bytes. */
 cprune_status cprune_pack_weights(const cprune_plan *plan, const float *w, const float *b, void *w_packed,
