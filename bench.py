@@ -269,6 +269,8 @@ def main():
     barrier()
     ms_sus = e4.elapsed_time(e5)
     sus_clocks = sus_sampler.stop()
+    if clocks["sm_mhz"] is None and sus_clocks["sm_mhz"] is not None:       # the timed region ended before nvidia-smi's first sample
+        clocks = dict(sus_clocks, region="sustained run of the same step")
     cp.cprune_poll_device_status()
 
     ms, ms_e2e, ms_sus = max_over_ranks([ms, ms_e2e, ms_sus], dev if world > 1 else None)
