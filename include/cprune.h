@@ -287,13 +287,18 @@ cprune_status cprune_block_run(cprune_block *block, const void *x, const void *w
  */
 enum { CPRUNE_OP_CONV = 1, CPRUNE_OP_MAXPOOL = 2, CPRUNE_OP_GAP = 3, CPRUNE_OP_FC = 4, CPRUNE_OP_BLOCK = 5 };
 
+/* CONV, p0 of a depthwise task: the library may run it and the next task, a 1x1 stride-1 conv task that alone reads its result, as one
+ * kernel.  The values are those of the two tasks.  The tensor between them is then not stored by a pass: cprune_model_copy_tensor makes it from the
+ * depthwise task's stored input, and once cprune_model_tensor has handed out its address the two tasks run separately. */
+enum { CPRUNE_CONV_WITH_NEXT = 1 };
+
 typedef struct {
     int op;                 /* CPRUNE_OP_* */
     int in, out, res;       /* tensor ids; 0 is the model input (after the cast to bf16); res < 0: none */
     cprune_plan *plan;      /* CONV: the task's plan (borrowed; must outlive the model) */
     const void *w;          /* CONV / FC: packed weights, device, borrowed */
     const float *b;         /* CONV / FC: packed bias, device, borrowed */
-    int p0, p1, p2, p3;     /* MAXPOOL: k, stride, pad, -.  FC: in_features, out_features, activation, - */
+    int p0, p1, p2, p3;     /* MAXPOOL: k, stride, pad, -.  FC: in_features, out_features, activation, -.  CONV: 0 or CPRUNE_CONV_WITH_NEXT, -, -, - */
     cprune_block *block;    /* BLOCK: the fused block's plan (borrowed); w and b are its packed buffers, res is unused
                                (the block's residual is its own input) */
 } cprune_task_desc;
@@ -314,7 +319,8 @@ cprune_status cprune_model_run(cprune_model *model, const float *x, float *logit
  * x_host unchanged until then.  Two device-side input buffers alternate, so the copy of one call
  * overlaps the kernels of the previous one.  The first call allocates those buffers (cudaMalloc). */
 cprune_status cprune_model_run_host(cprune_model *model, const float *x_host, float *logits_host, void *stream);
-/* Device pointer and element count of tensor `id` of the model (for tests). */
+/* Device pointer and element count of tensor `id` of the model (for tests).  ptr may be NULL.  Synchronises the device the first time it
+ * gives the address of a tensor that passes have not stored (CPRUNE_CONV_WITH_NEXT). */
 cprune_status cprune_model_tensor(const cprune_model *model, int id, const void **ptr, int *n, int *h, int *w, int *c_pad);
 /* Copies tensor `id` (bf16 [n][h][w][c_pad]) into dst (device) on `stream`. */
 cprune_status cprune_model_copy_tensor(const cprune_model *model, int id, void *dst, void *stream);

@@ -20,6 +20,7 @@ KERNEL = {"auto": 0, "direct": 1, "tensor": 2, "depthwise": 3}
 KERNEL_NAMES = {v: k for k, v in KERNEL.items()}
 FLAGS = {"im2col_only": 1, "pool_on_epilogue_warps": 2}
 OP_CONV, OP_MAXPOOL, OP_GAP, OP_FC, OP_BLOCK = 1, 2, 3, 4, 5
+CONV_WITH_NEXT = 1
 
 # every symbol include/cprune.h declares
 EXPORTS = [
@@ -477,7 +478,9 @@ class Model:
 
     def copy_tensor(self, tid, stream=None):
         """A bf16 copy [n, h, w, c_pad] of an activation buffer."""
-        _, shape = self.tensor(tid)
+        n, h, w, c = c_int(), c_int(), c_int(), c_int()
+        _check(lib().cprune_model_tensor(self.handle, tid, None, byref(n), byref(h), byref(w), byref(c)), "cprune_model_tensor")
+        shape = (n.value, h.value, w.value, c.value)
         dev = torch.device("cuda", torch.cuda.current_device())
         out = torch.empty(shape, dtype=torch.bfloat16, device=dev)
         _check(lib().cprune_model_copy_tensor(self.handle, tid, _ptr(out), _stream(stream)), "cprune_model_copy_tensor")
@@ -545,4 +548,4 @@ def cprune_selftest_wait_timeout(stream=None):
 
 __all__ = [n for n in dir() if n.startswith("cprune_")] + ["Plan", "Model", "TaskDesc", "CpruneError", "lib",
                                                            "EXPORTS", "KERNEL_NAMES", "OP_CONV", "OP_MAXPOOL",
-                                                           "OP_GAP", "OP_FC", "OP_BLOCK", "Block"]
+                                                           "OP_GAP", "OP_FC", "OP_BLOCK", "CONV_WITH_NEXT", "Block"]

@@ -21,6 +21,7 @@
 #include <cstring>
 
 #include "common.cuh"
+#include "depthwise_rows.cuh"
 #include "plan.h"
 #include "sm100_ptx.cuh"
 
@@ -43,39 +44,11 @@ struct DwParams {
     int *status;
 };
 
-// x * w + a on a pair of float32 values: one instruction issues both fused multiply-adds
-__device__ __forceinline__ unsigned long long fma2(unsigned long long x, unsigned long long w, unsigned long long a) {
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(x), "l"(w), "l"(a));
-    return d;
-}
-__device__ __forceinline__ unsigned long long widen2(uint32_t v) {       // the float32 values of a bf16 pair
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(v << 16), "r"(v & 0xffff0000u));
-    return r;
-}
-__device__ __forceinline__ float2 split2(unsigned long long a) {
-    float2 f;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(a));
-    return f;
-}
-template <int NW>
-__device__ __forceinline__ void load_words(const uint32_t *p, uint32_t *v) {
-    if constexpr (NW == 2) {
-        const uint2 t = *reinterpret_cast<const uint2 *>(p);
-        v[0] = t.x; v[1] = t.y;
-    } else {
-        v[0] = *p;
-    }
-}
-
 template <int R, int STRIDE, int CH, int COLS, int ACT>
 __global__ void __launch_bounds__(256, 2) depthwise_kernel(const __grid_constant__ CUtensorMap tm_x, const DwParams p) {
     extern __shared__ __align__(128) uint8_t dw_smem[];
     __shared__ __align__(8) unsigned long long bars[2];
     __shared__ int abort_word;
-    constexpr int NACC = (R + STRIDE - 1) / STRIDE;      // output rows one input row can belong to
-    constexpr int NPX = (COLS - 1) * STRIDE + R;         // input pixels per row of a thread's window
     constexpr int NW = CH / 2;                           // words (channel pairs) per pixel
 
     pdl_trigger();
@@ -156,83 +129,34 @@ __global__ void __launch_bounds__(256, 2) depthwise_kernel(const __grid_constant
         const int rows = min(p.TR, p.P - ps);
         if (ok && in_tile && rows > 0 && qs < p.Q) {
             const uint32_t *in = reinterpret_cast<const uint32_t *>(dw_smem + buf * p.patch_bytes) + in0;
-            unsigned long long acc[NACC][COLS][NW];
-#pragma unroll
-            for (int a = 0; a < NACC; ++a)
-#pragma unroll
-                for (int c = 0; c < COLS; ++c)
-#pragma unroll
-                    for (int k = 0; k < NW; ++k) acc[a][c][k] = 0ull;
             const size_t o0 = (((size_t)n * p.P + ps) * p.Q + qs) * p.c2 + word;
             uint32_t *dst = p.y + o0;
             const uint32_t *rsrc = p.res + o0;
-            const int steps = rows + NACC - 1;           // STRIDE input rows each; step t completes output row t - NACC + 1
-            for (int t0 = 0; t0 < steps; t0 += NACC) {
+            depthwise_rows<R, STRIDE, CH, COLS>(
+                in, pix, row_words, rows, wf, bf,
+                [&](int c, const unsigned long long (&sum)[NW]) {
+                    if (c == 0 || qs + c < p.Q) {
+                        uint32_t o[NW];
 #pragma unroll
-                for (int u = 0; u < NACC; ++u) {
-                    const int t = t0 + u;
-                    if (t >= steps) break;
-#pragma unroll
-                    for (int j = 0; j < STRIDE; ++j) {
-                        if (j > 0 && t * STRIDE + j >= (rows - 1) * STRIDE + R) break;      // below the last row the segment needs
-#pragma unroll
-                        for (int k = 0; k < NPX; ++k) {
-                            uint32_t raw[NW];
-                            unsigned long long xv[NW];
-                            load_words<NW>(in + k * pix, raw);
-#pragma unroll
-                            for (int q = 0; q < NW; ++q) xv[q] = widen2(raw[q]);
-#pragma unroll
-                            for (int a = 0; a < NACC; ++a) {
-                                const int r = a * STRIDE + j;    // this input row is tap row r of output row t - a
-                                if (r < R) {
-#pragma unroll
-                                    for (int c = 0; c < COLS; ++c) {
-                                        const int s = k - c * STRIDE;
-                                        if (s >= 0 && s < R) {
-#pragma unroll
-                                            for (int q = 0; q < NW; ++q) {
-                                                unsigned long long &d = acc[(u - a + NACC) % NACC][c][q];
-                                                d = fma2(xv[q], wf[r][s][q], (r == 0 && s == 0) ? bf[q] : d);    // an output row starts from the bias
-                                            }
-                                        }
-                                    }
-                                }
+                        for (int q = 0; q < NW; ++q) {
+                            float2 f = split2(sum[q]);
+                            if (has_res) {
+                                const uint32_t rv = rsrc[(uint32_t)c * p.c2 + q];
+                                f.x += __uint_as_float(rv << 16);
+                                f.y += __uint_as_float(rv & 0xffff0000u);
                             }
+                            // 0 and 6 are bf16 values, so the clamp commutes with the rounding
+                            __nv_bfloat162 v = __floats2bfloat162_rn(f.x, f.y);
+                            if (ACT != CPRUNE_ACT_NONE) v = __hmax2(v, zero2);
+                            if (ACT == CPRUNE_ACT_RELU6) v = __hmin2(v, six2);
+                            o[q] = *reinterpret_cast<const uint32_t *>(&v);
                         }
-                        in += row_words;
-                        if (j == 0 && t >= NACC - 1) {
-                            // output row t - NACC + 1 is complete (R is odd: its last tap row is the first row of a step)
-                            unsigned long long (&fin)[COLS][NW] = acc[(u + 1) % NACC];
-#pragma unroll
-                            for (int c = 0; c < COLS; ++c) {
-                                if (c == 0 || qs + c < p.Q) {
-                                    uint32_t o[NW];
-#pragma unroll
-                                    for (int q = 0; q < NW; ++q) {
-                                        float2 f = split2(fin[c][q]);
-                                        if (has_res) {
-                                            const uint32_t rv = rsrc[(uint32_t)c * p.c2 + q];
-                                            f.x += __uint_as_float(rv << 16);
-                                            f.y += __uint_as_float(rv & 0xffff0000u);
-                                        }
-                                        // 0 and 6 are bf16 values, so the clamp commutes with the rounding
-                                        __nv_bfloat162 v = __floats2bfloat162_rn(f.x, f.y);
-                                        if (ACT != CPRUNE_ACT_NONE) v = __hmax2(v, zero2);
-                                        if (ACT == CPRUNE_ACT_RELU6) v = __hmin2(v, six2);
-                                        o[q] = *reinterpret_cast<const uint32_t *>(&v);
-                                    }
-                                    uint32_t *d = dst + (uint32_t)c * p.c2;
-                                    if constexpr (NW == 2) *reinterpret_cast<uint2 *>(d) = make_uint2(o[0], o[1]);
-                                    else *d = o[0];
-                                }
-                            }
-                            dst += out_step;
-                            rsrc += out_step;
-                        }
+                        uint32_t *d = dst + (uint32_t)c * p.c2;
+                        if constexpr (NW == 2) *reinterpret_cast<uint2 *>(d) = make_uint2(o[0], o[1]);
+                        else *d = o[0];
                     }
-                }
-            }
+                },
+                [&]() { dst += out_step; rsrc += out_step; });
         }
         advance(n, th, tw);
         if (__syncthreads_or(ok ? 0 : 1)) break;         // the buffer has been read by everyone (or somebody gave up)

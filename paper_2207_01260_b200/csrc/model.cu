@@ -16,6 +16,7 @@ struct ModelTensor {
 struct cprune_model {
     int N, H, W, C;
     std::vector<cprune_task_desc> tasks;
+    std::vector<DwProjTiling> pairs;     // per task; ok: a depthwise task that runs as one kernel with the next task
     std::map<int, ModelTensor> tensors;
     char *arena = nullptr;
     size_t arena_bytes = 0;
@@ -59,6 +60,31 @@ static cprune_status enqueue(cprune_model *m, const float *x, float *logits, cud
     return s;
 }
 
+// Pairs of a depthwise task and the 1x1 task that reads its result, run as one kernel where the caller allows it
+// (CPRUNE_CONV_WITH_NEXT) and nothing else reads the tensor between them, which is then not stored.
+static void find_pairs(cprune_model *m) {
+    m->pairs.assign(m->tasks.size(), DwProjTiling());
+    for (size_t t = 0; t + 1 < m->tasks.size(); ++t) {
+        const cprune_task_desc &d = m->tasks[t], &e = m->tasks[t + 1];
+        if (d.op != CPRUNE_OP_CONV || e.op != CPRUNE_OP_CONV || d.p0 != CPRUNE_CONV_WITH_NEXT || e.in != d.out || e.res == d.out) continue;
+        bool read = false;
+        for (size_t u = t + 2; u < m->tasks.size(); ++u) read = read || m->tasks[u].in == d.out || m->tasks[u].res == d.out;
+        if (!read) plan_depthwise_project(d.plan, e.plan, &m->pairs[t]);
+    }
+}
+
+// The depthwise task whose result the passes do not store, or -1.
+static int unstored(const cprune_model *m, int id) {
+    for (size_t t = 0; t < m->pairs.size(); ++t)
+        if (m->pairs[t].ok && m->tasks[t].out == id) return (int)t;
+    return -1;
+}
+
+static cprune_status store_tensor(const cprune_model *m, int t, cudaStream_t st) {
+    const cprune_task_desc &d = m->tasks[t];
+    return task_run_internal(d.plan, tensor_ptr(m, d.in), d.w, d.b, nullptr, tensor_ptr(m, d.out), m->workspace, st, false);
+}
+
 // How the model's first task gets at the float32 image when it is the only reader of the input: straight (the stem kernel
 // casts on the way in), through the regrouped copy of the patch kernel (cast and regrouping in one pass), or, otherwise,
 // from the bf16 NHWC copy that every model can make.  The stem kernel's bulk copies need an image on a 16-byte boundary.
@@ -100,7 +126,12 @@ static cprune_status enqueue_chain(cprune_model *m, const float *x, float *logit
         void *pout = last ? (void *)logits : tensor_ptr(m, d.out);
         switch (d.op) {
             case CPRUNE_OP_CONV:
-                if (t == 0 && path != INPUT_CAST) s = run_first_task(m, path, x, pout, st);
+                if (m->pairs[t].ok) {
+                    const cprune_task_desc &e = m->tasks[t + 1];
+                    s = launch_depthwise_project(d.plan, e.plan, m->pairs[t], pin, d.w, d.b, e.w, e.b, e.res >= 0 ? tensor_ptr(m, e.res) : nullptr,
+                                                 tensor_ptr(m, e.out), st);
+                    ++t;
+                } else if (t == 0 && path != INPUT_CAST) s = run_first_task(m, path, x, pout, st);
                 else s = task_run_internal(d.plan, pin, d.w, d.b, d.res >= 0 ? tensor_ptr(m, d.res) : nullptr, pout, m->workspace, st, false);
                 break;
             case CPRUNE_OP_BLOCK:
@@ -210,6 +241,9 @@ cprune_status cprune_model_create(int N, int H, int W, int C, const cprune_task_
     const int path = input_path(m);
     if (path != INPUT_CAST) m->launches -= 1;               // no separate cast of the image
     if (path == INPUT_DIRECT) m->launches += 1 - conv_launches(m->tasks[0].plan);
+    find_pairs(m);
+    for (size_t t = 0; t < m->pairs.size(); ++t)
+        if (m->pairs[t].ok) m->launches -= conv_launches(m->tasks[t + 1].plan);
     size_t off = 0;
     for (auto &kv : m->tensors) {
         kv.second.bytes = (size_t)kv.second.n * kv.second.h * kv.second.w * kv.second.c_pad * 2;
@@ -295,7 +329,21 @@ cprune_status cprune_model_tensor(const cprune_model *m, int id, const void **pt
     if (!m) return CPRUNE_ERR_INVALID_ARG;
     auto it = m->tensors.find(id);
     if (it == m->tensors.end()) return CPRUNE_ERR_INVALID_ARG;
-    if (ptr) *ptr = m->arena + it->second.offset;
+    if (ptr) {
+        if (const int t = unstored(m, id); t >= 0) {
+            // from now on the passes store it; what the last one left out is made up for
+            cprune_model *own = const_cast<cprune_model *>(m);
+            CPRUNE_CUDA_CHECK(cudaDeviceSynchronize());
+            own->pairs[t].ok = 0;
+            own->launches += conv_launches(m->tasks[t + 1].plan);
+            for (auto &g : own->graphs)
+                if (g.exec) { cudaGraphExecDestroy(g.exec); g.exec = nullptr; }
+            const cprune_status s = store_tensor(m, t, nullptr);
+            if (s != CPRUNE_OK) return s;
+            CPRUNE_CUDA_CHECK(cudaDeviceSynchronize());
+        }
+        *ptr = m->arena + it->second.offset;
+    }
     if (n) *n = it->second.n;
     if (h) *h = it->second.h;
     if (w) *w = it->second.w;
@@ -307,6 +355,10 @@ cprune_status cprune_model_copy_tensor(const cprune_model *m, int id, void *dst,
     if (!m || !dst) return CPRUNE_ERR_INVALID_ARG;
     auto it = m->tensors.find(id);
     if (it == m->tensors.end()) return CPRUNE_ERR_INVALID_ARG;
+    if (const int t = unstored(m, id); t >= 0) {
+        const cprune_status s = store_tensor(m, t, (cudaStream_t)stream);      // (its input is stored)
+        if (s != CPRUNE_OK) return s;
+    }
     CPRUNE_CUDA_CHECK(cudaMemcpyAsync(dst, m->arena + it->second.offset, it->second.bytes, cudaMemcpyDeviceToDevice,
                                       (cudaStream_t)stream));
     return CPRUNE_OK;

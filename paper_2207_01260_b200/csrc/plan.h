@@ -33,6 +33,15 @@ struct DwTiling {
     int patch_bytes;
 };
 
+// Tiling of the depthwise kernel with the 1x1 task behind it (depthwise_project.cu)
+struct DwProjTiling {
+    int ok;
+    int MT, G, chunks, lanes, panels;        // 128-pixel blocks of a tile, channel groups (of 8) per chunk, chunks, threads per strip, 64-channel panels of a chunk
+    int strips, segs, TR, TH, TW, IH, IW;    // tile: column strips x row segments of TR rows; its input patch
+    int tiles_h, tiles_w, tiles, ctas, threads;
+    int patch_bytes, panel_bytes, w_bytes, wstages, k16, k_part, tmem_cols, smem_bytes;
+};
+
 // Tiling of the stem kernel that reads a model's float32 image (conv_stem.cu): a step is D conv rows of KF filters each
 struct StemTiling {
     int ok;
@@ -91,6 +100,10 @@ cprune_status launch_depthwise(cprune_plan *plan, const void *x, const void *w, 
 // channel groups (of 8 channels) one depthwise CTA handles, for c8 groups in the tensor
 int depthwise_groups(int c8);
 cprune_status plan_depthwise(cprune_plan *plan);    // fills plan->dw
+// a depthwise task and the 1x1 task that reads its result as one kernel
+bool plan_depthwise_project(const cprune_plan *dw, const cprune_plan *proj, DwProjTiling *out);
+cprune_status launch_depthwise_project(const cprune_plan *dw, const cprune_plan *proj, const DwProjTiling &t, const void *x, const void *w, const float *b,
+                                       const void *w2, const float *b2, const void *res, void *y, cudaStream_t st);
 // tcgen05 implicit GEMM
 cprune_status plan_conv_tensor(cprune_plan *plan);  // fills tile fields of plan->info; UNSUPPORTED if not eligible
 cprune_status launch_conv_tensor(cprune_plan *plan, const void *x, const void *w, const float *b, const void *res,

@@ -947,6 +947,80 @@ def test_fused_inverted_residual_block(cp, case):
     assert np.max(np.abs(sep - got) / (MATCH_REL * np.abs(ref_m) + 1e-3 * bound_m)) <= 2.0
 
 
+@pytest.mark.parametrize("case", [
+    # N, C, H, W, K, R, act, res: one and two pixel blocks per tile, several tiles per thread block, rows and columns beyond the image,
+    # an odd number of 8-channel groups, two chunks of channels, more than 64 and more than 256 filters (two MMAs), a residual
+    (64, 32, 57, 55, 16, 3, "relu6", False), (40, 40, 21, 23, 40, 3, "relu", True), (70, 200, 14, 14, 72, 3, "relu6", False),
+    (150, 296, 9, 11, 100, 3, "none", False), (80, 72, 28, 28, 320, 5, "relu", False), (64, 144, 13, 13, 144, 5, "none", True),
+    (3, 24, 56, 56, 20, 3, "relu", False)])
+def test_depthwise_and_1x1_tasks_as_one_kernel(cp, case):
+    N, C, H, W, K, R, act, res = case
+    x, w, b, _ = wl.conv_task_tensors(110, N, C, H, W, C, R, R, C)
+    _, w2, b2, _ = wl.conv_task_tensors(111, 1, C, 1, 1, K, 1, 1)
+    dw = cp.cprune_task_plan(N, C, H, W, C, R, R, 1, R // 2, C, act)
+    pj = cp.cprune_task_plan(N, C, H, W, K, 1, 1, 1, 0, 1, act, res)
+    p1, p2, fc = cp.cprune_pack_weights(dw, _dev(w), _dev(b)), cp.cprune_pack_weights(pj, _dev(w2), _dev(b2)), cp.cprune_fc_pack(torch.ones((8, K), device="cuda"))
+    def build(flag):
+        tasks = [cp.TaskDesc(op=cp.OP_CONV, in_=0, out=1, res=-1, plan=dw.handle, w=p1[0].data_ptr(), b=p1[1].data_ptr(), p0=flag),
+                 cp.TaskDesc(op=cp.OP_CONV, in_=1, out=2, res=0 if res else -1, plan=pj.handle, w=p2[0].data_ptr(), b=p2[1].data_ptr()),
+                 cp.TaskDesc(op=cp.OP_GAP, in_=2, out=3, res=-1),
+                 cp.TaskDesc(op=cp.OP_FC, in_=3, out=4, res=-1, w=fc[0].data_ptr(), b=fc[1].data_ptr(), p0=K, p1=8)]
+        return cp.cprune_model_create(N, H, W, C, tasks, keep_alive=(dw, pj, p1, p2, fc))
+    model, plain = build(cp.CONV_WITH_NEXT), build(0)
+    assert model.launches == plain.launches - 1
+    for use_graph in (False, True):
+        cp.cprune_model_run(model, _dev(x), use_graph=use_graph)
+    cp.cprune_model_run(plain, _dev(x))
+    y = model.copy_tensor(2).float().cpu().numpy()
+    cp.cprune_poll_device_status()
+    # the tensor in between is not stored, but can be had; the second product against the oracle on these very values
+    h = model.copy_tensor(1)
+    assert torch.equal(h, plain.copy_tensor(1))
+    h, rb = h.float().cpu().numpy()[..., :C], oracle.round_bf16
+    r = rb(x) if res else None
+    ref, bound = oracle.conv2d(h, w2, b2, 1, 0, 1, act, r, with_bound=True)
+    ref_m, bound_m = oracle.conv2d(h, rb(w2), b2, 1, 0, 1, act, r, with_bound=True)
+    assert np.all(y[..., K:] == 0)
+    check_values("pair %s" % (case,), y[..., :K], ref, bound, ref_m, bound_m)
+    # a pixel that is no number reaches only the outputs whose window holds it
+    bad = x.copy()
+    bad[N - 1, 4, 3, 5] = np.nan
+    cp.cprune_model_run(model, _dev(bad))
+    cp.cprune_model_run(plain, _dev(bad))
+    z, want = model.copy_tensor(2).float().cpu().numpy(), plain.copy_tensor(2).float().cpu().numpy()
+    cp.cprune_poll_device_status()
+    lo, hi = 4 - R // 2, 4 + R // 2 + 1
+    out = np.ones(y.shape[:3], dtype=bool)
+    out[N - 1, max(0, lo):hi, max(0, lo - 1):hi - 1] = False
+    assert np.array_equal(z[out], y[out]) and np.array_equal(np.isnan(z), np.isnan(want))
+    # an address handed out is kept up to date from then on: the tasks run separately
+    cp.cprune_model_run(model, _dev(x), use_graph=True)
+    model.tensor(1)
+    assert model.launches == plain.launches
+    cp.cprune_model_run(model, _dev(x), use_graph=True)
+    cp.cprune_model_run(plain, _dev(x))
+    assert torch.equal(model.copy_tensor(2), plain.copy_tensor(2))
+
+
+def test_mobilenet_v2_with_and_without_pairs(cp):
+    from paper_2207_01260_b200.pipeline import PrunedNetwork
+    table = wl.mobilenet_v2()
+    weights = wl.model_weights(table)
+    x = wl.model_input(table, 1)
+    pairs, plain = PrunedNetwork(table, weights, 1), PrunedNetwork(table, weights, 1, fuse_blocks=False)
+    assert pairs.model.launches < plain.model.launches
+    a, b = pairs.run(_dev(x)).cpu().numpy(), plain.run(_dev(x)).cpu().numpy()
+    cp.cprune_poll_device_status()
+    assert np.linalg.norm(a - b) <= 1e-2 * np.linalg.norm(b)           # the order of the float32 sums differs, at batch 1 in 4 of 17 blocks
+    pw, _ = oracle.prune_model(table, weights)
+    ref = oracle.model_ref(table, pw, x, matched=True)
+    assert np.linalg.norm(a - ref) <= 1e-2 * np.linalg.norm(ref)
+    for name in ("b1_dw", "b3_dw", "b9_dw"):                           # depthwise results can be had whether stored or not
+        out = wl.layer_by_name(table)[name]["out"]
+        u, v = pairs.activation(out), plain.activation(out)
+        assert np.linalg.norm(u - v) <= 1e-2 * np.linalg.norm(v)
+
+
 def test_fused_block_argument_errors_and_unsupported_shapes(cp):
     for args in ((2, 64, 28, 28, 288, 64), (2, 256, 14, 14, 512, 64), (2, 64, 14, 14, 288, 320)):   # image too large, C_in, C_out
         with pytest.raises(cp.CpruneError) as e:
