@@ -25,6 +25,14 @@
 // most, and every wait, commit and counter between taps is exposed (60 to 220 cycles a tap).  Hence one wait per filter row where
 // two rows of filters fit, and one instantiation per kind of ring and epilogue, which keeps the code between the loops short.
 //
+// Pairs.  Where filters are streamed that port carries them twice over: 16 KB of a tap of 64 channels and 128 filters arrive for every 128 or
+// 256 pixels, and every MMA reads them again.  Two CTAs of a cluster therefore take neighbouring tiles of the same filters, each with its own
+// patch, staging and accumulator, and each holds half of the filters: one tcgen05.mma of cta_group::2 multiplies both patches, the
+// barriers of the first CTA count what arrives in both, and its commits free the stages of both.  Cold, alone (us, one CTA / pairs): 131 -> 203
+// 28x28, 64 images 36.9 / 32.2; 70 -> 160 with a residual 35.8 / 28.4; 101 -> 96 16x16, 128 images 18.8 / 14.1 (all filters fit, halved); in the network
+// 512 -> 358 7x7 18.4 / 15.7, 179 -> 256 14x14 16.3 / 14.8.  Filters that fit one CTA gain nothing (45 -> 58 32x32 14.7 / 17.4).  An expect_tx that the other
+// CTA sends across (release at cluster scope) cost 700 cycles a tap; the first CTA expects the bytes of both instead.
+//
 //   warp 0       patch loads (one per channel block); with a residual, one more load per group of
 //                64 filters brings the residual tile in through the same ring;
 //   warps 1, 2   filter loads, one per (channel block, tap), taken in turn; small filter sets
@@ -139,9 +147,21 @@ __device__ __forceinline__ bf16x8 bias_act8(const uint32_t *v, const unsigned lo
     return r;
 }
 
+// One MMA of 16 channels, and the arrival of those issued so far, for one CTA or for a pair.
+template <bool PAIR>
+__device__ __forceinline__ void mma_words(uint32_t d_tmem, uint32_t a_lo, uint32_t w_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate) {
+    if (PAIR) umma_bf16_words_pair(d_tmem, a_lo, w_lo, desc_hi, idesc, accumulate);
+    else umma_bf16_words(d_tmem, a_lo, w_lo, desc_hi, idesc, accumulate);
+}
+template <bool PAIR>
+__device__ __forceinline__ void mma_commit(uint32_t bar) {
+    if (PAIR) umma_commit_pair(bar);
+    else umma_commit(bar);
+}
 // All MMAs of one filter tap for one accumulator block: nk steps of 16 channels.  a_lo and w_lo are
 // the low words of the operand descriptors (start address in 16-byte units).  Called by the whole warp: the
 // operands are computed by all lanes (they stay in uniform registers) and one elected lane issues.
+template <bool PAIR>
 __device__ __forceinline__ void issue_tap(uint32_t d_tmem, uint32_t a_lo, uint32_t w_lo, uint32_t desc_hi, uint32_t idesc,
                                           uint32_t accumulate, int nk, uint32_t commit_w, uint32_t commit_p) {
     uint32_t al[4], wl[4];
@@ -150,20 +170,21 @@ __device__ __forceinline__ void issue_tap(uint32_t d_tmem, uint32_t a_lo, uint32
     if (elect_one()) {
         if (nk == 4) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) umma_bf16_words(d_tmem, al[kk], wl[kk], desc_hi, idesc, kk ? 1u : accumulate);
+            for (int kk = 0; kk < 4; ++kk) mma_words<PAIR>(d_tmem, al[kk], wl[kk], desc_hi, idesc, kk ? 1u : accumulate);
         } else {
-            umma_bf16_words(d_tmem, al[0], wl[0], desc_hi, idesc, accumulate);
+            mma_words<PAIR>(d_tmem, al[0], wl[0], desc_hi, idesc, accumulate);
 #pragma unroll
             for (int kk = 1; kk < 3; ++kk)
-                if (kk < nk) umma_bf16_words(d_tmem, al[kk], wl[kk], desc_hi, idesc, 1u);
+                if (kk < nk) mma_words<PAIR>(d_tmem, al[kk], wl[kk], desc_hi, idesc, 1u);
         }
-        if (commit_w) umma_commit(commit_w);
-        if (commit_p) umma_commit(commit_p);
+        if (commit_w) mma_commit<PAIR>(commit_w);
+        if (commit_p) mma_commit<PAIR>(commit_p);
     }
     __syncwarp();
 }
 
 // A whole filter row (S taps) from one elected block: nothing has to be waited for between its taps.
+template <bool PAIR>
 __device__ __forceinline__ void issue_row(uint32_t d_tmem, uint32_t a_lo, uint32_t w_lo, uint32_t desc_hi, uint32_t idesc,
                                           uint32_t accumulate, int nk, int S, uint32_t slot_step, uint32_t w_step, uint32_t commit_w, uint32_t commit_p) {
     if (elect_one()) {
@@ -171,19 +192,19 @@ __device__ __forceinline__ void issue_row(uint32_t d_tmem, uint32_t a_lo, uint32
             if (nk == 4) {
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
-                    umma_bf16_words(d_tmem, a_lo + (uint32_t)(2 * kk), w_lo + (uint32_t)(2 * kk), desc_hi, idesc, kk ? 1u : accumulate);
+                    mma_words<PAIR>(d_tmem, a_lo + (uint32_t)(2 * kk), w_lo + (uint32_t)(2 * kk), desc_hi, idesc, kk ? 1u : accumulate);
             } else {
-                umma_bf16_words(d_tmem, a_lo, w_lo, desc_hi, idesc, accumulate);
+                mma_words<PAIR>(d_tmem, a_lo, w_lo, desc_hi, idesc, accumulate);
 #pragma unroll
                 for (int kk = 1; kk < 3; ++kk)
-                    if (kk < nk) umma_bf16_words(d_tmem, a_lo + (uint32_t)(2 * kk), w_lo + (uint32_t)(2 * kk), desc_hi, idesc, 1u);
+                    if (kk < nk) mma_words<PAIR>(d_tmem, a_lo + (uint32_t)(2 * kk), w_lo + (uint32_t)(2 * kk), desc_hi, idesc, 1u);
             }
             accumulate = 1;
             a_lo += slot_step;
             w_lo += w_step;
-            if (commit_w) { umma_commit(commit_w); commit_w += 8u; }     // every tap frees its own stage
+            if (commit_w) { mma_commit<PAIR>(commit_w); commit_w += 8u; }     // every tap frees its own stage
         }
-        if (commit_p) umma_commit(commit_p);
+        if (commit_p) mma_commit<PAIR>(commit_p);
     }
     __syncwarp();
 }
@@ -210,7 +231,7 @@ __device__ __forceinline__ void tile_origin(const PatchParams &p, int tm, int &n
     q0 = tx * p.step_w + p.org;
 }
 
-template <int MODE, bool RESIDENT, bool POOLED = false, int WIDTH = 0>
+template <int MODE, bool RESIDENT, bool POOLED = false, int WIDTH = 0, bool PAIR = false>
 __global__ void __launch_bounds__(pk_threads(MODE), 1)
 conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                   const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_res, const PatchParams p) {
@@ -231,7 +252,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *smem = smem_raw + (base - raw);
     const uint32_t w_bytes = (uint32_t)p.w_stage_bytes;                   // stage stride
-    const uint32_t w_tx_bytes = (uint32_t)p.FT * 16u * (uint32_t)p.rb16;  // bytes one filter load delivers
+    const uint32_t w_tx_bytes = (uint32_t)p.FT * (PAIR ? 8u : 16u) * (uint32_t)p.rb16;  // bytes one filter load delivers
     const uint32_t patch0 = base;
     const uint32_t w0 = patch0 + (uint32_t)p.pstages * (uint32_t)p.patch_bytes;
     const uint32_t staging0 = w0 + (uint32_t)p.wstages * w_bytes;
@@ -259,13 +280,23 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     constexpr bool FLAT = MODE == PK_DENSE || MODE == PK_FLAT;      // 1x1 tasks: one image of one row
     const int FR = FLAT ? 1 : WIDTH ? WIDTH : p.R, FS = FLAT || SPLIT ? 1 : WIDTH ? WIDTH : p.S, RS = FR * FS;
     const int ipt = FLAT || SPLIT ? 0 : p.ipt;
+    // Pairs: two CTAs take neighbouring tiles of the same filters, each with its own patch and half of the filters; the first one's
+    // MMA warps issue for both, and its barriers count what arrives in both.
+    const int rank = PAIR ? (int)(blockIdx.x & 1u) : 0, first_item = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+    const int item_step = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x, total_items = PAIR ? ((p.tiles_m + 1) >> 1) * p.tiles_n : p.tiles_m * p.tiles_n;
+    auto tile_of = [&](int item, int &tm, int &nt) {
+        tm = item; nt = 0;
+        if (p.tiles_n > 1) { tm = item / p.tiles_n; nt = item - tm * p.tiles_n; }
+        if (PAIR) tm = tm * 2 + rank;
+    };
 
     // barrier set-up, spread over the lanes of warp 0 (one thread doing up to 70 initialisations costs microseconds).
     // Every accumulator block has its own issuing warp: stages are free, and a tile is complete, once all have committed.
     if (threadIdx.x < 32) {
         const int l = threadIdx.x;
+        constexpr int CTAS = PAIR ? 2 : 1;
         if (l < p.pstages) { mbar_init(pfull(l), 1); mbar_init(pempty(l), p.MT); }
-        if (l < 2) { mbar_init(tfull(l), p.MT); mbar_init(tempty(l), EPI_WARPS); mbar_init(res_full(l), 1); }
+        if (l < 2) { mbar_init(tfull(l), p.MT); mbar_init(tempty(l), EPI_WARPS * CTAS); mbar_init(res_full(l), 1); }
         if (l == 2) { mbar_init(epi_bar, EPI_WARPS); *abort_flag = 0; }
         if (SPLIT && l >= 4 && l < 6) { mbar_init(sfull(l - 4), EPI_WARPS); mbar_init(sempty(l - 4), PK_POOL_WARPS); }
         if (l < p.wstages) { mbar_init(wfull(l), p.wgroup); mbar_init(wempty(l), p.MT); }
@@ -282,14 +313,16 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     if (p.res_blocks) {
         uint8_t *ident = smem + (ident0 - base);
         for (int e = threadIdx.x; e < 64 * 8; e += blockDim.x) {
-            const int r = e >> 3, c = e & 7;
+            // (pairs: this CTA's half of the rows, for blocks of 64 filters and, from row 32 on, for the last block)
+            const int i = e >> 3, c = e & 7, last = (p.FT & 63) ? (p.FT & 63) >> 1 : 32;
+            const int r = !PAIR ? i : i < 32 ? rank * 32 + i : i < 32 + last ? rank * last + i - 32 : 64;
             uint4 v = make_uint4(0u, 0u, 0u, 0u);
             if (c == (r >> 3)) {
                 const uint32_t one = (r & 1) ? 0x3F800000u : 0x00003F80u;      // bf16 1.0 in the odd or even half
                 const int word = (r & 7) >> 1;
                 if (word == 0) v.x = one; else if (word == 1) v.y = one; else if (word == 2) v.z = one; else v.w = one;
             }
-            *(uint4 *)(ident + sub_off(r, c)) = v;
+            *(uint4 *)(ident + sub_off(i, c)) = v;
         }
         fence_async_smem();
     }
@@ -317,35 +350,43 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         lut[e] = v;
     }
     if (warp == PK_MMA_WARP) {
-        tmem_alloc(smem_u32(tmem_slot), 512);
-        tmem_relinquish();
+        if (PAIR) { tmem_alloc_pair(smem_u32(tmem_slot), 512); tmem_relinquish_pair(); }
+        else { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
     }
     tc_fence_before();
-    __syncthreads();
+    if (PAIR) cluster_sync();
+    else __syncthreads();
     tc_fence_after();
     // Set-up done.  Only the patch (and residual) loads of warp 0 read what the preceding kernel wrote, and everything
     // else in this kernel follows from them, so warp 0 alone waits for the predecessor; filters and bias were written
     // when the task was packed and are fetched right away.
     const uint32_t tmem_base = *tmem_slot;
-    const int total_items = p.tiles_m * p.tiles_n;
 
+    auto expect = [&](uint32_t bar, uint32_t bytes) {
+        // (pairs: the first CTA expects the bytes of both; what the other's loads deliver before that is counted all the same)
+        if (rank == 0) mbar_expect_tx(bar, PAIR ? 2 * bytes : bytes);
+    };
+    auto load_4d = [&](uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1, int c2, int c3) {
+        if (PAIR) tma_load_4d_pair(dst, map, leader_addr(bar), c0, c1, c2, c3);
+        else tma_load_4d(dst, map, bar, c0, c1, c2, c3);
+    };
     if (warp == 0) {
         // ------------------------------------------------------------------ patch loads
         pdl_wait();
         int ps = 0;
         uint32_t pphase = 0;
         bool ok = true;
-        for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
-            int tm = item, nt = 0;
-            if (p.tiles_n > 1) { tm = item / p.tiles_n; nt = item - tm * p.tiles_n; }
+        for (int item = first_item; item < total_items && ok; item += item_step) {
+            int tm, nt;
+            tile_of(item, tm, nt);
             int n, p0, q0;
             tile_origin<FLAT>(p, tm, n, p0, q0);
             for (int cb = 0; cb < p.cblks; ++cb) {
                 ok = __all_sync(0xffffffffu, mbar_wait(pempty(ps), pphase ^ 1u, abort_flag, p.status));
                 if (!ok) break;
                 if (elect_one()) {
-                    mbar_expect_tx(pfull(ps), (uint32_t)p.patch_box_bytes);
-                    tma_load_4d(patch0 + (uint32_t)ps * p.patch_bytes, &tm_x, pfull(ps), cb * 64, q0 - p.pad_w, p0 - p.pad, n);
+                    expect(pfull(ps), (uint32_t)p.patch_box_bytes);
+                    load_4d(patch0 + (uint32_t)ps * p.patch_bytes, &tm_x, pfull(ps), cb * 64, q0 - p.pad_w, p0 - p.pad, n);
                 }
                 __syncwarp();
                 if (++ps == p.pstages) { ps = 0; pphase ^= 1u; }
@@ -357,8 +398,8 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 ok = __all_sync(0xffffffffu, mbar_wait(pempty(ps), pphase ^ 1u, abort_flag, p.status));
                 if (!ok) break;
                 if (elect_one()) {
-                    mbar_expect_tx(pfull(ps), (uint32_t)(p.TH * p.Wp * 128));
-                    tma_load_4d(patch0 + (uint32_t)ps * p.patch_bytes, &tm_res, pfull(ps), nt * p.FT + j * 64, q0, p0, n);
+                    expect(pfull(ps), (uint32_t)(p.TH * p.Wp * 128));
+                    load_4d(patch0 + (uint32_t)ps * p.patch_bytes, &tm_res, pfull(ps), nt * p.FT + j * 64, q0, p0, n);
                 }
                 __syncwarp();
                 if (++ps == p.pstages) { ps = 0; pphase ^= 1u; }
@@ -370,11 +411,11 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         uint32_t wphase = 0;
         bool ok = true;
         const int me = warp - 1;
-        for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
-            if (RESIDENT && item != (int)blockIdx.x) break;     // the filters of the first tile stay
+        for (int item = first_item; item < total_items && ok; item += item_step) {
+            if (RESIDENT && item != first_item) break;     // the filters of the first tile stay
             int nt = 0;
             if (p.tiles_n > 1) nt = item % p.tiles_n;
-            const int k0 = nt * p.FT;
+            const int k0 = nt * p.FT + (PAIR ? rank * (p.FT >> 1) : 0);
             for (int cb = 0; cb < p.cblks && ok; ++cb) {
                 for (int tap = 0; tap < RS; ++tap) {
                     const bool mine = turn == me;
@@ -384,8 +425,9 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                         if (!ok) break;
                         if (elect_one()) {
                             const uint32_t wb = wfull(MODE == PK_GENERAL ? ws - wsub : ws);   // the taps of a row complete one barrier
-                            mbar_expect_tx(wb, w_tx_bytes);
-                            tma_load_3d(w0 + (uint32_t)ws * w_bytes, &tm_w, wb, cb * 64, tap, k0);
+                            expect(wb, w_tx_bytes);
+                            if (PAIR) tma_load_3d_pair(w0 + (uint32_t)ws * w_bytes, &tm_w, leader_addr(wb), cb * 64, tap, k0);
+                            else tma_load_3d(w0 + (uint32_t)ws * w_bytes, &tm_w, wb, cb * 64, tap, k0);
                         }
                         __syncwarp();
                     }
@@ -400,8 +442,9 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         // bookkeeping between taps would leave the tensor pipe idle if one warp issued everything: with MT = 2
         // each accumulator block gets its own issuing warp and the two interleave.
         const int mb = warp == PK_MMA_WARP ? 0 : 1;
-        if (mb < p.MT) {
-        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.FT >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+        if (mb < p.MT && rank == 0) {
+        constexpr uint32_t M_BITS = (uint32_t)((PAIR ? 256 : 128) >> 4) << 24;
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.FT >> 3) << 17) | M_BITS;
         int ps = 0, ws = 0, acc = 0;
         uint32_t pphase = 0, wphase = 0, acc_phase = 0;
         bool ok = true;
@@ -413,7 +456,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         const uint32_t patch_step = (uint32_t)p.patch_bytes >> 4, w_step = w_bytes >> 4;
         const uint32_t row_step = (uint32_t)(p.Wp - FS + 1) * slot_step;   // from tap (r, S-1) to (r+1, 0)
         uint32_t patch_lo = patch_lo0, w_lo = w_lo0;
-        for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
+        for (int item = first_item; item < total_items && ok; item += item_step) {
             ok = __all_sync(0xffffffffu, mbar_wait(tempty(acc), acc_phase ^ 1u, abort_flag, p.status));
             if (!ok) break;
             tc_fence_after();
@@ -424,10 +467,10 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 if (!ok) break;
                 const int nk = cb == p.cblks - 1 ? p.ksteps_last : 4;
                 uint32_t tap_lo = patch_lo + (uint32_t)(mb * 128) * slot_step;      // the second block's slots follow the first's
-                if (RESIDENT && item != (int)blockIdx.x) {
+                if (RESIDENT && item != first_item) {
                     // resident filters, loaded during the first tile: nothing to wait for, a filter row per elected block
                     for (int r = 0; r < FR; ++r) {
-                        issue_row(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, FS, slot_step, w_step, 0u, r == FR - 1 ? pempty(ps) : 0u);
+                        issue_row<PAIR>(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, FS, slot_step, w_step, 0u, r == FR - 1 ? pempty(ps) : 0u);
                         accumulate = 1;
                         tap_lo += (uint32_t)p.Wp * slot_step;
                         w_lo += (uint32_t)FS * w_step;
@@ -439,7 +482,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                     for (int r = 0; r < FR; ++r) {
                         ok = __all_sync(0xffffffffu, mbar_wait(wfull(ws), RESIDENT ? 0u : wphase, abort_flag, p.status));
                         if (!ok) break;
-                        issue_row(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, FS, slot_step, w_step, RESIDENT ? 0u : wempty(ws),
+                        issue_row<PAIR>(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, FS, slot_step, w_step, RESIDENT ? 0u : wempty(ws),
                                   r == FR - 1 ? pempty(ps) : 0u);
                         accumulate = 1;
                         tap_lo += (uint32_t)p.Wp * slot_step;
@@ -454,7 +497,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                         if (!ok) break;
                         {
                             const uint32_t cw = RESIDENT ? 0u : wempty(ws), cp = tap == RS - 1 ? pempty(ps) : 0u;
-                            issue_tap(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, cw, cp);
+                            issue_tap<PAIR>(d_tmem, tap_lo, w_lo, desc_hi, idesc, accumulate, nk, cw, cp);
                         }
                         accumulate = 1;
                         w_lo += w_step;
@@ -472,13 +515,13 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                 ok = __all_sync(0xffffffffu, mbar_wait(pfull(ps), pphase, abort_flag, p.status));
                 if (!ok) break;
                 const int nres = min(64, p.FT - j * 64);
-                const uint32_t idesc_r = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nres >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-                issue_tap(d_tmem + (uint32_t)(j * 64), patch_lo + (uint32_t)(mb * 128) * slot_step, desc_lo(ident0), DESC_HI_SW128, idesc_r, 1u,
+                const uint32_t idesc_r = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nres >> 3) << 17) | M_BITS;
+                issue_tap<PAIR>(d_tmem + (uint32_t)(j * 64), patch_lo + (uint32_t)(mb * 128) * slot_step, desc_lo(ident0 + (PAIR && nres < 64 ? 4096u : 0u)), DESC_HI_SW128, idesc_r, 1u,
                           nres >> 4, 0u, pempty(ps));
                 patch_lo += patch_step;
                 if (++ps == p.pstages) { ps = 0; pphase ^= 1u; patch_lo = patch_lo0; }
             }
-            if (ok && elect_one()) umma_commit(tfull(acc));
+            if (ok && elect_one()) mma_commit<PAIR>(tfull(acc));
             __syncwarp();
             if (p.acc_bufs == 2) { if (++acc == 2) { acc = 0; acc_phase ^= 1u; } }
             else acc_phase ^= 1u;
@@ -513,9 +556,9 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         // pixels outside the image never win: after ReLU / ReLU6 every value is >= 0 (and every window holds a real
         // pixel), so they can be replaced by 0 and the maximum taken on the bit patterns; else by -inf
         const uint4 fill = clamp_lo ? make_uint4(0u, 0u, 0u, 0u) : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
-        for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
-            int tm = item, nt = 0;
-            if (p.tiles_n > 1) { tm = item / p.tiles_n; nt = item - tm * p.tiles_n; }
+        for (int item = first_item; item < total_items && ok; item += item_step) {
+            int tm, nt;
+            tile_of(item, tm, nt);
             int n, p0, q0;
             tile_origin<FLAT>(p, tm, n, p0, q0);
             const int pr0 = (p0 + 1) >> 1, pc0 = (q0 + 1) >> 1;
@@ -623,13 +666,13 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             pdl_wait();        // the residual is the result of an earlier kernel of the chain
             load_residual_dense(blockIdx.x, 0);
         }
-        for (int item = blockIdx.x; item < total_items && ok; item += gridDim.x) {
-            int tm = item, nt = 0;
-            if (p.tiles_n > 1) { tm = item / p.tiles_n; nt = item - tm * p.tiles_n; }
+        for (int item = first_item; item < total_items && ok; item += item_step) {
+            int tm, nt;
+            tile_of(item, tm, nt);
             int n, p0, q0;
             tile_origin<FLAT>(p, tm, n, p0, q0);
             const int k0 = nt * p.FT;
-            const int rows_valid = ipt ? p.imgs - n : p.P - p0;    // tile rows (or images) below this are real ones
+            const int rows_valid = PAIR && tm >= p.tiles_m ? 0 : ipt ? p.imgs - n : p.P - p0;    // tile rows (or images) below this are real ones
             // first pooled pixel of the tile (2x2 pool: full-width tiles from an even row)
             __nv_bfloat16 *ytile = p.pool == 1 ? p.y + ((size_t)n * (p.P >> 1) + (p0 >> 1)) * (p.Q >> 1) * p.k_pad : nullptr;
             ok = __all_sync(0xffffffffu, mbar_wait(tfull(acc), acc_phase, abort_flag, p.status, false));
@@ -719,7 +762,10 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
                     if (q == UNITS - 1 && g == groups - 1) {     // accumulator fully read: hand it back
                         tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(tempty(acc));
+                        if (lane == 0) {
+                            if (PAIR) mbar_arrive_cluster(leader_addr(tempty(acc)));
+                            else mbar_arrive(tempty(acc));
+                        }
                     }
                     if (do_a) {
                         uint8_t *blk = buf + mb_a * PK_BLOCK_BYTES;
@@ -833,10 +879,16 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         for (int i = 0; i < 200; ++i) __nanosleep(1000);   // let copies in flight land before the memory goes away
     }
     tc_fence_before();
-    __syncthreads();
+    if (PAIR) {
+        __syncwarp();
+        cluster_sync();        // (the other CTA's MMAs read this one's memory and arrive on its barriers)
+    } else {
+        __syncthreads();
+    }
     if (warp == PK_MMA_WARP) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, 512);
+        if (PAIR) tmem_dealloc_pair(tmem_base, 512);
+        else tmem_dealloc(tmem_base, 512);
     }
 }
 
@@ -845,13 +897,15 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
 // Estimated cycles of one tile.  Per tcgen05.mma (M = 128, N = FT, K = 16) the tensor pipe needs FT / 2 cycles
 // and the operand reads (128 + FT) * 32 bytes of the 128 bytes per clock that shared memory delivers; the TMA
 // writes of filters and patches share that port (measured on B200).
+// Pairs: half of the filters in either CTA; an MMA costs max(N / 2, 35 + N / 8) cycles (measured: 39 / 43 / 50 / 64 at N = 32 / 64 / 96 / 128).
 static double tile_cycles(int MT, int FT, int RS, int cblks, int ksteps_last, int row_bytes, int Wp, int TH, int R, bool resident,
-                          int acc_bufs) {
+                          int acc_bufs, int pair) {
     double total = 0;
     for (int cb = 0; cb < cblks; ++cb) {
         const int nk = cb == cblks - 1 ? ksteps_last : 4;
         const double tensor = MT * nk * (FT / 2.0);
-        const double smem = (MT * nk * (128.0 + FT) * 32.0 + (resident ? 0.0 : FT * (double)row_bytes)) / 128.0;
+        const double own = pair ? FT / 2.0 : FT;           // filters in this CTA's shared memory
+        const double smem = (MT * nk * ((128.0 + own) * 32.0 + (pair ? 384.0 : 0.0)) + (resident ? 0.0 : own * row_bytes)) / 128.0;
         total += RS * (tensor > smem ? tensor : smem) + Wp * (TH + R - 1) * row_bytes / 128.0;
     }
     const double epilogue = MT * ((FT + 63) / 64) * 1200.0;
@@ -936,7 +990,9 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
     const int RS = g.kR * g.kS;
     double best = 1e30;
     PatchTiling bt = {};
-    for (int MT = 1; MT <= 2; ++MT) {
+    const int pairs_allowed = !g.flat && !g.stem && !pool3 && g.kR == 3 && g.kS == 3 ? 1 : 0;
+    for (int MT = 1; MT <= 2; ++MT)
+      for (int pair = 0; pair <= pairs_allowed; ++pair) {
       // candidate tile shapes: whole-width rows; for the 3x3 pool (2 tpr + 1) x (2 tpc + 1) conv pixels around tpr x tpc pooled ones
       // and whole images next to each other where several fit
       const int n_shapes = pool3 ? 32 * 32 : 2;
@@ -977,7 +1033,7 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
         for (int tiles_n = 1; tiles_n <= 8; ++tiles_n) {
             // with several filter tiles every tile ends on a 64-filter boundary: the stores are 64 filters wide and
             // only the tensor's own edge clips them
-            const int FT = round_up((k16 + tiles_n - 1) / tiles_n, tiles_n > 1 ? 64 : 16);
+            const int FT = round_up((k16 + tiles_n - 1) / tiles_n, tiles_n > 1 ? 64 : pair ? 32 : 16);
             if (FT > 256 || MT * FT > 512) continue;
             if ((k16 + FT - 1) / FT != tiles_n) continue;
             const int acc_bufs = 2 * MT * FT <= 512 ? 2 : 1;
@@ -1006,7 +1062,7 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
             const int fixed = 1024 + pstages * patch_bytes + PK_CTRL_BYTES + ident_bytes;
             const int budget = 227 * 1024 - fixed;
             const int sb_max = 2, sb_min = 1;
-            const int w_stage = round_up(FT * RB, 1024);
+            const int w_stage = round_up((pair ? FT / 2 : FT) * RB, 1024);
             // flat tasks with one filter tile stage the tile as it lies in memory (k_pad filters per pixel) when that fits,
             // with the pixel pitch made an odd number of 16-byte pieces (no bank conflicts between neighbouring pixels;
             // 32-byte pixels conflict two-way and still gain, measured)
@@ -1029,7 +1085,7 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
                 wstages = (budget - staging_bufs * stage_bytes) / w_stage;
                 if (wstages < 3) continue;
                 // (four rows for tiles of whole images, which pass a row in 700 cycles: VGG-16 143.0 -> 141.4 us)
-                const int most = ipt ? 12 : 8;
+                const int most = ipt || pair ? 12 : 8;
                 if (wstages > most) wstages = 2 * wgroup > most ? 2 * wgroup : most;
                 wstages -= wstages % wgroup;
             }
@@ -1037,21 +1093,26 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
             // the fused 3x3 pool runs on its own warps only beside two staging buffers, which is worth more than a deeper ring
             if (pool3 && staging_bufs != 2 && pstages > 2) continue;
             const long long tiles = (ipt ? ceil_div(g.vN, ipt) : (long long)g.vN * tiles_per_img) * tiles_n;
-            const double waves = (double)((tiles + 147) / 148);
-            double tile = tile_cycles(MT, FT, RS, cblks, ksteps_last, RB, Wp, TH, g.kR, resident != 0, acc_bufs);
+            const long long tiles_of_pairs = ((ipt ? ceil_div(g.vN, ipt) : (long long)g.vN * tiles_per_img) + 1) / 2 * tiles_n;
+            const double waves = (double)(pair ? ceil_div(tiles_of_pairs, 74) : ceil_div(tiles, 148));
+            double tile = tile_cycles(MT, FT, RS, cblks, ksteps_last, RB, Wp, TH, g.kR, resident != 0, acc_bufs, pair);
             // between two filter barriers the tensor pipe idles for as long as its queue of two MMAs is shorter than a wait
             // (measured: 221 cycles with 64 filters, 117 with 128, 65 with 192; the second issuing warp hides most of it)
             if (!resident && !g.flat) tile += cblks * (RS / wgroup) * (MT == 2 ? 60.0 : FT < 200 ? 280.0 - 1.2 * FT : 40.0);
+            // a stage's round trip through both CTAs is longer than two filter rows
+            if (pair && !resident) tile += cblks * (RS / wgroup) * (wstages >= 3 * wgroup ? 0.0 : 200.0);
             if (ipt) tile -= cblks * Wp * (g.kR - 1) * RB / 128.0;     // (no border rows beside the TH counted)
             if (res_blocks_plan && !dense) tile += res_blocks_plan * (MT * 4 * 48.0 + TH * Wp);   // residual MMAs and their loads
             double t = waves * tile;
             if (resident) t += RS * cblks * FT;    // one-time filter load
             if (staging_bufs == 1 && !g.flat) t += ((FT + 63) / 64) * 900.0;     // the last tile's stores, one after the other
+            // what the estimate leaves out, fitted to 25 shapes: waits across the pair, a cluster's start
+            if (pair) t = 1.15 * t + 800.0;
             if (t < best) {
                 best = t;
-                bt = {MT, TH, FT, tiles_n, tiles_per_img, wstages, resident, acc_bufs, staging_bufs, patch_bytes, TW, tiles_w, step_h, step_w, org, pstages, dense, stage_bytes, dense_pitch, ipt, wgroup};
+                bt = {MT, TH, FT, tiles_n, tiles_per_img, wstages, resident, acc_bufs, staging_bufs, patch_bytes, TW, tiles_w, step_h, step_w, org, pstages, dense, stage_bytes, dense_pitch, ipt, wgroup, pair};
             }
-            if (resident || wgroup == g.kS) break;      // the deepest patch ring beside which the filters fit
+            if (!pair && (resident || wgroup == g.kS)) break;      // the deepest patch ring beside which the filters fit
           }
         }
       }
@@ -1078,13 +1139,13 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
     i.tile_m = 128 * bt.MT;
     i.tile_n = bt.FT;
     i.tile_k = 64;
-    i.stages = bt.wstages;
+    i.stages = bt.pair ? (bt.wstages + 1) / 2 : bt.wstages;      // (of whole filters)
     i.tiles_m = (int)tiles_m;
     i.tiles_n = bt.tiles_n;
     i.k_alloc = bt.tiles_n * bt.FT;
     const int ksteps = (cblks - 1) * 4 + ksteps_last;
     i.padded_flops = 2.0 * (double)i.tiles_m * i.tile_m * (double)i.k_alloc * RS * ksteps * 16.0;
-    plan->smem_bytes = 1024 + bt.pstages * bt.patch_bytes + bt.wstages * round_up(bt.FT * RB, 1024) +
+    plan->smem_bytes = 1024 + bt.pstages * bt.patch_bytes + bt.wstages * round_up((bt.pair ? bt.FT / 2 : bt.FT) * RB, 1024) +
                        bt.staging_bufs * bt.stage_bytes + PK_CTRL_BYTES + ((plan->opts.residual && !bt.dense) ? PK_IDENT_BYTES : 0);
     plan->est_us = best / 1900.0 + 4.0;      // cycles at about 1.9 GHz plus launch, set-up and drain
     return CPRUNE_OK;
@@ -1266,7 +1327,7 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
             const unsigned long long taps = (unsigned long long)(g.kR * g.kS);
             const unsigned long long dims[3] = {ctap, taps, (unsigned long long)i.k_alloc};
             const unsigned long long strides[2] = {ctap * 2, taps * ctap * 2};
-            const unsigned box[3] = {64, 1, (unsigned)t.FT};
+            const unsigned box[3] = {64, 1, (unsigned)(t.pair ? t.FT / 2 : t.FT)};
             cprune_status s = encode_tiled_bf16_swz(&plan->tm_b, w, 3, dims, strides, box, 128, true);
             if (s != CPRUNE_OK) return s;
             plan->map_w = w;
@@ -1314,6 +1375,9 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
             const void *kernels[] = {(const void *)conv_patch_kernel<PK_GENERAL, false>, (const void *)conv_patch_kernel<PK_GENERAL, false, false, 3>, (const void *)conv_patch_kernel<PK_GENERAL, false, true, 3>, (const void *)conv_patch_kernel<PK_GENERAL, false, true>,
                                      (const void *)conv_patch_kernel<PK_GENERAL, true>, (const void *)conv_patch_kernel<PK_GENERAL, true, false, 3>, (const void *)conv_patch_kernel<PK_GENERAL, true, true, 3>,  (const void *)conv_patch_kernel<PK_GENERAL, true, true>,
                                      (const void *)conv_patch_kernel<PK_TAPS, false>,    (const void *)conv_patch_kernel<PK_TAPS, false, true>,
+                                     (const void *)conv_patch_kernel<PK_GENERAL, false, false, 3, true>, (const void *)conv_patch_kernel<PK_GENERAL, false, true, 3, true>,
+                                     (const void *)conv_patch_kernel<PK_GENERAL, true, false, 3, true>, (const void *)conv_patch_kernel<PK_GENERAL, true, true, 3, true>,
+                                     (const void *)conv_patch_kernel<PK_TAPS, false, false, 3, true>, (const void *)conv_patch_kernel<PK_TAPS, false, true, 3, true>,
                                      (const void *)conv_patch_kernel<PK_FLAT, false>,    (const void *)conv_patch_kernel<PK_FLAT, true>,
                                      (const void *)conv_patch_kernel<PK_DENSE, false>,   (const void *)conv_patch_kernel<PK_DENSE, true>,
                                      (const void *)conv_patch_kernel<PK_POOL3, false>,   (const void *)conv_patch_kernel<PK_POOL3, true>};
@@ -1343,7 +1407,7 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
     p.patch_box_bytes = Wp * (int)(box_rows * box_imgs) * 128;
     p.rb16 = 8;
     p.dense = t.dense; p.stage_bytes = t.stage_bytes; p.dense_pitch = t.dense_pitch;
-    p.w_stage_bytes = t.FT * 128;
+    p.w_stage_bytes = t.FT * (t.pair ? 64 : 128);
     p.bias = b;
     // dense staging takes the residual through the staging buffer; everywhere else the MMA warps add it
     p.res = t.dense ? (const __nv_bfloat16 *)res : nullptr;
@@ -1356,7 +1420,8 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
     int sms = 148, dev = 0;
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 148;
-    const int grid = total < sms ? total : sms;
+    const int pair_items = (i.tiles_m + 1) / 2 * i.tiles_n;
+    const int grid = t.pair ? 2 * (pair_items < sms / 2 ? pair_items : sms / 2) : total < sms ? total : sms;
     // a fused 3x3 pool with two staging buffers: the instantiation with separate pooling warps
     const bool split_pool = p.pool == CPRUNE_POOL_MAX3X3S2 && t.staging_bufs == 2 && !res && !(plan->opts.flags & CPRUNE_FLAG_POOL_ON_EPILOGUE_WARPS);
     // One instantiation per kind of epilogue and of filter set, and for 3x3 filters: a role is one warp that fetches its
@@ -1364,11 +1429,14 @@ cprune_status launch_conv_patch(cprune_plan *plan, const void *x, const void *w,
     // 1x1 24 -> 108 56x56 20.2 / 17.6, 96 -> 432 14x14 10.7 / 9.6, 32 -> 16 112x112 19.7 / 18.8, 3x3 512 -> 358 7x7 20.5 / 18.2,
     // 64 -> 44 56x56 20.8 / 19.9, 131 -> 203 28x28 37.0 / 36.2.
     const auto launch = [&](auto kernel, int mode) {
-        return launch_chained(kernel, dim3(grid), dim3(pk_threads(mode)), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, p);
+        return launch_chained_as(t.pair != 0, kernel, dim3(grid), dim3(pk_threads(mode)), (size_t)plan->smem_bytes, st, tm_x, tm_w, tm_y, tm_res, p);
     };
     const bool r = t.resident != 0, pooled = p.pool != 0;
     cudaError_t e;
-    if (t.dense) e = r ? launch(conv_patch_kernel<PK_DENSE, true>, PK_DENSE) : launch(conv_patch_kernel<PK_DENSE, false>, PK_DENSE);
+    if (t.pair && r) e = pooled ? launch(conv_patch_kernel<PK_GENERAL, true, true, 3, true>, PK_GENERAL) : launch(conv_patch_kernel<PK_GENERAL, true, false, 3, true>, PK_GENERAL);
+    else if (t.pair && t.wgroup == 3) e = pooled ? launch(conv_patch_kernel<PK_GENERAL, false, true, 3, true>, PK_GENERAL) : launch(conv_patch_kernel<PK_GENERAL, false, false, 3, true>, PK_GENERAL);
+    else if (t.pair) e = pooled ? launch(conv_patch_kernel<PK_TAPS, false, true, 3, true>, PK_TAPS) : launch(conv_patch_kernel<PK_TAPS, false, false, 3, true>, PK_TAPS);
+    else if (t.dense) e = r ? launch(conv_patch_kernel<PK_DENSE, true>, PK_DENSE) : launch(conv_patch_kernel<PK_DENSE, false>, PK_DENSE);
     else if (g.flat) e = r ? launch(conv_patch_kernel<PK_FLAT, true>, PK_FLAT) : launch(conv_patch_kernel<PK_FLAT, false>, PK_FLAT);
     else if (split_pool) e = r ? launch(conv_patch_kernel<PK_POOL3, true>, PK_POOL3) : launch(conv_patch_kernel<PK_POOL3, false>, PK_POOL3);
     else if (g.kR == 3 && g.kS == 3 && r) e = pooled ? launch(conv_patch_kernel<PK_GENERAL, true, true, 3>, PK_GENERAL) : launch(conv_patch_kernel<PK_GENERAL, true, false, 3>, PK_GENERAL);

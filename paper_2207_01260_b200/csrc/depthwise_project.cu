@@ -344,7 +344,7 @@ bool plan_depthwise_project(const cprune_plan *dw, const cprune_plan *proj, DwPr
     const double step_cycles = 0.37 * i.R * i.R + 34.3;
     double best = 1e30;
     for (t.MT = 1; t.MT <= 2; ++t.MT)
-        for (t.chunks = 1; t.chunks <= 16; ++t.chunks) {
+        for (t.chunks = 1; t.chunks <= 3; ++t.chunks) {     // (three only to see whether two are the better choice)
             t.G = (c8 + t.chunks - 1) / t.chunks;
             if (t.chunks > 1) t.G = (t.G + 1) & ~1;        // chunks begin at multiples of 16 channels
             if (t.chunks > 1 && (t.chunks - 1) * t.G >= c8) continue;

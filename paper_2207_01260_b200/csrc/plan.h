@@ -20,6 +20,7 @@ struct PatchTiling {
     int dense_pitch;                        // dense staging: bytes between neighbouring pixels in the staging buffer
     int ipt;                                // whole images per tile where several fit (0: tiles are rows of one image)
     int wgroup;                             // filter taps under one barrier of the filter ring
+    int pair;                               // two CTAs share the filters of a tile each (cta_group::2)
 };
 
 // Tiling of the depthwise kernel (depthwise.cu)

@@ -288,6 +288,19 @@ def test_patch_tiles_of_whole_images_and_streamed_filter_rows(cp, case):
     assert plan.variant == 1 and plan.tiles_m == tiles
 
 
+@pytest.mark.parametrize("case", [
+    # N, C, H, K, act, residual, pool, filters of a tile (a multiple of 32 above the 16 that K needs: only pairs of thread blocks have those):
+    # even and odd numbers of tiles (the second block of the last pair without one), one and several tiles per pair, a last residual
+    # block of 32 filters, whole small images, the 2x2 pool, filters that stay and filters that are streamed
+    (41, 72, 12, 203, "relu", True, None, 224), (41, 40, 16, 140, "none", False, None, 160), (75, 72, 16, 70, "relu6", True, None, 96),
+    (150, 72, 7, 203, "none", True, None, 224), (41, 40, 16, 140, "relu", False, "max2x2", 160), (75, 200, 8, 140, "none", False, "max2x2", 160),
+    (64, 131, 28, 203, "relu", False, None, 224)])
+def test_patch_tiles_of_pairs_of_thread_blocks(cp, case):
+    N, C, H, K, act, res, pool, tile_n = case
+    plan = check_task(cp, N, C, H, H, K, 3, 1, 1, act=act, with_res=res, pool=pool)
+    assert plan.variant == 1 and plan.tile_n == tile_n
+
+
 def test_stems_on_the_patch_kernel(cp):
     # enough tiles for the patch kernel: the input is regrouped into 16-channel pixels (stride 1 and 2)
     plan = check_task(cp, 16, 3, 64, 64, 64, 7, 2, 3, kernel="tensor")
