@@ -46,9 +46,10 @@ struct DwProjTiling {
 // Tiling of the stem kernel that reads a model's float32 image (conv_stem.cu): a step is D conv rows of KF filters each
 struct StemTiling {
     int ok;
-    int D, KF, RH, N, ktot;                  // input rows per step, MMA columns, packed row length
+    int D, KF, RH, N;                        // conv rows of KF filters per step, input rows per step, MMA columns
+    int used, ksteps, accs, acc_stride;      // MMA steps (16 values) per input row and per step; accumulators, their distance in columns
     int per, slot, tiles, adv;               // input rows per operand tile, bytes of a window, tiles a step reads, tiles from step to step
-    int row_bytes, tile_bytes, raw_bytes, ring, stage_bytes, xch_words, smem_bytes, steps_per_img;
+    int tile_bytes, raw_bytes, ring, stage_bytes, smem_bytes, steps_per_img;
     size_t weight_offset, weight_bytes;      // its filters behind the task's own in the packed weights
 };
 

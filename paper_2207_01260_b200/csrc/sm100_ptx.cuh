@@ -216,6 +216,18 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t *v) {
         : "r"(taddr)
         : "memory");
 }
+// 16 columns of 16 lanes: registers 4 g + 2 h + e hold lane 8 h + (thread / 4), column 8 g + 2 (thread % 4) + e
+__device__ __forceinline__ void tmem_ld_rows16(uint32_t taddr, uint32_t *v) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(taddr)
+                 : "memory");
+}
+// 8 x 8 matrices of 16-bit values whose rows lie along the threads (thread / 4; two columns each), stored by columns of 16 bytes; thread
+// 8 i + j has the address of column j of matrix i
+__device__ __forceinline__ void stmatrix4_trans(uint32_t addr, const uint32_t *v) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Shared-memory matrix descriptor of a K-major bf16 tile whose rows are 128 bytes, 128-byte
@@ -250,20 +262,37 @@ __device__ __forceinline__ void umma_bf16_words(uint32_t d_tmem, uint32_t a_lo, 
         : "memory");
 }
 
-// The same for some of the accumulator's lanes: bit i of `on` enables lanes 32 i to 32 i + 31, the others keep their contents.
-__device__ __forceinline__ void umma_bf16_words_lanes(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
-                                                      uint32_t accumulate, uint32_t on) {
-    const uint32_t m0 = (on & 1u) - 1u, m1 = ((on >> 1) & 1u) - 1u, m2 = ((on >> 2) & 1u) - 1u, m3 = ((on >> 3) & 1u) - 1u;
+// The same with the 128 rows of A in tensor memory, 16 values of a row in 8 columns.
+__device__ __forceinline__ void umma_bf16_tmem(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-        "mov.b64 da, {%1, %4};\n\t"
+        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
         "mov.b64 db, {%2, %4};\n\t"
         "setp.ne.b32 p, %5, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, {%6, %7, %8, %9}, p;\n\t}"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n\t}"
         :
-        : "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(desc_hi), "r"(accumulate), "r"(m0), "r"(m1), "r"(m2), "r"(m3)
+        : "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(desc_hi), "r"(accumulate)
         : "memory");
 }
+// ... for some of the accumulator's lanes: bit i of `on` enables lanes 32 i to 32 i + 31, the others keep their contents.
+__device__ __forceinline__ void umma_bf16_tmem_lanes(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
+                                                     uint32_t accumulate, uint32_t on) {
+    const uint32_t m0 = (on & 1u) - 1u, m1 = ((on >> 1) & 1u) - 1u, m2 = ((on >> 2) & 1u) - 1u, m3 = ((on >> 3) & 1u) - 1u;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
+        "mov.b64 db, {%2, %4};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, {%6, %7, %8, %9}, p;\n\t}"
+        :
+        : "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(desc_hi), "r"(accumulate), "r"(m0), "r"(m1), "r"(m2), "r"(m3)
+        : "memory");
+}
+// 32 bytes of a lane's row into 8 columns
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint4 &a, const uint4 &b) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w),
+                 "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // Descriptor of a K-major bf16 operand stored without swizzle as 8-row x 16-byte core matrices:
 // rows 16 bytes apart, 8-row groups 128 bytes apart, the next 8 channels `k_stride` bytes away

@@ -356,6 +356,30 @@ def stem_model(cp, plan, w, b):
 
 
 @pytest.mark.parametrize("case", [
+    # N, H, W, K, R, stride, pad, act, pool: rows that leave room for one accumulator, windows read as pairs of floats (3, 5 and 7 wide)
+    # and value by value (1, 6 and 8 wide; 18 and 24 values), one and two MMA steps a row, blocks of one to four steps;
+    # pooled rows of 64 columns and of 8 filters
+    (9, 40, 480, 32, 3, 2, 1, "relu6", None), (7, 41, 472, 24, 5, 2, 2, "none", None), (17, 70, 132, 100, 5, 2, 1, "relu", None),
+    (9, 64, 68, 40, 6, 1, 2, "none", None), (9, 66, 140, 33, 8, 2, 3, "relu", None), (40, 64, 128, 16, 1, 2, 0, "none", None),
+    (40, 32, 256, 64, 7, 2, 3, "relu", "max3x3s2"), (20, 32, 132, 8, 3, 2, 1, "none", "max3x3s2")])
+def test_stems_with_every_kind_of_window(cp, case):
+    N, H, W, K, R, stride, pad, act, pool = case
+    x, w, b, _ = wl.conv_task_tensors(97, N, 3, H, W, K, R, R)
+    plan = cp.cprune_task_plan(N, 3, H, W, K, R, R, stride, pad, 1, act, False, pool)
+    model = stem_model(cp, plan, w, b)
+    assert model.reads_image
+    for _ in range(2):
+        cp.cprune_model_run(model, _dev(x))
+    y = model.copy_tensor(1).float().cpu().numpy()
+    cp.cprune_poll_device_status()
+    ref, bound = _pooled(*oracle.conv2d(x, w, b, stride, pad, 1, act, None, with_bound=True), pool)
+    rb = oracle.round_bf16
+    ref_m, bound_m = _pooled(*oracle.conv2d(rb(x), rb(w), b, stride, pad, 1, act, None, with_bound=True), pool)
+    assert np.all(y[..., K:] == 0)
+    check_values("stem %s" % (case,), y[..., :K], ref, bound, ref_m, bound_m)
+
+
+@pytest.mark.parametrize("case", [
     # N, H, W, K, R, stride, pad, act: images too large for a step of 128 filter rows, so that a step has one or two conv rows of 32
     # or 64 filters and the other rows of the MMA go nowhere; two or three steps per block (both staging buffers), every step's bias
     # other than zero
