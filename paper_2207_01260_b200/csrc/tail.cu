@@ -38,7 +38,10 @@ __global__ void __launch_bounds__(256) maxpool_kernel(const bf16x8 *__restrict__
 }
 
 // One block per (image, 32 channel groups): 8 pixel lanes x 32 channel groups; each thread sums every 8th pixel of
-// its channel group in float32, the lanes are added through shared memory in a fixed order, mean stored as bf16.
+// its channel group in float32, the lanes are added through shared memory in a fixed order, mean stored as bf16.  Bound by the
+// latency of its loads: eight go out together, all of a 7x7 image (one by one 64 images of 1280 channels took 4.8 us
+// in MobileNetV2, now 2.5; 8 x 56x56 x 64 channels by themselves 57 and 33 us).
+constexpr int GAP_AHEAD = 8;
 __global__ void __launch_bounds__(256) gap_kernel(const bf16x8 *__restrict__ x, int N, int HW, int c8,
                                                   bf16x8 *__restrict__ y) {
     __shared__ float part[8][32][9];
@@ -53,11 +56,19 @@ __global__ void __launch_bounds__(256) gap_kernel(const bf16x8 *__restrict__ x, 
     for (int i = 0; i < 8; ++i) s[i] = 0.f;
     if (cg < c8) {
         const bf16x8 *px = x + (size_t)n * HW * c8 + cg;
-        for (int i = pl; i < HW; i += 8) {
-            float f[8];
-            unpack8(ldg8(px + (size_t)i * c8), f);
+        for (int i0 = pl; i0 < HW; i0 += 8 * GAP_AHEAD) {
+            bf16x8 v[GAP_AHEAD];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) s[j] += f[j];
+            for (int i = 0; i < GAP_AHEAD; ++i)
+                if (i0 + 8 * i < HW) v[i] = ldg8(px + (size_t)(i0 + 8 * i) * c8);
+#pragma unroll
+            for (int i = 0; i < GAP_AHEAD; ++i) {
+                if (i0 + 8 * i >= HW) break;
+                float f[8];
+                unpack8(v[i], f);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) s[j] += f[j];
+            }
         }
     }
 #pragma unroll
@@ -77,10 +88,10 @@ __global__ void __launch_bounds__(256) gap_kernel(const bf16x8 *__restrict__ x, 
     }
 }
 
-// Fully connected layer.  A block computes 8 output features of 16 * MT images; its eight warps share out the input
+// Fully connected layer.  A block computes 8 * NT output features of 16 images; its eight warps share out the input
 // features, 32 at a time, and their sums meet in shared memory in a fixed order.  The work is tiny (a few MFLOP per SM) and
 // what it costs is the latency of reading a few megabytes of weights once, so everything is arranged for loads in flight:
-// eight output features per block give 125 blocks for 1000 classes, operands go straight from global memory into MMA
+// eight output features per block give 125 blocks for 1000 classes and up to 16 images, operands go straight from global memory into MMA
 // registers (a thread's 16-byte piece of 8 neighbouring features serves two MMA steps: the order of the contraction index is
 // free as long as both operands use the same), and the first pieces of the weights, which no kernel of the chain writes, are
 // requested before the preceding kernel has finished.
@@ -88,66 +99,72 @@ __global__ void __launch_bounds__(256) gap_kernel(const bf16x8 *__restrict__ x, 
 // MMAs (32 features) start from zero and are added to the running sum with a rounded addition; the eight warps' sums meet in
 // float64.  Relative error (2-norm, against 64 bits): 512 features 5.4e-8, 1280 6.5e-8, 4096 9.0e-8, 25088 1.9e-7; as one chain per
 // warp 8.7e-8, 1.5e-7, 4.7e-7, 3.3e-6; float32 fused multiply-adds 6.7e-8, 7.7e-8, 9.8e-8, 2.2e-7.
-// Back to back, cold weights: 1280 -> 1000 at 64 images 14.3 us with one warp per 4 features x 8 images on the FMA pipe, 5.3 us
-// with this one (5.0 as one chain); 512 -> 1000 7.0 and 3.8 us; one image 5.0 and 3.0, 3.2 and 2.5 us.
+// More images take 16 features per block: the reads of the images' rows, one line per row and 64 bytes, are halved and the sums of a
+// block stay few.  (Two tiles of images and 8 features, as it was, read the weights half as often, but a block needed 6.3 us whether its
+// grid was one wave or two.)  In the networks, before and now: 1280 -> 1000 at 64 images 6.6 and 3.7 us, at 20 images 6.3 and 3.0 us;
+// 512 -> 1000 at 64 images 6.4 and 3.3 us.  By themselves: 25088 -> 4096 at 8 images 119 and 45 us, at 128 images 751 and 297 us.
+// (64 images 14.3 us with one warp per 4 features x 8 images on the FMA pipe.)
 constexpr int FC_WARPS = 8, FC_AHEAD = 5;
+constexpr int FC_NARROW_BLOCKS = 148;     // one per SM
 
-template <int MT>
+template <int NT>
 __global__ void __launch_bounds__(FC_WARPS * 32) fc_kernel(const bf16x8 *__restrict__ x, int N, int in8,
                                                            const bf16x8 *__restrict__ w, const float *__restrict__ b, int out,
                                                            int out_pad, int act, int out_is_f32, void *__restrict__ y) {
-    __shared__ float part[FC_WARPS][MT * 16][9];
+    __shared__ float part[FC_WARPS][16][NT * 8 + 1];
     pdl_trigger();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
-    const int o0 = (blockIdx.x % (out_pad >> 3)) * 8, n0 = (int)(blockIdx.x / (out_pad >> 3)) * (MT * 16);
+    const int tiles_o = (out_pad + NT * 8 - 1) / (NT * 8);
+    const int o0 = (int)(blockIdx.x % tiles_o) * (NT * 8), n0 = (int)(blockIdx.x / tiles_o) * 16;
     const bf16x8 zero = {{0u, 0u, 0u, 0u}};
     const bf16x8 *wrow = w + (size_t)(o0 + g) * in8 + t;
-    auto load_w = [&](int c) { return c * 4 + t < in8 ? ldg8(wrow + c * 4) : zero; };
-    bf16x8 wq[FC_AHEAD];
+    auto load_w = [&](int c, bf16x8 *v) {
 #pragma unroll
-    for (int i = 0; i < FC_AHEAD; ++i) wq[i] = load_w(warp + i * FC_WARPS);
+        for (int f = 0; f < NT; ++f) v[f] = c * 4 + t < in8 && (f == 0 || o0 + f * 8 < out_pad) ? ldg8(wrow + (size_t)(f * 8) * in8 + c * 4) : zero;
+    };
+    bf16x8 wq[FC_AHEAD][NT];
+#pragma unroll
+    for (int i = 0; i < FC_AHEAD; ++i) load_w(warp + i * FC_WARPS, wq[i]);
     pdl_wait();
-    float acc[MT][4];
+    float acc[NT][4];
 #pragma unroll
-    for (int m = 0; m < MT; ++m)
+    for (int f = 0; f < NT; ++f)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[m][j] = 0.f;
+        for (int j = 0; j < 4; ++j) acc[f][j] = 0.f;
     const int chunks = (in8 + 3) >> 2;
     for (int c0 = warp; c0 < chunks; c0 += FC_AHEAD * FC_WARPS) {
-        bf16x8 xq[FC_AHEAD][MT][2];
+        bf16x8 xq[FC_AHEAD][2];
 #pragma unroll
         for (int i = 0; i < FC_AHEAD; ++i) {
             const int q = (c0 + i * FC_WARPS) * 4 + t;
 #pragma unroll
-            for (int m = 0; m < MT; ++m)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int n = n0 + m * 16 + h * 8 + g;
-                    xq[i][m][h] = (n < N && q < in8) ? ldg8(x + (size_t)n * in8 + q) : zero;
-                }
+            for (int h = 0; h < 2; ++h) {
+                const int n = n0 + h * 8 + g;
+                xq[i][h] = (n < N && q < in8) ? ldg8(x + (size_t)n * in8 + q) : zero;
+            }
         }
 #pragma unroll
         for (int i = 0; i < FC_AHEAD; ++i) {
 #pragma unroll
-            for (int m = 0; m < MT; ++m) {
+            for (int f = 0; f < NT; ++f) {
                 float s[4] = {0.f, 0.f, 0.f, 0.f};
-                mma_16816(s, xq[i][m][0].w[0], xq[i][m][1].w[0], xq[i][m][0].w[1], xq[i][m][1].w[1], wq[i].w[0], wq[i].w[1]);
-                mma_16816(s, xq[i][m][0].w[2], xq[i][m][1].w[2], xq[i][m][0].w[3], xq[i][m][1].w[3], wq[i].w[2], wq[i].w[3]);
+                mma_16816(s, xq[i][0].w[0], xq[i][1].w[0], xq[i][0].w[1], xq[i][1].w[1], wq[i][f].w[0], wq[i][f].w[1]);
+                mma_16816(s, xq[i][0].w[2], xq[i][1].w[2], xq[i][0].w[3], xq[i][1].w[3], wq[i][f].w[2], wq[i][f].w[3]);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[m][j] += s[j];
+                for (int j = 0; j < 4; ++j) acc[f][j] += s[j];
             }
-            wq[i] = load_w(c0 + (FC_AHEAD + i) * FC_WARPS);
+            load_w(c0 + (FC_AHEAD + i) * FC_WARPS, wq[i]);
         }
     }
 #pragma unroll
-    for (int m = 0; m < MT; ++m)
+    for (int f = 0; f < NT; ++f)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) part[warp][m * 16 + (j >> 1) * 8 + g][t * 2 + (j & 1)] = acc[m][j];
+        for (int j = 0; j < 4; ++j) part[warp][(j >> 1) * 8 + g][f * 8 + t * 2 + (j & 1)] = acc[f][j];
     __syncthreads();
-    for (int e = threadIdx.x; e < MT * 16 * 8; e += FC_WARPS * 32) {
-        const int r = e >> 3, c = e & 7, n = n0 + r, o = o0 + c;
-        if (n >= N) continue;
+    for (int e = threadIdx.x; e < 16 * NT * 8; e += FC_WARPS * 32) {
+        const int r = e / (NT * 8), c = e % (NT * 8), n = n0 + r, o = o0 + c;
+        if (n >= N || o >= out_pad) continue;
         double s[FC_WARPS];
 #pragma unroll
         for (int q = 0; q < FC_WARPS; ++q) s[q] = part[q][r][c];
@@ -203,12 +220,14 @@ cprune_status cprune_fc(const void *x, int N, int in, const void *w_packed, cons
     if (!x || !w_packed || !b_packed || !y || N <= 0 || in <= 0 || out <= 0) return CPRUNE_ERR_INVALID_ARG;
     int in8 = cprune_padded_channels(in) / 8, out_pad = cprune_padded_channels(out);
     if ((long long)(out_pad >> 3) * ((N + 15) / 16) > 0x7fffffffLL) return CPRUNE_ERR_UNSUPPORTED;
-    // up to 16 images one 16-row tile; more images take two at a time, which halves the reads of the weights
-    if (N <= 16)
-        CPRUNE_CUDA_CHECK(launch_chained(fc_kernel<1>, dim3((unsigned)(out_pad >> 3)), dim3(FC_WARPS * 32), 0, (cudaStream_t)stream,
+    // One tile of 8 features per SM as long as there are SMs for them: one image 2.4 us.  Beyond that 16 features: 20 images of 1280
+    // features 5.0 us with 8 (252 blocks, two or three to an SM) and 3.0 us with 16 (126 blocks).
+    const long long tiles_n = (N + 15) / 16, blocks = (out_pad >> 3) * tiles_n;
+    if (blocks <= FC_NARROW_BLOCKS)
+        CPRUNE_CUDA_CHECK(launch_chained(fc_kernel<1>, dim3((unsigned)blocks), dim3(FC_WARPS * 32), 0, (cudaStream_t)stream,
                                          (const bf16x8 *)x, N, in8, (const bf16x8 *)w_packed, b_packed, out, out_pad, act, out_is_f32, y));
     else
-        CPRUNE_CUDA_CHECK(launch_chained(fc_kernel<2>, dim3((unsigned)((out_pad >> 3) * ((N + 31) / 32))), dim3(FC_WARPS * 32), 0, (cudaStream_t)stream,
+        CPRUNE_CUDA_CHECK(launch_chained(fc_kernel<2>, dim3((unsigned)((out_pad + 15) / 16 * tiles_n)), dim3(FC_WARPS * 32), 0, (cudaStream_t)stream,
                                          (const bf16x8 *)x, N, in8, (const bf16x8 *)w_packed, b_packed, out, out_pad, act, out_is_f32, y));
     return CPRUNE_OK;
 }

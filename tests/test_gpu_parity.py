@@ -928,6 +928,30 @@ def test_fully_connected_sums_are_as_exact_as_float32_additions(cp, N, inn, out)
         assert rel <= bound, (rel, bound)
 
 
+@pytest.mark.parametrize("N,inn,out,act", [(2369, 24, 8, "none"), (161, 72, 120, "relu"), (300, 1290, 130, "none")])
+def test_fully_connected_tiles_of_sixteen_features(cp, N, inn, out, act):
+    # more tiles of eight features than the GPU has SMs: the second eight beyond the padded output, half of the last tile, several
+    # rounds of input pieces; the values are those of a small call, whose tiles have eight features, bit by bit
+    x, w, b = wl.normal_f32(92, 0, (N, inn)), wl.normal_f32(92, 1, (out, inn), 0.1), wl.normal_f32(92, 2, (out,), 0.05)
+    xb = cp.cprune_cast_input(_dev(x.reshape(N, 1, 1, inn))).reshape(N, -1)
+    packed = cp.cprune_fc_pack(_dev(w), _dev(b))
+    for f32 in (True, False):
+        y = cp.cprune_fc(xb, inn, *packed, out, act, out_f32=f32)
+        for n0 in (0, N // 16 * 16, 16):
+            n1 = min(N, n0 + 16)
+            assert torch.equal(y[n0:n1], cp.cprune_fc(xb[n0:n1].contiguous(), inn, *packed, out, act, out_f32=f32))
+
+
+@pytest.mark.parametrize("hw", [(1, 1), (1, 7), (8, 8), (5, 13), (9, 14), (16, 17)])
+def test_global_average_over_one_and_several_rounds_of_loads(cp, hw):
+    x = wl.normal_f32(93, 0, (3, *hw, 270))
+    g = cp.cprune_global_avgpool(cp.cprune_cast_input(_dev(x)), 270).float().cpu().numpy()
+    ref = oracle.gap(oracle.round_bf16(x))
+    scale = np.abs(oracle.round_bf16(x)).mean(axis=(1, 2))
+    # one rounding to bf16 (8 significant bits: half a unit is at most 2^-8 of the value), float32 sums of at most 272 values
+    assert np.all(np.abs(g[:, :270] - ref) <= 2.0 ** -8 * np.abs(ref) + 2.0 ** -18 * scale) and np.all(g[:, 270:] == 0)
+
+
 def block_tensors(seed, N, C_in, H, W, hidden, C_out):
     x = wl.normal_f32(seed, 0, (N, H, W, C_in))
     we = wl.normal_f32(seed, 1, (hidden, C_in, 1, 1), np.sqrt(2.0 / C_in))
