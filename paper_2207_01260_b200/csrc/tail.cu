@@ -115,13 +115,14 @@ __global__ void __launch_bounds__(FC_WARPS * 32) fc_kernel(const bf16x8 *__restr
     pdl_trigger();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
-    const int tiles_o = (out_pad + NT * 8 - 1) / (NT * 8);
-    const int o0 = (int)(blockIdx.x % tiles_o) * (NT * 8), n0 = (int)(blockIdx.x / tiles_o) * 16;
+    constexpr int SHIFT = NT == 1 ? 3 : 4;
+    const int tiles_o = (out_pad + NT * 8 - 8) >> SHIFT;
+    const int o0 = (blockIdx.x % tiles_o) * (NT * 8), n0 = (int)(blockIdx.x / tiles_o) * 16;
     const bf16x8 zero = {{0u, 0u, 0u, 0u}};
     const bf16x8 *wrow = w + (size_t)(o0 + g) * in8 + t;
     auto load_w = [&](int c, bf16x8 *v) {
 #pragma unroll
-        for (int f = 0; f < NT; ++f) v[f] = c * 4 + t < in8 && (f == 0 || o0 + f * 8 < out_pad) ? ldg8(wrow + (size_t)(f * 8) * in8 + c * 4) : zero;
+        for (int f = 0; f < NT; ++f) v[f] = c * 4 + t < in8 && (f == 0 || o0 + f * 8 < out_pad) ? ldg8(wrow + f * 8 * (size_t)in8 + c * 4) : zero;
     };
     bf16x8 wq[FC_AHEAD][NT];
 #pragma unroll
@@ -163,8 +164,8 @@ __global__ void __launch_bounds__(FC_WARPS * 32) fc_kernel(const bf16x8 *__restr
         for (int j = 0; j < 4; ++j) part[warp][(j >> 1) * 8 + g][f * 8 + t * 2 + (j & 1)] = acc[f][j];
     __syncthreads();
     for (int e = threadIdx.x; e < 16 * NT * 8; e += FC_WARPS * 32) {
-        const int r = e / (NT * 8), c = e % (NT * 8), n = n0 + r, o = o0 + c;
-        if (n >= N || o >= out_pad) continue;
+        const int r = e >> SHIFT, c = e & (NT * 8 - 1), n = n0 + r, o = o0 + c;
+        if (n >= N || (NT > 1 && o >= out_pad)) continue;
         double s[FC_WARPS];
 #pragma unroll
         for (int q = 0; q < FC_WARPS; ++q) s[q] = part[q][r][c];
