@@ -31,8 +31,8 @@
 //               instead of 40.6 us).
 // A block works through consecutive steps; with a pool it recomputes one step where it starts inside an image (the odd conv
 // row above).
-// What bounds it: the shared-memory port and the issue of the epilogue.  A step of the pooled 7x7 stem of 224x224 images takes 2400 cycles; the
-// MMAs are 1010 of them on the tensor pipe, and the port moves some 1900 x 128 bytes (MMA 500, windows 480, staged rows 800, rows in 90).
+// What bounds it: the epilogue's chain, whose warps share the issue slots (45 % of them busy at 8 images, 33 % before) with the converters'.  A
+// step of the pooled 7x7 stem of 224x224 images takes 2400 cycles, of which the epilogue works 1950, the converters 1500 and the MMAs 1010.
 // The plain 3x3 stem is at 4.1 TB/s (of 90 MB, 51 written).
 // Stem of 64 224x224 images inside the network: 7x7 stride 2, 64 filters, pooled 49.6 us before the changes above, 38.0 now;
 // 3x3 stride 2, 32 filters 29.5 and 22.0; 20 images 13.6 and 10.6; one image, pooled 9.4 and 8.2.
