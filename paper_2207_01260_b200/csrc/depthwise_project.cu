@@ -190,7 +190,8 @@ depthwise_project_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
         const int piece = (ch0 >> 3) & 7;
         const __nv_bfloat162 zero2 = __floats2bfloat162_rn(0.f, 0.f), six2 = __floats2bfloat162_rn(6.f, 6.f);
         const uint32_t lo2 = p.act2 == CPRUNE_ACT_NONE ? 0x7fff7fffu : 0u, hi2 = p.act2 == CPRUNE_ACT_RELU6 ? 0x40C040C0u : 0x7fff7fffu;
-        const int quarter = warp & 3, of_quarter = (warps - quarter + 3) >> 2, units = (p.k16 >> 4) * p.MT;
+        // (more than 256 filters: the accumulator's two halves hold up to 16 columns more than a stored pixel has channels)
+        const int quarter = warp & 3, of_quarter = (warps - quarter + 3) >> 2, block_units = (p.k_pad2 + 15) >> 4, units = block_units * p.MT;
         const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
         const int erow0 = (quarter * 32 + lane) / p.TW, ecol0 = quarter * 32 + lane - erow0 * p.TW;      // this lane's pixel in either block
         const int erow1 = (128 + quarter * 32 + lane) / p.TW, ecol1 = 128 + quarter * 32 + lane - erow1 * p.TW;
@@ -257,11 +258,13 @@ depthwise_project_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
             // a unit: 16 filters of a pixel block; a lane has one pixel
             size_t o0 = 0;
             bool pixel = false;
+            uint32_t column = 0;
             bf16x8 rv[2] = {};
             auto locate = [&](int u, int &c) {
-                const bool second = u >= (p.k16 >> 4);
+                const bool second = u >= block_units;
                 const int erow = second ? erow1 : erow0, ph = th * p.TH + erow, pw = tw * p.TW + (second ? ecol1 : ecol0);
-                c = (u - (second ? p.k16 >> 4 : 0)) * 16;
+                c = (u - (second ? block_units : 0)) * 16;
+                column = (uint32_t)(c + (second ? p.k16 : 0));
                 pixel = erow < p.TH && ph < p.P && pw < p.Q;
                 o0 = (((size_t)n * p.P + ph) * p.Q + pw) * p.k_pad2 + c;
                 if (p.res && pixel) {
@@ -277,7 +280,7 @@ depthwise_project_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
             tc_fence_after();
             while (u < units) {
                 uint32_t v[16];
-                tmem_ld16(t_lane + (uint32_t)(u * 16), v);
+                tmem_ld16(t_lane + column, v);
                 float f[16];
                 const float4 *src = reinterpret_cast<const float4 *>(bias2_s + c);
                 tmem_ld_wait();

@@ -1063,6 +1063,46 @@ def test_depthwise_and_1x1_tasks_as_one_kernel(cp, case):
     assert torch.equal(model.copy_tensor(2), plain.copy_tensor(2))
 
 
+@pytest.mark.parametrize("case", [
+    # N, C, H, K, R, act, res: more than 256 filters, whose two MMAs are wider than the stored pixel; one tile and several per thread block
+    (1, 32, 56, 257, 5, "relu", False), (64, 72, 14, 272, 3, "none", False), (64, 72, 14, 260, 3, "none", True), (64, 32, 28, 300, 5, "relu6", False),
+    (90, 32, 16, 304, 3, "relu", True)])
+def test_depthwise_and_wide_1x1_tasks_as_one_kernel_stay_in_their_pixels(cp, case):
+    N, C, H, K, R, act, res = case
+    x, w, b, _ = wl.conv_task_tensors(112, N, C, H, H, C, R, R, C)
+    _, w2, b2, _ = wl.conv_task_tensors(113, 1, C, 1, 1, K, 1, 1)
+    _, w3, b3, _ = wl.conv_task_tensors(114, 1, C, 1, 1, K, 1, 1)
+    dw = cp.cprune_task_plan(N, C, H, H, C, R, R, 1, R // 2, C, act)
+    pj = cp.cprune_task_plan(N, C, H, H, K, 1, 1, 1, 0, 1, act, res)
+    side = cp.cprune_task_plan(N, C, H, H, K, 1, 1, 1, 0, 1, "none")
+    p1, p2, p3 = (cp.cprune_pack_weights(*t) for t in ((dw, _dev(w), _dev(b)), (pj, _dev(w2), _dev(b2)), (side, _dev(w3), _dev(b3))))
+    fc = cp.cprune_fc_pack(torch.ones((8, K), device="cuda"))
+
+    def build(flag):
+        # tensors lie in memory in the order of their ids: behind the pair's result (3) comes a copy of the image (4), its input
+        conv = lambda i, o, plan, p, r=-1, f=0: cp.TaskDesc(op=cp.OP_CONV, in_=i, out=o, res=r, plan=plan.handle, w=p[0].data_ptr(), b=p[1].data_ptr(), p0=f)
+        tasks = [cp.TaskDesc(op=cp.OP_MAXPOOL, in_=0, out=4, res=-1, p0=1, p1=1), conv(4, 6, side, p3), conv(4, 5, dw, p1, f=flag),
+                 conv(5, 3, pj, p2, 6 if res else -1), cp.TaskDesc(op=cp.OP_GAP, in_=3, out=7, res=-1),
+                 cp.TaskDesc(op=cp.OP_FC, in_=7, out=8, res=-1, w=fc[0].data_ptr(), b=fc[1].data_ptr(), p0=K, p1=8)]
+        return cp.cprune_model_create(N, H, H, C, tasks, keep_alive=(dw, pj, side, p1, p2, p3, fc))
+
+    model, plain = build(cp.CONV_WITH_NEXT), build(0)
+    assert model.launches == plain.launches - 1
+    for m in (model, plain):
+        for _ in range(2):
+            cp.cprune_model_run(m, _dev(x))
+    y, want = model.copy_tensor(3).float().cpu().numpy(), plain.copy_tensor(3).float().cpu().numpy()
+    h = model.copy_tensor(5).float().cpu().numpy()[..., :C]
+    assert torch.equal(model.copy_tensor(4), plain.copy_tensor(4)) and torch.equal(model.copy_tensor(6), plain.copy_tensor(6))
+    r = plain.copy_tensor(6).float().cpu().numpy()[..., :K] if res else None
+    cp.cprune_poll_device_status()
+    assert np.all(y[..., K:] == 0)
+    ref, bound = oracle.conv2d(h, w2, b2, 1, 0, 1, act, r, with_bound=True)
+    ref_m, bound_m = oracle.conv2d(h, oracle.round_bf16(w2), b2, 1, 0, 1, act, r, with_bound=True)
+    check_values("wide pair %s" % (case,), y[..., :K], ref, bound, ref_m, bound_m)
+    check_values("wide pair, separate %s" % (case,), want[..., :K], ref, bound, ref_m, bound_m)
+
+
 def test_mobilenet_v2_with_and_without_pairs(cp):
     from paper_2207_01260_b200.pipeline import PrunedNetwork
     table = wl.mobilenet_v2()
