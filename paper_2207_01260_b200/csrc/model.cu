@@ -61,7 +61,8 @@ static cprune_status enqueue(cprune_model *m, const float *x, float *logits, cud
 }
 
 // Pairs of a depthwise task and the 1x1 task that reads its result, run as one kernel where the caller allows it
-// (CPRUNE_CONV_WITH_NEXT) and nothing else reads the tensor between them, which is then not stored.
+// (CPRUNE_CONV_WITH_NEXT) and nothing else reads the tensor between them, which is then not stored.  Filters and biases that the
+// kernel cannot read where they are (off 16 and 4 bytes) leave the tasks separate, and a pass refuses them as the tasks do.
 static void find_pairs(cprune_model *m) {
     m->pairs.assign(m->tasks.size(), DwProjTiling());
     for (size_t t = 0; t + 1 < m->tasks.size(); ++t) {
@@ -69,7 +70,8 @@ static void find_pairs(cprune_model *m) {
         if (d.op != CPRUNE_OP_CONV || e.op != CPRUNE_OP_CONV || d.p0 != CPRUNE_CONV_WITH_NEXT || e.in != d.out || e.res == d.out) continue;
         bool read = false;
         for (size_t u = t + 2; u < m->tasks.size(); ++u) read = read || m->tasks[u].in == d.out || m->tasks[u].res == d.out;
-        if (!read) plan_depthwise_project(d.plan, e.plan, &m->pairs[t]);
+        const bool aligned = !(((uintptr_t)d.w | (uintptr_t)e.w) & 15) && !(((uintptr_t)d.b | (uintptr_t)e.b) & 3);
+        if (!read && aligned) plan_depthwise_project(d.plan, e.plan, &m->pairs[t]);
     }
 }
 

@@ -1103,6 +1103,40 @@ def test_depthwise_and_wide_1x1_tasks_as_one_kernel_stay_in_their_pixels(cp, cas
     check_values("wide pair, separate %s" % (case,), want[..., :K], ref, bound, ref_m, bound_m)
 
 
+@pytest.mark.parametrize("which,offset", [(0, 4), (0, 8), (1, 4), (2, 1), (3, 2)])
+def test_a_pair_refuses_the_parameters_that_its_tasks_refuse(cp, which, offset):
+    # 0, 1: depthwise and 1x1 filters off a 16-byte boundary; 2, 3: their biases off a 4-byte one.  The host refuses: no kernel reads them
+    N, C, H, K = 64, 32, 28, 16
+    _, w, b, _ = wl.conv_task_tensors(115, 1, C, H, H, C, 3, 3, C)
+    _, w2, b2, _ = wl.conv_task_tensors(116, 1, C, 1, 1, K, 1, 1)
+    dw, pj = cp.cprune_task_plan(N, C, H, H, C, 3, 3, 1, 1, C, "relu"), cp.cprune_task_plan(N, C, H, H, K, 1, 1, 1, 0)
+    packed = [cp.cprune_pack_weights(dw, _dev(w), _dev(b)), cp.cprune_pack_weights(pj, _dev(w2), _dev(b2))]
+    bytes_ = [t.contiguous().view(torch.uint8).reshape(-1) for t in (packed[0][0], packed[1][0], packed[0][1], packed[1][1])]
+    moved = torch.empty(bytes_[which].numel() + 16, dtype=torch.uint8, device="cuda")
+    moved[offset:offset + bytes_[which].numel()] = bytes_[which]
+    ptr = [t.data_ptr() for t in bytes_]
+    fc = cp.cprune_fc_pack(torch.ones((8, K), device="cuda"))
+
+    def build(p):
+        tasks = [cp.TaskDesc(op=cp.OP_CONV, in_=0, out=1, res=-1, plan=dw.handle, w=p[0], b=p[2], p0=cp.CONV_WITH_NEXT),
+                 cp.TaskDesc(op=cp.OP_CONV, in_=1, out=2, res=-1, plan=pj.handle, w=p[1], b=p[3]),
+                 cp.TaskDesc(op=cp.OP_GAP, in_=2, out=3, res=-1),
+                 cp.TaskDesc(op=cp.OP_FC, in_=3, out=4, res=-1, w=fc[0].data_ptr(), b=fc[1].data_ptr(), p0=K, p1=8)]
+        return cp.cprune_model_create(N, H, H, C, tasks, keep_alive=(dw, pj, packed, moved, fc))
+
+    good = build(ptr)
+    ptr[which] = moved.data_ptr() + offset
+    bad = build(ptr)
+    x = _dev(wl.normal_f32(117, 0, (N, H, H, C)))
+    for use_graph in (False, True):
+        with pytest.raises(cp.CpruneError) as e:
+            cp.cprune_model_run(bad, x, use_graph=use_graph)
+        assert e.value.status == 1                    # CPRUNE_ERR_INVALID_ARG
+    assert bad.launches == good.launches + 1
+    cp.cprune_model_run(good, x)
+    cp.cprune_poll_device_status()
+
+
 def test_mobilenet_v2_with_and_without_pairs(cp):
     from paper_2207_01260_b200.pipeline import PrunedNetwork
     table = wl.mobilenet_v2()
