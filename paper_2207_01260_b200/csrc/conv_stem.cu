@@ -645,7 +645,7 @@ static cprune_status launch_stem_width(const StemParams &p, unsigned grid, size_
 cprune_status launch_conv_stem(const cprune_plan *plan, const float *x, const void *w_packed, const float *b, void *y, cudaStream_t st) {
     const cprune_plan_info &i = plan->info;
     const StemTiling &s = plan->stem;
-    if (!s.ok || ((uintptr_t)x & 15)) return CPRUNE_ERR_INVALID_ARG;
+    if (!s.ok || (((uintptr_t)x | (uintptr_t)w_packed) & 15) || ((uintptr_t)b & 3)) return CPRUNE_ERR_INVALID_ARG;
     StemParams p;
     p.x = x; p.w = (const uint4 *)((const char *)w_packed + s.weight_offset); p.bias = b; p.y = (__nv_bfloat16 *)y;
     p.H = i.H; p.W = i.W; p.P = i.P; p.Q = i.Q; p.out_h = i.out_h; p.out_w = i.out_w;

@@ -379,6 +379,24 @@ def test_stems_with_every_kind_of_window(cp, case):
     check_values("stem %s" % (case,), y[..., :K], ref, bound, ref_m, bound_m)
 
 
+@pytest.mark.parametrize("filters,bias", [(4, 0), (8, 0), (0, 1)])
+def test_a_stem_from_the_image_refuses_misaligned_parameters(cp, filters, bias):
+    # on the host, as the task by itself does: no kernel reads them
+    plan = cp.cprune_task_plan(9, 3, 40, 480, 32, 3, 3, 2, 1)
+    x, w, b, _ = wl.conv_task_tensors(98, 9, 3, 40, 480, 32, 3, 3)
+    wp, bp = cp.cprune_pack_weights(plan, _dev(w), _dev(b))
+    fc = cp.cprune_fc_pack(torch.ones((8, 32), device="cuda"))
+    room = torch.zeros(wp.numel() * wp.element_size() + 16, dtype=torch.uint8, device="cuda")
+    tasks = [cp.TaskDesc(op=cp.OP_CONV, in_=0, out=1, res=-1, plan=plan.handle, w=room.data_ptr() + filters if filters else wp.data_ptr(), b=bp.data_ptr() + bias),
+             cp.TaskDesc(op=cp.OP_GAP, in_=1, out=2, res=-1),
+             cp.TaskDesc(op=cp.OP_FC, in_=2, out=3, res=-1, w=fc[0].data_ptr(), b=fc[1].data_ptr(), p0=32, p1=8)]
+    model = cp.cprune_model_create(9, 40, 480, 3, tasks, keep_alive=(plan, wp, bp, fc, room))
+    assert model.reads_image
+    with pytest.raises(cp.CpruneError) as e:
+        cp.cprune_model_run(model, _dev(x))
+    assert e.value.status == 1                        # CPRUNE_ERR_INVALID_ARG
+
+
 @pytest.mark.parametrize("case", [
     # N, H, W, K, R, stride, pad, act: images too large for a step of 128 filter rows, so that a step has one or two conv rows of 32
     # or 64 filters and the other rows of the MMA go nowhere; two or three steps per block (both staging buffers), every step's bias
