@@ -33,6 +33,8 @@ cprune_status cuda_fail(cudaError_t e, const char *what);
 // Programmatic dependent launch.  A kernel of a model's launch chain lets its successor start as early as possible
 // (pdl_trigger) and waits for its predecessor's results (pdl_wait) only after its own set-up, so that launch
 // latency and set-up overlap the predecessor's tail.  Both are no-ops in a kernel launched the ordinary way.
+// A kernel that uses tensor memory lets its successor start only once it has its columns: a block of a later kernel that got them first
+// would keep them while it waits for this kernel, which would wait for them, and an allocation has no limit.  (The warp that allocates triggers.)
 // A chain begins with a kernel that waits BEFORE it lets its successor start (cast, regrouping, stem): everything that was enqueued
 // before the chain is then complete when the second kernel starts.  Kernels may therefore read packed parameters ahead of their wait,
 // even those that a kernel just before the chain packed, and no kernel of a pass starts while the pass before it still reads the

@@ -240,7 +240,6 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
     constexpr bool SPLIT = MODE == PK_POOL3;      // staging by the epilogue warps, pooling by PK_POOL_WARPS further warps
     constexpr int EPI_WARPS = pk_epi_warps(MODE);
     constexpr int MMA_WARP2 = PK_FIRST_EPI + EPI_WARPS;
-    pdl_trigger();
     if (threadIdx.x == 0) {
         // the descriptors are fetched on first use otherwise, which the first loads would wait for
         asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_x) : "memory");
@@ -290,6 +289,11 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         if (PAIR) tm = tm * 2 + rank;
     };
 
+    if (warp == PK_MMA_WARP) {
+        if (PAIR) { tmem_alloc_pair(smem_u32(tmem_slot), 512); tmem_relinquish_pair(); }
+        else { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
+        pdl_trigger();
+    }
     // barrier set-up, spread over the lanes of warp 0 (one thread doing up to 70 initialisations costs microseconds).
     // Every accumulator block has its own issuing warp: stages are free, and a tile is complete, once all have committed.
     if (threadIdx.x < 32) {
@@ -348,10 +352,6 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
             } else if (i2 < (p.TH >> 1)) v = make_int2((2 * i2 * p.Wp + 2 * j2) | ((2 * i2) << 16), (i2 * hq + j2) * p.k_pad);
         }
         lut[e] = v;
-    }
-    if (warp == PK_MMA_WARP) {
-        if (PAIR) { tmem_alloc_pair(smem_u32(tmem_slot), 512); tmem_relinquish_pair(); }
-        else { tmem_alloc(smem_u32(tmem_slot), 512); tmem_relinquish(); }
     }
     tc_fence_before();
     if (PAIR) cluster_sync();

@@ -176,9 +176,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const StemPara
         mbar_init(wbar, ST_EPI_WARPS);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        // first kernel of a chain: before its successor may start, and before the image and the parameters are read
-        pdl_wait();
-        pdl_trigger();
+        pdl_wait();                        // the image
         lmore = next_segment<POOL>(p, lt, t1, ls);
         ltile = ls.first * p.adv;
         for (int s = 0; s < ST_RAW && lmore; ++s) load_next();
@@ -190,6 +188,9 @@ __global__ void __launch_bounds__(ST_THREADS, 1) conv_stem_kernel(const StemPara
     if (warp == ST_MMA_WARP) {
         tmem_alloc(smem_u32(tmem_slot), 512);
         tmem_relinquish();
+        // first kernel of a chain: before its successor may start
+        pdl_wait();
+        pdl_trigger();
     }
     fence_async_smem();                    // the tensor core reads the zeros
     tc_fence_before();

@@ -100,7 +100,6 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__
                const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_res,
                const __grid_constant__ CUtensorMap tm_id, const TcParams p) {
     extern __shared__ uint8_t smem_raw[];
-    pdl_trigger();
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;          // swizzled tiles need 1024-byte alignment
     uint8_t *smem = smem_raw + (base - raw);
@@ -143,6 +142,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__
     if (warp == MMA_WARP) {
         tmem_alloc(smem_u32(tmem_slot), TMEM_COLS);
         tmem_relinquish();
+        pdl_trigger();
     }
     tc_fence_before();
     __syncthreads();

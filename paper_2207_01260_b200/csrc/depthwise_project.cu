@@ -63,7 +63,6 @@ __global__ void __launch_bounds__(DP_MAX_THREADS + 32, 1)
 depthwise_project_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w, const DpParams p) {
     constexpr int COLS = 2, NW = CH / 2;
     extern __shared__ uint8_t smem_raw[];
-    pdl_trigger();
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *smem = smem_raw + (base - raw);
@@ -83,6 +82,9 @@ depthwise_project_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int warps = (int)(blockDim.x >> 5) - 1;          // of the depthwise half
     if (warp == warps) {
+        tmem_alloc(smem_u32(tmem_slot), (uint32_t)p.tmem_cols);
+        tmem_relinquish();
+        pdl_trigger();
         if (lane == 0) {
             mbar_init(pfull(0), 1); mbar_init(pfull(1), 1);
             for (int s = 0; s < p.wstages; ++s) mbar_init(wfull(s), 1);
@@ -92,8 +94,6 @@ depthwise_project_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         __syncwarp();
-        tmem_alloc(smem_u32(tmem_slot), (uint32_t)p.tmem_cols);
-        tmem_relinquish();
     } else {
         // channels that fill up the last 16 have to be numbers: zeros
         if (p.G & 1)

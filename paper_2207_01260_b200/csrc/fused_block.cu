@@ -67,7 +67,6 @@ __global__ void __launch_bounds__(FB_THREADS, 1)
 fused_block_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_we,
                    const __grid_constant__ CUtensorMap tm_wp, const BlockParams p) {
     extern __shared__ uint8_t smem_raw[];
-    pdl_trigger();
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *smem = smem_raw + (base - raw);
@@ -104,6 +103,7 @@ fused_block_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     if (warp == 1) {
         tmem_alloc(smem_u32(tmem_slot), 512);
         tmem_relinquish();
+        pdl_trigger();
     }
     // the border of the expanded image is the depthwise layer's zero padding: cleared once, only the interior is rewritten
     for (uint32_t e = tid; e < h1_bytes / 16; e += FB_THREADS) ((uint4 *)h1)[e] = make_uint4(0u, 0u, 0u, 0u);

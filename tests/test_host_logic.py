@@ -229,3 +229,23 @@ def test_plan_flags_are_part_of_the_cache_key(cp):
         st = L.cprune_task_plan(1, 8, 8, 8, 8, 3, 3, 1, 1, 1, ctypes.byref(TaskOpts(1, 0, 0, 0, 64)), ctypes.byref(h))
         raise cp.CpruneError(st, "cprune_task_plan")
     assert e.value.status == 1
+
+
+def test_kernels_let_their_successor_start_only_with_their_tensor_memory():
+    # An allocation of tensor memory has no time limit: a later kernel of a launch chain must not be resident, and allocate, while a
+    # block of an earlier one still waits for its columns.  In every kernel that allocates, the trigger follows the allocation
+    # in the same warp.
+    csrc = os.path.join(ROOT, "paper_2207_01260_b200", "csrc")
+    seen = 0
+    for name in sorted(os.listdir(csrc)):
+        if not name.endswith(".cu"):
+            continue
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        for kernel in text.split("__global__")[1:]:
+            allocs = [m.start() for m in re.finditer(r"\btmem_alloc(?:_pair)?\s*\(", kernel)]
+            if allocs:
+                seen += 1
+                triggers = [m.start() for m in re.finditer(r"\bpdl_trigger\s*\(", kernel)]
+                assert len(triggers) == 1 and triggers[0] > max(allocs), name
+                assert kernel.count("}", max(allocs), triggers[0]) <= 1, name
+    assert seen >= 5
