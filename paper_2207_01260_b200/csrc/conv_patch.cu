@@ -354,7 +354,7 @@ conv_patch_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constan
         lut[e] = v;
     }
     tc_fence_before();
-    if (PAIR) cluster_sync();
+    if (PAIR) { __syncwarp(); cluster_sync(); }      // (.aligned: the loops above may have left a warp's threads apart)
     else __syncthreads();
     tc_fence_after();
     // Set-up done.  Only the patch (and residual) loads of warp 0 read what the preceding kernel wrote, and everything
