@@ -96,16 +96,25 @@ def test_one_latency_gated_iteration_of_the_pruning_loop(cp):
 
 
 def _time_task(cp, plan, x, wp, bp, reps=20):
+    # The runs are replayed as a CUDA graph.  Launched one by one they begin on a grid of about 2.06 us: a task then takes 18.6 or 20.6 us
+    # (a ratio of 0.902, whatever the kernel does in between), and the bounds below could not be told from a step of that clock.
+    # In graphs the levels of the three shapes are flat to 4 % (the bound is 15 %), and the cheapest is 0.86, 0.66 and 0.54 of the dearest
+    # (the bound is 0.9).
     y = torch.empty((plan.N, plan.out_h, plan.out_w, plan.k_pad), dtype=torch.bfloat16, device="cuda")
     ws = torch.empty(max(plan.workspace_bytes, 16), dtype=torch.uint8, device="cuda")
     for _ in range(3):
         cp.cprune_task_run(plan, x, wp, bp, None, y, ws)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(reps):
+            cp.cprune_task_run(plan, x, wp, bp, None, y, ws)
+    graph.replay()
     best = 1e9
     for _ in range(3):
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record()
-        for _ in range(reps):
-            cp.cprune_task_run(plan, x, wp, bp, None, y, ws)
+        graph.replay()
         e1.record()
         torch.cuda.synchronize()
         best = min(best, e0.elapsed_time(e1) / reps)
