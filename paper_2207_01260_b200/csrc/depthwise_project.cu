@@ -435,10 +435,8 @@ static cprune_status launch_dp_act(int act, const CUtensorMap *tm, const DpParam
     return launch_dp<R, CH, CPRUNE_ACT_RELU6>(tm, p, t, st);
 }
 
-cprune_status launch_depthwise_project(const cprune_plan *dw, const cprune_plan *proj, const DwProjTiling &t, const void *x, const void *w, const float *b,
-                                       const void *w2, const float *b2, const void *res, void *y, cudaStream_t st) {
+cprune_status encode_depthwise_project(const cprune_plan *dw, const cprune_plan *proj, const DwProjTiling &t, const void *x, const void *w2, CUtensorMap *tm) {
     const cprune_plan_info &i = dw->info;
-    CUtensorMap tm[2];
     {
         const unsigned long long dims[4] = {(unsigned long long)i.c_pad, (unsigned long long)i.W, (unsigned long long)i.H, (unsigned long long)i.N};
         const unsigned long long strides[3] = {(unsigned long long)i.c_pad * 2, (unsigned long long)i.W * i.c_pad * 2, (unsigned long long)i.H * i.W * i.c_pad * 2};
@@ -453,6 +451,12 @@ cprune_status launch_depthwise_project(const cprune_plan *dw, const cprune_plan 
         cprune_status s = encode_tiled_bf16_swz(&tm[1], w2, 2, dims, strides, box, 128, true);
         if (s != CPRUNE_OK) return s;
     }
+    return CPRUNE_OK;
+}
+
+cprune_status launch_depthwise_project(const cprune_plan *dw, const cprune_plan *proj, const DwProjTiling &t, const CUtensorMap *tm, const void *w, const float *b,
+                                       const float *b2, const void *res, void *y, cudaStream_t st) {
+    const cprune_plan_info &i = dw->info;
     DpParams p;
     p.w = (const uint32_t *)w;
     p.b = b; p.b2 = b2;

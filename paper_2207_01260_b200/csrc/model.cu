@@ -13,10 +13,16 @@ struct ModelTensor {
     bool defined = false;
 };
 
+// A depthwise task that runs as one kernel with the next task
+struct ModelPair {
+    DwProjTiling t = {};                 // t.ok: it does
+    CUtensorMap tm[2];
+};
+
 struct cprune_model {
     int N, H, W, C;
     std::vector<cprune_task_desc> tasks;
-    std::vector<DwProjTiling> pairs;     // per task; ok: a depthwise task that runs as one kernel with the next task
+    std::vector<ModelPair> pairs;        // per task
     std::map<int, ModelTensor> tensors;
     char *arena = nullptr;
     size_t arena_bytes = 0;
@@ -64,21 +70,21 @@ static cprune_status enqueue(cprune_model *m, const float *x, float *logits, cud
 // (CPRUNE_CONV_WITH_NEXT) and nothing else reads the tensor between them, which is then not stored.  Filters and biases that the
 // kernel cannot read where they are (off 16 and 4 bytes) leave the tasks separate, and a pass refuses them as the tasks do.
 static void find_pairs(cprune_model *m) {
-    m->pairs.assign(m->tasks.size(), DwProjTiling());
+    m->pairs.assign(m->tasks.size(), ModelPair());
     for (size_t t = 0; t + 1 < m->tasks.size(); ++t) {
         const cprune_task_desc &d = m->tasks[t], &e = m->tasks[t + 1];
         if (d.op != CPRUNE_OP_CONV || e.op != CPRUNE_OP_CONV || d.p0 != CPRUNE_CONV_WITH_NEXT || e.in != d.out || e.res == d.out) continue;
         bool read = false;
         for (size_t u = t + 2; u < m->tasks.size(); ++u) read = read || m->tasks[u].in == d.out || m->tasks[u].res == d.out;
         const bool aligned = !(((uintptr_t)d.w | (uintptr_t)e.w) & 15) && !(((uintptr_t)d.b | (uintptr_t)e.b) & 3);
-        if (!read && aligned) plan_depthwise_project(d.plan, e.plan, &m->pairs[t]);
+        if (!read && aligned) plan_depthwise_project(d.plan, e.plan, &m->pairs[t].t);
     }
 }
 
 // The depthwise task whose result the passes do not store, or -1.
 static int unstored(const cprune_model *m, int id) {
     for (size_t t = 0; t < m->pairs.size(); ++t)
-        if (m->pairs[t].ok && m->tasks[t].out == id) return (int)t;
+        if (m->pairs[t].t.ok && m->tasks[t].out == id) return (int)t;
     return -1;
 }
 
@@ -115,6 +121,12 @@ static cprune_status run_first_task(const cprune_model *m, int path, const float
     return s != CPRUNE_OK ? s : task_run_internal(d.plan, tensor_ptr(m, 0), d.w, d.b, nullptr, y, m->workspace, st, true);
 }
 
+static cprune_status run_pair(const cprune_model *m, size_t t, cudaStream_t st) {
+    const cprune_task_desc &d = m->tasks[t], &e = m->tasks[t + 1];
+    return launch_depthwise_project(d.plan, e.plan, m->pairs[t].t, m->pairs[t].tm, d.w, d.b, e.b, e.res >= 0 ? tensor_ptr(m, e.res) : nullptr,
+                                    tensor_ptr(m, e.out), st);
+}
+
 static cprune_status enqueue_chain(cprune_model *m, const float *x, float *logits, cudaStream_t st) {
     const int path = input_path(m, ((uintptr_t)x & 15) == 0);
     cprune_status s = CPRUNE_OK;
@@ -128,10 +140,8 @@ static cprune_status enqueue_chain(cprune_model *m, const float *x, float *logit
         void *pout = last ? (void *)logits : tensor_ptr(m, d.out);
         switch (d.op) {
             case CPRUNE_OP_CONV:
-                if (m->pairs[t].ok) {
-                    const cprune_task_desc &e = m->tasks[t + 1];
-                    s = launch_depthwise_project(d.plan, e.plan, m->pairs[t], pin, d.w, d.b, e.w, e.b, e.res >= 0 ? tensor_ptr(m, e.res) : nullptr,
-                                                 tensor_ptr(m, e.out), st);
+                if (m->pairs[t].t.ok) {
+                    s = run_pair(m, t, st);
                     ++t;
                 } else if (t == 0 && path != INPUT_CAST) s = run_first_task(m, path, x, pout, st);
                 else s = task_run_internal(d.plan, pin, d.w, d.b, d.res >= 0 ? tensor_ptr(m, d.res) : nullptr, pout, m->workspace, st, false);
@@ -245,7 +255,7 @@ cprune_status cprune_model_create(int N, int H, int W, int C, const cprune_task_
     if (path == INPUT_DIRECT) m->launches += 1 - conv_launches(m->tasks[0].plan);
     find_pairs(m);
     for (size_t t = 0; t < m->pairs.size(); ++t)
-        if (m->pairs[t].ok) m->launches -= conv_launches(m->tasks[t + 1].plan);
+        if (m->pairs[t].t.ok) m->launches -= conv_launches(m->tasks[t + 1].plan);
     size_t off = 0;
     for (auto &kv : m->tensors) {
         kv.second.bytes = (size_t)kv.second.n * kv.second.h * kv.second.w * kv.second.c_pad * 2;
@@ -260,6 +270,11 @@ cprune_status cprune_model_create(int N, int H, int W, int C, const cprune_task_
         delete m;
         return cuda_fail(e, "cudaMalloc(model activations)");
     }
+    for (size_t t = 0; t < m->pairs.size() && st == CPRUNE_OK; ++t) {
+        const cprune_task_desc &d = m->tasks[t];
+        if (m->pairs[t].t.ok) st = encode_depthwise_project(d.plan, m->tasks[t + 1].plan, m->pairs[t].t, tensor_ptr(m, d.in), m->tasks[t + 1].w, m->pairs[t].tm);
+    }
+    if (st != CPRUNE_OK) { cprune_model_destroy(m); return st; }
     *out = m;
     return CPRUNE_OK;
 }
@@ -336,7 +351,7 @@ cprune_status cprune_model_tensor(const cprune_model *m, int id, const void **pt
             // from now on the passes store it; what the last one left out is made up for
             cprune_model *own = const_cast<cprune_model *>(m);
             CPRUNE_CUDA_CHECK(cudaDeviceSynchronize());
-            own->pairs[t].ok = 0;
+            own->pairs[t].t.ok = 0;
             own->launches += conv_launches(m->tasks[t + 1].plan);
             for (auto &g : own->graphs)
                 if (g.exec) { cudaGraphExecDestroy(g.exec); g.exec = nullptr; }

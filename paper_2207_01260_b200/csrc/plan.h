@@ -104,8 +104,10 @@ int depthwise_groups(int c8);
 cprune_status plan_depthwise(cprune_plan *plan);    // fills plan->dw
 // a depthwise task and the 1x1 task that reads its result as one kernel
 bool plan_depthwise_project(const cprune_plan *dw, const cprune_plan *proj, DwProjTiling *out);
-cprune_status launch_depthwise_project(const cprune_plan *dw, const cprune_plan *proj, const DwProjTiling &t, const void *x, const void *w, const float *b,
-                                       const void *w2, const float *b2, const void *res, void *y, cudaStream_t st);
+// (its tensor maps, of the input and of the 1x1 filters: once for all passes of a model, whose buffers stay where they are)
+cprune_status encode_depthwise_project(const cprune_plan *dw, const cprune_plan *proj, const DwProjTiling &t, const void *x, const void *w2, CUtensorMap *tm);
+cprune_status launch_depthwise_project(const cprune_plan *dw, const cprune_plan *proj, const DwProjTiling &t, const CUtensorMap *tm, const void *w, const float *b,
+                                       const float *b2, const void *res, void *y, cudaStream_t st);
 // tcgen05 implicit GEMM
 cprune_status plan_conv_tensor(cprune_plan *plan);  // fills tile fields of plan->info; UNSUPPORTED if not eligible
 cprune_status launch_conv_tensor(cprune_plan *plan, const void *x, const void *w, const float *b, const void *res,
