@@ -343,7 +343,8 @@ cprune_status cprune_model_task_table(const cprune_model *model, cprune_task_ent
 /* Times every entry of the task table on the device: the entry's first subgraph is run `reps` times back to back
  * on the model's own buffers between two CUDA events (after one untimed run), the model's first task as the model runs it, from
  * a float32 image of zeros that takes the place of tensor 0; ms (host, one value per table entry)
- * receives the mean milliseconds per run.  Blocks until the measurements are done.  Feed ms and the counts to
+ * receives the mean milliseconds per run.  Two tasks that the model runs as one kernel (CPRUNE_CONV_WITH_NEXT) are timed as that kernel,
+ * whose time is shared out in proportion to the times of the two by themselves; an entry with subgraphs of both kinds gets their mean.  Blocks until the measurements are done.  Feed ms and the counts to
  * cprune_task_order to get the paper's pruning priority. */
 cprune_status cprune_model_time_tasks(cprune_model *model, int reps, double *ms, void *stream);
 cprune_status cprune_model_destroy(cprune_model *model);

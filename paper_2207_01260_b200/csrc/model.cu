@@ -419,20 +419,45 @@ cprune_status cprune_model_time_tasks(cprune_model *m, int reps, double *ms, voi
     const int path = image_bytes <= t0.bytes ? input_path(m) : (int)INPUT_CAST;
     float *image = (float *)tensor_ptr(m, 0);
     if (path != INPUT_CAST && cudaMemsetAsync(image, 0, image_bytes, st) != cudaSuccess) s = cuda_fail(cudaGetLastError(), "cudaMemsetAsync");
-    for (int j = 0; j < n && s == CPRUNE_OK; ++j) {
-        const bool first = table[j].first_task == 0 && path != INPUT_CAST;
-        const cprune_task_desc &d = m->tasks[table[j].first_task];
-        void *pin = tensor_ptr(m, d.in), *pout = tensor_ptr(m, d.out);
-        const void *res = d.res >= 0 ? tensor_ptr(m, d.res) : nullptr;
+    // mean milliseconds of `run` over reps back-to-back runs, 0 after an error
+    auto time = [&](auto run) -> double {
         for (int r = 0; r <= reps && s == CPRUNE_OK; ++r) {
             if (r == 1 && cudaEventRecord(e0, st) != cudaSuccess) s = CPRUNE_ERR_CUDA;   // run 0 is the untimed one
-            if (s == CPRUNE_OK) s = first ? run_first_task(m, path, image, pout, st) : task_run_internal(d.plan, pin, d.w, d.b, res, pout, m->workspace, st, false);
+            if (s == CPRUNE_OK) s = run();
         }
-        if (s != CPRUNE_OK) break;
         float t = 0.f;
-        if (cudaEventRecord(e1, st) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
-            cudaEventElapsedTime(&t, e0, e1) != cudaSuccess) { s = cuda_fail(cudaGetLastError(), "task timing"); break; }
-        ms[j] = (double)t / reps;
+        if (s == CPRUNE_OK && (cudaEventRecord(e1, st) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+                               cudaEventElapsedTime(&t, e0, e1) != cudaSuccess)) s = cuda_fail(cudaGetLastError(), "task timing");
+        return s == CPRUNE_OK ? (double)t / reps : 0.0;
+    };
+    auto time_task = [&](int t) {
+        const cprune_task_desc &d = m->tasks[t];
+        void *pin = tensor_ptr(m, d.in), *pout = tensor_ptr(m, d.out);
+        const void *res = d.res >= 0 ? tensor_ptr(m, d.res) : nullptr;
+        return time([&] { return t == 0 && path != INPUT_CAST ? run_first_task(m, path, image, pout, st) : task_run_internal(d.plan, pin, d.w, d.b, res, pout, m->workspace, st, false); });
+    };
+    // a pair's kernel, shared out in proportion to the two tasks' own times (the depthwise task first: it stores what the other one reads)
+    std::map<std::pair<const cprune_plan *, const cprune_plan *>, std::pair<double, double>> pair_times;
+    auto time_pair = [&](int t) {
+        auto &p = pair_times[{m->tasks[t].plan, m->tasks[t + 1].plan}];
+        if (p.first == 0.0 && s == CPRUNE_OK) {
+            const double a = time_task(t), b = time_task(t + 1), both = time([&] { return run_pair(m, t, st); });
+            if (s == CPRUNE_OK) p = {both * (a / (a + b)), both * (b / (a + b))};
+        }
+        return p;
+    };
+    for (int j = 0; j < n && s == CPRUNE_OK; ++j) {
+        double sum = 0.0, alone = -1.0;
+        for (int t = 0; t < (int)m->tasks.size() && s == CPRUNE_OK; ++t) {
+            if (m->tasks[t].op != CPRUNE_OP_CONV || m->tasks[t].plan != table[j].plan) continue;
+            if (m->pairs[t].t.ok) sum += time_pair(t).first;
+            else if (t > 0 && m->pairs[t - 1].t.ok) sum += time_pair(t - 1).second;
+            else {
+                if (alone < 0.0) alone = time_task(t);
+                sum += alone;
+            }
+        }
+        ms[j] = sum / table[j].count;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
