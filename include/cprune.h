@@ -288,7 +288,7 @@ cprune_status cprune_block_run(cprune_block *block, const void *x, const void *w
 enum { CPRUNE_OP_CONV = 1, CPRUNE_OP_MAXPOOL = 2, CPRUNE_OP_GAP = 3, CPRUNE_OP_FC = 4, CPRUNE_OP_BLOCK = 5 };
 
 /* CONV, p0 of a depthwise task: the library may run it and the next task, a 1x1 stride-1 conv task that alone reads its result, as one
- * kernel.  The values are those of the two tasks.  The tensor between them is then not stored by a pass: cprune_model_copy_tensor makes it from the
+ * kernel.  The values are those of the two tasks up to the order of the float32 additions.  The tensor between them is then not stored by a pass: cprune_model_copy_tensor makes it from the
  * depthwise task's stored input, and once cprune_model_tensor has handed out its address the two tasks run separately. */
 enum { CPRUNE_CONV_WITH_NEXT = 1 };
 
@@ -319,8 +319,11 @@ cprune_status cprune_model_run(cprune_model *model, const float *x, float *logit
  * x_host unchanged until then.  Two device-side input buffers alternate, so the copy of one call
  * overlaps the kernels of the previous one.  The first call allocates those buffers (cudaMalloc). */
 cprune_status cprune_model_run_host(cprune_model *model, const float *x_host, float *logits_host, void *stream);
-/* Device pointer and element count of tensor `id` of the model (for tests).  ptr may be NULL.  Synchronises the device the first time it
- * gives the address of a tensor that passes have not stored (CPRUNE_CONV_WITH_NEXT). */
+/* Device pointer and element count of tensor `id` of the model (for tests).  ptr may be NULL.  A look-up, with one exception: the first call
+ * that gives the address of a tensor that passes do not store (CPRUNE_CONV_WITH_NEXT) makes the model run the two tasks separately from
+ * then on.  It drops the model's recorded graphs (the next passes record them again), and if a pass has been enqueued it synchronises the
+ * device and makes the tensor of the last pass on a stream of the model's own; so not while a stream is being captured.  Other threads may
+ * enqueue passes meanwhile.  A graph that the caller captured around cprune_model_run before keeps running the one kernel. */
 cprune_status cprune_model_tensor(const cprune_model *model, int id, const void **ptr, int *n, int *h, int *w, int *c_pad);
 /* Copies tensor `id` (bf16 [n][h][w][c_pad]) into dst (device) on `stream`. */
 cprune_status cprune_model_copy_tensor(const cprune_model *model, int id, void *dst, void *stream);

@@ -2,6 +2,7 @@
 // (paper Sec. 3.1: the model is the aggregate of its tasks' programs and is timed as a whole),
 // optionally replayed as a CUDA graph so that one replay costs one host call.
 #include <map>
+#include <mutex>
 #include <vector>
 
 #include "common.cuh"
@@ -21,6 +22,8 @@ struct ModelPair {
 
 struct cprune_model {
     int N, H, W, C;
+    mutable std::mutex mu;               // pairs, graphs and launches change when a tensor's address is handed out, perhaps by another thread
+    bool ran = false;                    // a pass has been enqueued
     std::vector<cprune_task_desc> tasks;
     std::vector<ModelPair> pairs;        // per task
     std::map<int, ModelTensor> tensors;
@@ -309,12 +312,16 @@ static cprune_status run_graph(cprune_model *m, int slot, const float *x, float 
 cprune_status cprune_model_run(cprune_model *m, const float *x, float *logits, int use_graph, void *stream) {
     if (!m || !x || !logits) return CPRUNE_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
+    std::lock_guard<std::mutex> lock(m->mu);
+    m->ran = true;
     if (!use_graph) return enqueue(m, x, logits, st);
     return run_graph(m, 2, x, logits, st);
 }
 
 cprune_status cprune_model_run_host(cprune_model *m, const float *x_host, float *logits_host, void *stream) {
     if (!m || !x_host || !logits_host) return CPRUNE_ERR_INVALID_ARG;
+    std::lock_guard<std::mutex> lock(m->mu);
+    m->ran = true;
     cudaStream_t st = (cudaStream_t)stream;
     const size_t x_bytes = (size_t)m->N * m->H * m->W * m->C * sizeof(float);
     const size_t l_bytes = (size_t)m->N * m->classes * sizeof(float);
@@ -347,17 +354,21 @@ cprune_status cprune_model_tensor(const cprune_model *m, int id, const void **pt
     auto it = m->tensors.find(id);
     if (it == m->tensors.end()) return CPRUNE_ERR_INVALID_ARG;
     if (ptr) {
+        std::lock_guard<std::mutex> lock(m->mu);
         if (const int t = unstored(m, id); t >= 0) {
             // from now on the passes store it; what the last one left out is made up for
             cprune_model *own = const_cast<cprune_model *>(m);
-            CPRUNE_CUDA_CHECK(cudaDeviceSynchronize());
+            if (own->ran) {
+                if (!own->capture_stream) CPRUNE_CUDA_CHECK(cudaStreamCreateWithFlags(&own->capture_stream, cudaStreamNonBlocking));
+                CPRUNE_CUDA_CHECK(cudaDeviceSynchronize());
+                const cprune_status s = store_tensor(m, t, own->capture_stream);
+                if (s != CPRUNE_OK) return s;
+                CPRUNE_CUDA_CHECK(cudaStreamSynchronize(own->capture_stream));
+            }
             own->pairs[t].t.ok = 0;
             own->launches += conv_launches(m->tasks[t + 1].plan);
             for (auto &g : own->graphs)
                 if (g.exec) { cudaGraphExecDestroy(g.exec); g.exec = nullptr; }
-            const cprune_status s = store_tensor(m, t, nullptr);
-            if (s != CPRUNE_OK) return s;
-            CPRUNE_CUDA_CHECK(cudaDeviceSynchronize());
         }
         *ptr = m->arena + it->second.offset;
     }
@@ -372,6 +383,7 @@ cprune_status cprune_model_copy_tensor(const cprune_model *m, int id, void *dst,
     if (!m || !dst) return CPRUNE_ERR_INVALID_ARG;
     auto it = m->tensors.find(id);
     if (it == m->tensors.end()) return CPRUNE_ERR_INVALID_ARG;
+    std::lock_guard<std::mutex> lock(m->mu);
     if (const int t = unstored(m, id); t >= 0) {
         const cprune_status s = store_tensor(m, t, (cudaStream_t)stream);      // (its input is stored)
         if (s != CPRUNE_OK) return s;
@@ -381,7 +393,11 @@ cprune_status cprune_model_copy_tensor(const cprune_model *m, int id, void *dst,
     return CPRUNE_OK;
 }
 
-int cprune_model_launches(const cprune_model *m) { return m ? m->launches : 0; }
+int cprune_model_launches(const cprune_model *m) {
+    if (!m) return 0;
+    std::lock_guard<std::mutex> lock(m->mu);
+    return m->launches;
+}
 
 int cprune_model_reads_image(const cprune_model *m) { return m && input_path(m) == INPUT_DIRECT ? 1 : 0; }
 
@@ -410,6 +426,7 @@ cprune_status cprune_model_time_tasks(cprune_model *m, int reps, double *ms, voi
     s = cprune_model_task_table(m, table.data(), n, &n);
     if (s != CPRUNE_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
+    std::lock_guard<std::mutex> lock(m->mu);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CPRUNE_CUDA_CHECK(cudaEventCreate(&e0));
     CPRUNE_CUDA_CHECK(cudaEventCreate(&e1));
