@@ -27,7 +27,6 @@
 namespace cprune {
 
 constexpr int DP_MAX_THREADS = 480;        // of the depthwise half
-constexpr int DP_MAX_W = 8;                // chunks whose filters can stay
 constexpr int DP_CTRL = 128;
 
 struct DpParams {
@@ -40,7 +39,7 @@ struct DpParams {
     int strips, segs, TR, TH, TW, IH, IW;
     int tiles_h, tiles_w, tiles;
     int dn, dth, dtw;      // the grid's size as images, tile rows, tile columns
-    int patch_bytes, panels, panel_bytes, w_bytes, wstages;      // panels of 64 channels per chunk; filters of one panel; chunks of them kept
+    int patch_bytes, panels, panel_bytes, w_bytes;      // panels of 64 channels per chunk; filters of one panel
     int MT;                // 128-pixel blocks of a tile
     int k16, k_part, k_pad2, act2, tmem_cols;              // k_part: columns of an MMA (at most 256)
     int *status;
@@ -69,14 +68,14 @@ depthwise_project_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
     const uint32_t a_bytes = (uint32_t)p.panels * (uint32_t)p.panel_bytes;
     const uint32_t w0 = base + a_bytes;
     const uint32_t w_chunk = (uint32_t)(p.panels * p.w_bytes);
-    const uint32_t patch0 = w0 + (uint32_t)p.wstages * w_chunk;
+    const uint32_t patch0 = w0 + (uint32_t)p.chunks * w_chunk;
     const uint32_t ctrl0 = patch0 + 2u * (uint32_t)p.patch_bytes;
     uint8_t *ctrl = smem + (ctrl0 - base);
     auto pfull = [&](int s) { return ctrl0 + 8u * s; };
-    auto wfull = [&](int s) { return ctrl0 + 16u + 8u * s; };           // DP_MAX_W
-    const uint32_t afull = ctrl0 + 80u, adone = ctrl0 + 88u;
-    uint32_t *tmem_slot = (uint32_t *)(ctrl + 96);
-    volatile int *abort_flag = (volatile int *)(ctrl + 100);
+    auto wfull = [&](int s) { return ctrl0 + 16u + 8u * s; };           // the filters of a chunk: at most two, and they stay
+    const uint32_t afull = ctrl0 + 32u, adone = ctrl0 + 40u;
+    uint32_t *tmem_slot = (uint32_t *)(ctrl + 48);
+    volatile int *abort_flag = (volatile int *)(ctrl + 52);
     float *bias2_s = (float *)(ctrl + DP_CTRL);
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
@@ -87,7 +86,7 @@ depthwise_project_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
         pdl_trigger();
         if (lane == 0) {
             mbar_init(pfull(0), 1); mbar_init(pfull(1), 1);
-            for (int s = 0; s < p.wstages; ++s) mbar_init(wfull(s), 1);
+            for (int s = 0; s < p.chunks; ++s) mbar_init(wfull(s), 1);
             mbar_init(afull, warps);
             mbar_init(adone, 1);
             *abort_flag = 0;
@@ -132,31 +131,28 @@ depthwise_project_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
             __syncwarp();
             if (++lchunk == p.chunks) { lchunk = 0; advance(n, th, tw); }
         };
-        auto load_w = [&](int stage, int chunk) {
+        for (int s = 0; s < p.chunks && s < steps; ++s) {
             if (elect_one()) {
-                mbar_expect_tx(wfull(stage), (uint32_t)(p.panels * p.k16) * 128u);
+                mbar_expect_tx(wfull(s), (uint32_t)(p.panels * p.k16) * 128u);
                 for (int q = 0; q < p.panels; ++q)
                     for (int k = 0; k < p.k16; k += p.k_part)
-                        tma_load_2d(w0 + (uint32_t)stage * w_chunk + (uint32_t)(q * p.w_bytes + k * 128), &tm_w, wfull(stage), chunk * p.G * 8 + q * 64, k);
+                        tma_load_2d(w0 + (uint32_t)s * w_chunk + (uint32_t)(q * p.w_bytes + k * 128), &tm_w, wfull(s), s * p.G * 8 + q * 64, k);
             }
             __syncwarp();
-        };
-        const bool w_stay = p.wstages >= p.chunks;
-        for (int s = 0; s < p.wstages && s < steps; ++s) load_w(s, s);
+        }
         pdl_wait();
         load_patch(0);
         if (steps > 1) load_patch(1);
         const int ksteps_last = (((p.c2 + 3) >> 2) - (p.chunks - 1) * p.G + 1) >> 1;
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.k_part >> 3) << 17) | (8u << 24);
-        int chunk = 0, ws = 0;
-        uint32_t wphase = 0;
+        int chunk = 0;
         for (int i = 0; i < steps && ok; ++i) {
-            ok = __all_sync(0xffffffffu, mbar_wait(wfull(ws), wphase, abort_flag, p.status));
+            ok = __all_sync(0xffffffffu, mbar_wait(wfull(chunk), 0u, abort_flag, p.status));
             ok = ok && __all_sync(0xffffffffu, mbar_wait(afull, (uint32_t)(i & 1), abort_flag, p.status));
             if (!ok) break;
             tc_fence_after();
             if (i + 2 < steps) load_patch(i & 1);          // (its last patch has been read)
-            const uint32_t a_lo = desc_lo(base), b_lo = desc_lo(w0 + (uint32_t)ws * w_chunk);
+            const uint32_t a_lo = desc_lo(base), b_lo = desc_lo(w0 + (uint32_t)chunk * w_chunk);
             if (elect_one()) {
                 const int ksteps = chunk + 1 == p.chunks ? ksteps_last : p.G >> 1;
                 for (int k = 0; k < ksteps; ++k) {
@@ -169,14 +165,6 @@ depthwise_project_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_
             }
             __syncwarp();
             if (++chunk == p.chunks) chunk = 0;
-            if (w_stay) {
-                if (++ws == p.chunks) ws = 0;
-            } else {
-                // the next filters of this stage, once the MMAs have read these
-                ok = __all_sync(0xffffffffu, mbar_wait(adone, (uint32_t)(i & 1), abort_flag, p.status));
-                if (ok && i + p.wstages < steps) load_w(ws, (i + p.wstages) % p.chunks);
-                if (++ws == p.wstages) { ws = 0; wphase ^= 1u; }
-            }
         }
     } else {
         // ------------------------------------------------------------------ depthwise half and epilogue
@@ -347,7 +335,7 @@ bool plan_depthwise_project(const cprune_plan *dw, const cprune_plan *proj, DwPr
     const double step_cycles = 0.37 * i.R * i.R + 34.3;
     double best = 1e30;
     for (t.MT = 1; t.MT <= 2; ++t.MT)
-        for (t.chunks = 1; t.chunks <= 3; ++t.chunks) {     // (three only to see whether two are the better choice)
+        for (t.chunks = 1; t.chunks <= 3; ++t.chunks) {     // (three, which are not run, only to see whether two are the better choice)
             t.G = (c8 + t.chunks - 1) / t.chunks;
             if (t.chunks > 1) t.G = (t.G + 1) & ~1;        // chunks begin at multiples of 16 channels
             if (t.chunks > 1 && (t.chunks - 1) * t.G >= c8) continue;
@@ -376,33 +364,29 @@ bool plan_depthwise_project(const cprune_plan *dw, const cprune_plan *proj, DwPr
                         if (tiles > 0x3fffffffLL / t.chunks) continue;
                         int warps = (t.lanes * t.strips * t.segs + 31) / 32;
                         if (warps < 4) warps = 4;          // (the four quarters of the accumulator's lanes)
-                        // the filters of all chunks, or of two at a time
-                        for (int stay = 1; stay >= 0; --stay) {
-                            t.wstages = stay ? t.chunks : 2;
-                            if (stay ? t.chunks > DP_MAX_W : t.chunks <= 2) continue;
-                            t.smem_bytes = 1024 + t.panels * (t.panel_bytes + t.wstages * t.w_bytes) + 2 * t.patch_bytes + DP_CTRL + t.k16 * 4;
-                            if (t.smem_bytes > 227 * 1024) continue;
-                            int resident = 227 * 1024 / (t.smem_bytes + 1024);
-                            if (resident > 16 / (warps + 1)) resident = 16 / (warps + 1);                // by registers
-                            if (resident > 512 / t.tmem_cols) resident = 512 / t.tmem_cols;
-                            if (resident < 1) resident = 1;
-                            long long ctas = 148LL * resident;
-                            if (ctas > tiles) ctas = tiles;
-                            const double on_sm = (double)ceil_div(ctas, 148), active = on_sm * warps;
-                            const double share = (double)ceil_div(tiles, ctas) * on_sm * 0.78 + (double)tiles / 148.0 * 0.22;
-                            const double hide = active < 12.0 ? 12.0 / active : 1.0;
-                            const double work = share * t.chunks * warps * (t.TR + i.R + 1.0 + (t.chunks > 1 ? 1.0 : 0.0)) * step_cycles * hide;
-                            const double load = share * t.chunks * t.patch_bytes / 50.0;
-                            const double tail = share / on_sm * (600.0 + t.chunks * 300.0 + t.k16 * 8.0) * (on_sm > 1 ? 0.6 : 1.0);
-                            const double total = (work > load ? work + 0.3 * load : load + 0.3 * work) + tail + active * 200.0;
-                            if (total < best) {
-                                best = total;
-                                *out = t;
-                                out->tiles = (int)tiles;
-                                out->ctas = (int)ctas;
-                                out->threads = (warps + 1) * 32;
-                            }
-                            break;
+                        t.smem_bytes = 1024 + t.panels * (t.panel_bytes + t.chunks * t.w_bytes) + 2 * t.patch_bytes + DP_CTRL + t.k16 * 4;
+                        // (three chunks, which are not run, are compared as if two of them could be kept)
+                        if (t.chunks == 3 && t.smem_bytes > 227 * 1024) t.smem_bytes -= t.panels * t.w_bytes;
+                        if (t.smem_bytes > 227 * 1024) continue;
+                        int resident = 227 * 1024 / (t.smem_bytes + 1024);
+                        if (resident > 16 / (warps + 1)) resident = 16 / (warps + 1);                // by registers
+                        if (resident > 512 / t.tmem_cols) resident = 512 / t.tmem_cols;
+                        if (resident < 1) resident = 1;
+                        long long ctas = 148LL * resident;
+                        if (ctas > tiles) ctas = tiles;
+                        const double on_sm = (double)ceil_div(ctas, 148), active = on_sm * warps;
+                        const double share = (double)ceil_div(tiles, ctas) * on_sm * 0.78 + (double)tiles / 148.0 * 0.22;
+                        const double hide = active < 12.0 ? 12.0 / active : 1.0;
+                        const double work = share * t.chunks * warps * (t.TR + i.R + 1.0 + (t.chunks > 1 ? 1.0 : 0.0)) * step_cycles * hide;
+                        const double load = share * t.chunks * t.patch_bytes / 50.0;
+                        const double tail = share / on_sm * (600.0 + t.chunks * 300.0 + t.k16 * 8.0) * (on_sm > 1 ? 0.6 : 1.0);
+                        const double total = (work > load ? work + 0.3 * load : load + 0.3 * work) + tail + active * 200.0;
+                        if (total < best) {
+                            best = total;
+                            *out = t;
+                            out->tiles = (int)tiles;
+                            out->ctas = (int)ctas;
+                            out->threads = (warps + 1) * 32;
                         }
                     }
             }
@@ -470,7 +454,7 @@ cprune_status launch_depthwise_project(const cprune_plan *dw, const cprune_plan 
     p.dth = (t.ctas - p.dn * t.tiles_h * t.tiles_w) / t.tiles_w;
     p.dtw = t.ctas - (p.dn * t.tiles_h + p.dth) * t.tiles_w;
     p.MT = t.MT;
-    p.patch_bytes = t.patch_bytes; p.panels = t.panels; p.panel_bytes = t.panel_bytes; p.w_bytes = t.w_bytes; p.wstages = t.wstages;
+    p.patch_bytes = t.patch_bytes; p.panels = t.panels; p.panel_bytes = t.panel_bytes; p.w_bytes = t.w_bytes;
     p.k16 = t.k16; p.k_part = t.k_part; p.k_pad2 = proj->info.k_pad; p.act2 = proj->opts.activation; p.tmem_cols = t.tmem_cols;
     p.status = device_status_word();
     if (!p.status) return cuda_fail(cudaGetLastError(), "status word");

@@ -40,7 +40,7 @@ struct DwProjTiling {
     int MT, G, chunks, lanes, panels;        // 128-pixel blocks of a tile, channel groups (of 8) per chunk, chunks, threads per strip, 64-channel panels of a chunk
     int strips, segs, TR, TH, TW, IH, IW;    // tile: column strips x row segments of TR rows; its input patch
     int tiles_h, tiles_w, tiles, ctas, threads;
-    int patch_bytes, panel_bytes, w_bytes, wstages, k16, k_part, tmem_cols, smem_bytes;
+    int patch_bytes, panel_bytes, w_bytes, k16, k_part, tmem_cols, smem_bytes;
 };
 
 // Tiling of the stem kernel that reads a model's float32 image (conv_stem.cu): a step is D conv rows of KF filters each
