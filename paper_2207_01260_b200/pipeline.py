@@ -30,14 +30,15 @@ class PrunedNetwork:
     FUSE_BLOCKS_BATCH = 2
     FUSE_BLOCKS_MAX_PIXELS = 64
 
-    def __init__(self, table: dict, weights: dict, batch: int, device="cuda:0", kernel="auto", fuse_pool=True, fuse_blocks="auto"):
+    def __init__(self, table: dict, weights: dict, batch: int, device="cuda:0", kernel="auto", fuse_pool=True, fuse_blocks="auto",
+                 fuse_pairs="auto"):
         self.table, self.batch, self.device = table, batch, torch.device(device)
         self.kernel = kernel
         self.fuse_pool = fuse_pool
         # A depthwise layer and the 1x1 layer behind it may run as one kernel where the caller leaves the choice to the library, which takes it where
         # it is faster (us per batch, without / with: pruned MobileNetV2 batch 1 145 / 137, 64 506 / 479; MnasNet, 60 % kept, 20 333 / 309).
-        # With True or False every layer but those of the fused blocks is a kernel of its own.
-        self.fuse_pairs = fuse_blocks == "auto" and kernel == "auto"
+        # Where fuse_blocks or kernel is chosen, every layer but those of the fused blocks is a kernel of its own unless fuse_pairs says otherwise.
+        self.fuse_pairs = (fuse_blocks == "auto" and kernel == "auto") if fuse_pairs == "auto" else bool(fuse_pairs)
         self.fuse_pixels = None              # largest image of a fused block (None: whatever the library supports)
         if fuse_blocks == "auto":
             fuse_blocks = batch == self.FUSE_BLOCKS_BATCH

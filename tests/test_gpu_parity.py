@@ -1081,6 +1081,20 @@ def test_depthwise_and_1x1_tasks_as_one_kernel(cp, case):
     assert torch.equal(model.copy_tensor(2), plain.copy_tensor(2))
 
 
+def test_pairs_are_an_option_of_their_own(cp):
+    from paper_2207_01260_b200.pipeline import PrunedNetwork
+    table = wl.mobilenet_v2()
+    table["input"] = (96, 96, 3)
+    weights, x = wl.model_weights(table), _dev(wl.normal_f32(120, 0, (20, 96, 96, 3)))
+    nets = {kw: PrunedNetwork(table, weights, 20, **dict(kw)) for kw in ((), (("fuse_blocks", False),), (("fuse_blocks", False), ("fuse_pairs", True)), (("fuse_pairs", False),))}
+    auto, separate, pairs, off = nets.values()
+    assert auto.model.launches == pairs.model.launches < separate.model.launches == off.model.launches
+    assert torch.equal(pairs.run(x), auto.run(x)) and torch.equal(off.run(x), separate.run(x))
+    ref = separate.run(x)
+    assert torch.linalg.vector_norm(pairs.run(x) - ref) <= 1e-2 * torch.linalg.vector_norm(ref)
+    cp.cprune_poll_device_status()
+
+
 def test_the_address_of_a_tensor_between_two_tasks_beside_passes_of_another_thread(cp):
     import threading
     N, C, H, K = 32, 48, 28, 24
