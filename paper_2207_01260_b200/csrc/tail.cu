@@ -104,11 +104,17 @@ __global__ void __launch_bounds__(256) gap_kernel(const bf16x8 *__restrict__ x, 
 // grid was one wave or two.)  In the networks, before and now: 1280 -> 1000 at 64 images 6.6 and 3.7 us, at 20 images 6.3 and 3.0 us;
 // 512 -> 1000 at 64 images 6.4 and 3.3 us.  By themselves: 25088 -> 4096 at 8 images 119 and 45 us, at 128 images 751 and 297 us.
 // (64 images 14.3 us with one warp per 4 features x 8 images on the FMA pipe.)
-constexpr int FC_WARPS = 8, FC_AHEAD = 5;
-constexpr int FC_NARROW_BLOCKS = 148;     // one per SM
+// Five pieces of 16 features ahead take 116 registers and let two blocks onto an SM, which is what a latency asks for as long as the grid
+// fits; a grid of more blocks than that is bound by how many are resident, and goes three pieces ahead with three blocks to an SM (80
+// registers): where a warp has no more than three pieces, and up to 4096 features where that saves a round of blocks.  us, two blocks to an SM / three /
+// the tiles of 8 features by 32 images that these replaced (in graphs): 64 -> 4096 at 1024 images 88.8 / 55.7 / 69.0, 512 -> 4096 at 1024 images
+// 114 / 80 / 104, 4096 -> 1000 at 256 images (three rounds, or four of two blocks) 27.6 / 24.6 / 34.6; with as many rounds 1280 -> 1000 at 128 images
+// 7.1 / 7.5 / 9.4; 25088 -> 1000 at 512 images, where a block's own stream of loads counts for more, 227 / 260 / 723.
+constexpr int FC_WARPS = 8, FC_AHEAD = 5, FC_AHEAD_MANY = 3, FC_BLOCKS_MANY = 3, FC_FEATURES_MANY = 4096;
+constexpr int FC_SMS = 148;
 
-template <int NT>
-__global__ void __launch_bounds__(FC_WARPS * 32) fc_kernel(const bf16x8 *__restrict__ x, int N, int in8,
+template <int NT, int AHEAD, int BLOCKS>
+__global__ void __launch_bounds__(FC_WARPS * 32, BLOCKS) fc_kernel(const bf16x8 *__restrict__ x, int N, int in8,
                                                            const bf16x8 *__restrict__ w, const float *__restrict__ b, int out,
                                                            int out_pad, int act, int out_is_f32, void *__restrict__ y) {
     __shared__ float part[FC_WARPS][16][NT * 8 + 1];
@@ -124,9 +130,9 @@ __global__ void __launch_bounds__(FC_WARPS * 32) fc_kernel(const bf16x8 *__restr
 #pragma unroll
         for (int f = 0; f < NT; ++f) v[f] = c * 4 + t < in8 && (f == 0 || o0 + f * 8 < out_pad) ? ldg8(wrow + f * 8 * (size_t)in8 + c * 4) : zero;
     };
-    bf16x8 wq[FC_AHEAD][NT];
+    bf16x8 wq[AHEAD][NT];
 #pragma unroll
-    for (int i = 0; i < FC_AHEAD; ++i) load_w(warp + i * FC_WARPS, wq[i]);
+    for (int i = 0; i < AHEAD; ++i) load_w(warp + i * FC_WARPS, wq[i]);
     pdl_wait();
     float acc[NT][4];
 #pragma unroll
@@ -134,10 +140,10 @@ __global__ void __launch_bounds__(FC_WARPS * 32) fc_kernel(const bf16x8 *__restr
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[f][j] = 0.f;
     const int chunks = (in8 + 3) >> 2;
-    for (int c0 = warp; c0 < chunks; c0 += FC_AHEAD * FC_WARPS) {
-        bf16x8 xq[FC_AHEAD][2];
+    for (int c0 = warp; c0 < chunks; c0 += AHEAD * FC_WARPS) {
+        bf16x8 xq[AHEAD][2];
 #pragma unroll
-        for (int i = 0; i < FC_AHEAD; ++i) {
+        for (int i = 0; i < AHEAD; ++i) {
             const int q = (c0 + i * FC_WARPS) * 4 + t;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -146,7 +152,7 @@ __global__ void __launch_bounds__(FC_WARPS * 32) fc_kernel(const bf16x8 *__restr
             }
         }
 #pragma unroll
-        for (int i = 0; i < FC_AHEAD; ++i) {
+        for (int i = 0; i < AHEAD; ++i) {
 #pragma unroll
             for (int f = 0; f < NT; ++f) {
                 float s[4] = {0.f, 0.f, 0.f, 0.f};
@@ -155,7 +161,7 @@ __global__ void __launch_bounds__(FC_WARPS * 32) fc_kernel(const bf16x8 *__restr
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[f][j] += s[j];
             }
-            load_w(c0 + (FC_AHEAD + i) * FC_WARPS, wq[i]);
+            load_w(c0 + (AHEAD + i) * FC_WARPS, wq[i]);
         }
     }
 #pragma unroll
@@ -223,13 +229,16 @@ cprune_status cprune_fc(const void *x, int N, int in, const void *w_packed, cons
     if ((long long)(out_pad >> 3) * ((N + 15) / 16) > 0x7fffffffLL) return CPRUNE_ERR_UNSUPPORTED;
     // One tile of 8 features per SM as long as there are SMs for them: one image 2.4 us.  Beyond that 16 features: 20 images of 1280
     // features 5.0 us with 8 (252 blocks, two or three to an SM) and 3.0 us with 16 (126 blocks).
-    const long long tiles_n = (N + 15) / 16, blocks = (out_pad >> 3) * tiles_n;
-    if (blocks <= FC_NARROW_BLOCKS)
-        CPRUNE_CUDA_CHECK(launch_chained(fc_kernel<1>, dim3((unsigned)blocks), dim3(FC_WARPS * 32), 0, (cudaStream_t)stream,
-                                         (const bf16x8 *)x, N, in8, (const bf16x8 *)w_packed, b_packed, out, out_pad, act, out_is_f32, y));
-    else
-        CPRUNE_CUDA_CHECK(launch_chained(fc_kernel<2>, dim3((unsigned)((out_pad + 15) / 16 * tiles_n)), dim3(FC_WARPS * 32), 0, (cudaStream_t)stream,
-                                         (const bf16x8 *)x, N, in8, (const bf16x8 *)w_packed, b_packed, out, out_pad, act, out_is_f32, y));
+    const long long tiles_n = (N + 15) / 16, narrow = (out_pad >> 3) * tiles_n, wide = (out_pad + 15) / 16 * tiles_n;
+    const bool saves_a_round = ceil_div(wide, FC_BLOCKS_MANY * FC_SMS) < ceil_div(wide, 2 * FC_SMS);
+    const bool many = wide > 2 * FC_SMS && (in <= FC_AHEAD_MANY * FC_WARPS * 32 || (in <= FC_FEATURES_MANY && saves_a_round));
+    auto launch = [&](auto kernel, long long blocks) {
+        return launch_chained(kernel, dim3((unsigned)blocks), dim3(FC_WARPS * 32), 0, (cudaStream_t)stream, (const bf16x8 *)x, N, in8, (const bf16x8 *)w_packed, b_packed, out,
+                              out_pad, act, out_is_f32, y);
+    };
+    if (narrow <= FC_SMS) CPRUNE_CUDA_CHECK(launch(fc_kernel<1, FC_AHEAD, 0>, narrow));
+    else if (many) CPRUNE_CUDA_CHECK(launch(fc_kernel<2, FC_AHEAD_MANY, FC_BLOCKS_MANY>, wide));
+    else CPRUNE_CUDA_CHECK(launch(fc_kernel<2, FC_AHEAD, 0>, wide));
     return CPRUNE_OK;
 }
 

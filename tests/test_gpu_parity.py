@@ -960,6 +960,20 @@ def test_fully_connected_tiles_of_sixteen_features(cp, N, inn, out, act):
             assert torch.equal(y[n0:n1], cp.cprune_fc(xb[n0:n1].contiguous(), inn, *packed, out, act, out_f32=f32))
 
 
+@pytest.mark.parametrize("N,inn,out,act", [(2353, 72, 24, "none"), (2369, 40, 40, "relu"), (700, 768, 130, "none"), (700, 1290, 136, "none"), (1100, 1290, 136, "none"),
+                                           (1100, 4090, 120, "none"), (1100, 4100, 130, "relu")])
+def test_fully_connected_grids_of_many_blocks(cp, N, inn, out, act):
+    # more than 296 blocks of 16 features by 16 images, up to 768 and 4096 input features and beyond, two and three rounds of blocks: the values are those of a small call, bit by bit
+    x, w, b = wl.normal_f32(94, 0, (N, inn)), wl.normal_f32(94, 1, (out, inn), 0.1), wl.normal_f32(94, 2, (out,), 0.05)
+    xb = cp.cprune_cast_input(_dev(x.reshape(N, 1, 1, inn))).reshape(N, -1)
+    packed = cp.cprune_fc_pack(_dev(w), _dev(b))
+    for f32 in (True, False):
+        y = cp.cprune_fc(xb, inn, *packed, out, act, out_f32=f32)
+        for n0 in (0, 16, N // 32 * 16, N // 16 * 16 if N % 16 else N - 16):
+            n1 = min(N, n0 + 16)
+            assert torch.equal(y[n0:n1], cp.cprune_fc(xb[n0:n1].contiguous(), inn, *packed, out, act, out_f32=f32))
+
+
 @pytest.mark.parametrize("hw", [(1, 1), (1, 7), (8, 8), (5, 13), (9, 14), (16, 17)])
 def test_global_average_over_one_and_several_rounds_of_loads(cp, hw):
     x = wl.normal_f32(93, 0, (3, *hw, 270))
