@@ -988,8 +988,9 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
     const int k16 = round_up(i.K, 16);
     const int cblks = g.cblks, ksteps_last = g.ksteps_last, RB = 128;
     const int RS = g.kR * g.kS;
-    double best = 1e30;
-    PatchTiling bt = {};
+    double best_of[2] = {1e30, 1e30};        // of single blocks, of pairs
+    PatchTiling tiling_of[2] = {};
+    double pair_rounds = 1.0;
     const int pairs_allowed = !g.flat && !g.stem && !pool3 && g.kR == 3 && g.kS == 3 ? 1 : 0;
     for (int MT = 1; MT <= 2; ++MT)
       for (int pair = 0; pair <= pairs_allowed; ++pair) {
@@ -1108,15 +1109,36 @@ cprune_status plan_conv_patch(cprune_plan *plan) {
             if (staging_bufs == 1 && !g.flat) t += ((FT + 63) / 64) * 900.0;     // the last tile's stores, one after the other
             // what the estimate leaves out, fitted to 25 shapes: waits across the pair, a cluster's start
             if (pair) t = 1.15 * t + 800.0;
-            if (t < best) {
-                best = t;
-                bt = {MT, TH, FT, tiles_n, tiles_per_img, wstages, resident, acc_bufs, staging_bufs, patch_bytes, TW, tiles_w, step_h, step_w, org, pstages, dense, stage_bytes, dense_pitch, ipt, wgroup, pair};
+            if (t < best_of[pair]) {
+                best_of[pair] = t;
+                if (pair) pair_rounds = waves;
+                tiling_of[pair] = {MT, TH, FT, tiles_n, tiles_per_img, wstages, resident, acc_bufs, staging_bufs, patch_bytes, TW, tiles_w, step_h, step_w, org, pstages, dense, stage_bytes, dense_pitch, ipt, wgroup, pair};
             }
             if (!pair && (resident || wgroup == g.kS)) break;      // the deepest patch ring beside which the filters fit
           }
         }
       }
     }
+    // Where pairs begin.  The estimate says by how much they gain to within 6 %, and what it leaves out weighs most where a block goes
+    // through few channel blocks, all its rounds together: pairs that go through one or two have to promise 4 %, through three 5 %, and filters that could
+    // stay, 97 of them and more, 3 %.  Not so where a single block would take its filters tap by tap (256 of them, for instance): by themselves
+    // such tasks say the same, but in networks they are the slower ones, 102 -> 256 14x14 with a residual, batch 40, by 6 us a task.
+    // By themselves, in graphs, both ways in turn, 734 shapes that the cheaper estimate alone gave to pairs (16 to 512 channels and filters, 4x4 to 56x56, batch 1
+    // to 128): 60 took more than 5 % longer than as single blocks, of those that are left 28; none that gains 2 % is given up.  128 -> 179 12x12, batch 64,
+    // 10.4 us single and 11.2 as pairs; 60 -> 152 56x56, batch 128, 70 and 83; 131 -> 203 28x28, batch 64, 35.1 and 29.6.  Networks (us, single blocks
+    // everywhere / the estimate alone / this line): ResNet-18 with 50 % kept, batch 20, 182.9 / 189.6 / 183.2; with 60 %, batch 48, 289.5 / 279.0 / 276.7, block outputs
+    // pruned too 258.3 / 258.1 / 254.3; with 70 %, batch 64, 324.1 / 313.8 / 314.6.  256 -> 179 14x14, batch 64, stays a pair: by itself 16.1 us instead of
+    // 15.1, in that network 1.3 us less.
+    const PatchTiling &single = tiling_of[0], &paired = tiling_of[1];
+    const double blocks_through = pair_rounds * cblks;
+    double promise = 1.0;
+    if (single.wgroup == g.kS && paired.FT > 96) {      // (79 of 79 pairs of up to 96 filters gain)
+        if (paired.resident) promise = 0.97;
+        if (blocks_through <= 3) promise = blocks_through <= 2 ? 0.96 : 0.95;
+    }
+    const bool pairs = best_of[0] >= 1e30 || best_of[1] < best_of[0] * promise;
+    const double best = best_of[pairs ? 1 : 0];
+    const PatchTiling bt = tiling_of[pairs ? 1 : 0];
     if (best >= 1e30) return CPRUNE_ERR_UNSUPPORTED;
     // share of accumulator rows that hold real pixels; below one half the im2col kernel is the better choice
     const long long tiles_m = bt.ipt ? ceil_div(g.vN, bt.ipt) : (long long)g.vN * bt.tiles_per_img;

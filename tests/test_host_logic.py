@@ -249,3 +249,13 @@ def test_kernels_let_their_successor_start_only_with_their_tensor_memory():
                 assert len(triggers) == 1 and triggers[0] > max(allocs), name
                 assert kernel.count("}", max(allocs), triggers[0]) <= 1, name
     assert seen >= 5
+
+
+def test_pairs_of_thread_blocks_have_to_promise_enough(cp):
+    # tiles of a pair have multiples of 32 filters, those of single blocks of 16.  Few channel blocks in all, or resident filters, and a gain that the
+    # estimate puts at 1 to 4 %: single blocks.  The last three promise more: pairs.
+    for (N, C, hw, K, res), tile_n in [((64, 153, 14, 133, False), 144), ((48, 156, 16, 99, False), 112), ((128, 64, 12, 135, False), 144),
+                                       ((64, 50, 16, 136, False), 144), ((128, 148, 8, 134, True), 144), ((64, 131, 28, 203, False), 224),
+                                       ((41, 40, 16, 140, False), 160), ((41, 72, 12, 203, True), 224)]:
+        plan = cp.cprune_task_plan(N, C, hw, hw, K, 3, 3, 1, 1, 1, "relu", res)
+        assert plan.variant == 1 and plan.tile_n == tile_n, (N, C, hw, K, plan.tile_n)
